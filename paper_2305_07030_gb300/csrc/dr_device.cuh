@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "f64_soft.cuh"
 #include "fe2_internal.h"
 
 namespace fe2 {
@@ -15,8 +16,9 @@ namespace fe2 {
 __device__ __forceinline__ double dadd(double a, double b) { return __dadd_rn(a, b); }
 __device__ __forceinline__ double dsub(double a, double b) { return __dsub_rn(a, b); }
 __device__ __forceinline__ double dmul(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ double ddiv(double a, double b) { return __ddiv_rn(a, b); }
-__device__ __forceinline__ double dsqrt(double a) { return __dsqrt_rn(a); }
+// division and square root off the FP64 pipe (same bits as __ddiv_rn, __dsqrt_rn)
+__device__ __forceinline__ double ddiv(double a, double b) { return f64_div(a, b); }
+__device__ __forceinline__ double dsqrt(double a) { return f64_sqrt(a); }
 
 // Sum over the CTA; every thread gets the total. `red` holds >= 32 doubles and
 // must not be in use by another reduction until the next barrier.
