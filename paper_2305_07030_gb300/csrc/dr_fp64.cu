@@ -21,7 +21,7 @@ template <bool SM>
 __global__ void __launch_bounds__(512) dr_fp64_kernel(DevMesh M, DevState S, DevResults O,
                                                        SolveParams P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ double red[32];
+    __shared__ double red[9 * kStressWarps];
     __shared__ int s_item;
     for (;;) {
         if (threadIdx.x == 0) s_item = atomicAdd(P.counter, 1);

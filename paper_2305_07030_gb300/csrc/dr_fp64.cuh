@@ -46,6 +46,7 @@ __device__ __forceinline__ void gather_table_fp64(const DevMesh &M, const RveDes
     }
 }
 
+// `red` holds 9 * kStressWarps doubles.
 // ET: element forces through the per-element table S.tf (batched path);
 // otherwise every directed edge is evaluated by gather_force_fp64.
 template <bool SM, bool ET>
@@ -212,7 +213,9 @@ __device__ void solve_rve_fp64(const DevMesh &M, const DevState &S, const DevRes
         if (it >= P.max_iter) { status = RVE_MAXITER; break; }
     }
     __syncthreads();
-    rve_stress(M, R, F, x0, x1, x2, O.sigma + 9 * (int64_t)p, red);
+    stress_partials(M, R, x0, x1, x2, 0, 1, red);
+    __syncthreads();
+    stress_total(R, F, red, O.sigma + 9 * (int64_t)p);
     if (threadIdx.x == 0) {
         O.iters[p] = it;
         O.rel_res[p] = f_ref > 0.0 ? r / f_ref : (r > 0.0 ? INFINITY : 0.0);

@@ -87,17 +87,20 @@ F64_FN uint32_t f64_recip(uint64_t mb) {
     return (uint32_t)((int32_t)v0 + (int32_t)(((int64_t)(int32_t)v0 * eh) >> 42)) - 1u;
 }
 
-// RN(a / b).
+// RN(a / b) from v = 2^83 / mb - d for b's significand mb; d < 2.1 as
+// f64_recip gives it, or d < 8 with WIDE (f64_sqrt_recip).
 //
 // With A the numerator's significand, doubled when it is below mb, the
 // quotient's significand is A 2^52 / mb in [2^52, 2^53). Digits from v:
-//   q1 = A 2^29 / mb, short by d (d < 2.1 from v, 0.5 from the truncation of
-//        A, 1 from that of the product: < 3.6): remainder R1 < 3.6 mb < 2^55;
-//   q2 = R1 2^23 / mb, short by < 1.1: R2 < 1.1 mb;
-// so the rounded significand is q1 2^23 + q2, plus one when 2 R2 > mb (2 R2 =
-// mb never: mb would be a multiple of 2^53). All remainders fit in 64 bits and
-// are exact; the products are taken modulo 2^64.
-F64_FN double f64_div(double a, double b) {
+//   q1 = A 2^29 / mb, short by d (from v), 0.5 (truncation of A) and 1 (of the
+//        product): remainder R1 < 3.6 mb < 2^55, WIDE 9.5 mb < 2^57;
+//   q2 = R1 2^23 / mb, short by < 1.1, WIDE < 1.7: R2 < 1.1 mb, WIDE 1.7 mb;
+// so the rounded significand is q1 2^23 + q2, plus one when 2 R2 > mb, plus one
+// when 2 R2 > 3 mb (WIDE only). (2 R2 = mb never: mb would be a multiple of
+// 2^53.) All remainders fit in 64 bits and are exact; the products are taken
+// modulo 2^64.
+template <bool WIDE>
+F64_FN double f64_div_v(double a, double b, uint32_t v) {
     const uint64_t ua = f64_bits(a), ub = f64_bits(b);
     const int ea = (int)(ua >> 52) & 0x7ff, eb = (int)(ub >> 52) & 0x7ff;
     const uint64_t ma = (ua & kF64Man) | kF64One, mb = (ub & kF64Man) | kF64One;
@@ -106,14 +109,19 @@ F64_FN double f64_div(double a, double b) {
     if ((unsigned)(ea - 1) >= 2046u || (unsigned)(eb - 1) >= 2046u || (unsigned)e >= 2045u)
         return f64_hw_div(a, b);
     const uint64_t A = low ? ma << 1 : ma;
-    const uint32_t v = f64_recip(mb);
     const uint32_t q1 = f64_mulhi((uint32_t)(A >> 22), v);
     const uint64_t R1 = (A << 29) - (uint64_t)q1 * mb;
-    const uint32_t q2 = f64_mulhi((uint32_t)(R1 >> 24), v) >> 4;
+    const uint32_t q2 = WIDE ? f64_mulhi((uint32_t)(R1 >> 25), v) >> 3 : f64_mulhi((uint32_t)(R1 >> 24), v) >> 4;
     const uint64_t R2 = ((R1 << 23) - (uint64_t)q2 * mb) << 1;
-    const uint64_t Q = ((uint64_t)q1 << 23) + q2 + (R2 > mb);
+    const uint64_t Q = ((uint64_t)q1 << 23) + q2 + (R2 > mb) + (WIDE ? (R2 > 3 * mb) : 0);
     return f64_from(((ua ^ ub) & 0x8000000000000000ull) | (((uint64_t)e << 52) + Q));
 }
+
+// the reciprocal digit estimate of a divisor, for f64_div_v<false>
+F64_FN uint32_t f64_recip_of(double b) { return f64_recip((f64_bits(b) & kF64Man) | kF64One); }
+
+// RN(a / b)
+F64_FN double f64_div(double a, double b) { return f64_div_v<false>(a, b, f64_recip_of(b)); }
 
 // RN(sqrt(a)).
 //
@@ -127,10 +135,17 @@ F64_FN double f64_div(double a, double b) {
 // R2 = m 2^52 - Q^2, Q = q1 2^23 + q2, is exact modulo 2^64, and the root
 // rounds to Q + k, k = -1 .. 2, where (Q + k - 1/2)^2 < m 2^52 <
 // (Q + k + 1/2)^2 (never equal: the square of a half-integer is no integer).
-F64_FN double f64_sqrt(double a) {
+//
+// vr receives v: the root's significand is at most 2^53 - 1 (m <= 2^54 - 2), so
+// v is also 2^83 / (the root's significand) - d for f64_div_v<true>.
+F64_FN double f64_sqrt_recip(double a, uint32_t &vr) {
     const uint64_t ua = f64_bits(a);
     const int ea = (int)(ua >> 52);  // the sign bit makes it >= 2048
-    if ((unsigned)(ea - 1) >= 2046u) return f64_hw_sqrt(a);
+    if ((unsigned)(ea - 1) >= 2046u) {
+        const double r = f64_hw_sqrt(a);
+        vr = f64_recip_of(r);
+        return r;
+    }
     const int odd = (ea & 1) ^ 1;  // biased exponent even: true exponent odd
     const uint64_t m = ((ua & kF64Man) | kF64One) << odd;
     const int e = (ea - 1023 - odd) >> 1;
@@ -140,6 +155,7 @@ F64_FN double f64_sqrt(double a) {
     const uint32_t w = f64_mulhi(v0, v0);                             // 2^30 / mu
     const int32_t d = (int32_t)(0x10000000u - f64_mulhi(w, mh));      // 2^28 (1 - mu v0^2)
     const uint32_t v = (uint32_t)((int32_t)v0 + (int32_t)(((int64_t)(int32_t)v0 * d) >> 29)) - 6u;
+    vr = v;
     const uint32_t q1 = f64_mulhi(mh, v);                             // 2^29 sqrt(mu)
     const uint64_t R1 = (m << 6) - (uint64_t)q1 * q1;
     const uint32_t q2 = f64_mulhi((uint32_t)(R1 >> 3), v) >> 3;
@@ -148,6 +164,10 @@ F64_FN double f64_sqrt(double a) {
     const int64_t s = (int64_t)Q;
     const int k = (R2 > -s) + (R2 > s) + (R2 > 3 * s + 2) - 1;
     return f64_from(((uint64_t)(e + 1022) << 52) + Q + (uint64_t)(int64_t)k);
+}
+F64_FN double f64_sqrt(double a) {
+    uint32_t v;
+    return f64_sqrt_recip(a, v);
 }
 
 }  // namespace fe2

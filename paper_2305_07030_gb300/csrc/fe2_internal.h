@@ -42,9 +42,26 @@ struct RveDesc {
     int32_t part_elem_max;  // FP32 kernel: most table elements of one part
     int32_t part_slot_max;  // FP32 kernel: most row slots (ELL, 32-node slabs) of one part
     int64_t slot0;          // FP64 cluster kernel: first element slot of this RVE
-    int32_t part_fslot_max; // FP64 cluster kernel: most element slots of one part
+    // FP64 cluster kernel: its parts (a multiple of n_parts), the largest of
+    // them, and their most free nodes, element slots and row entries
+    int32_t fp_parts;
+    int32_t fp_part_max;
+    int32_t fp_free_max;
+    int32_t fp_slot_max;
+    int32_t fp_row_max;
     int32_t pad_;
 };
+
+// Launch shape of the FP64 cluster kernel: CTAs per cluster, capacities of one
+// CTA, and what it keeps in shared memory beside the positions (tsm: element
+// table and rows, ssm: the own free nodes' state).
+struct Fp64Shape {
+    int parts, part_max, free_max, slot_max, row_max;
+    bool tsm, ssm;
+};
+// doubles per free node of that state: velocity, displacement, reference
+// position, mass, damping factor, the mass's division estimate
+constexpr int kStateDoubles = 12;
 
 // Read-only, create-time arrays.
 struct DevMesh {
@@ -69,9 +86,16 @@ struct DevMesh {
                                   // (caller orientation)
     const int4 *fp_slot;          // FP64 cluster kernel, per element slot: (element,
                                   // first end, second end, 0), ends as (part << 16 | index)
-    const int32_t *fp_csr_slot;   // per CSR entry of a free node: part-relative slot << 1
-                                  // | 1 when the node is the element's second end
+    const int32_t *fp_csr_slot;   // per row entry of a free node, in FP64 order from csr0:
+                                  // part-relative slot << 1 | 1 when the node is the
+                                  // element's second end
     const int32_t *fp_part_slot;  // per RVE kMaxParts+1 part slot offsets (from slot0)
+    const int32_t *fp_node;       // FP64 order: RVE-local ids part by part, a part's free
+                                  // nodes first, then its fixed ones
+    const int32_t *fp_part_off;   // per RVE 2*(kMaxParts+1): the parts' first entries of
+                                  // fp_node, and of the free nodes counted alone
+    const int32_t *fp_row;        // per RVE n_free + 1 (from rp0): row offsets into
+                                  // fp_csr_slot, free nodes in FP64 order
 };
 
 // Mutable solver state (device).
@@ -89,8 +113,8 @@ struct DevState {
     float2 *sa;                   //   (v, a.x) and (a.y, a.z)
     double *gp, *fdp;             // FP64 energy check: previous internal and damping
                                   // force per free DOF [3][N]
-    double *ualt;                 // FP64 cluster kernel: displacement of odd evaluations,
-                                  // per RVE [3][n] at 3 node0
+    double *ualt;                 // FP64 cluster kernel: displacements of the last three
+                                  // evaluations, per RVE [3][3][n] at 9 node0, FP64 order
     double *fpt;                  // FP64 cluster kernel: element forces [3][part slots]
                                   // when the table does not fit in shared memory
 };
@@ -159,16 +183,13 @@ size_t mixed_fp32_smem(int part_cap, int free_cap, int elem_cap, int slot_cap, s
 size_t mixed_lead_smem(int part_cap, int free_cap, int elem_cap, int slot_cap, size_t limit);
 // Whether a launch with `smem` bytes uses the shared-memory element table.
 bool mixed_staged(int lead, size_t smem, int part_cap);
-// FP64 cluster kernel (dr_fp64_cluster.cu): dynamic shared memory (two
-// position buffers, and the element table when tsm), launch, occupancy.
-// ssm: the own free nodes' state (displacement, velocity, acceleration, mass)
-// in shared memory as well.
-size_t fp64_cluster_smem(int part_cap, int free_cap, int slot_cap, bool tsm, bool ssm);
+// FP64 cluster kernel (dr_fp64_cluster.cu): dynamic shared memory, launch,
+// co-resident clusters. `block`: threads per CTA, the last warp of which tests
+// the residual.
+size_t fp64_cluster_smem(const Fp64Shape &sp);
 int launch_dr_fp64_cluster(const DevMesh &m, const DevState &s, const DevResults &r, const SolveParams &p,
-                           int clusters, int parts, int block, int part_cap, int free_cap, int slot_cap,
-                           bool tsm, bool ssm, void *stream);
-int occupancy_dr_fp64_cluster(int parts, int block, int part_cap, int free_cap, int slot_cap, bool tsm,
-                              bool ssm);
+                           int clusters, int block, const Fp64Shape &sp, void *stream);
+int occupancy_dr_fp64_cluster(int block, const Fp64Shape &sp);
 // Shared memory per node of a kernel without its element table.
 size_t mixed_plain_node_bytes(int lead);
 // Resident CTAs per SM (FP64) / co-resident clusters (mixed) for a launch shape.

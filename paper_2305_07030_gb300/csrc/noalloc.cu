@@ -100,7 +100,7 @@ __device__ __forceinline__ int block_excl_scan(int v, int *tmp) {
 
 __global__ void __launch_bounds__(kNaThreads) k_noalloc_solve(NaArgs A, SolveParams P, unsigned char *scr) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ double red[32];
+    __shared__ double red[9 * kStressWarps];
     __shared__ int tmp[32];
     __shared__ int err, nfree_s;
     RveDesc *rve = reinterpret_cast<RveDesc *>(scr + kOffRve);

@@ -68,9 +68,7 @@ struct SizeClass {
     int block_fp32 = 0;
     int smem_positions = 1;     // FP64: positions in shared memory
     bool fp64_cluster = false;  // FP64: one cluster of `parts` CTAs per RVE
-    bool fp64_tsm = false;      // FP64 cluster: element table in shared memory
-    bool fp64_ssm = false;      // FP64 cluster: free-node state in shared memory
-    int fslot_max = 0;          // FP64 cluster: most element slots of one part
+    Fp64Shape fp = {};          // FP64 cluster: launch shape
     size_t smem_bytes = 0;      // dynamic shared memory per CTA
     int part_max = 0;           // mixed: largest part (nodes)
     int free_max = 0;           // mixed: most free nodes in one part
@@ -125,7 +123,7 @@ struct fe2_batch {
     DevBuf<double> d_X, d_mass, d_EA_csr, d_L_csr, d_el_EA, d_el_L;
     DevBuf<float> d_Xh, d_Xl, d_imh, d_iml;
     DevBuf<int32_t> d_rowptr, d_col, d_col_part, d_part_off, d_el_a, d_el_b, d_csr_el;
-    DevBuf<int32_t> d_fp_csr_slot, d_fp_part_slot;
+    DevBuf<int32_t> d_fp_csr_slot, d_fp_part_slot, d_fp_node, d_fp_part_off, d_fp_row;
     DevBuf<int4> d_fp_slot;
     DevBuf<double> d_ualt, d_fpt;
     DevBuf<float2> d_eaf, d_eaf_lo, d_sa;
@@ -198,6 +196,9 @@ struct fe2_batch {
         m.fp_slot = d_fp_slot.p;
         m.fp_csr_slot = d_fp_csr_slot.p;
         m.fp_part_slot = d_fp_part_slot.p;
+        m.fp_node = d_fp_node.p;
+        m.fp_part_off = d_fp_part_off.p;
+        m.fp_row = d_fp_row.p;
         return m;
     }
     DevState state() const {
@@ -228,7 +229,7 @@ struct fe2_batch {
         d_rve.release(); d_X.release(); d_mass.release(); d_EA_csr.release(); d_L_csr.release();
         d_el_EA.release(); d_el_L.release(); d_Xh.release(); d_Xl.release(); d_imh.release();
         d_iml.release(); d_rowptr.release(); d_col.release(); d_col_part.release();
-        d_part_off.release(); d_el_a.release(); d_el_b.release(); d_csr_el.release(); d_fp_csr_slot.release(); d_fp_part_slot.release(); d_fp_slot.release(); d_ualt.release(); d_fpt.release(); d_tf.release(); d_sv.release(); d_sa.release(); d_eaf.release();
+        d_part_off.release(); d_el_a.release(); d_el_b.release(); d_csr_el.release(); d_fp_csr_slot.release(); d_fp_part_slot.release(); d_fp_node.release(); d_fp_part_off.release(); d_fp_row.release(); d_fp_slot.release(); d_ualt.release(); d_fpt.release(); d_tf.release(); d_sv.release(); d_sa.release(); d_eaf.release();
         d_eaf_lo.release(); d_dh.release(); d_dl.release(); d_u.release(); d_v.release(); d_a.release(); d_xg.release();
         d_uh.release(); d_ul.release(); d_vh.release(); d_vl.release(); d_ah.release();
         d_al.release(); d_fg.release(); d_F.release(); d_sigma.release(); d_rel.release();
@@ -365,51 +366,48 @@ void build_classes(const std::vector<RveDesc> &rve, const std::vector<int32_t> &
     });
     const size_t cap = smem_optin - 16384;  // room for static shared memory
     if (precision == FE2_PREC_FP64) {
-        // RVEs of several parts run on a cluster (one part per CTA) when its
-        // position buffers fit; classes by (parts, table in shared memory).
-        // FE2_FP64_CLUSTER=0 keeps every RVE on the single-CTA kernel.
+        // RVEs run on a cluster (one FP64 part per CTA) when its position
+        // buffers fit, else on the single-CTA kernel; classes by parts and by
+        // what fits in shared memory. FE2_FP64_CLUSTER=0 keeps every RVE on
+        // the single-CTA kernel.
         const bool clusters = env_int("FE2_FP64_CLUSTER", 1) != 0;
-        auto on_cluster = [&](const RveDesc &R) {
-            return clusters && R.n_parts >= 2 && fp64_cluster_smem(R.part_max, 0, 0, false, false) <= cap;
+        auto shape_of = [&](const RveDesc &R) {
+            return Fp64Shape{R.fp_parts, R.fp_part_max, R.fp_free_max, R.fp_slot_max, R.fp_row_max, false, false};
         };
-        // shared-memory variant of an RVE: the element table first, then the
-        // free-node state, as far as they fit
-        auto variant = [&](int pm, int fm, int sm, bool &tsm, bool &ssm) {
-            const bool opts[4][2] = {{true, true}, {true, false}, {false, true}, {false, false}};
-            for (const auto &o : opts)
-                if (fp64_cluster_smem(pm, fm, sm, o[0], o[1]) <= cap) {
-                    tsm = o[0];
-                    ssm = o[1];
-                    return;
-                }
-        };
+        auto on_cluster = [&](const RveDesc &R) { return clusters && fp64_cluster_smem(shape_of(R)) <= cap; };
         for (int32_t p : order) {
-            const RveDesc &R = rve[p];
-            if (!on_cluster(R)) continue;
-            bool tsm = false, ssm = false;
-            variant(R.part_max, part_free_max[p], R.part_fslot_max, tsm, ssm);
+            if (!on_cluster(rve[p])) continue;
+            // shared-memory variant of an RVE: the element table first, then
+            // the free-node state, as far as they fit
+            Fp64Shape one = shape_of(rve[p]);
+            const bool opts[4][2] = {{true, true}, {true, false}, {false, true}, {false, false}};
+            for (const auto &o : opts) {
+                one.tsm = o[0];
+                one.ssm = o[1];
+                if (fp64_cluster_smem(one) <= cap) break;
+            }
             SizeClass *c = nullptr;
-            for (auto &k : out)
-                if (k.parts == R.n_parts && k.fp64_tsm == tsm && k.fp64_ssm == ssm &&
-                    fp64_cluster_smem(std::max(k.part_max, R.part_max), std::max(k.free_max, part_free_max[p]),
-                                      std::max(k.fslot_max, R.part_fslot_max), tsm, ssm) <= cap) {
-                    c = &k;
-                    break;
-                }
+            for (auto &k : out) {
+                if (k.fp.parts != one.parts || k.fp.tsm != one.tsm || k.fp.ssm != one.ssm) continue;
+                Fp64Shape t = one;
+                t.part_max = std::max(t.part_max, k.fp.part_max);
+                t.free_max = std::max(t.free_max, k.fp.free_max);
+                t.slot_max = std::max(t.slot_max, k.fp.slot_max);
+                t.row_max = std::max(t.row_max, k.fp.row_max);
+                if (fp64_cluster_smem(t) > cap) continue;
+                k.fp = t;
+                c = &k;
+                break;
+            }
             if (!c) {
                 out.emplace_back();
                 c = &out.back();
-                c->parts = R.n_parts;
                 c->fp64_cluster = true;
-                c->fp64_tsm = tsm;
-                c->fp64_ssm = ssm;
                 c->smem_positions = 0;
+                c->parts = one.parts;
+                c->fp = one;
             }
             c->rves.push_back(p);
-            c->part_max = std::max(c->part_max, R.part_max);
-            c->free_max = std::max(c->free_max, part_free_max[p]);
-            c->fslot_max = std::max(c->fslot_max, R.part_fslot_max);
-            c->smem_bytes = fp64_cluster_smem(c->part_max, c->free_max, c->fslot_max, c->fp64_tsm, c->fp64_ssm);
         }
         std::stable_sort(out.begin(), out.end(), [](const SizeClass &a, const SizeClass &b) {
             return a.parts > b.parts;
@@ -585,9 +583,79 @@ struct HostLayout {
     // the part's free nodes (first use in row order); per slot (element,
     // first end, second end) with ends as (part << 16 | index in part); per
     // CSR entry of a free node its slot << 1 | 1 when the node is the second
-    // end; per RVE the parts' slot offsets (relative to RveDesc::slot0)
-    std::vector<int32_t> fpSlot, fpCsrSlot, fpPartSlot;
+    // end; per RVE the parts' slot offsets (relative to RveDesc::slot0). The
+    // FP64 order of the nodes, the parts' offsets in it, and the free nodes'
+    // row offsets (DevMesh::fp_node, fp_part_off, fp_row)
+    std::vector<int32_t> fpSlot, fpCsrSlot, fpPartSlot, fpNode, fpPartOff, fpRow;
 };
+
+// The FP64 cluster kernel's part of the layout (see HostLayout): its parts are
+// the mixed solver's.
+void build_fp64_parts(const int64_t *elem_off, HostLayout &L) {
+    const int32_t n_rve = (int32_t)L.rve.size();
+    for (int32_t p = 0; p < n_rve; ++p) {
+        RveDesc &R = L.rve[p];
+        const int n = R.n_nodes, nf = R.n_free, C = R.n_parts;
+        const int32_t *pf = L.part.data() + (size_t)p * 2 * (kMaxParts + 1), *pg = pf + (kMaxParts + 1);
+        std::vector<std::vector<int>> fr(C), fx(C);  // per part: free and fixed nodes
+        for (int r = 0; r < C; ++r) {
+            for (int k = pf[r]; k < pf[r + 1]; ++k) fr[r].push_back(k);
+            for (int k = pg[r]; k < pg[r + 1]; ++k) fx[r].push_back(nf + k);
+        }
+        int32_t *node = L.fpNode.data() + R.node0, *frow = L.fpRow.data() + R.rp0;
+        int32_t *off = L.fpPartOff.data() + (size_t)p * 2 * (kMaxParts + 1), *ffree = off + (kMaxParts + 1);
+        int32_t *ps = L.fpPartSlot.data() + (size_t)p * (kMaxParts + 1);
+        std::vector<int32_t> ref(n);  // (part << 16 | index in part)
+        int32_t at = 0, nfree = 0;
+        for (int r = 0; r < C; ++r) {
+            off[r] = at;
+            ffree[r] = nfree;
+            nfree += (int32_t)fr[r].size();
+            int32_t k = 0;
+            for (const auto *ids : {&fr[r], &fx[r]})
+                for (int i : *ids) {
+                    ref[i] = (r << 16) | k++;
+                    node[at++] = i;
+                }
+        }
+        for (int r = C; r <= kMaxParts; ++r) {
+            off[r] = at;
+            ffree[r] = nfree;
+        }
+        R.slot0 = (int64_t)(L.fpSlot.size() / 4);
+        R.fp_parts = C;
+        R.fp_part_max = R.fp_free_max = R.fp_slot_max = R.fp_row_max = 0;
+        std::vector<int32_t> slot_of(R.n_elems, -1);
+        const int32_t *row = L.row.data() + R.rp0;
+        const int64_t e0 = elem_off[p];
+        int32_t ns = 0, pos = 0, x = 0;
+        for (int r = 0; r < C; ++r) {
+            ps[r] = ns;
+            const int32_t first = ns, pos0 = pos;
+            for (int k : fr[r]) {
+                frow[x++] = pos;
+                for (int32_t q = row[k]; q < row[k + 1]; ++q, ++pos) {
+                    const int32_t w = L.csrEl[R.csr0 + q];
+                    const int32_t e = w >> 1;
+                    if (slot_of[e] < first) {  // not yet a slot of this part
+                        slot_of[e] = ns++;
+                        L.fpSlot.push_back(e);
+                        L.fpSlot.push_back(ref[L.Ela[e0 + e]]);
+                        L.fpSlot.push_back(ref[L.Elb[e0 + e]]);
+                        L.fpSlot.push_back(0);
+                    }
+                    L.fpCsrSlot[R.csr0 + pos] = ((slot_of[e] - first) << 1) | (w & 1);
+                }
+            }
+            R.fp_part_max = std::max(R.fp_part_max, (int32_t)(fr[r].size() + fx[r].size()));
+            R.fp_free_max = std::max(R.fp_free_max, (int32_t)fr[r].size());
+            R.fp_slot_max = std::max(R.fp_slot_max, ns - first);
+            R.fp_row_max = std::max(R.fp_row_max, pos - pos0);
+        }
+        frow[x] = pos;
+        for (int r = C; r <= kMaxParts; ++r) ps[r] = ns;
+    }
+}
 
 void build_layout(int32_t n_rve, const int64_t *node_off, const double *X, const int64_t *elem_off,
                   const int32_t *conn, const double *EA, const uint8_t *fixed, const double *V0,
@@ -604,6 +672,9 @@ void build_layout(int32_t n_rve, const int64_t *node_off, const double *X, const
     L.csrEl.assign(2 * E, 0);
     L.fpCsrSlot.assign(2 * E, -1);
     L.fpPartSlot.assign((size_t)n_rve * (kMaxParts + 1), 0);
+    L.fpNode.assign(N, 0);
+    L.fpPartOff.assign((size_t)n_rve * 2 * (kMaxParts + 1), 0);
+    L.fpRow.assign((size_t)N + n_rve, 0);
     L.fpSlot.clear();
     L.Ela.assign(E, 0);
     L.Elb.assign(E, 0);
@@ -747,35 +818,6 @@ void build_layout(int32_t n_rve, const int64_t *node_off, const double *X, const
             }
         }
         hrow[R.rp0 + n] = pos;
-        // FP64 cluster slot tables (see HostLayout)
-        {
-            R.slot0 = (int64_t)(L.fpSlot.size() / 4);
-            int32_t *ps = L.fpPartSlot.data() + (size_t)p * (kMaxParts + 1);
-            std::vector<int32_t> slot_of(ne, -1);
-            int32_t ns = 0, fslot_max = 0;
-            for (int r = 0; r < C; ++r) {
-                ps[r] = ns;
-                const int32_t first = ns;
-                for (int k = pf[r]; k < pf[r + 1]; ++k) {
-                    for (int32_t q = hrow[R.rp0 + k]; q < hrow[R.rp0 + k + 1]; ++q) {
-                        const int32_t w = L.csrEl[csr_pos + q];
-                        const int32_t e = w >> 1;
-                        if (slot_of[e] < first) {  // not yet a slot of this part
-                            slot_of[e] = ns++;
-                            const int a = conn[2 * (e0 + e)], c2 = conn[2 * (e0 + e) + 1];
-                            L.fpSlot.push_back(e);
-                            L.fpSlot.push_back((owner[a] << 16) | local[a]);
-                            L.fpSlot.push_back((owner[c2] << 16) | local[c2]);
-                            L.fpSlot.push_back(0);
-                        }
-                        L.fpCsrSlot[csr_pos + q] = ((slot_of[e] - first) << 1) | (w & 1);
-                    }
-                }
-                fslot_max = std::max(fslot_max, ns - first);
-            }
-            for (int r = C; r <= kMaxParts; ++r) ps[r] = ns;
-            R.part_fslot_max = fslot_max;
-        }
         csr_pos += pos;
         for (int64_t e = e0; e < e0 + ne; ++e) {
             // the caller's orientation (a, b) is kept for lengths and the stress sum
@@ -786,7 +828,7 @@ void build_layout(int32_t n_rve, const int64_t *node_off, const double *X, const
             hElEA[e] = EA[e];
         }
     }
-
+    build_fp64_parts(elem_off, L);
 }
 
 }  // namespace
@@ -865,7 +907,10 @@ extern "C" fe2_status fe2_batch_create(int32_t n_rve, const int64_t *node_off, c
     A(b->d_fp_slot.alloc(std::max<size_t>(1, n_fslots)), "fp_slot");
     A(b->d_fp_csr_slot.alloc(2 * E), "fp_csr_slot");
     A(b->d_fp_part_slot.alloc(L.fpPartSlot.size()), "fp_part_slot");
-    A(b->d_ualt.alloc(3 * N), "ualt");
+    A(b->d_fp_node.alloc(N), "fp_node");
+    A(b->d_fp_part_off.alloc(L.fpPartOff.size()), "fp_part_off");
+    A(b->d_fp_row.alloc(N + n_rve), "fp_row");
+    A(b->d_ualt.alloc(9 * N), "ualt");
     A(b->d_fpt.alloc(3 * std::max<size_t>(1, n_fslots)), "fpt");
     A(b->d_tf.alloc(3 * E), "tf");
     A(b->d_sv.alloc(N), "sv");
@@ -916,6 +961,9 @@ extern "C" fe2_status fe2_batch_create(int32_t n_rve, const int64_t *node_off, c
     if (n_fslots) H2D(b->d_fp_slot.p, L.fpSlot.data(), sizeof(int4) * n_fslots, "fp_slot");
     H2D(b->d_fp_csr_slot.p, L.fpCsrSlot.data(), sizeof(int32_t) * 2 * E, "fp_csr_slot");
     H2D(b->d_fp_part_slot.p, L.fpPartSlot.data(), sizeof(int32_t) * L.fpPartSlot.size(), "fp_part_slot");
+    H2D(b->d_fp_node.p, L.fpNode.data(), sizeof(int32_t) * N, "fp_node");
+    H2D(b->d_fp_part_off.p, L.fpPartOff.data(), sizeof(int32_t) * L.fpPartOff.size(), "fp_part_off");
+    H2D(b->d_fp_row.p, L.fpRow.data(), sizeof(int32_t) * (N + n_rve), "fp_row");
     H2D(b->d_rowptr.p, hrow.data(), sizeof(int32_t) * (N + n_rve), "rowptr");
     H2D(b->d_part_off.p, hpart.data(), sizeof(int32_t) * hpart.size(), "part_off");
     H2D(b->d_el_a.p, hEla.data(), sizeof(int32_t) * E, "el_a");
@@ -1161,12 +1209,11 @@ int resident_of(fe2_batch *b, int kind, int parts, int block, size_t smem, int p
 // Resident clusters of an FP64 cluster class (cached like resident_of; the
 // key's kind 3 + 2 tsm + ssm and the smem size identify the variant).
 int resident_fp64_cluster(fe2_batch *b, const SizeClass &c, int block) {
-    const auto key = std::make_tuple(3 + 2 * (int)c.fp64_tsm + (int)c.fp64_ssm, c.parts, block, c.smem_bytes,
-                                     c.part_max);
+    const auto key = std::make_tuple(3 + 2 * (int)c.fp.tsm + (int)c.fp.ssm, c.parts, block, fp64_cluster_smem(c.fp),
+                                     c.fp.part_max);
     auto it = b->occ.find(key);
     if (it != b->occ.end()) return it->second;
-    const int r = occupancy_dr_fp64_cluster(c.parts, block, c.part_max, c.free_max, c.fslot_max, c.fp64_tsm,
-                                            c.fp64_ssm);
+    const int r = occupancy_dr_fp64_cluster(block, c.fp);
     b->occ[key] = r;
     return r;
 }
@@ -1196,8 +1243,7 @@ fe2_status launch_class(fe2_batch *b, const fe2_opts &o, const SizeClass &c, Sol
             if (*timed + 2 > (int)b->tev.size()) return fail(FE2_ECUDA, "too many launch classes");
             CUDA_TRY(record_timing(b->tev[*timed], s, capturing));
         }
-        const int e = launch_dr_fp64_cluster(M, S, R, P, std::min(nq, resident), c.parts, block, c.part_max,
-                                             c.free_max, c.fslot_max, c.fp64_tsm, c.fp64_ssm, s);
+        const int e = launch_dr_fp64_cluster(M, S, R, P, std::min(nq, resident), block, c.fp, s);
         if (e != 0) return fail(FE2_ECUDA, std::string("launch: ") + cudaGetErrorString((cudaError_t)e));
         if (timed) {
             CUDA_TRY(record_timing(b->tev[*timed + 1], s, capturing));

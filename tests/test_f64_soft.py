@@ -33,6 +33,9 @@ int main(int, char **argv) {
                     div(make(m & 1, e, m), make(n & 1, f, n));
                     root(make(0, e, m));
                     root(make(1, f, n));
+                    uint32_t v;
+                    const double l = f64_sqrt_recip(make(0, f, n), v);
+                    bad += !same(f64_div_v<true>(make(m & 1, e, m), l, v), make(m & 1, e, m) / l);
                 }
     for (long i = 0; i < 400000; ++i) {
         const uint64_t x = g(), y = g();
@@ -45,6 +48,11 @@ int main(int, char **argv) {
         root(f64_from(f64_bits(s) + y % 5 - 2));
         const double h = make(0, 1000, (x >> 11) & ~0x3ffffffull);  // 26-bit root: its square is exact
         root(h * h);
+        // a root as divisor, with the root's own estimate
+        uint32_t v;
+        const double l = f64_sqrt_recip(f64_from(f64_bits(s) + y % 5 - 2), v);
+        bad += !same(f64_div_v<true>(a, l, v), a / l);
+        bad += !same(f64_div_v<true>(f64_from(f64_bits(a * l) + x % 5 - 2), l, v), f64_from(f64_bits(a * l) + x % 5 - 2) / l);
         div(a, make(0, 1000, (y >> 11) & (~0ull << (y % 53))));
         div(make(0, 1010, (y >> 11) + x % 7 - 3), make(0, 1003, y >> 11));
     }
