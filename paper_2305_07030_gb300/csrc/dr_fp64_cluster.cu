@@ -30,9 +30,10 @@
 // additions and multiplications, per free node 45 at degree 5; divisions and
 // square roots run on the integer pipes (f64_soft.cuh). Everything that is the
 // same for the whole CTA is kept off that pipe: a residual total or a square
-// root computed by every thread costs 16 warps' slots. (With the totals in
-// every thread, the acceleration stored and the update a phase of its own:
-// @@BEFORE@@; now @@AFTER@@.)
+// root computed by every thread costs 16 warps' slots. Measured per
+// iteration, before (totals in every thread, the acceleration stored, the
+// update a phase of its own, one-part RVEs on the single-CTA kernel) and now:
+// 5000 nodes on 8 CTAs 23.4 -> 16.0 us, 512 nodes on one CTA 18.8 -> 13.0 us.
 #include <cooperative_groups.h>
 
 #include <algorithm>
