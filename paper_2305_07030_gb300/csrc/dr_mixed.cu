@@ -32,21 +32,26 @@
 //    and across warps and CTAs in double-float; the threshold (tol f_ref)^2 is
 //    formed in FP64 once per RVE; the stress sum is FP64.
 //
-// Synchronisation of the FP32 kernel. One cluster barrier per iteration.
-// Five displacement-increment buffers rotate. Each node's owner thread
-// computes the next iteration's increment right after the node's velocity
-// update, so an iteration begins at the barrier. Between the barrier's arrive
-// and wait, every warp publishes its residual partial of the previous
-// evaluation to its own CTA, and one warp per CTA totals evaluation n-3 across
-// the cluster (DSMEM reads) and leaves a verdict. All warps read the verdict
-// after the next barrier. If the test succeeded, they finish with the state of
-// the tested evaluation, whose buffer is still intact.
+// The FP32 phase runs in dr_mixed_node.cu's kernel, one thread per free node
+// with its row tables on chip. The FP32 kernel of this file, which re-reads the
+// CSR rows from L2, remains for parts whose increments alone (with the copies
+// of neighbours in other parts) do not fit in shared memory.
 //
-// The element forces of the FP32 kernel and of the lead come from a
-// shared-memory element table. Each element with an end among a CTA's free
-// nodes is evaluated once per iteration, spread evenly over the threads. Each
-// node then sums the +- results of its CSR row in row order. The two ends see
-// exactly opposite values, so this equals the per-direction evaluation.
+// Synchronisation of this file's FP32 kernel. One cluster barrier per
+// iteration. Five displacement-increment buffers rotate. Each node's owner
+// thread computes the next iteration's increment right after the node's
+// velocity update, so an iteration begins at the barrier. Between the
+// barrier's arrive and wait, every warp publishes its residual partial of the
+// previous evaluation to its own CTA, and one warp per CTA totals evaluation
+// n-3 across the cluster (DSMEM reads) and leaves a verdict. All warps read
+// the verdict after the next barrier. If the test succeeded, they finish with
+// the state of the tested evaluation, whose buffer is still intact.
+//
+// The element forces of the lead come from a shared-memory element table. Each
+// element with an end among a CTA's free nodes is evaluated once per
+// iteration, spread evenly over the threads. Each node then sums the +-
+// results of its CSR row in row order. The two ends see exactly opposite
+// values, so this equals the per-direction evaluation.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -54,35 +59,24 @@
 #include <mutex>
 #include <utility>
 
-#include "df64.cuh"
-#include "dr_device.cuh"
-
-namespace cg = cooperative_groups;
+#include "dr_mixed.cuh"
 
 namespace fe2 {
 
 namespace {
 
-constexpr int kMaxWarps = 16;  // blocks of at most 512 threads
 constexpr int kLeadBufs = 3;   // lead kernel: rotating partial buffers
-constexpr int kBufs = 5;       // FP32 kernel: rotating increment / partial buffers
-// FP32 kernel shared memory per node with the element table: reference
-// position, five increment buffers (float4 each), velocity + a.x (float4),
-// a.yz (float2). Without the table, velocity and acceleration live in global
-// memory and a node takes the first six float4 only.
-constexpr size_t kFp32NodeBytes = (1 + kBufs + 1) * sizeof(float4) + sizeof(float2);
+// FP32 kernel without row tables (this file): shared memory per node, the
+// reference position and five increment buffers (float4 each); velocity and
+// acceleration live in global memory.
 constexpr size_t kFp32PlainNodeBytes = (1 + kBufs) * sizeof(float4);
+// Per-node bytes of the footprint rule that sets the cluster size
+// (mixed_fp32_smem).
+constexpr size_t kFp32NodeBytes = (1 + kBufs + 1) * sizeof(float4) + sizeof(float2);
 // Lead kernel shared memory per node without the element table: one
 // double-float displacement (hi, lo float4); with the table, two of them.
 constexpr size_t kLeadPlainNodeBytes = 2 * sizeof(float4);
 __host__ __device__ constexpr size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
-
-// Convergence verdict on one evaluation (FP32 kernel): code -1 = go on, else
-// the RVE status; the double-float squared residual and kinetic energy.
-struct Verdict {
-    int code;
-    float r2h, r2l, k2h, k2l;
-};
 
 struct MixedShared {
     // lead kernel: per-warp residual partials of every CTA, dense: entry
@@ -109,35 +103,6 @@ struct MixedShared {
     int slots;                                // FP32 kernel: row slots of this CTA's part
 };
 
-struct Part {
-    int me, C;
-    int f0, nfr;   // own free nodes: RVE-local [f0, f0 + nfr)
-    int g0, nfx;   // own fixed nodes: RVE-local n_free + [g0, g0 + nfx)
-    int nf;        // RVE free count
-    __device__ int gidx(int k) const { return k < nfr ? f0 + k : nf + g0 + (k - nfr); }
-    __device__ int m() const { return nfr + nfx; }
-};
-
-__device__ __forceinline__ Part make_part(const DevMesh &M, const RveDesc &R, int p, int me, int C) {
-    const int32_t *po = M.part_off + (int64_t)p * 2 * (kMaxParts + 1);
-    Part pt;
-    pt.me = me;
-    pt.C = C;
-    pt.nf = R.n_free;
-    pt.f0 = po[me];
-    pt.nfr = po[me + 1] - pt.f0;
-    pt.g0 = po[kMaxParts + 1 + me];
-    pt.nfx = po[kMaxParts + 1 + me + 1] - pt.g0;
-    return pt;
-}
-
-__device__ __forceinline__ void cluster_arrive() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
-}
-__device__ __forceinline__ void cluster_wait() {
-    asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-}
-
 // Double-float total of the cluster's per-warp partials (buffer `buf`),
 // computed warp-parallel on the FP32 pipes: lane l adds entries l, l+32, ...
 // and a butterfly of double-float additions finishes the sum. The order is
@@ -155,9 +120,6 @@ __device__ __forceinline__ df cluster_total(const float (*red)[kMaxParts * kMaxW
     }
     return acc;
 }
-
-// a <= b for double-float values.
-__device__ __forceinline__ bool df_le(df a, df b) { return a.hi < b.hi || (a.hi == b.hi && a.lo <= b.lo); }
 
 // Publish this thread's FP32 partials (warp-reduced) into every CTA's buffer.
 __device__ __forceinline__ void publish(MixedShared &sh, const Part &pt, float v, float kv, bool want_k,
@@ -205,25 +167,8 @@ __device__ __forceinline__ void gather_df(const DevMesh &M, const RveDesc &R, co
         const int r = cp >> 16, loc = cp & 0xffff;
         const float4 pj = r == pt.me ? Pl[loc] : sh.P[r][loc];
         const float4 qj = r == pt.me ? Ql[loc] : sh.Q[qbuf][r][loc];
-        const float4 Dh = M.dh[kk], Dl = M.dl[kk];
-        // relative displacement and current element vector
-        const df e0 = df_sub({pj.x, qj.x}, ui0), e1 = df_sub({pj.y, qj.y}, ui1),
-                 e2 = df_sub({pj.z, qj.z}, ui2);
-        const df D0 = {Dh.x, Dl.x}, D1 = {Dh.y, Dl.y}, D2 = {Dh.z, Dl.z}, L = {Dh.w, Dl.w};
-        const df d0 = df_add(D0, e0), d1 = df_add(D1, e1), d2 = df_add(D2, e2);
-        // h = l^2 - L^2 = e.(D + d)
-        const df h = df_add(df_add(df_mul(e0, df_add(D0, d0)), df_mul(e1, df_add(D1, d1))),
-                            df_mul(e2, df_add(D2, d2)));
-        const df l2 = df_add(df_sqr(L), h);
-        const df rl = df_rsqrt(l2);
-        const df l = df_mul(l2, rl);
-        const float2 eh = M.eaf[kk], el = M.eaf_lo[kk];
-        // N/l = EA (l - L) / (L l) = (EA/L) h / (l (l + L))
-        const df kax = df_mul({eh.x, el.x}, {eh.y, el.y});
-        const df q = df_mul(df_mul(kax, df_mul(h, rl)), df_rcp(df_add(l, L)));
-        g0 = df_add(g0, df_mul(q, d0));
-        g1 = df_add(g1, df_mul(q, d1));
-        g2 = df_add(g2, df_mul(q, d2));
+        df_entry_force(M, kk, df_sub({pj.x, qj.x}, ui0), df_sub({pj.y, qj.y}, ui1), df_sub({pj.z, qj.z}, ui2),
+                       g0, g1, g2);
     }
 }
 
@@ -271,35 +216,25 @@ __device__ __forceinline__ void edge_increment(const float4 &pi, const float4 &q
     g2 += qref * e2 + dq * (r2 + e2);
 }
 
-// Per-part element tables of the FP32 kernel, in shared memory when they fit
+// Per-part element tables of the lead kernel, in shared memory when they fit
 // (STAGE); otherwise every row is re-read from the global CSR each iteration.
 //
 // Element list: each element with at least one end among this CTA's free
 // nodes appears once. An element between two own free nodes belongs to the
 // row of its lower local index (end a) and is used with the opposite sign by
 // the other row (end b); any other element belongs to the row of its own free
-// end a. Element u holds
-//   K0 = (r, |r|^2), r = x_ref,b - x_ref,a,
-//   K1 = (q_ref, EA, 1/|r|, address of b's increment in buffer 0: shared::cta,
-//        or shared::cluster with bit 0 set when b lives in another CTA),
-//   EI = shared::cta address of a's increment in buffer 0,
-//   TF = the iteration's force increment on a (on b it is -TF, exactly).
-// The reference geometry only changes when the reference state moves.
+// end a (lead_loop_staged gives an element's entries).
 // Node rows are laid out ELL-style in slabs of 32 consecutive own free nodes:
 // entry j of node k sits at slot SS[k / 32] + 32 j + k % 32 and holds
 // (element << 1 | 1 if the node is end b), so a warp reads 32 consecutive
 // slots at every step; the entries keep the CSR row order.
 struct Staged {
-    float4 *SG;    // per own free node: (g_ref, 1/m)
     float4 *K0;    // per element
     float4 *K1;    // per element
-    float4 *TF;    // per element
-    uint32_t *EI;  // per element
     uint32_t *NS;  // per slot
     int *SD;       // per own free node: row length
     int *EB;       // per own free node: first element of its row
     int *SS;       // per slab + 1: first slot
-    // lead kernel only (K0, K1 then hold the double-float D and L)
     float4 *KA;    // per element
     float4 *TA;    // per element
     float2 *TB;    // per element
@@ -308,15 +243,6 @@ struct Staged {
     float4 *AY;    // per own free node: (a.hi y, a.hi z, a.lo y, a.lo z)
 };
 
-// 32-bit shared-memory address of p and its image in cluster CTA `rank`.
-__device__ __forceinline__ uint32_t smem_addr(const void *p) {
-    return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ uint32_t cluster_addr(uint32_t a, uint32_t rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-    return r;
-}
 __device__ __forceinline__ float4 ld_cluster(uint32_t a) {
     float4 v;
     asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
@@ -330,23 +256,6 @@ __device__ __forceinline__ float4 ld_local(uint32_t a) {
                  : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
                  : "r"(a));
     return v;
-}
-
-// The FP32 increment of edge_increment with the reference geometry taken from
-// an element's K0, K1 (same operations, same order).
-__device__ __forceinline__ void edge_increment_slot(const float4 &qi, const float4 &qj, const float4 &k0,
-                                                    const float4 &k1, float &g0, float &g1, float &g2) {
-    const float r0 = k0.x, r1 = k0.y, r2 = k0.z, lr2 = k0.w;
-    const float qref = k1.x, ea = k1.y, ril = k1.z;
-    const float e0 = qj.x - qi.x, e1 = qj.y - qi.y, e2 = qj.z - qi.z;
-    const float lr = lr2 * ril;
-    const float h = 2.f * (r0 * e0 + r1 * e1 + r2 * e2) + (e0 * e0 + e1 * e1 + e2 * e2);
-    const float rl = rsqrtf(lr2 + h);
-    const float l = (lr2 + h) * rl;
-    const float dq = __fdividef(ea * h * rl * ril, l + lr);
-    g0 += qref * e0 + dq * (r0 + e0);
-    g1 += qref * e1 + dq * (r1 + e1);
-    g2 += qref * e2 + dq * (r2 + e2);
 }
 
 // Whether CSR entry (rank r, local loc) of own free node k is used with the
@@ -390,86 +299,11 @@ __device__ void element_offsets(MixedShared &sh, const Part &pt, const Staged &s
     sh.slots = slots;
 }
 
-// Fill the element table from the current reference positions (every CTA's Pl
-// must be final): K0 and K1.xyz always; with `full` also the addresses and the
-// node rows.
-__device__ void element_setup(const MixedShared &sh, const DevMesh &M, const RveDesc &R, const Part &pt,
-                              const int32_t *rowptr, const float4 *Pl, const float4 *Q0,
-                              const Staged &st, bool full) {
-    for (int k = threadIdx.x; k < pt.nfr; k += blockDim.x) {
-        const int beg = rowptr[pt.f0 + k], deg = st.SD[k];
-        const float4 pa = Pl[k];
-        int u = st.EB[k];
-        int slot = st.SS[k >> 5] + (k & 31);
-        for (int e = 0; e < deg; ++e, slot += 32) {
-            const int64_t kk = R.csr0 + beg + e;
-            const int cp = M.col_part[kk];
-            const int r = cp >> 16, loc = cp & 0xffff;
-            if (b_end(r, loc, k, pt)) {
-                if (full) {
-                    // the element's index in row loc
-                    const int jb = rowptr[pt.f0 + loc], jd = st.SD[loc];
-                    int v = st.EB[loc];
-                    for (int x = 0; x < jd; ++x) {
-                        const int cq = M.col_part[R.csr0 + jb + x];
-                        const int rq = cq >> 16, lq = cq & 0xffff;
-                        if (rq == pt.me && lq == k) break;
-                        v += !b_end(rq, lq, loc, pt);
-                    }
-                    st.NS[slot] = ((uint32_t)v << 1) | 1u;
-                }
-                continue;
-            }
-            const float4 pb = r == pt.me ? Pl[loc] : sh.P[r][loc];
-            const float2 ei = M.eaf[kk];
-            const float r0 = pb.x - pa.x, r1 = pb.y - pa.y, r2 = pb.z - pa.z;
-            const float lr2 = r0 * r0 + r1 * r1 + r2 * r2;
-            const float ril = rsqrtf(lr2);
-            const float qref = ei.x * (ei.y - ril);
-            uint32_t ab;
-            if (full) {
-                const uint32_t qb = smem_addr(Q0 + loc);
-                ab = r == pt.me ? qb : (cluster_addr(qb, (uint32_t)r) | 1u);
-                st.EI[u] = smem_addr(Q0 + k);
-                st.NS[slot] = (uint32_t)u << 1;
-            } else {
-                ab = __float_as_uint(st.K1[u].w);
-            }
-            st.K0[u] = make_float4(r0, r1, r2, lr2);
-            st.K1[u] = make_float4(qref, ei.x, ril, __uint_as_float(ab));
-            ++u;
-        }
-    }
-}
-
-// Convergence verdict on one evaluation: the double-float total of every
-// CTA's per-warp partials (fixed order: rank, then warp), read through
-// distributed shared memory.
-__device__ __forceinline__ Verdict residual_verdict(const MixedShared &sh, const Part &pt, int buf, int64_t done,
-                                         const df &thresh2, bool want_k, int64_t max_iter) {
-    const int nw = (int)(blockDim.x >> 5), total = pt.C * nw, lane = threadIdx.x & 31;
-    df r2 = df_from(0.f), k2 = df_from(0.f);
-    for (int j = lane; j < total; j += 32) {
-        const int r = j / nw, w = j - r * nw;
-        r2 = df_add_f(r2, sh.ownp[r][(buf * 2 + 0) * kMaxWarps + w]);
-        if (want_k) k2 = df_add_f(k2, sh.ownp[r][(buf * 2 + 1) * kMaxWarps + w]);
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        r2 = df_add(r2, {__shfl_xor_sync(0xffffffffu, r2.hi, o), __shfl_xor_sync(0xffffffffu, r2.lo, o)});
-        if (want_k)
-            k2 = df_add(k2, {__shfl_xor_sync(0xffffffffu, k2.hi, o), __shfl_xor_sync(0xffffffffu, k2.lo, o)});
-    }
-    Verdict v;
-    v.code = !isfinite(r2.hi) ? RVE_NAN : df_le(r2, thresh2) ? RVE_OK : done >= max_iter ? RVE_MAXITER : -1;
-    v.r2h = r2.hi; v.r2l = r2.lo; v.k2h = k2.hi; v.k2l = k2.lo;
-    return v;
-}
-
 // ---------------------------------------------------------------------------
 // lead kernel with the element table (STAGE)
 // ---------------------------------------------------------------------------
-// The lead's element table: the same element list and node rows as the FP32
-// kernel's (element_counts, element_offsets), with per element
+// The lead's element table (element list and node rows: element_counts,
+// element_offsets), with per element
 //   K0 = (D, L).hi, K1 = (D, L).lo  (D = X_b - X_a, double-float),
 //   KA = ((EA/L).hi, (EA/L).lo, shared::cta address of a's displacement in
 //        buffer 0, address of b's: shared::cta, or shared::cluster with bit 0
@@ -721,84 +555,10 @@ __device__ void lead_loop_staged(cg::cluster_group &cl, MixedShared &sh, const D
     }
 }
 
-// End of a mixed solve of RVE p: the final displacement (FP64 output; the
-// double-float displacement plus the FP32 increment Qfin when given), the
-// FP64 stress sum split across the cluster, and the per-RVE outputs.
-__device__ void mixed_finish(cg::cluster_group &cl, MixedShared &sh, const DevMesh &M, const DevState &S,
-                             const DevResults &O, const SolveParams &P, int p, const RveDesc &R,
-                             const Part &pt, const double *F, const float4 *Qfin, int status, int64_t it,
-                             df r2, df k2, double f_ref) {
-    const int n = R.n_nodes, m = pt.m();
-    const int64_t n0 = R.node0, b3 = 3 * n0;
-    const float *uh = S.uh + b3, *ul = S.ul + b3;
-    double *xg = S.xg + b3;
-    const bool want_k = P.want_ke != 0;
-    const int fin = Qfin ? 0 : -1;
-    // ---- final displacement (FP64 output) and positions for the stress ----
-    for (int k = threadIdx.x; k < m; k += blockDim.x) {
-        const int i = pt.gidx(k);
-        float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (fin >= 0 && k < pt.nfr) d = Qfin[k];
-        const float dd[3] = {d.x, d.y, d.z};
-        double *uo[3] = {S.u0 + n0, S.u1 + n0, S.u2 + n0};
-        const double *Xd[3] = {M.X0 + n0, M.X1 + n0, M.X2 + n0};
-        for (int c = 0; c < 3; ++c) {
-            df u = {uh[c * n + i], ul[c * n + i]};
-            if (fin >= 0 && k < pt.nfr) u = df_add_f(u, dd[c]);
-            const double ud = df_to_double(u);
-            uo[c][i] = ud;
-            xg[c * n + i] = dadd(Xd[c][i], ud);
-        }
-    }
-    cl.sync();
-    // stress: elements split across the cluster, partials reduced on rank 0
-    double s[9];
-#pragma unroll
-    for (int k = 0; k < 9; ++k) s[k] = 0.0;
-    {
-        const double *x0 = xg, *x1 = xg + n, *x2 = xg + 2 * n;
-        for (int e = pt.me * blockDim.x + threadIdx.x; e < R.n_elems; e += pt.C * blockDim.x) {
-            const int64_t ee = R.elem0 + e;
-            const int a = M.el_a[ee], bb = M.el_b[ee];
-            double d[3] = {dsub(x0[bb], x0[a]), dsub(x1[bb], x1[a]), dsub(x2[bb], x2[a])};
-            const double l = dsqrt(dadd(dadd(dmul(d[0], d[0]), dmul(d[1], d[1])), dmul(d[2], d[2])));
-            const double q = ddiv(dmul(M.el_EA[ee], dsub(ddiv(l, M.el_L[ee]), 1.0)), l);
-#pragma unroll
-            for (int rr = 0; rr < 3; ++rr)
-#pragma unroll
-                for (int c = 0; c < 3; ++c) s[3 * rr + c] = dadd(s[3 * rr + c], dmul(dmul(q, d[rr]), d[c]));
-        }
-    }
-    {
-        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            double v = s[k];
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (lane == 0) sh.wsum[warp][k] = v;
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x < 9) {
-        double t = 0.0;
-        for (int w = 0; w < (int)((blockDim.x + 31) >> 5); ++w) t += sh.wsum[w][threadIdx.x];
-        sh.sigp[pt.me * 9 + threadIdx.x] = t;
-    }
-    cl.sync();
-    if (pt.me == 0 && threadIdx.x < 9) {
-        double t = 0.0;
-        for (int q = 0; q < pt.C; ++q) t += sh.sig[q][threadIdx.x];
-        O.sigma[9 * (int64_t)p + threadIdx.x] = ddiv(t, dmul(det3(F), R.V0));
-    }
-    if (pt.me == 0 && threadIdx.x == 0) {
-        const double r = sqrt(df_to_double(r2));
-        O.iters[p] = it;
-        O.rel_res[p] = f_ref > 0.0 ? r / f_ref : (r > 0.0 ? INFINITY : 0.0);
-        O.status[p] = status;
-        O.ke[p] = want_k ? df_to_double(k2) : 0.0;
-    }
-    cl.sync();
-}
+// No FP32 increment on top of the double-float displacement.
+struct NoInc {
+    __device__ float4 operator()(int) const { return make_float4(0.f, 0.f, 0.f, 0.f); }
+};
 
 // ---------------------------------------------------------------------------
 // lead kernel: setup (Algorithm 1 lines up to the loop) and the double-float
@@ -986,7 +746,7 @@ __device__ void lead_rve(cg::cluster_group &cl, MixedShared &sh, const DevMesh &
     }
     if (P.resume) {
         if (pt.me == 0 && threadIdx.x == 0) O.lead[p] += it - it0;
-        mixed_finish(cl, sh, M, S, O, P, p, R, pt, F, nullptr, status, it, r2, k2, f_ref);
+        mixed_finish(cl, sh, M, S, O, P, p, R, pt, F, false, NoInc{}, status, it, r2, k2, f_ref);
         return;
     }
     if (pt.me == 0 && threadIdx.x == 0) {
@@ -1003,33 +763,18 @@ __device__ void lead_rve(cg::cluster_group &cl, MixedShared &sh, const DevMesh &
 // ---------------------------------------------------------------------------
 // FP32 kernel: increment iterations, reference refreshes, final state, stress
 // ---------------------------------------------------------------------------
-// The next iteration's partial velocity update (Algorithm 1: v += dt/2 a)
-// and displacement increment (u += dt v, as an increment on top of d) for one
-// node, from its velocity w and acceleration a after this iteration.
-__device__ __forceinline__ void next_increment(float w0, float w1, float w2, float a0, float a1, float a2,
-                                               const float4 &d, float hdtf, float dtf, float4 &sv,
-                                               float2 &sa, float4 &next) {
-    const float v0 = w0 + hdtf * a0, v1 = w1 + hdtf * a1, v2 = w2 + hdtf * a2;
-    sv = make_float4(v0, v1, v2, a0);
-    sa = make_float2(a1, a2);
-    next = make_float4(d.x + dtf * v0, d.y + dtf * v1, d.z + dtf * v2, 0.f);
-}
-
-template <bool STAGE>
 __device__ void fp32_rve(cg::cluster_group &cl, MixedShared &sh, const DevMesh &M, const DevState &S,
                          const DevResults &O, const SolveParams &P, int p, float4 *Pl,
-                         float4 *const *Qb, float4 *SVs, float2 *SAs, const Staged &st, int elem_cap,
-                         int slot_cap, uint32_t bstride) {
+                         float4 *const *Qb) {
     const RveDesc R = M.rve[p];
     const Part pt = make_part(M, R, p, (int)cl.block_rank(), (int)cl.num_blocks());
     const int n = R.n_nodes, m = pt.m();
     const int64_t n0 = R.node0, b3 = 3 * n0;
     const int32_t *rowptr = M.rowptr + R.rp0;
-    // velocity (+ a.x) and a.yz of the own free nodes: shared memory with the
-    // element table; otherwise global (L2-resident) arrays, which keeps the
-    // unstaged kernel's shared memory at 96 bytes per node
-    float4 *SV = STAGE ? SVs : S.sv + n0 + pt.f0;
-    float2 *SA = STAGE ? SAs : S.sa + n0 + pt.f0;
+    // velocity (+ a.x) and a.yz of the own free nodes: global (L2-resident)
+    // arrays, which keeps the shared memory at 96 bytes per node
+    float4 *SV = S.sv + n0 + pt.f0;
+    float2 *SA = S.sa + n0 + pt.f0;
     const float *Xh = M.Xh + b3, *Xl = M.Xl + b3;
     float *uh = S.uh + b3, *ul = S.ul + b3, *vh = S.vh + b3, *ah = S.ah + b3, *fg = S.fg + b3;
     const float *imh = M.imh + n0;
@@ -1051,13 +796,12 @@ __device__ void fp32_rve(cg::cluster_group &cl, MixedShared &sh, const DevMesh &
         const double dt64 = dmul(P.alpha, R.dtc);
         const float dtf = (float)dt64, hdtf = (float)dmul(0.5, dt64), cf = (float)R.c;
         const int K = P.rebase_every > 0 ? P.rebase_every : 512;
-        // lanes per node: with the element table one (element forces are spread
-        // over all threads, node sums are short); otherwise as many as the CTA
-        // size allows for this RVE's largest part. Node k's velocity and
+        // lanes per node: as many as the CTA size allows for this RVE's largest
+        // part. Node k's velocity and
         // acceleration are owned by lane 0 of group k in every phase, so
         // consecutive phases need no barrier between them.
         int lanes = 1;
-        while (!STAGE && lanes < 4 && (int)blockDim.x >= 2 * lanes * R.part_free_max) lanes *= 2;
+        while (lanes < 4 && (int)blockDim.x >= 2 * lanes * R.part_free_max) lanes *= 2;
         const int L = lanes;
         const int sub = threadIdx.x & (L - 1), grp = threadIdx.x / L, ngrp = blockDim.x / L;
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1076,13 +820,7 @@ __device__ void fp32_rve(cg::cluster_group &cl, MixedShared &sh, const DevMesh &
             if (k < pt.nfr) {
                 SV[k] = make_float4(vh[i], vh[n + i], vh[2 * n + i], ah[i]);
                 SA[k] = make_float2(ah[n + i], ah[2 * n + i]);
-                if (STAGE) st.SG[k] = make_float4(fg[i], fg[n + i], fg[2 * n + i], imh[i]);
             }
-        }
-        if (STAGE) {
-            element_counts(M, R, pt, rowptr, st);
-            __syncthreads();
-            if (threadIdx.x == 0) element_offsets(sh, pt, st);
         }
         if (threadIdx.x == 0) {
             sh.st_h = INFINITY;
@@ -1090,19 +828,6 @@ __device__ void fp32_rve(cg::cluster_group &cl, MixedShared &sh, const DevMesh &
             sh.st_e = it;
         }
         cl.sync();
-        int n_el = 0;
-        if (STAGE) {
-            // The capacities are sized on the host for every part. Should a
-            // part not fit, every CTA of the cluster sees it (so all leave the
-            // loop together) and the RVE is reported failed.
-            bool over = false;
-            for (int r = 0; r < pt.C; ++r)
-                over |= *cl.map_shared_rank(&sh.elems, r) > elem_cap ||
-                        *cl.map_shared_rank(&sh.slots, r) > slot_cap;
-            if (over) status = RVE_NAN;
-            else element_setup(sh, M, R, pt, rowptr, Pl, Qb[0], st, true);
-            n_el = sh.elems;
-        }
         const int64_t first = it;  // evaluation index of the first FP32 iteration
         int64_t chk = first;       // next evaluation whose residual is still untested
         int chkb = 0;              // its buffer
@@ -1261,7 +986,6 @@ __device__ void fp32_rve(cg::cluster_group &cl, MixedShared &sh, const DevMesh &
                     df g[3];
                     gather_df(M, R, rowptr, sh, pt, k, Pl, cur, b, g[0], g[1], g[2]);
                     fg[i] = g[0].hi; fg[n + i] = g[1].hi; fg[2 * n + i] = g[2].hi;
-                    if (STAGE) st.SG[k] = make_float4(g[0].hi, g[1].hi, g[2].hi, imh[i]);
                 }
                 cl.sync();
                 // back to FP32 reference positions and zero increments
@@ -1274,7 +998,6 @@ __device__ void fp32_rve(cg::cluster_group &cl, MixedShared &sh, const DevMesh &
                     cur[k] = make_float4(0.f, 0.f, 0.f, 0.f);
                 }
                 cl.sync();
-                if (STAGE) element_setup(sh, M, R, pt, rowptr, Pl, Qb[0], st, false);
                 for (int k = grp; k < pt.nfr; k += ngrp) {
                     if (sub != 0) continue;
                     const int i = pt.f0 + k;
@@ -1291,97 +1014,58 @@ __device__ void fp32_rve(cg::cluster_group &cl, MixedShared &sh, const DevMesh &
                 since = 0;
             } else {
                 vpend = tnow; veval = teval; vbuf = tbuf;
-                const uint32_t boff = (uint32_t)b * bstride;
-                if (STAGE) {
-                    // element forces, spread evenly over the CTA's threads
-                    for (int u = threadIdx.x; u < n_el; u += blockDim.x) {
-                        const float4 k0 = st.K0[u], k1 = st.K1[u];
-                        const float4 qa = ld_local(st.EI[u] + boff);
-                        const uint32_t ab = __float_as_uint(k1.w);
-                        const float4 qb = (ab & 1u) ? ld_cluster((ab & ~1u) + boff) : ld_local(ab + boff);
-                        float t0 = 0.f, t1 = 0.f, t2 = 0.f;
-                        edge_increment_slot(qa, qb, k0, k1, t0, t1, t2);
-                        st.TF[u] = make_float4(t0, t1, t2, 0.f);
-                    }
-                    __syncthreads();
-                    // node sums in CSR row order, then the velocity update
-                    for (int k = threadIdx.x; k < pt.nfr; k += blockDim.x) {
-                        const int deg = st.SD[k];
-                        int sl = st.SS[k >> 5] + (k & 31);
-                        float g0 = 0.f, g1 = 0.f, g2 = 0.f;
-                        for (int j = 0; j < deg; ++j, sl += 32) {
-                            const uint32_t w = st.NS[sl];
-                            const float4 t = st.TF[w >> 1];
-                            if (w & 1u) { g0 -= t.x; g1 -= t.y; g2 -= t.z; }
-                            else { g0 += t.x; g1 += t.y; g2 += t.z; }
+                // L lanes share a node's edges (lane s takes edges s, s+L, ...,
+                // two at a time) and combine with shuffles; L is fixed per RVE
+                // so its result does not depend on the launch it runs in.
+                for (int kb = 0; kb < pt.nfr; kb += ngrp) {
+                    const int k = kb + grp;
+                    const bool valid = k < pt.nfr;
+                    float g0 = 0.f, g1 = 0.f, g2 = 0.f;
+                    if (valid) {
+                        const float4 qi = cur[k];
+                        const int i = pt.f0 + k;
+                        const float4 pi = Pl[k];
+                        const int end = rowptr[i + 1];
+                        int e = rowptr[i] + sub;
+                        for (; e + L < end; e += 2 * L) {
+                            const int ca = __ldg(colp + e), cb = __ldg(colp + e + L);
+                            const float2 ea = __ldg(eafp + e), eb = __ldg(eafp + e + L);
+                            const int ra = ca >> 16, la = ca & 0xffff, rb2 = cb >> 16, lb = cb & 0xffff;
+                            const float4 pa = ra == pt.me ? Pl[la] : sh.P[ra][la];
+                            const float4 qa = ra == pt.me ? cur[la] : sh.Q[b][ra][la];
+                            const float4 pb = rb2 == pt.me ? Pl[lb] : sh.P[rb2][lb];
+                            const float4 qb = rb2 == pt.me ? cur[lb] : sh.Q[b][rb2][lb];
+                            edge_increment(pi, qi, pa, qa, ea, g0, g1, g2);
+                            edge_increment(pi, qi, pb, qb, eb, g0, g1, g2);
                         }
-                        const float4 gr = st.SG[k];
-                        g0 += gr.x; g1 += gr.y; g2 += gr.z;
-                        const float im = gr.w;
+                        if (e < end) {
+                            const int ca = __ldg(colp + e);
+                            const float2 ea = __ldg(eafp + e);
+                            const int ra = ca >> 16, la = ca & 0xffff;
+                            const float4 pa = ra == pt.me ? Pl[la] : sh.P[ra][la];
+                            const float4 qa = ra == pt.me ? cur[la] : sh.Q[b][ra][la];
+                            edge_increment(pi, qi, pa, qa, ea, g0, g1, g2);
+                        }
+                    }
+                    for (int o = 1; o < L; o <<= 1) {
+                        g0 += __shfl_xor_sync(0xffffffffu, g0, o);
+                        g1 += __shfl_xor_sync(0xffffffffu, g1, o);
+                        g2 += __shfl_xor_sync(0xffffffffu, g2, o);
+                    }
+                    if (valid && sub == 0) {
+                        const int i = pt.f0 + k;
+                        g0 += fg[i]; g1 += fg[n + i]; g2 += fg[2 * n + i];
+                        const float im = imh[i];
                         const float4 va = SV[k];
                         float w0 = va.x, w1 = va.y, w2 = va.z;
                         const float a0 = g0 * im - cf * w0;
                         const float a1 = g1 * im - cf * w1;
                         const float a2 = g2 * im - cf * w2;
                         w0 += hdtf * a0; w1 += hdtf * a1; w2 += hdtf * a2;
-                        next_increment(w0, w1, w2, a0, a1, a2, cur[k], hdtf, dtf, SV[k], SA[k], Qb[bn][k]);
+                        next_increment(w0, w1, w2, a0, a1, a2, cur[k], hdtf, dtf, SV[k], SA[k],
+                                       Qb[bn][k]);
                         rs += g0 * g0 + g1 * g1 + g2 * g2;
                         if (want_k) kes += 0.5f * (w0 * w0 + w1 * w1 + w2 * w2) / im;
-                    }
-                } else {
-                    // L lanes share a node's edges (lane s takes edges s, s+L, ...,
-                    // two at a time) and combine with shuffles; L is fixed per RVE
-                    // so its result does not depend on the launch it runs in.
-                    for (int kb = 0; kb < pt.nfr; kb += ngrp) {
-                        const int k = kb + grp;
-                        const bool valid = k < pt.nfr;
-                        float g0 = 0.f, g1 = 0.f, g2 = 0.f;
-                        if (valid) {
-                            const float4 qi = cur[k];
-                            const int i = pt.f0 + k;
-                            const float4 pi = Pl[k];
-                            const int end = rowptr[i + 1];
-                            int e = rowptr[i] + sub;
-                            for (; e + L < end; e += 2 * L) {
-                                const int ca = __ldg(colp + e), cb = __ldg(colp + e + L);
-                                const float2 ea = __ldg(eafp + e), eb = __ldg(eafp + e + L);
-                                const int ra = ca >> 16, la = ca & 0xffff, rb2 = cb >> 16, lb = cb & 0xffff;
-                                const float4 pa = ra == pt.me ? Pl[la] : sh.P[ra][la];
-                                const float4 qa = ra == pt.me ? cur[la] : sh.Q[b][ra][la];
-                                const float4 pb = rb2 == pt.me ? Pl[lb] : sh.P[rb2][lb];
-                                const float4 qb = rb2 == pt.me ? cur[lb] : sh.Q[b][rb2][lb];
-                                edge_increment(pi, qi, pa, qa, ea, g0, g1, g2);
-                                edge_increment(pi, qi, pb, qb, eb, g0, g1, g2);
-                            }
-                            if (e < end) {
-                                const int ca = __ldg(colp + e);
-                                const float2 ea = __ldg(eafp + e);
-                                const int ra = ca >> 16, la = ca & 0xffff;
-                                const float4 pa = ra == pt.me ? Pl[la] : sh.P[ra][la];
-                                const float4 qa = ra == pt.me ? cur[la] : sh.Q[b][ra][la];
-                                edge_increment(pi, qi, pa, qa, ea, g0, g1, g2);
-                            }
-                        }
-                        for (int o = 1; o < L; o <<= 1) {
-                            g0 += __shfl_xor_sync(0xffffffffu, g0, o);
-                            g1 += __shfl_xor_sync(0xffffffffu, g1, o);
-                            g2 += __shfl_xor_sync(0xffffffffu, g2, o);
-                        }
-                        if (valid && sub == 0) {
-                            const int i = pt.f0 + k;
-                            g0 += fg[i]; g1 += fg[n + i]; g2 += fg[2 * n + i];
-                            const float im = imh[i];
-                            const float4 va = SV[k];
-                            float w0 = va.x, w1 = va.y, w2 = va.z;
-                            const float a0 = g0 * im - cf * w0;
-                            const float a1 = g1 * im - cf * w1;
-                            const float a2 = g2 * im - cf * w2;
-                            w0 += hdtf * a0; w1 += hdtf * a1; w2 += hdtf * a2;
-                            next_increment(w0, w1, w2, a0, a1, a2, cur[k], hdtf, dtf, SV[k], SA[k],
-                                           Qb[bn][k]);
-                            rs += g0 * g0 + g1 * g1 + g2 * g2;
-                            if (want_k) kes += 0.5f * (w0 * w0 + w1 * w1 + w2 * w2) / im;
-                        }
                     }
                 }
             }
@@ -1403,7 +1087,8 @@ __device__ void fp32_rve(cg::cluster_group &cl, MixedShared &sh, const DevMesh &
         cl.sync();
         return;
     }
-    mixed_finish(cl, sh, M, S, O, P, p, R, pt, F, fin >= 0 ? Qb[fin] : nullptr, status, it, r2, k2, f_ref);
+    const float4 *Qfin = fin >= 0 ? Qb[fin] : nullptr;
+    mixed_finish(cl, sh, M, S, O, P, p, R, pt, F, fin >= 0, [&](int k) { return Qfin[k]; }, status, it, r2, k2, f_ref);
 }
 
 }  // namespace
@@ -1453,48 +1138,19 @@ __global__ void __launch_bounds__(512, 1) dr_mixed_lead_kernel(DevMesh M, DevSta
     }
 }
 
-template <bool STAGE>
 __global__ void __launch_bounds__(512, 1) dr_mixed_fp32_kernel(DevMesh M, DevState S, DevResults O,
-                                                               SolveParams P, int part_cap,
-                                                               int free_cap, int elem_cap,
-                                                               int slot_cap) {
+                                                               SolveParams P, int part_cap) {
     extern __shared__ __align__(16) float4 dsm[];
     __shared__ MixedShared sh;
     cg::cluster_group cl = cg::this_cluster();
     float4 *Pl = dsm;
     float4 *Qb[kBufs];
     for (int b = 0; b < kBufs; ++b) Qb[b] = dsm + (1 + b) * part_cap;
-    float4 *SV = dsm + (1 + kBufs) * part_cap;
-    float2 *SA = reinterpret_cast<float2 *>(dsm + (2 + kBufs) * part_cap);
-    Staged st = {};
-    if (STAGE) {
-        // layout as in mixed_fp32_smem
-        char *base = reinterpret_cast<char *>(dsm) + align16(kFp32NodeBytes * part_cap);
-        st.SG = reinterpret_cast<float4 *>(base);
-        base += 16 * (size_t)free_cap;
-        st.K0 = reinterpret_cast<float4 *>(base);
-        base += 16 * (size_t)elem_cap;
-        st.K1 = reinterpret_cast<float4 *>(base);
-        base += 16 * (size_t)elem_cap;
-        st.TF = reinterpret_cast<float4 *>(base);
-        base += 16 * (size_t)elem_cap;
-        st.EI = reinterpret_cast<uint32_t *>(base);
-        base += 4 * (size_t)elem_cap;
-        st.NS = reinterpret_cast<uint32_t *>(base);
-        base += 4 * (size_t)slot_cap;
-        st.SD = reinterpret_cast<int *>(base);
-        base += 4 * (size_t)free_cap;
-        st.EB = reinterpret_cast<int *>(base);
-        base += 4 * (size_t)free_cap;
-        st.SS = reinterpret_cast<int *>(base);
-    }
     map_remote(cl, sh, Pl, Qb, (int)cl.num_blocks());
-    const uint32_t bstride = (uint32_t)(sizeof(float4) * part_cap);
     for (;;) {
         const int item = next_item(cl, sh, P.counter + 1);
         if (item >= P.queue_len) return;
-        fp32_rve<STAGE>(cl, sh, M, S, O, P, P.queue[item], Pl, Qb, SV, SA, st, elem_cap, slot_cap,
-                        bstride);
+        fp32_rve(cl, sh, M, S, O, P, P.queue[item], Pl, Qb);
     }
 }
 
@@ -1535,6 +1191,10 @@ void prepare(K kernel, size_t smem) {
 }
 }  // namespace
 
+// Footprint rule of the cluster size: a part's node state (120 B per node) and
+// 52 B per element of its rows within the limit. A part that meets it has its
+// row tables wholly in shared memory in dr_mixed_node.cu's kernel, whose own
+// need is smaller.
 size_t mixed_fp32_smem(int part_cap, int free_cap, int elem_cap, int slot_cap, size_t limit) {
     const size_t plain = kFp32PlainNodeBytes * (size_t)part_cap;
     const size_t F = (size_t)free_cap, U = (size_t)elem_cap, S = (size_t)slot_cap;
@@ -1573,14 +1233,9 @@ int launch_dr_mixed(const DevMesh &m, const DevState &s, const DevResults &r, co
         prepare(dr_mixed_lead_kernel<false>, smem);
         e = cudaLaunchKernelEx(&cfg, dr_mixed_lead_kernel<false>, m, s, r, p, part_cap, free_cap,
                                elem_cap, slot_cap);
-    } else if (staged) {
-        prepare(dr_mixed_fp32_kernel<true>, smem);
-        e = cudaLaunchKernelEx(&cfg, dr_mixed_fp32_kernel<true>, m, s, r, p, part_cap, free_cap,
-                               elem_cap, slot_cap);
     } else {
-        prepare(dr_mixed_fp32_kernel<false>, smem);
-        e = cudaLaunchKernelEx(&cfg, dr_mixed_fp32_kernel<false>, m, s, r, p, part_cap, free_cap,
-                               elem_cap, slot_cap);
+        prepare(dr_mixed_fp32_kernel, smem);
+        e = cudaLaunchKernelEx(&cfg, dr_mixed_fp32_kernel, m, s, r, p, part_cap);
     }
     if (e != cudaSuccess) return (int)e;
     return (int)cudaGetLastError();
@@ -1598,12 +1253,9 @@ int occupancy_dr_mixed(int lead, int parts, int block, size_t smem, int part_cap
     } else if (lead) {
         prepare(dr_mixed_lead_kernel<false>, smem);
         e = cudaOccupancyMaxActiveClusters(&n, dr_mixed_lead_kernel<false>, &cfg);
-    } else if (staged) {
-        prepare(dr_mixed_fp32_kernel<true>, smem);
-        e = cudaOccupancyMaxActiveClusters(&n, dr_mixed_fp32_kernel<true>, &cfg);
     } else {
-        prepare(dr_mixed_fp32_kernel<false>, smem);
-        e = cudaOccupancyMaxActiveClusters(&n, dr_mixed_fp32_kernel<false>, &cfg);
+        prepare(dr_mixed_fp32_kernel, smem);
+        e = cudaOccupancyMaxActiveClusters(&n, dr_mixed_fp32_kernel, &cfg);
     }
     if (e != cudaSuccess) {
         cudaGetLastError();

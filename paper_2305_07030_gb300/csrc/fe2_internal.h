@@ -49,7 +49,15 @@ struct RveDesc {
     int32_t fp_free_max;
     int32_t fp_slot_max;
     int32_t fp_row_max;
-    int32_t pad_;
+    // FP32 phase of the mixed solver (dr_mixed_node.cu): most entries of a part's
+    // increment array (free nodes, the zero entry, copies of other parts' nodes)
+    // and most copies of its own nodes elsewhere; first copy; first global slot
+    // of the rows that do not fit in shared memory
+    int32_t part_q_max;
+    int32_t part_push_max;
+    int32_t flush_ok;  // lengths and rigidities far from FP32's limits (node_range_ok)
+    int64_t push0;
+    int64_t ell0;
 };
 
 // Launch shape of the FP64 cluster kernel: CTAs per cluster, capacities of one
@@ -59,7 +67,14 @@ struct Fp64Shape {
     int parts, part_max, free_max, slot_max, row_max;
     bool tsm, ssm;
 };
-// doubles per free node of that state: velocity, displacement, reference
+// CTAs per cluster of the FP32-phase kernel (dr_mixed_node.cu) and capacities of
+// one CTA: increment entries, free nodes, row slots, copies of own nodes, and the row slots held in
+// shared memory (the others are streamed from global memory).
+struct NodeShape {
+    int parts, q_cap, free_cap, slot_cap, push_cap, smem_slots;
+    int alt;  // order of the fused operations in an element's force (entry_forces)
+};
+// doubles per free node of the FP64 cluster kernel's state: velocity, displacement, reference
 // position, mass, damping factor, the mass's division estimate
 constexpr int kStateDoubles = 12;
 
@@ -96,6 +111,11 @@ struct DevMesh {
                                   // fp_node, and of the free nodes counted alone
     const int32_t *fp_row;        // per RVE n_free + 1 (from rp0): row offsets into
                                   // fp_csr_slot, free nodes in FP64 order
+    const uint16_t *qidx;         // FP32 phase, per CSR entry of a free node: the neighbour's
+                                  // place in the part's increment array
+    const int32_t *push_off;      // per RVE n_free + 1 (from rp0): copies of a free node in
+                                  // other parts, offsets from push0
+    const uint32_t *push;         // per copy: (part << 16 | place in its increment array)
 };
 
 // Mutable solver state (device).
@@ -114,7 +134,10 @@ struct DevState {
     double *gp, *fdp;             // FP64 energy check: previous internal and damping
                                   // force per free DOF [3][N]
     double *ualt;                 // FP64 cluster kernel: displacements of the last three
-                                  // evaluations, per RVE [3][3][n] at 9 node0, FP64 order
+                                  // evaluations, per RVE [3][3][n] at 9 node0, FP64 order;
+                                  // FP32 phase: increments of the last four, float4 [4][n]
+    float4 *ek0;                  // FP32 phase, row slots beyond shared memory: (r, EA)
+    float *ek1;                   //   and q_ref
     double *fpt;                  // FP64 cluster kernel: element forces [3][part slots]
                                   // when the table does not fit in shared memory
 };
@@ -181,6 +204,12 @@ size_t mixed_fp32_smem(int part_cap, int free_cap, int elem_cap, int slot_cap, s
 // Dynamic shared memory of the lead kernel for a class: one double-float
 // displacement per node, or two plus the element table when they fit.
 size_t mixed_lead_smem(int part_cap, int free_cap, int elem_cap, int slot_cap, size_t limit);
+// FP32 phase with row tables (dr_mixed_node.cu): dynamic shared memory, launch,
+// co-resident clusters.
+size_t mixed_node_smem(const NodeShape &sp);
+int launch_dr_mixed_node(const DevMesh &m, const DevState &s, const DevResults &r, const SolveParams &p,
+                         int clusters, int block, size_t smem, const NodeShape &sp, bool pair, void *stream);
+int occupancy_dr_mixed_node(int block, size_t smem, const NodeShape &sp, bool pair);
 // Whether a launch with `smem` bytes uses the shared-memory element table.
 bool mixed_staged(int lead, size_t smem, int part_cap);
 // FP64 cluster kernel (dr_fp64_cluster.cu): dynamic shared memory, launch,

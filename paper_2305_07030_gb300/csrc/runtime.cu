@@ -74,6 +74,9 @@ struct SizeClass {
     int free_max = 0;           // mixed: most free nodes in one part
     int elem_max = 0;           // mixed: most FP32-kernel table elements of one part
     int slot_max = 0;           // mixed: most FP32-kernel row slots of one part
+    // mixed, FP32 phase: how the row tables are held (node_kind_of), capacities
+    int node_kind = 0;
+    NodeShape node = {};
     std::vector<int32_t> rves;  // in scheduling order
     int32_t queue_off = 0;      // offset of its queue in the device queue buffer
 };
@@ -126,6 +129,11 @@ struct fe2_batch {
     DevBuf<int32_t> d_fp_csr_slot, d_fp_part_slot, d_fp_node, d_fp_part_off, d_fp_row;
     DevBuf<int4> d_fp_slot;
     DevBuf<double> d_ualt, d_fpt;
+    DevBuf<uint16_t> d_qidx;
+    DevBuf<int32_t> d_push_off;
+    DevBuf<uint32_t> d_push;
+    DevBuf<float4> d_ek0;
+    DevBuf<float> d_ek1;
     DevBuf<float2> d_eaf, d_eaf_lo, d_sa;
     DevBuf<float4> d_sv;
     DevBuf<float4> d_dh, d_dl;
@@ -199,6 +207,9 @@ struct fe2_batch {
         m.fp_node = d_fp_node.p;
         m.fp_part_off = d_fp_part_off.p;
         m.fp_row = d_fp_row.p;
+        m.qidx = d_qidx.p;
+        m.push_off = d_push_off.p;
+        m.push = d_push.p;
         return m;
     }
     DevState state() const {
@@ -214,6 +225,8 @@ struct fe2_batch {
         s.gp = d_gp.p;
         s.ualt = d_ualt.p;
         s.fpt = d_fpt.p;
+        s.ek0 = d_ek0.p;
+        s.ek1 = d_ek1.p;
         s.fdp = d_fdp.p;
         s.sa = d_sa.p;
         return s;
@@ -229,7 +242,7 @@ struct fe2_batch {
         d_rve.release(); d_X.release(); d_mass.release(); d_EA_csr.release(); d_L_csr.release();
         d_el_EA.release(); d_el_L.release(); d_Xh.release(); d_Xl.release(); d_imh.release();
         d_iml.release(); d_rowptr.release(); d_col.release(); d_col_part.release();
-        d_part_off.release(); d_el_a.release(); d_el_b.release(); d_csr_el.release(); d_fp_csr_slot.release(); d_fp_part_slot.release(); d_fp_node.release(); d_fp_part_off.release(); d_fp_row.release(); d_fp_slot.release(); d_ualt.release(); d_fpt.release(); d_tf.release(); d_sv.release(); d_sa.release(); d_eaf.release();
+        d_part_off.release(); d_el_a.release(); d_el_b.release(); d_csr_el.release(); d_fp_csr_slot.release(); d_fp_part_slot.release(); d_fp_node.release(); d_fp_part_off.release(); d_fp_row.release(); d_fp_slot.release(); d_ualt.release(); d_fpt.release(); d_qidx.release(); d_push_off.release(); d_push.release(); d_ek0.release(); d_ek1.release(); d_tf.release(); d_sv.release(); d_sa.release(); d_eaf.release();
         d_eaf_lo.release(); d_dh.release(); d_dl.release(); d_u.release(); d_v.release(); d_a.release(); d_xg.release();
         d_uh.release(); d_ul.release(); d_vh.release(); d_vl.release(); d_ah.release();
         d_al.release(); d_fg.release(); d_F.release(); d_sigma.release(); d_rel.release();
@@ -352,6 +365,16 @@ void rcb(std::vector<int> ids, int parts, const double *X, int64_t base,
     rcb(std::vector<int>(ids.begin() + half, ids.end()), parts / 2, X, base, out);
 }
 
+// How the FP32 phase holds an RVE's (or a class's) row tables: 2 = in shared
+// memory, 1 = the slots that do not fit in global memory, 0 = not even the
+// increments fit (the kernel without tables).
+int node_kind_of(NodeShape s, size_t limit) {
+    s.smem_slots = s.slot_cap;
+    if (mixed_node_smem(s) <= limit) return 2;
+    s.smem_slots = 0;
+    return mixed_node_smem(s) <= limit ? 1 : 0;
+}
+
 // Bucket RVEs into launch classes. FP64: by staged footprint (24 B/node), so
 // small RVEs are not limited by the occupancy of the largest; RVEs too big for
 // shared memory stage in L2 scratch. Mixed: by cluster size.
@@ -436,9 +459,7 @@ void build_classes(const std::vector<RveDesc> &rve, const std::vector<int32_t> &
         auto fits = [&](const SizeClass &c) {
             const bool l = !c.lead_staged || mixed_staged(1, mixed_lead_smem(c.part_max, c.free_max, c.elem_max,
                                                                              c.slot_max, limit), c.part_max);
-            const bool f = !c.fp32_staged || mixed_staged(0, mixed_fp32_smem(c.part_max, c.free_max, c.elem_max,
-                                                                             c.slot_max, limit), c.part_max);
-            return l && f;
+            return l && node_kind_of(c.node, limit) >= c.node_kind;
         };
         // first-fit decreasing: the RVEs with the largest shared-memory needs
         // open the classes, so that smaller ones fit under their maxima (the
@@ -461,21 +482,29 @@ void build_classes(const std::vector<RveDesc> &rve, const std::vector<int32_t> &
             one.slot_max = R.part_slot_max;
             one.lead_staged = mixed_staged(1, mixed_lead_smem(one.part_max, one.free_max, one.elem_max,
                                                               one.slot_max, limit), one.part_max);
-            one.fp32_staged = mixed_staged(0, mixed_fp32_smem(one.part_max, one.free_max, one.elem_max,
+            one.node = NodeShape{R.n_parts, R.part_q_max, one.free_max, one.slot_max, R.part_push_max, one.slot_max, 0};
+            one.node_kind = R.flush_ok ? node_kind_of(one.node, limit) : 0;
+            one.fp32_staged = one.node_kind > 0 &&
+                              mixed_staged(0, mixed_fp32_smem(one.part_max, one.free_max, one.elem_max,
                                                               one.slot_max, limit), one.part_max);
+            one.node.alt = !one.fp32_staged;
             const int bk = node_bucket(R.n_nodes);
             one.block_lead = g_tuning.block_lead[bk];
             one.block_fp32 = g_tuning.block_fp32[bk];
             bool placed = false;
             for (auto &c : out) {
                 if (c.parts != one.parts || c.lead_staged != one.lead_staged || c.fp32_staged != one.fp32_staged ||
-                    c.block_lead != one.block_lead || c.block_fp32 != one.block_fp32)
+                    c.node_kind != one.node_kind || c.block_lead != one.block_lead || c.block_fp32 != one.block_fp32)
                     continue;
                 SizeClass t = c;
                 t.part_max = std::max(t.part_max, one.part_max);
                 t.free_max = std::max(t.free_max, one.free_max);
                 t.elem_max = std::max(t.elem_max, one.elem_max);
                 t.slot_max = std::max(t.slot_max, one.slot_max);
+                t.node.q_cap = std::max(t.node.q_cap, one.node.q_cap);
+                t.node.free_cap = t.free_max;
+                t.node.slot_cap = t.node.smem_slots = t.slot_max;
+                t.node.push_cap = std::max(t.node.push_cap, one.node.push_cap);
                 if (!fits(t)) continue;
                 t.rves.push_back(p);
                 c = std::move(t);
@@ -493,8 +522,14 @@ void build_classes(const std::vector<RveDesc> &rve, const std::vector<int32_t> &
         std::stable_sort(out.begin(), out.end(), [](const SizeClass &a, const SizeClass &b) {
             return a.parts > b.parts;
         });
-        for (auto &c : out)
+        for (auto &c : out) {
             c.smem_bytes = mixed_plain_node_bytes(0) * c.part_max;
+            if (c.node_kind != 1) continue;
+            // as many row slots in shared memory as fit beside the rest
+            c.node.smem_slots = 0;
+            const size_t rest = mixed_node_smem(c.node), slot = sizeof(float4) + sizeof(float);
+            c.node.smem_slots = (int)((limit - rest) / slot) & ~31;
+        }
     }
     int32_t off = 0;
     for (auto &c : out) {
@@ -509,9 +544,11 @@ int mixed_block(int requested, bool lead, bool staged);
 // with the element table when the class is staged for that kernel.
 size_t class_smem(const SizeClass &c, int lead, size_t limit) {
     const bool st = lead ? c.lead_staged : c.fp32_staged;
-    if (!st) return mixed_plain_node_bytes(lead) * (size_t)c.part_max;
-    return lead ? mixed_lead_smem(c.part_max, c.free_max, c.elem_max, c.slot_max, limit)
-                : mixed_fp32_smem(c.part_max, c.free_max, c.elem_max, c.slot_max, limit);
+    const size_t plain = mixed_plain_node_bytes(lead) * (size_t)c.part_max;
+    if (lead) return st ? mixed_lead_smem(c.part_max, c.free_max, c.elem_max, c.slot_max, limit) : plain;
+    // the plain footprint bounds the part size whatever the kernel
+    const size_t node = c.node_kind > 0 ? mixed_node_smem(c.node) : 0;
+    return st ? node : std::max(plain, node);
 }
 
 // CTA size of a mixed class's kernel: the caller's request, else the tuned
@@ -587,6 +624,11 @@ struct HostLayout {
     // FP64 order of the nodes, the parts' offsets in it, and the free nodes'
     // row offsets (DevMesh::fp_node, fp_part_off, fp_row)
     std::vector<int32_t> fpSlot, fpCsrSlot, fpPartSlot, fpNode, fpPartOff, fpRow;
+    // FP32-phase kernel: DevMesh::qidx, push_off and push; total global row slots
+    std::vector<uint16_t> qidx;
+    std::vector<int32_t> pushOff;
+    std::vector<uint32_t> push;
+    int64_t n_ell = 0;
 };
 
 // The FP64 cluster kernel's part of the layout (see HostLayout): its parts are
@@ -654,6 +696,85 @@ void build_fp64_parts(const int64_t *elem_off, HostLayout &L) {
         }
         frow[x] = pos;
         for (int r = C; r <= kMaxParts; ++r) ps[r] = ns;
+    }
+}
+
+// Whether the FP32 phase may use the flush-to-zero forms of the reciprocal square
+// root and the division: they differ from the others only where a squared length
+// or a force is subnormal. A squared length of the iterations is lr2 + h, zero or
+// at least 6e-8 lr2, so lengths from 1e-12 to 1e6 keep it normal; with
+// rigidities from 1e-15 to 1e15 a flushed force term is below 1e-31 of the force
+// at unit strain.
+bool node_range_ok(const HostLayout &L, const RveDesc &R) {
+    const int64_t N = (int64_t)L.perm_to_orig.size();
+    for (int64_t e = R.elem0; e < R.elem0 + R.n_elems; ++e) {
+        double l2 = 0.0;
+        for (int c = 0; c < 3; ++c) {
+            const double d = L.X[c * N + R.node0 + L.Elb[e]] - L.X[c * N + R.node0 + L.Ela[e]];
+            l2 += d * d;
+        }
+        if (!(l2 >= 1e-24 && l2 <= 1e12 && L.ElEA[e] >= 1e-15 && L.ElEA[e] <= 1e15)) return false;
+    }
+    return true;
+}
+
+// FP32-phase tables (dr_mixed_node.cu). A part's increment array holds its free
+// nodes, one zero entry for every fixed node, and a copy of each free neighbour
+// of another part; a node's copies are listed with the node, one per part that
+// has a free neighbour of it.
+void build_node_tables(size_t smem_cap, HostLayout &L) {
+    L.qidx.assign(L.colp.size(), 0);
+    L.pushOff.assign(L.row.size(), 0);
+    L.push.clear();
+    L.n_ell = 0;
+    for (RveDesc &R : L.rve) {
+        const int p = (int)(&R - L.rve.data()), C = R.n_parts;
+        const int32_t *pf = L.part.data() + (size_t)p * 2 * (kMaxParts + 1);
+        const int32_t *row = L.row.data() + R.rp0, *colp = L.colp.data() + R.csr0;
+        int32_t *off = L.pushOff.data() + R.rp0;
+        auto n_free = [&](int r) { return pf[r + 1] - pf[r]; };
+        std::vector<int32_t> q(C);  // entries of each part's increment array
+        for (int r = 0; r < C; ++r) q[r] = n_free(r) + 1;
+        R.push0 = (int64_t)L.push.size();
+        R.part_push_max = 0;
+        R.ell0 = L.n_ell;
+        R.flush_ok = 0;
+        if (R.part_max > 0xffff) {  // beyond the mixed solver (and its 16-bit indices)
+            R.part_q_max = R.part_max;
+            continue;
+        }
+        for (int s = 0; s < C; ++s) {
+            for (int k = pf[s]; k < pf[s + 1]; ++k) {
+                off[k] = (int32_t)(L.push.size() - R.push0);
+                uint32_t seen = 0;
+                for (int32_t e = row[k]; e < row[k + 1]; ++e) {
+                    const int r = colp[e] >> 16, loc = colp[e] & 0xffff;
+                    if (r == s || loc >= n_free(r) || (seen >> r & 1)) continue;
+                    seen |= 1u << r;
+                    L.push.push_back(((uint32_t)r << 16) | (uint32_t)(q[r]++ & 0xffff));
+                }
+            }
+            R.part_push_max = std::max(R.part_push_max, (int32_t)(L.push.size() - R.push0) - off[pf[s]]);
+        }
+        off[R.n_free] = (int32_t)(L.push.size() - R.push0);
+        for (int s = 0; s < C; ++s)
+            for (int k = pf[s]; k < pf[s + 1]; ++k)
+                for (int32_t e = row[k]; e < row[k + 1]; ++e) {
+                    const int r = colp[e] >> 16, loc = colp[e] & 0xffff;
+                    int at = n_free(s);  // fixed: the zero entry
+                    if (loc < n_free(r)) {
+                        at = loc;
+                        for (int32_t x = off[pf[r] + loc]; r != s && x < off[pf[r] + loc + 1]; ++x)
+                            if ((int)(L.push[R.push0 + x] >> 16) == s) at = (int)(L.push[R.push0 + x] & 0xffff);
+                    }
+                    L.qidx[R.csr0 + e] = (uint16_t)at;
+                }
+        R.part_q_max = *std::max_element(q.begin(), q.end());
+        // global row slots, where shared memory does not hold them all (also
+        // when the RVE shares a launch with others)
+        const NodeShape sp = {C, R.part_q_max, R.part_free_max, R.part_slot_max, R.part_push_max, R.part_slot_max, 0};
+        R.flush_ok = node_range_ok(L, R);
+        if (R.flush_ok && node_kind_of(sp, smem_cap) == 1) L.n_ell += (int64_t)C * R.part_slot_max;
     }
 }
 
@@ -829,6 +950,7 @@ void build_layout(int32_t n_rve, const int64_t *node_off, const double *X, const
         }
     }
     build_fp64_parts(elem_off, L);
+    build_node_tables(smem_cap, L);
 }
 
 }  // namespace
@@ -911,6 +1033,11 @@ extern "C" fe2_status fe2_batch_create(int32_t n_rve, const int64_t *node_off, c
     A(b->d_fp_part_off.alloc(L.fpPartOff.size()), "fp_part_off");
     A(b->d_fp_row.alloc(N + n_rve), "fp_row");
     A(b->d_ualt.alloc(9 * N), "ualt");
+    A(b->d_qidx.alloc(2 * E), "qidx");
+    A(b->d_push_off.alloc(N + n_rve), "push_off");
+    A(b->d_push.alloc(std::max<size_t>(1, L.push.size())), "push");
+    A(b->d_ek0.alloc(L.n_ell), "ek0");
+    A(b->d_ek1.alloc(L.n_ell), "ek1");
     A(b->d_fpt.alloc(3 * std::max<size_t>(1, n_fslots)), "fpt");
     A(b->d_tf.alloc(3 * E), "tf");
     A(b->d_sv.alloc(N), "sv");
@@ -964,6 +1091,9 @@ extern "C" fe2_status fe2_batch_create(int32_t n_rve, const int64_t *node_off, c
     H2D(b->d_fp_node.p, L.fpNode.data(), sizeof(int32_t) * N, "fp_node");
     H2D(b->d_fp_part_off.p, L.fpPartOff.data(), sizeof(int32_t) * L.fpPartOff.size(), "fp_part_off");
     H2D(b->d_fp_row.p, L.fpRow.data(), sizeof(int32_t) * (N + n_rve), "fp_row");
+    H2D(b->d_qidx.p, L.qidx.data(), sizeof(uint16_t) * 2 * E, "qidx");
+    H2D(b->d_push_off.p, L.pushOff.data(), sizeof(int32_t) * (N + n_rve), "push_off");
+    H2D(b->d_push.p, L.push.data(), sizeof(uint32_t) * L.push.size(), "push");
     H2D(b->d_rowptr.p, hrow.data(), sizeof(int32_t) * (N + n_rve), "rowptr");
     H2D(b->d_part_off.p, hpart.data(), sizeof(int32_t) * hpart.size(), "part_off");
     H2D(b->d_el_a.p, hEla.data(), sizeof(int32_t) * E, "el_a");
@@ -1218,6 +1348,18 @@ int resident_fp64_cluster(fe2_batch *b, const SizeClass &c, int block) {
     return r;
 }
 
+// Resident clusters of a mixed class's kernel (cached likewise; kinds 7 to 10:
+// the FP32-phase kernel with row tables, by its capacities).
+int resident_mixed(fe2_batch *b, const SizeClass &c, int lead, int block, size_t smem, bool pair = false) {
+    if (lead || c.node_kind == 0) return resident_of(b, lead, c.parts, block, smem, c.part_max);
+    const auto key = std::make_tuple(7 + (c.node_kind == 1) + 2 * pair, c.parts, block, smem, c.node.free_cap);
+    auto it = b->occ.find(key);
+    if (it != b->occ.end()) return it->second;
+    const int r = occupancy_dr_mixed_node(block, smem, c.node, pair);
+    b->occ[key] = r;
+    return r;
+}
+
 // Timing event around a launch: recorded as a graph node while capturing.
 cudaError_t record_timing(cudaEvent_t e, cudaStream_t s, bool capturing) {
     return capturing ? cudaEventRecordWithFlags(e, s, cudaEventRecordExternal) : cudaEventRecord(e, s);
@@ -1275,16 +1417,24 @@ fe2_status launch_class(fe2_batch *b, const fe2_opts &o, const SizeClass &c, Sol
             const size_t limit = b->smem_optin - 16384;
             const size_t smem = class_smem(c, lead, limit);
             const int block = class_block(c, lead, o.block_threads);
-            const int resident = resident_of(b, lead, c.parts, block, smem, c.part_max);
-            if (resident < 1)
-                return fail(FE2_ECUDA, "no cluster of " + std::to_string(c.parts) + " CTAs with " +
-                                           std::to_string(smem) + " B shared memory fits");
+            const bool node = !lead && c.node_kind > 0;
+            // FP32 phase with two CTAs per SM when the queue is longer than one
+            // round at one per SM. An iteration then takes 1.2 to 1.6 times as
+            // long on twice the clusters: 64 RVEs of 5000 nodes x 3600
+            // iterations 22.2 ms against 30.5, 256 of 1000 x 1800 9.0 against
+            // 11.2.
+            const int one = resident_mixed(b, c, lead, block, smem);
+            const int two = node && nq > one && c.node_kind == 2 && !c.node.alt ? resident_mixed(b, c, lead, block, smem, true) : 0;
+            const bool pair = two >= 2 * one;
+            const int resident = pair ? two : one;
             if (timed) {
                 if (*timed + 2 > (int)b->tev.size()) return fail(FE2_ECUDA, "too many launch classes");
                 CUDA_TRY(record_timing(b->tev[*timed], s, capturing));
             }
-            const int e = launch_dr_mixed(M, S, R, P, lead, std::min(nq, resident), c.parts, block, smem,
-                                          c.part_max, c.free_max, c.elem_max, c.slot_max, s);
+            const int clusters = std::min(nq, resident);
+            const int e = node ? launch_dr_mixed_node(M, S, R, P, clusters, block, smem, c.node, pair, s)
+                               : launch_dr_mixed(M, S, R, P, lead, clusters, c.parts, block, smem, c.part_max,
+                                                 c.free_max, c.elem_max, c.slot_max, s);
             if (e != 0) return fail(FE2_ECUDA, std::string("launch: ") + cudaGetErrorString((cudaError_t)e));
             if (timed) {
                 CUDA_TRY(record_timing(b->tev[*timed + 1], s, capturing));
@@ -1377,7 +1527,8 @@ fe2_status warm_shapes(fe2_batch *b, const fe2_opts &o) {
                                             std::to_string(b->rve[big].n_nodes) +
                                             " nodes) exceeds the mixed solver's shared memory; use FE2_PREC_FP64");
             }
-            if (resident_of(b, lead, c.parts, class_block(c, lead, o.block_threads), smem, c.part_max) < 1)
+            if (!lead) resident_mixed(b, c, lead, class_block(c, lead, o.block_threads), smem, true);
+            if (resident_mixed(b, c, lead, class_block(c, lead, o.block_threads), smem) < 1)
                 return fail(FE2_ECUDA, "no cluster of " + std::to_string(c.parts) + " CTAs with " +
                                            std::to_string(smem) + " B shared memory fits");
         }
