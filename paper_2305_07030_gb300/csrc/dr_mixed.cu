@@ -2,9 +2,16 @@
 // thread-block cluster per RVE, three persistent launches per size class (the
 // double-float lead, the FP32 phase, the double-float resume of stalled RVEs).
 //
+// The lead runs in dr_mixed_lead.cu's kernel and the FP32 phase in
+// dr_mixed_node.cu's, both with their tables on chip. The kernels of this file,
+// which re-read the CSR rows from L2, remain for parts whose displacements or
+// increments (with the copies of neighbours in other parts) do not fit in shared
+// memory, and for lengths and rigidities near the limits of FP32.
+//
 // Layout. The RVE is split spatially into `parts` pieces, one per CTA of the
-// cluster; a CTA stages the state of its own nodes in its shared memory and
-// reads neighbours owned by other CTAs through distributed shared memory. The
+// cluster; a CTA stages the state of its own nodes in its shared memory and (in
+// this file) reads neighbours owned by other CTAs through distributed shared
+// memory. The
 // paper used one thread team per sub-problem (Section III); a cluster lets one
 // sub-problem span several SMs.
 //
@@ -32,11 +39,6 @@
 //    and across warps and CTAs in double-float; the threshold (tol f_ref)^2 is
 //    formed in FP64 once per RVE; the stress sum is FP64.
 //
-// The FP32 phase runs in dr_mixed_node.cu's kernel, one thread per free node
-// with its row tables on chip. The FP32 kernel of this file, which re-reads the
-// CSR rows from L2, remains for parts whose increments alone (with the copies
-// of neighbours in other parts) do not fit in shared memory.
-//
 // Synchronisation of this file's FP32 kernel. One cluster barrier per
 // iteration. Five displacement-increment buffers rotate. Each node's owner
 // thread computes the next iteration's increment right after the node's
@@ -46,12 +48,6 @@
 // n-3 across the cluster (DSMEM reads) and leaves a verdict. All warps read
 // the verdict after the next barrier. If the test succeeded, they finish with
 // the state of the tested evaluation, whose buffer is still intact.
-//
-// The element forces of the lead come from a shared-memory element table. Each
-// element with an end among a CTA's free nodes is evaluated once per
-// iteration, spread evenly over the threads. Each node then sums the +-
-// results of its CSR row in row order. The two ends see exactly opposite
-// values, so this equals the per-direction evaluation.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -73,8 +69,8 @@ constexpr size_t kFp32PlainNodeBytes = (1 + kBufs) * sizeof(float4);
 // Per-node bytes of the footprint rule that sets the cluster size
 // (mixed_fp32_smem).
 constexpr size_t kFp32NodeBytes = (1 + kBufs + 1) * sizeof(float4) + sizeof(float2);
-// Lead kernel shared memory per node without the element table: one
-// double-float displacement (hi, lo float4); with the table, two of them.
+// Lead kernel without tables (this file): shared memory per node, one
+// double-float displacement (hi, lo float4).
 constexpr size_t kLeadPlainNodeBytes = 2 * sizeof(float4);
 __host__ __device__ constexpr size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
 
@@ -216,345 +212,6 @@ __device__ __forceinline__ void edge_increment(const float4 &pi, const float4 &q
     g2 += qref * e2 + dq * (r2 + e2);
 }
 
-// Per-part element tables of the lead kernel, in shared memory when they fit
-// (STAGE); otherwise every row is re-read from the global CSR each iteration.
-//
-// Element list: each element with at least one end among this CTA's free
-// nodes appears once. An element between two own free nodes belongs to the
-// row of its lower local index (end a) and is used with the opposite sign by
-// the other row (end b); any other element belongs to the row of its own free
-// end a (lead_loop_staged gives an element's entries).
-// Node rows are laid out ELL-style in slabs of 32 consecutive own free nodes:
-// entry j of node k sits at slot SS[k / 32] + 32 j + k % 32 and holds
-// (element << 1 | 1 if the node is end b), so a warp reads 32 consecutive
-// slots at every step; the entries keep the CSR row order.
-struct Staged {
-    float4 *K0;    // per element
-    float4 *K1;    // per element
-    uint32_t *NS;  // per slot
-    int *SD;       // per own free node: row length
-    int *EB;       // per own free node: first element of its row
-    int *SS;       // per slab + 1: first slot
-    float4 *KA;    // per element
-    float4 *TA;    // per element
-    float2 *TB;    // per element
-    float4 *VH;    // per own free node: (v.hi, a.hi x)
-    float4 *VL;    // per own free node: (v.lo, a.lo x)
-    float4 *AY;    // per own free node: (a.hi y, a.hi z, a.lo y, a.lo z)
-};
-
-__device__ __forceinline__ float4 ld_cluster(uint32_t a) {
-    float4 v;
-    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-                 : "r"(a));
-    return v;
-}
-__device__ __forceinline__ float4 ld_local(uint32_t a) {
-    float4 v;
-    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-                 : "r"(a));
-    return v;
-}
-
-// Whether CSR entry (rank r, local loc) of own free node k is used with the
-// opposite sign: its element belongs to the lower own free end.
-__device__ __forceinline__ bool b_end(int r, int loc, int k, const Part &pt) {
-    return r == pt.me && loc < pt.nfr && loc < k;
-}
-
-// Row lengths and element counts of this CTA's free nodes (first pass), then
-// (thread 0) element offsets and slab bases. The caller synchronises the CTA
-// before the second part.
-__device__ void element_counts(const DevMesh &M, const RveDesc &R, const Part &pt, const int32_t *rowptr,
-                               const Staged &st) {
-    for (int k = threadIdx.x; k < pt.nfr; k += blockDim.x) {
-        const int beg = rowptr[pt.f0 + k], deg = rowptr[pt.f0 + k + 1] - beg;
-        int own = 0;
-        for (int e = 0; e < deg; ++e) {
-            const int cp = M.col_part[R.csr0 + beg + e];
-            own += !b_end(cp >> 16, cp & 0xffff, k, pt);
-        }
-        st.SD[k] = deg;
-        st.EB[k] = own;
-    }
-}
-__device__ void element_offsets(MixedShared &sh, const Part &pt, const Staged &st) {
-    int base = 0;
-    for (int k = 0; k < pt.nfr; ++k) {
-        const int c = st.EB[k];
-        st.EB[k] = base;
-        base += c;
-    }
-    sh.elems = base;
-    int slots = 0, s = 0;
-    for (int k0 = 0; k0 < pt.nfr; k0 += 32, ++s) {
-        int w = 0;
-        for (int k = k0; k < k0 + 32 && k < pt.nfr; ++k) w = max(w, st.SD[k]);
-        st.SS[s] = slots;
-        slots += 32 * w;
-    }
-    st.SS[s] = slots;
-    sh.slots = slots;
-}
-
-// ---------------------------------------------------------------------------
-// lead kernel with the element table (STAGE)
-// ---------------------------------------------------------------------------
-// The lead's element table (element list and node rows: element_counts,
-// element_offsets), with per element
-//   K0 = (D, L).hi, K1 = (D, L).lo  (D = X_b - X_a, double-float),
-//   KA = ((EA/L).hi, (EA/L).lo, shared::cta address of a's displacement in
-//        buffer 0, address of b's: shared::cta, or shared::cluster with bit 0
-//        set when b lives in another CTA),
-//   TA, TB = the iteration's double-float force on a (hi xyz + lo x; lo yz).
-// Displacements rotate through two buffers (hi then lo arrays per buffer), so
-// one cluster barrier per iteration suffices.
-__device__ void lead_elements(const MixedShared &sh, const DevMesh &M, const RveDesc &R, const Part &pt,
-                              const int32_t *rowptr, const float4 *U0, const Staged &st) {
-    for (int k = threadIdx.x; k < pt.nfr; k += blockDim.x) {
-        const int beg = rowptr[pt.f0 + k], deg = st.SD[k];
-        int u = st.EB[k];
-        int slot = st.SS[k >> 5] + (k & 31);
-        for (int e = 0; e < deg; ++e, slot += 32) {
-            const int64_t kk = R.csr0 + beg + e;
-            const int cp = M.col_part[kk];
-            const int r = cp >> 16, loc = cp & 0xffff;
-            if (b_end(r, loc, k, pt)) {
-                const int jb = rowptr[pt.f0 + loc], jd = st.SD[loc];
-                int v = st.EB[loc];
-                for (int x = 0; x < jd; ++x) {
-                    const int cq = M.col_part[R.csr0 + jb + x];
-                    const int rq = cq >> 16, lq = cq & 0xffff;
-                    if (rq == pt.me && lq == k) break;
-                    v += !b_end(rq, lq, loc, pt);
-                }
-                st.NS[slot] = ((uint32_t)v << 1) | 1u;
-                continue;
-            }
-            const float2 eh = M.eaf[kk], el = M.eaf_lo[kk];
-            const df kax = df_mul({eh.x, el.x}, {eh.y, el.y});
-            const uint32_t qb = smem_addr(U0 + loc);
-            const uint32_t ab = r == pt.me ? qb : (cluster_addr(qb, (uint32_t)r) | 1u);
-            st.K0[u] = M.dh[kk];
-            st.K1[u] = M.dl[kk];
-            st.KA[u] = make_float4(kax.hi, kax.lo, __uint_as_float(smem_addr(U0 + k)), __uint_as_float(ab));
-            st.NS[slot] = (uint32_t)u << 1;
-            ++u;
-        }
-    }
-}
-
-__device__ __forceinline__ float4 ld_any(uint32_t a) {
-    return (a & 1u) ? ld_cluster(a & ~1u) : ld_local(a);
-}
-
-// Double-float element force in displacement form (the operations of
-// gather_df) for element u, written to TA/TB.
-__device__ __forceinline__ void lead_element_force(const Staged &st, int u, const float4 &pi,
-                                                   const float4 &qi, const float4 &pj, const float4 &qj) {
-    const float4 Dh = st.K0[u], Dl = st.K1[u];
-    const float2 kax = make_float2(st.KA[u].x, st.KA[u].y);
-    const df e0 = df_sub({pj.x, qj.x}, {pi.x, qi.x}), e1 = df_sub({pj.y, qj.y}, {pi.y, qi.y}),
-             e2 = df_sub({pj.z, qj.z}, {pi.z, qi.z});
-    const df D0 = {Dh.x, Dl.x}, D1 = {Dh.y, Dl.y}, D2 = {Dh.z, Dl.z}, L = {Dh.w, Dl.w};
-    const df d0 = df_add(D0, e0), d1 = df_add(D1, e1), d2 = df_add(D2, e2);
-    const df h = df_add(df_add(df_mul(e0, df_add(D0, d0)), df_mul(e1, df_add(D1, d1))),
-                        df_mul(e2, df_add(D2, d2)));
-    const df l2 = df_add(df_sqr(L), h);
-    const df rl = df_rsqrt(l2);
-    const df l = df_mul(l2, rl);
-    const df q = df_mul(df_mul({kax.x, kax.y}, df_mul(h, rl)), df_rcp(df_add(l, L)));
-    const df t0 = df_mul(q, d0), t1 = df_mul(q, d1), t2 = df_mul(q, d2);
-    st.TA[u] = make_float4(t0.hi, t1.hi, t2.hi, t0.lo);
-    st.TB[u] = make_float2(t1.lo, t2.lo);
-}
-
-// Elements ua and ub (ub < 0: none) of displacement buffer offset toff: all
-// loads first, then the two independent chains.
-__device__ __forceinline__ void lead_element_pair(const Staged &st, int ua, int ub, uint32_t toff,
-                                                  uint32_t lo_off) {
-    const float4 ka = st.KA[ua];
-    const uint32_t a0 = __float_as_uint(ka.z) + toff, a1 = __float_as_uint(ka.w) + toff;
-    const float4 pi = ld_local(a0), qi = ld_local(a0 + lo_off);
-    const float4 pj = ld_any(a1), qj = ld_any(a1 + lo_off);
-    if (ub >= 0) {
-        const float4 kb = st.KA[ub];
-        const uint32_t b0 = __float_as_uint(kb.z) + toff, b1 = __float_as_uint(kb.w) + toff;
-        const float4 pi2 = ld_local(b0), qi2 = ld_local(b0 + lo_off);
-        const float4 pj2 = ld_any(b1), qj2 = ld_any(b1 + lo_off);
-        lead_element_force(st, ua, pi, qi, pj, qj);
-        lead_element_force(st, ub, pi2, qi2, pj2, qj2);
-    } else {
-        lead_element_force(st, ua, pi, qi, pj, qj);
-    }
-}
-
-// Double-float iterations until the relative residual first drops below
-// lead_tol (or lead_iters), NaN or max_iter. The residual test of evaluation
-// n-2 runs in one testing warp per CTA between the arrive and the wait of
-// iteration n; the others read its verdict after the next barrier, and the
-// hand-over happens at the end of that iteration, so the handed-over state
-// (u, v, a and g_ref of one evaluation) is consistent. The hand-over state's
-// own residual is then totalled by every warp.
-__device__ void lead_loop_staged(cg::cluster_group &cl, MixedShared &sh, const DevMesh &M,
-                                 const DevState &S, const RveDesc &R, const Part &pt,
-                                 const SolveParams &P, float4 *U0, const Staged &st, int part_cap,
-                                 int elem_cap, int slot_cap, const df &lead2, const df &thresh2,
-                                 const df &dt, const df &hdt, const df &cdf, int64_t &it,
-                                 int &status, df &r2, df &k2) {
-    const int64_t it0 = it;  // evaluations before this call (resume: > 0)
-    const int n = R.n_nodes, m = pt.m();
-    const int64_t n0 = R.node0, b3 = 3 * n0;
-    const int32_t *rowptr = M.rowptr + R.rp0;
-    float *uh = S.uh + b3, *ul = S.ul + b3, *vh = S.vh + b3, *vl = S.vl + b3;
-    float *ah = S.ah + b3, *al = S.al + b3, *fg = S.fg + b3;
-    const float *imh = M.imh + n0, *iml = M.iml + n0;
-    const bool want_k = P.want_ke != 0;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const bool test_warp = warp == (int)(blockDim.x >> 5) - 1;
-    // buffer t: hi at U0 + 2 t part_cap, lo at U0 + (2 t + 1) part_cap
-    const uint32_t lo_off = (uint32_t)(sizeof(float4) * part_cap), buf_off = 2 * lo_off;
-    // buffer 1 starts as a copy of buffer 0 (the fixed nodes never change)
-    for (int k = threadIdx.x; k < m; k += blockDim.x) {
-        U0[2 * part_cap + k] = U0[k];
-        U0[3 * part_cap + k] = U0[part_cap + k];
-    }
-    element_counts(M, R, pt, rowptr, st);
-    __syncthreads();
-    if (threadIdx.x == 0) element_offsets(sh, pt, st);
-    cl.sync();
-    bool over = false;
-    for (int r = 0; r < pt.C; ++r)
-        over |= *cl.map_shared_rank(&sh.elems, r) > elem_cap || *cl.map_shared_rank(&sh.slots, r) > slot_cap;
-    if (over) {  // sized on the host for every part; all CTAs agree
-        status = RVE_NAN;
-        return;
-    }
-    lead_elements(sh, M, R, pt, rowptr, U0, st);
-    const int n_el = sh.elems;
-    // velocity and acceleration of the own free nodes live in shared memory
-    // during the loop (owner thread k in every phase)
-    for (int k = threadIdx.x; k < pt.nfr; k += blockDim.x) {
-        const int i = pt.f0 + k;
-        st.VH[k] = make_float4(vh[i], vh[n + i], vh[2 * n + i], ah[i]);
-        st.VL[k] = make_float4(vl[i], vl[n + i], vl[2 * n + i], al[i]);
-        st.AY[k] = make_float4(ah[n + i], ah[2 * n + i], al[n + i], al[2 * n + i]);
-    }
-    __syncthreads();
-
-    bool vpend = false;
-    for (;;) {
-        const int64_t nidx = it + 1;  // this iteration's evaluation
-        const int t = (int)(nidx & 1), tp = t ^ 1;
-        const int vb = (int)(nidx & 3);
-        {
-            const float4 *Hp = U0 + 2 * tp * part_cap, *Lp = Hp + part_cap;
-            float4 *Hc = U0 + 2 * t * part_cap, *Lc = Hc + part_cap;
-            for (int k = threadIdx.x; k < pt.nfr; k += blockDim.x) {
-                const float4 ph = Hp[k], pl = Lp[k];
-                const float4 vhk = st.VH[k], vlk = st.VL[k], ay = st.AY[k];
-                const float uh0[3] = {ph.x, ph.y, ph.z}, ul0[3] = {pl.x, pl.y, pl.z};
-                const float v_h[3] = {vhk.x, vhk.y, vhk.z}, v_l[3] = {vlk.x, vlk.y, vlk.z};
-                const float a_h[3] = {vhk.w, ay.x, ay.y}, a_l[3] = {vlk.w, ay.z, ay.w};
-                df u[3], v[3];
-                for (int c = 0; c < 3; ++c) {
-                    v[c] = df_add({v_h[c], v_l[c]}, df_mul(hdt, {a_h[c], a_l[c]}));
-                    u[c] = df_add({uh0[c], ul0[c]}, df_mul(dt, v[c]));
-                }
-                st.VH[k] = make_float4(v[0].hi, v[1].hi, v[2].hi, vhk.w);
-                st.VL[k] = make_float4(v[0].lo, v[1].lo, v[2].lo, vlk.w);
-                Hc[k] = make_float4(u[0].hi, u[1].hi, u[2].hi, 0.f);
-                Lc[k] = make_float4(u[0].lo, u[1].lo, u[2].lo, 0.f);
-            }
-        }
-        const bool test_now = nidx >= it0 + 3;  // two evaluations of this call published
-        cluster_arrive();
-        if (test_now && test_warp) {
-            const Verdict v = residual_verdict(sh, pt, (int)((nidx - 2) & 3), 0, lead2, want_k, INT64_MAX);
-            if (lane == 0) sh.vd[vb] = v;
-        }
-        cluster_wait();
-        const int code = vpend ? sh.vd[(nidx - 1) & 3].code : -1;
-        vpend = test_now;
-        // element forces in displacement form (gather_df's operations), two
-        // elements per thread in flight
-        const uint32_t toff = (uint32_t)t * buf_off;
-        const int step = blockDim.x;
-        for (int u0 = threadIdx.x; u0 < n_el; u0 += 2 * step) {
-            lead_element_pair(st, u0, u0 + step < n_el ? u0 + step : -1, toff, lo_off);
-        }
-        __syncthreads();
-        // node sums in CSR row order, then acceleration and velocity
-        float rs = 0.f, kes = 0.f;
-        for (int k = threadIdx.x; k < pt.nfr; k += blockDim.x) {
-            const int deg = st.SD[k];
-            int sl = st.SS[k >> 5] + (k & 31);
-            df g[3] = {df_from(0.f), df_from(0.f), df_from(0.f)};
-            for (int j = 0; j < deg; ++j, sl += 32) {
-                const uint32_t w = st.NS[sl];
-                const float4 ta = st.TA[w >> 1];
-                const float2 tb = st.TB[w >> 1];
-                df f0 = {ta.x, ta.w}, f1 = {ta.y, tb.x}, f2 = {ta.z, tb.y};
-                if (w & 1u) {
-                    f0 = {-f0.hi, -f0.lo}; f1 = {-f1.hi, -f1.lo}; f2 = {-f2.hi, -f2.lo};
-                }
-                g[0] = df_add(g[0], f0); g[1] = df_add(g[1], f1); g[2] = df_add(g[2], f2);
-            }
-            const int i = pt.f0 + k;
-            const df im = {imh[i], iml[i]};
-            const float4 vhk = st.VH[k], vlk = st.VL[k];
-            const float v_h[3] = {vhk.x, vhk.y, vhk.z}, v_l[3] = {vlk.x, vlk.y, vlk.z};
-            float vv = 0.f;
-            df v[3], a[3];
-            for (int c = 0; c < 3; ++c) {
-                v[c] = {v_h[c], v_l[c]};
-                a[c] = df_sub(df_mul(g[c], im), df_mul(cdf, v[c]));
-                v[c] = df_add(v[c], df_mul(hdt, a[c]));
-                fg[c * n + i] = g[c].hi;
-                rs += g[c].hi * g[c].hi;
-                vv += v[c].hi * v[c].hi;
-            }
-            st.VH[k] = make_float4(v[0].hi, v[1].hi, v[2].hi, a[0].hi);
-            st.VL[k] = make_float4(v[0].lo, v[1].lo, v[2].lo, a[0].lo);
-            st.AY[k] = make_float4(a[1].hi, a[2].hi, a[1].lo, a[2].lo);
-            if (want_k) kes += 0.5f * vv / imh[i];
-        }
-        for (int o = 16; o > 0; o >>= 1) rs += __shfl_xor_sync(0xffffffffu, rs, o);
-        if (want_k)
-            for (int o = 16; o > 0; o >>= 1) kes += __shfl_xor_sync(0xffffffffu, kes, o);
-        if (lane == 0) {
-            sh.own[vb][0][warp] = rs;
-            if (want_k) sh.own[vb][1][warp] = kes;
-        }
-        it = nidx;
-        if (code == RVE_NAN) break;
-        if (it >= P.max_iter) break;
-        if (P.lead_iters >= 0 ? it >= P.lead_iters : code == RVE_OK) break;
-    }
-    // the hand-over evaluation's own residual, by every warp
-    cl.sync();
-    const Verdict v = residual_verdict(sh, pt, (int)(it & 3), it, thresh2, want_k, P.max_iter);
-    r2 = {v.r2h, v.r2l};
-    k2 = {v.k2h, v.k2l};
-    status = v.code >= 0 ? v.code : RVE_PENDING;
-    // the double-float displacement for the FP32 kernel and the output
-    const int t = (int)(it & 1);
-    const float4 *Hc = U0 + 2 * t * part_cap, *Lc = Hc + part_cap;
-    for (int k = threadIdx.x; k < pt.nfr; k += blockDim.x) {
-        const int i = pt.f0 + k;
-        const float4 ph = Hc[k], pl = Lc[k];
-        uh[i] = ph.x; uh[n + i] = ph.y; uh[2 * n + i] = ph.z;
-        ul[i] = pl.x; ul[n + i] = pl.y; ul[2 * n + i] = pl.z;
-        const float4 vhk = st.VH[k], vlk = st.VL[k], ay = st.AY[k];
-        vh[i] = vhk.x; vh[n + i] = vhk.y; vh[2 * n + i] = vhk.z;
-        vl[i] = vlk.x; vl[n + i] = vlk.y; vl[2 * n + i] = vlk.z;
-        ah[i] = vhk.w; ah[n + i] = ay.x; ah[2 * n + i] = ay.y;
-        al[i] = vlk.w; al[n + i] = ay.z; al[2 * n + i] = ay.w;
-    }
-}
-
 // No FP32 increment on top of the double-float displacement.
 struct NoInc {
     __device__ float4 operator()(int) const { return make_float4(0.f, 0.f, 0.f, 0.f); }
@@ -564,10 +221,9 @@ struct NoInc {
 // lead kernel: setup (Algorithm 1 lines up to the loop) and the double-float
 // iterations
 // ---------------------------------------------------------------------------
-template <bool STAGE>
 __device__ void lead_rve(cg::cluster_group &cl, MixedShared &sh, const DevMesh &M, const DevState &S,
                          const DevResults &O, const SolveParams &P, int p, float4 *Pl, float4 *Q0,
-                         const Staged &st, int part_cap, int elem_cap, int slot_cap, int &rb) {
+                         int &rb) {
     const RveDesc R = M.rve[p];
     const Part pt = make_part(M, R, p, (int)cl.block_rank(), (int)cl.num_blocks());
     const int n = R.n_nodes, m = pt.m();
@@ -669,24 +325,6 @@ __device__ void lead_rve(cg::cluster_group &cl, MixedShared &sh, const DevMesh &
     const int64_t it0 = it;
     int status = RVE_PENDING;
     df r2 = df_from(0.f), k2 = df_from(0.f);
-    if (STAGE) {
-        SolveParams Q = P;
-        Q.lead_iters = lead_iters;
-        for (;;) {
-            lead_loop_staged(cl, sh, M, S, R, pt, Q, Pl, st, part_cap, elem_cap, slot_cap, lead2, thresh2,
-                             dt, hdt, cdf, it, status, r2, k2);
-            // The loop stops two evaluations after the tested one; when
-            // resuming, the state it stops at must itself be converged, else
-            // the iteration goes on from that state.
-            if (!P.resume || status != RVE_PENDING) break;
-            for (int k = threadIdx.x; k < m; k += blockDim.x) {
-                const int i = pt.gidx(k);
-                Pl[k] = make_float4(uh[i], uh[n + i], uh[2 * n + i], 0.f);
-                Q0[k] = make_float4(ul[i], ul[n + i], ul[2 * n + i], 0.f);
-            }
-            cl.sync();
-        }
-    } else {
     // L lanes share a node's edges; lane 0 of group k owns node k's state in
     // every phase, so consecutive phases need no barrier between them.
     int L = 1;
@@ -742,7 +380,6 @@ __device__ void lead_rve(cg::cluster_group &cl, MixedShared &sh, const DevMesh &
         if (df_le(r2, thresh2)) { status = RVE_OK; break; }
         if (it >= P.max_iter) { status = RVE_MAXITER; break; }
         if (lead_iters >= 0 ? it >= lead_iters : df_le(r2, lead2)) break;
-    }
     }
     if (P.resume) {
         if (pt.me == 0 && threadIdx.x == 0) O.lead[p] += it - it0;
@@ -1093,48 +730,20 @@ __device__ void fp32_rve(cg::cluster_group &cl, MixedShared &sh, const DevMesh &
 
 }  // namespace
 
-template <bool STAGE>
-__global__ void __launch_bounds__(512, 1) dr_mixed_lead_kernel(DevMesh M, DevState S, DevResults O,
-                                                            SolveParams P, int part_cap, int free_cap,
-                                                            int elem_cap, int slot_cap) {
+__global__ void __launch_bounds__(512, 1) dr_mixed_plain_lead_kernel(DevMesh M, DevState S, DevResults O,
+                                                                     SolveParams P, int part_cap) {
     extern __shared__ __align__(16) float4 dsm[];
     __shared__ MixedShared sh;
     cg::cluster_group cl = cg::this_cluster();
     float4 *Pl = dsm, *Q0 = dsm + part_cap;
     float4 *Qb[kBufs];
     for (int b = 0; b < kBufs; ++b) Qb[b] = Q0;
-    Staged st = {};
-    if (STAGE) {
-        // layout as in mixed_lead_smem: two displacement buffers, velocity and
-        // acceleration, then the tables
-        st.VH = dsm + 4 * (size_t)part_cap;
-        st.VL = st.VH + free_cap;
-        st.AY = st.VL + free_cap;
-        char *base = reinterpret_cast<char *>(st.AY + free_cap);
-        st.K0 = reinterpret_cast<float4 *>(base);
-        base += 16 * (size_t)elem_cap;
-        st.K1 = reinterpret_cast<float4 *>(base);
-        base += 16 * (size_t)elem_cap;
-        st.KA = reinterpret_cast<float4 *>(base);
-        base += 16 * (size_t)elem_cap;
-        st.TA = reinterpret_cast<float4 *>(base);
-        base += 16 * (size_t)elem_cap;
-        st.TB = reinterpret_cast<float2 *>(base);
-        base += 8 * (size_t)elem_cap;
-        st.NS = reinterpret_cast<uint32_t *>(base);
-        base += 4 * (size_t)slot_cap;
-        st.SD = reinterpret_cast<int *>(base);
-        base += 4 * (size_t)free_cap;
-        st.EB = reinterpret_cast<int *>(base);
-        base += 4 * (size_t)free_cap;
-        st.SS = reinterpret_cast<int *>(base);
-    }
     map_remote(cl, sh, Pl, Qb, (int)cl.num_blocks());
     int rb = 0;
     for (;;) {
         const int item = next_item(cl, sh, P.counter + (P.resume ? 2 : 0));
         if (item >= P.queue_len) return;
-        lead_rve<STAGE>(cl, sh, M, S, O, P, P.queue[item], Pl, Q0, st, part_cap, elem_cap, slot_cap, rb);
+        lead_rve(cl, sh, M, S, O, P, P.queue[item], Pl, Q0, rb);
     }
 }
 
@@ -1203,6 +812,9 @@ size_t mixed_fp32_smem(int part_cap, int free_cap, int elem_cap, int slot_cap, s
     return staged <= limit ? staged : plain;
 }
 
+// Footprint rule of the lead: with the table (dr_mixed_lead.cu, STAGED) when a
+// part's displacements, state and element records are within the limit by this
+// count; that kernel's own need is smaller.
 size_t mixed_lead_smem(int part_cap, int free_cap, int elem_cap, int slot_cap, size_t limit) {
     const size_t plain = kLeadPlainNodeBytes * (size_t)part_cap;
     const size_t F = (size_t)free_cap, U = (size_t)elem_cap, S = (size_t)slot_cap;
@@ -1218,46 +830,23 @@ bool mixed_staged(int lead, size_t smem, int part_cap) {
 size_t mixed_plain_node_bytes(int lead) { return lead ? kLeadPlainNodeBytes : kFp32PlainNodeBytes; }
 
 int launch_dr_mixed(const DevMesh &m, const DevState &s, const DevResults &r, const SolveParams &p,
-                    int lead, int clusters, int parts, int block, size_t smem, int part_cap,
-                    int free_cap, int elem_cap, int slot_cap, void *stream) {
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
+                    int lead, int clusters, int parts, int block, size_t smem, int part_cap, void *stream) {
     cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = mixed_config(clusters, parts, block, smem, attr, st);
-    const bool staged = mixed_staged(lead, smem, part_cap);
-    cudaError_t e;
-    if (lead && staged) {
-        prepare(dr_mixed_lead_kernel<true>, smem);
-        e = cudaLaunchKernelEx(&cfg, dr_mixed_lead_kernel<true>, m, s, r, p, part_cap, free_cap,
-                               elem_cap, slot_cap);
-    } else if (lead) {
-        prepare(dr_mixed_lead_kernel<false>, smem);
-        e = cudaLaunchKernelEx(&cfg, dr_mixed_lead_kernel<false>, m, s, r, p, part_cap, free_cap,
-                               elem_cap, slot_cap);
-    } else {
-        prepare(dr_mixed_fp32_kernel, smem);
-        e = cudaLaunchKernelEx(&cfg, dr_mixed_fp32_kernel, m, s, r, p, part_cap);
-    }
+    cudaLaunchConfig_t cfg = mixed_config(clusters, parts, block, smem, attr, static_cast<cudaStream_t>(stream));
+    const auto kernel = lead ? dr_mixed_plain_lead_kernel : dr_mixed_fp32_kernel;
+    prepare(kernel, smem);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, m, s, r, p, part_cap);
     if (e != cudaSuccess) return (int)e;
     return (int)cudaGetLastError();
 }
 
-int occupancy_dr_mixed(int lead, int parts, int block, size_t smem, int part_cap) {
+int occupancy_dr_mixed(int lead, int parts, int block, size_t smem) {
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = mixed_config(parts * 64, parts, block, smem, attr, nullptr);
-    const bool staged = mixed_staged(lead, smem, part_cap);
+    const auto kernel = lead ? dr_mixed_plain_lead_kernel : dr_mixed_fp32_kernel;
+    prepare(kernel, smem);
     int n = 0;
-    cudaError_t e;
-    if (lead && staged) {
-        prepare(dr_mixed_lead_kernel<true>, smem);
-        e = cudaOccupancyMaxActiveClusters(&n, dr_mixed_lead_kernel<true>, &cfg);
-    } else if (lead) {
-        prepare(dr_mixed_lead_kernel<false>, smem);
-        e = cudaOccupancyMaxActiveClusters(&n, dr_mixed_lead_kernel<false>, &cfg);
-    } else {
-        prepare(dr_mixed_fp32_kernel, smem);
-        e = cudaOccupancyMaxActiveClusters(&n, dr_mixed_fp32_kernel, &cfg);
-    }
-    if (e != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }

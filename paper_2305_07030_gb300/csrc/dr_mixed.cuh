@@ -1,6 +1,6 @@
-// Helpers shared by the mixed-precision kernels (dr_mixed.cu, dr_mixed_node.cu):
-// a part of an RVE, cluster barriers, the residual verdict and the end of a
-// solve.
+// Helpers shared by the mixed-precision kernels (dr_mixed.cu, dr_mixed_lead.cu,
+// dr_mixed_node.cu): a part of an RVE, cluster barriers, row tables, the residual
+// test and the end of a solve.
 #pragma once
 #include <cooperative_groups.h>
 

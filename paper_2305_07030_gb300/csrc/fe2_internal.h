@@ -55,8 +55,10 @@ struct RveDesc {
     // of the rows that do not fit in shared memory
     int32_t part_q_max;
     int32_t part_push_max;
+    int32_t part_u_max;   // lead: most entries of a part's displacement array
     int32_t flush_ok;  // lengths and rigidities far from FP32's limits (node_range_ok)
     int64_t push0;
+    int64_t fix0;         // lead: first entry of lead_fix
     int64_t ell0;
 };
 
@@ -73,6 +75,14 @@ struct Fp64Shape {
 struct NodeShape {
     int parts, q_cap, free_cap, slot_cap, push_cap, smem_slots;
     int alt;  // order of the fused operations in an element's force (entry_forces)
+};
+// CTAs per cluster of the lead kernel (dr_mixed_lead.cu) and capacities of one
+// CTA: displacement entries, free nodes, element slots, row entries (ELL), copies
+// of own nodes; whether the part meets the footprint rule (staged) and whether
+// the element constants are in shared memory.
+struct LeadShape {
+    int parts, u_cap, free_cap, elem_cap, slot_cap, push_cap;
+    bool staged, ksm;
 };
 // doubles per free node of the FP64 cluster kernel's state: velocity, displacement, reference
 // position, mass, damping factor, the mass's division estimate
@@ -99,8 +109,9 @@ struct DevMesh {
     const int32_t *csr_el;        // per CSR entry: RVE-local element << 1, | 1 when
                                   // the row's node is the element's second node
                                   // (caller orientation)
-    const int4 *fp_slot;          // FP64 cluster kernel, per element slot: (element,
-                                  // first end, second end, 0), ends as (part << 16 | index)
+    const int4 *fp_slot;          // FP64 cluster kernel and lead, per element slot: (element,
+                                  // first end, second end, CSR entry << 1 | 1 when its row
+                                  // is the second end's), ends as (part << 16 | index)
     const int32_t *fp_csr_slot;   // per row entry of a free node, in FP64 order from csr0:
                                   // part-relative slot << 1 | 1 when the node is the
                                   // element's second end
@@ -115,6 +126,12 @@ struct DevMesh {
                                   // place in the part's increment array
     const int32_t *push_off;      // per RVE n_free + 1 (from rp0): copies of a free node in
                                   // other parts, offsets from push0
+    const uint32_t *lead_ends;    // lead, per element slot (fp_slot): places of its ends in the
+                                  // part's displacement array, first | second << 16
+    const int32_t *lead_fix;      // lead: per part the fixed neighbours of its free nodes
+                                  // (RVE-local ids, from fix0)
+    const int32_t *lead_fix_off;  // per RVE 2*(kMaxParts+1): the parts' offsets into them, and
+                                  // the place of each part's first in its displacement array
     const uint32_t *push;         // per copy: (part << 16 | place in its increment array)
 };
 
@@ -191,19 +208,23 @@ int launch_setup(int32_t n_rve, int64_t n_el, int64_t n_csr, RveDesc *rve,
                  void *stream);
 int launch_dr_fp64(const DevMesh &m, const DevState &s, const DevResults &r,
                    const SolveParams &p, int grid, int block, size_t smem, void *stream);
-// Mixed solver: one thread-block cluster of `parts` CTAs per RVE; two
-// persistent launches per class, the double-float lead (lead = 1) and then
-// the FP32 phase (lead = 0).
+// Mixed solver without tables (dr_mixed.cu): one thread-block cluster of `parts`
+// CTAs per RVE; lead = 1 the double-float lead, 0 the FP32 phase.
 int launch_dr_mixed(const DevMesh &m, const DevState &s, const DevResults &r,
                     const SolveParams &p, int lead, int clusters, int parts, int block,
-                    size_t smem, int part_cap, int free_cap, int elem_cap, int slot_cap,
-                    void *stream);
+                    size_t smem, int part_cap, void *stream);
 // Dynamic shared memory of the FP32 kernel for a class: the staged node state,
 // plus each part's element table and rows when they fit within `limit` bytes.
 size_t mixed_fp32_smem(int part_cap, int free_cap, int elem_cap, int slot_cap, size_t limit);
 // Dynamic shared memory of the lead kernel for a class: one double-float
 // displacement per node, or two plus the element table when they fit.
 size_t mixed_lead_smem(int part_cap, int free_cap, int elem_cap, int slot_cap, size_t limit);
+// Lead kernel (dr_mixed_lead.cu): dynamic shared memory, launch, co-resident
+// clusters.
+size_t lead_smem(const LeadShape &sp);
+int launch_dr_mixed_lead(const DevMesh &m, const DevState &s, const DevResults &r, const SolveParams &p,
+                         int clusters, int block, const LeadShape &sp, void *stream);
+int occupancy_dr_mixed_lead(int block, const LeadShape &sp);
 // FP32 phase with row tables (dr_mixed_node.cu): dynamic shared memory, launch,
 // co-resident clusters.
 size_t mixed_node_smem(const NodeShape &sp);
@@ -223,7 +244,7 @@ int occupancy_dr_fp64_cluster(int block, const Fp64Shape &sp);
 size_t mixed_plain_node_bytes(int lead);
 // Resident CTAs per SM (FP64) / co-resident clusters (mixed) for a launch shape.
 int occupancy_dr_fp64(int smem_positions, int block, size_t smem);
-int occupancy_dr_mixed(int lead, int parts, int block, size_t smem, int part_cap);
+int occupancy_dr_mixed(int lead, int parts, int block, size_t smem);
 
 // Naive comparator: scratch sized for the largest RVE, and one RVE's solve.
 struct NaiveScratch {

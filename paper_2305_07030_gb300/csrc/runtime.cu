@@ -77,6 +77,9 @@ struct SizeClass {
     // mixed, FP32 phase: how the row tables are held (node_kind_of), capacities
     int node_kind = 0;
     NodeShape node = {};
+    // mixed, lead: dr_mixed_lead.cu's kernel (false: the one without tables)
+    bool lead_kernel = false;
+    LeadShape lead = {};
     std::vector<int32_t> rves;  // in scheduling order
     int32_t queue_off = 0;      // offset of its queue in the device queue buffer
 };
@@ -131,7 +134,8 @@ struct fe2_batch {
     DevBuf<double> d_ualt, d_fpt;
     DevBuf<uint16_t> d_qidx;
     DevBuf<int32_t> d_push_off;
-    DevBuf<uint32_t> d_push;
+    DevBuf<uint32_t> d_push, d_lead_ends;
+    DevBuf<int32_t> d_lead_fix, d_lead_fix_off;
     DevBuf<float4> d_ek0;
     DevBuf<float> d_ek1;
     DevBuf<float2> d_eaf, d_eaf_lo, d_sa;
@@ -210,6 +214,9 @@ struct fe2_batch {
         m.qidx = d_qidx.p;
         m.push_off = d_push_off.p;
         m.push = d_push.p;
+        m.lead_ends = d_lead_ends.p;
+        m.lead_fix = d_lead_fix.p;
+        m.lead_fix_off = d_lead_fix_off.p;
         return m;
     }
     DevState state() const {
@@ -242,7 +249,7 @@ struct fe2_batch {
         d_rve.release(); d_X.release(); d_mass.release(); d_EA_csr.release(); d_L_csr.release();
         d_el_EA.release(); d_el_L.release(); d_Xh.release(); d_Xl.release(); d_imh.release();
         d_iml.release(); d_rowptr.release(); d_col.release(); d_col_part.release();
-        d_part_off.release(); d_el_a.release(); d_el_b.release(); d_csr_el.release(); d_fp_csr_slot.release(); d_fp_part_slot.release(); d_fp_node.release(); d_fp_part_off.release(); d_fp_row.release(); d_fp_slot.release(); d_ualt.release(); d_fpt.release(); d_qidx.release(); d_push_off.release(); d_push.release(); d_ek0.release(); d_ek1.release(); d_tf.release(); d_sv.release(); d_sa.release(); d_eaf.release();
+        d_part_off.release(); d_el_a.release(); d_el_b.release(); d_csr_el.release(); d_fp_csr_slot.release(); d_fp_part_slot.release(); d_fp_node.release(); d_fp_part_off.release(); d_fp_row.release(); d_fp_slot.release(); d_ualt.release(); d_fpt.release(); d_qidx.release(); d_push_off.release(); d_push.release(); d_lead_ends.release(); d_lead_fix.release(); d_lead_fix_off.release(); d_ek0.release(); d_ek1.release(); d_tf.release(); d_sv.release(); d_sa.release(); d_eaf.release();
         d_eaf_lo.release(); d_dh.release(); d_dl.release(); d_u.release(); d_v.release(); d_a.release(); d_xg.release();
         d_uh.release(); d_ul.release(); d_vh.release(); d_vl.release(); d_ah.release();
         d_al.release(); d_fg.release(); d_F.release(); d_sigma.release(); d_rel.release();
@@ -457,8 +464,7 @@ void build_classes(const std::vector<RveDesc> &rve, const std::vector<int32_t> &
         // packed first-fit into classes whose combined tables still fit.
         const size_t limit = cap;
         auto fits = [&](const SizeClass &c) {
-            const bool l = !c.lead_staged || mixed_staged(1, mixed_lead_smem(c.part_max, c.free_max, c.elem_max,
-                                                                             c.slot_max, limit), c.part_max);
+            const bool l = !c.lead_kernel || lead_smem(c.lead) <= limit;
             return l && node_kind_of(c.node, limit) >= c.node_kind;
         };
         // first-fit decreasing: the RVEs with the largest shared-memory needs
@@ -482,6 +488,12 @@ void build_classes(const std::vector<RveDesc> &rve, const std::vector<int32_t> &
             one.slot_max = R.part_slot_max;
             one.lead_staged = mixed_staged(1, mixed_lead_smem(one.part_max, one.free_max, one.elem_max,
                                                               one.slot_max, limit), one.part_max);
+            // element constants in shared memory when they fit
+            one.lead = LeadShape{R.n_parts, R.part_u_max, one.free_max, R.fp_slot_max, one.slot_max, R.part_push_max,
+                                 one.lead_staged, one.lead_staged};
+            if (lead_smem(one.lead) > limit) one.lead.ksm = false;
+            one.lead_kernel = R.part_max <= 0xffff && lead_smem(one.lead) <= limit;
+            one.lead_staged = one.lead_staged && one.lead_kernel;
             one.node = NodeShape{R.n_parts, R.part_q_max, one.free_max, one.slot_max, R.part_push_max, one.slot_max, 0};
             one.node_kind = R.flush_ok ? node_kind_of(one.node, limit) : 0;
             one.fp32_staged = one.node_kind > 0 &&
@@ -494,7 +506,8 @@ void build_classes(const std::vector<RveDesc> &rve, const std::vector<int32_t> &
             bool placed = false;
             for (auto &c : out) {
                 if (c.parts != one.parts || c.lead_staged != one.lead_staged || c.fp32_staged != one.fp32_staged ||
-                    c.node_kind != one.node_kind || c.block_lead != one.block_lead || c.block_fp32 != one.block_fp32)
+                    c.node_kind != one.node_kind || c.lead_kernel != one.lead_kernel || c.lead.ksm != one.lead.ksm ||
+                    c.block_lead != one.block_lead || c.block_fp32 != one.block_fp32)
                     continue;
                 SizeClass t = c;
                 t.part_max = std::max(t.part_max, one.part_max);
@@ -502,6 +515,11 @@ void build_classes(const std::vector<RveDesc> &rve, const std::vector<int32_t> &
                 t.elem_max = std::max(t.elem_max, one.elem_max);
                 t.slot_max = std::max(t.slot_max, one.slot_max);
                 t.node.q_cap = std::max(t.node.q_cap, one.node.q_cap);
+                t.lead.u_cap = std::max(t.lead.u_cap, one.lead.u_cap);
+                t.lead.free_cap = t.free_max;
+                t.lead.elem_cap = std::max(t.lead.elem_cap, one.lead.elem_cap);
+                t.lead.slot_cap = t.slot_max;
+                t.lead.push_cap = std::max(t.lead.push_cap, one.lead.push_cap);
                 t.node.free_cap = t.free_max;
                 t.node.slot_cap = t.node.smem_slots = t.slot_max;
                 t.node.push_cap = std::max(t.node.push_cap, one.node.push_cap);
@@ -542,10 +560,10 @@ int mixed_block(int requested, bool lead, bool staged);
 
 // Dynamic shared memory of a mixed class's lead (lead = 1) or FP32 kernel:
 // with the element table when the class is staged for that kernel.
-size_t class_smem(const SizeClass &c, int lead, size_t limit) {
+size_t class_smem(const SizeClass &c, int lead) {
     const bool st = lead ? c.lead_staged : c.fp32_staged;
     const size_t plain = mixed_plain_node_bytes(lead) * (size_t)c.part_max;
-    if (lead) return st ? mixed_lead_smem(c.part_max, c.free_max, c.elem_max, c.slot_max, limit) : plain;
+    if (lead) return !c.lead_kernel ? plain : st ? lead_smem(c.lead) : std::max(plain, lead_smem(c.lead));
     // the plain footprint bounds the part size whatever the kernel
     const size_t node = c.node_kind > 0 ? mixed_node_smem(c.node) : 0;
     return st ? node : std::max(plain, node);
@@ -628,6 +646,9 @@ struct HostLayout {
     std::vector<uint16_t> qidx;
     std::vector<int32_t> pushOff;
     std::vector<uint32_t> push;
+    // lead kernel: DevMesh::lead_ends, lead_fix, lead_fix_off
+    std::vector<uint32_t> leadEnds;
+    std::vector<int32_t> leadFix, leadFixOff;
     int64_t n_ell = 0;
 };
 
@@ -684,7 +705,7 @@ void build_fp64_parts(const int64_t *elem_off, HostLayout &L) {
                         L.fpSlot.push_back(e);
                         L.fpSlot.push_back(ref[L.Ela[e0 + e]]);
                         L.fpSlot.push_back(ref[L.Elb[e0 + e]]);
-                        L.fpSlot.push_back(0);
+                        L.fpSlot.push_back((q << 1) | (w & 1));
                     }
                     L.fpCsrSlot[R.csr0 + pos] = ((slot_of[e] - first) << 1) | (w & 1);
                 }
@@ -727,6 +748,10 @@ void build_node_tables(size_t smem_cap, HostLayout &L) {
     L.pushOff.assign(L.row.size(), 0);
     L.push.clear();
     L.n_ell = 0;
+    L.leadEnds.assign(L.fpSlot.size() / 4, 0);
+    L.leadFix.clear();
+    L.leadFixOff.assign(L.rve.size() * 2 * (kMaxParts + 1), 0);
+    std::vector<int32_t> fix_at, fix_part;  // a fixed node's place in the part that saw it last
     for (RveDesc &R : L.rve) {
         const int p = (int)(&R - L.rve.data()), C = R.n_parts;
         const int32_t *pf = L.part.data() + (size_t)p * 2 * (kMaxParts + 1);
@@ -740,7 +765,7 @@ void build_node_tables(size_t smem_cap, HostLayout &L) {
         R.ell0 = L.n_ell;
         R.flush_ok = 0;
         if (R.part_max > 0xffff) {  // beyond the mixed solver (and its 16-bit indices)
-            R.part_q_max = R.part_max;
+            R.part_q_max = R.part_u_max = R.part_max;
             continue;
         }
         for (int s = 0; s < C; ++s) {
@@ -770,6 +795,42 @@ void build_node_tables(size_t smem_cap, HostLayout &L) {
                     L.qidx[R.csr0 + e] = (uint16_t)at;
                 }
         R.part_q_max = *std::max_element(q.begin(), q.end());
+        // lead: the ends of every element slot in its part's displacement array
+        // (the increment array's places, then copies of the fixed neighbours)
+        const int32_t *pg = pf + (kMaxParts + 1), *ps = L.fpPartSlot.data() + (size_t)p * (kMaxParts + 1);
+        int32_t *fo = L.leadFixOff.data() + (size_t)p * 2 * (kMaxParts + 1), *fat = fo + (kMaxParts + 1);
+        R.fix0 = (int64_t)L.leadFix.size();
+        R.part_u_max = 0;
+        fix_at.assign(R.n_nodes - R.n_free, 0);
+        fix_part.assign(R.n_nodes - R.n_free, -1);
+        for (int s = 0; s < C; ++s) {
+            fo[s] = (int32_t)(L.leadFix.size() - R.fix0);
+            fat[s] = q[s];
+            int32_t at = q[s];
+            for (int32_t u = ps[s]; u < ps[s + 1]; ++u) {
+                const int32_t *sl = L.fpSlot.data() + 4 * (R.slot0 + u);
+                uint32_t place[2];
+                for (int e = 0; e < 2; ++e) {
+                    const int r = sl[1 + e] >> 16, loc = sl[1 + e] & 0xffff;
+                    if (loc >= n_free(r)) {
+                        const int f = pg[r] + loc - n_free(r);
+                        if (fix_part[f] != s) {
+                            fix_part[f] = s;
+                            fix_at[f] = at++;
+                            L.leadFix.push_back(R.n_free + f);
+                        }
+                        place[e] = (uint32_t)fix_at[f];
+                    } else {
+                        place[e] = (uint32_t)loc;
+                        for (int32_t x = off[pf[r] + loc]; r != s && x < off[pf[r] + loc + 1]; ++x)
+                            if ((int)(L.push[R.push0 + x] >> 16) == s) place[e] = L.push[R.push0 + x] & 0xffffu;
+                    }
+                }
+                L.leadEnds[R.slot0 + u] = place[0] | (place[1] << 16);
+            }
+            R.part_u_max = std::max(R.part_u_max, at);
+        }
+        for (int s = C; s <= kMaxParts; ++s) fo[s] = (int32_t)(L.leadFix.size() - R.fix0);
         // global row slots, where shared memory does not hold them all (also
         // when the RVE shares a launch with others)
         const NodeShape sp = {C, R.part_q_max, R.part_free_max, R.part_slot_max, R.part_push_max, R.part_slot_max, 0};
@@ -1036,6 +1097,9 @@ extern "C" fe2_status fe2_batch_create(int32_t n_rve, const int64_t *node_off, c
     A(b->d_qidx.alloc(2 * E), "qidx");
     A(b->d_push_off.alloc(N + n_rve), "push_off");
     A(b->d_push.alloc(std::max<size_t>(1, L.push.size())), "push");
+    A(b->d_lead_ends.alloc(std::max<size_t>(1, L.leadEnds.size())), "lead_ends");
+    A(b->d_lead_fix.alloc(std::max<size_t>(1, L.leadFix.size())), "lead_fix");
+    A(b->d_lead_fix_off.alloc(L.leadFixOff.size()), "lead_fix_off");
     A(b->d_ek0.alloc(L.n_ell), "ek0");
     A(b->d_ek1.alloc(L.n_ell), "ek1");
     A(b->d_fpt.alloc(3 * std::max<size_t>(1, n_fslots)), "fpt");
@@ -1093,6 +1157,9 @@ extern "C" fe2_status fe2_batch_create(int32_t n_rve, const int64_t *node_off, c
     H2D(b->d_fp_row.p, L.fpRow.data(), sizeof(int32_t) * (N + n_rve), "fp_row");
     H2D(b->d_qidx.p, L.qidx.data(), sizeof(uint16_t) * 2 * E, "qidx");
     H2D(b->d_push_off.p, L.pushOff.data(), sizeof(int32_t) * (N + n_rve), "push_off");
+    H2D(b->d_lead_ends.p, L.leadEnds.data(), sizeof(uint32_t) * L.leadEnds.size(), "lead_ends");
+    H2D(b->d_lead_fix.p, L.leadFix.data(), sizeof(int32_t) * L.leadFix.size(), "lead_fix");
+    H2D(b->d_lead_fix_off.p, L.leadFixOff.data(), sizeof(int32_t) * L.leadFixOff.size(), "lead_fix_off");
     H2D(b->d_push.p, L.push.data(), sizeof(uint32_t) * L.push.size(), "push");
     H2D(b->d_rowptr.p, hrow.data(), sizeof(int32_t) * (N + n_rve), "rowptr");
     H2D(b->d_part_off.p, hpart.data(), sizeof(int32_t) * hpart.size(), "part_off");
@@ -1249,7 +1316,6 @@ extern "C" fe2_status fe2_batch_plan(int32_t n_rve, const int64_t *node_off, con
     std::vector<SizeClass> cls;
     build_classes(L.rve, L.part_free_max, (size_t)smem_optin, FE2_PREC_MIXED, cls);
     if (n_classes) *n_classes = (int32_t)cls.size();
-    const size_t limit = (size_t)smem_optin - 16384;  // as in launch_class
     for (size_t k = 0; k < cls.size(); ++k) {
         const SizeClass &c = cls[k];
         if (rve_class)
@@ -1258,7 +1324,7 @@ extern "C" fe2_status fe2_batch_plan(int32_t n_rve, const int64_t *node_off, con
         if (class_parts) class_parts[k] = c.parts;
         if (class_rves) class_rves[k] = (int32_t)c.rves.size();
         for (int lead = 1; lead >= 0; --lead) {
-            const size_t sm = class_smem(c, lead, limit);
+            const size_t sm = class_smem(c, lead);
             const bool st = lead ? c.lead_staged : c.fp32_staged;
             const size_t at = 2 * k + (lead ? 0 : 1);
             if (smem) smem[at] = (int64_t)sm;
@@ -1331,7 +1397,7 @@ int resident_of(fe2_batch *b, int kind, int parts, int block, size_t smem, int p
     if (it != b->occ.end()) return it->second;
     // kind: 0/1 mixed FP32/lead, 2 FP64 single CTA (parts = positions staged)
     const int r = kind == 2 ? occupancy_dr_fp64(parts, block, smem)
-                            : occupancy_dr_mixed(kind, parts, block, smem, part_cap);
+                            : occupancy_dr_mixed(kind, parts, block, smem);
     b->occ[key] = r;
     return r;
 }
@@ -1349,8 +1415,16 @@ int resident_fp64_cluster(fe2_batch *b, const SizeClass &c, int block) {
 }
 
 // Resident clusters of a mixed class's kernel (cached likewise; kinds 7 to 10:
-// the FP32-phase kernel with row tables, by its capacities).
+// the FP32-phase kernel with row tables, 11 to 14: the lead kernel).
 int resident_mixed(fe2_batch *b, const SizeClass &c, int lead, int block, size_t smem, bool pair = false) {
+    if (lead && c.lead_kernel) {
+        const auto key = std::make_tuple(11 + 2 * c.lead.staged + c.lead.ksm, c.parts, block, lead_smem(c.lead), 0);
+        auto it = b->occ.find(key);
+        if (it != b->occ.end()) return it->second;
+        const int r = occupancy_dr_mixed_lead(block, c.lead);
+        b->occ[key] = r;
+        return r;
+    }
     if (lead || c.node_kind == 0) return resident_of(b, lead, c.parts, block, smem, c.part_max);
     const auto key = std::make_tuple(7 + (c.node_kind == 1) + 2 * pair, c.parts, block, smem, c.node.free_cap);
     auto it = b->occ.find(key);
@@ -1414,8 +1488,7 @@ fe2_status launch_class(fe2_batch *b, const fe2_opts &o, const SizeClass &c, Sol
         for (int step = 0; step < 3; ++step) {
             const int lead = step == 1 ? 0 : 1;
             P.resume = step == 2 ? 1 : 0;
-            const size_t limit = b->smem_optin - 16384;
-            const size_t smem = class_smem(c, lead, limit);
+            const size_t smem = class_smem(c, lead);
             const int block = class_block(c, lead, o.block_threads);
             const bool node = !lead && c.node_kind > 0;
             // FP32 phase with two CTAs per SM when the queue is longer than one
@@ -1432,9 +1505,9 @@ fe2_status launch_class(fe2_batch *b, const fe2_opts &o, const SizeClass &c, Sol
                 CUDA_TRY(record_timing(b->tev[*timed], s, capturing));
             }
             const int clusters = std::min(nq, resident);
-            const int e = node ? launch_dr_mixed_node(M, S, R, P, clusters, block, smem, c.node, pair, s)
-                               : launch_dr_mixed(M, S, R, P, lead, clusters, c.parts, block, smem, c.part_max,
-                                                 c.free_max, c.elem_max, c.slot_max, s);
+            const int e = node                    ? launch_dr_mixed_node(M, S, R, P, clusters, block, smem, c.node, pair, s)
+                          : lead && c.lead_kernel ? launch_dr_mixed_lead(M, S, R, P, clusters, block, c.lead, s)
+                                                  : launch_dr_mixed(M, S, R, P, lead, clusters, c.parts, block, smem, c.part_max, s);
             if (e != 0) return fail(FE2_ECUDA, std::string("launch: ") + cudaGetErrorString((cudaError_t)e));
             if (timed) {
                 CUDA_TRY(record_timing(b->tev[*timed + 1], s, capturing));
@@ -1519,7 +1592,7 @@ fe2_status warm_shapes(fe2_batch *b, const fe2_opts &o) {
             continue;
         }
         for (int lead = 1; lead >= 0; --lead) {
-            const size_t smem = class_smem(c, lead, limit);
+            const size_t smem = class_smem(c, lead);
             if (smem > limit) {
                 int32_t big = c.rves.front();
                 for (int32_t p : c.rves) if (b->rve[p].n_nodes > b->rve[big].n_nodes) big = p;

@@ -1,7 +1,8 @@
-"""The FP32 phase's kernel with row tables (csrc/dr_mixed_node.cu): its variants
-(one slab per warp in registers, several slabs, two CTAs per SM, tables partly in
-global memory) run the same arithmetic, so the displacement does not depend on
-the variant, the CTA size or the other RVEs of the launch."""
+"""The mixed solver's table kernels. The FP32 phase's (csrc/dr_mixed_node.cu): its
+variants (one slab per warp in registers, several slabs, two CTAs per SM, tables
+partly in global memory) run the same arithmetic, so the displacement does not
+depend on the variant, the CTA size or the other RVEs of the launch. The lead's
+(csrc/dr_mixed_lead.cu): likewise, and against the oracle."""
 import numpy as np
 import pytest
 
