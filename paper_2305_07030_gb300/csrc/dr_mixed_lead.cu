@@ -577,7 +577,7 @@ namespace {
 using LeadKernel = void (*)(DevMesh, DevState, DevResults, SolveParams, LeadShape);
 
 LeadKernel pick_lead(const LeadShape &sp) {
-    if (!sp.staged) return dr_mixed_lead_kernel<false, false>;
+    if (!sp.staged) return sp.ksm ? dr_mixed_lead_kernel<false, true> : dr_mixed_lead_kernel<false, false>;
     return sp.ksm ? dr_mixed_lead_kernel<true, true> : dr_mixed_lead_kernel<true, false>;
 }
 

@@ -490,7 +490,7 @@ void build_classes(const std::vector<RveDesc> &rve, const std::vector<int32_t> &
                                                               one.slot_max, limit), one.part_max);
             // element constants in shared memory when they fit
             one.lead = LeadShape{R.n_parts, R.part_u_max, one.free_max, R.fp_slot_max, one.slot_max, R.part_push_max,
-                                 one.lead_staged, one.lead_staged};
+                                 one.lead_staged, true};
             if (lead_smem(one.lead) > limit) one.lead.ksm = false;
             one.lead_kernel = R.part_max <= 0xffff && lead_smem(one.lead) <= limit;
             one.lead_staged = one.lead_staged && one.lead_kernel;
