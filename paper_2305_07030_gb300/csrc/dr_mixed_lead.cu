@@ -253,14 +253,14 @@ __device__ __forceinline__ void lead_loop(LeadShared &sh, const DevMesh &M, cons
     const int k0 = 32 * nslot + lane;
     const int W = (int)blockDim.x - 32;  // the element threads
     const bool test_warp = (int)threadIdx.x >= W;
-    const int32_t *ps = M.fp_part_slot + (int64_t)p * (kMaxParts + 1);
+    const int32_t *ps = M.ls_part_slot + (int64_t)p * (kMaxParts + 1);
     const int s0 = ps[pt.me], n_el = ps[pt.me + 1] - s0;
-    const int4 *slots = M.fp_slot + R.slot0 + s0;
-    const uint32_t *ends = M.lead_ends + R.slot0 + s0;
+    const int4 *slots = M.ls_slot + R.ls_slot0 + s0;
+    const uint32_t *ends = M.lead_ends + R.ls_slot0 + s0;
 
     // ---- tables ----
     {
-        const int32_t *frow = M.fp_row + R.rp0 + pt.f0, *fent = M.fp_csr_slot + R.csr0;
+        const int32_t *frow = M.ls_row + R.rp0 + pt.f0, *fent = M.ls_csr_slot + R.csr0;
         slab_offsets(T.SS, nfr, [&](int k) { return frow[k + 1] - frow[k]; });
         copy_lists(M, R, pt, T.PO, [&](int x, uint32_t w) { T.PA[x] = w; });
         const int32_t *fo = M.lead_fix_off + (int64_t)p * 2 * (kMaxParts + 1);

@@ -56,7 +56,9 @@ struct RveDesc {
     int32_t part_q_max;
     int32_t part_push_max;
     int32_t part_u_max;   // lead: most entries of a part's displacement array
+    int32_t ls_slot_max;  // lead: most element slots of a part
     int32_t flush_ok;  // lengths and rigidities far from FP32's limits (node_range_ok)
+    int64_t ls_slot0;     // lead: first element slot
     int64_t push0;
     int64_t fix0;         // lead: first entry of lead_fix
     int64_t ell0;
@@ -122,11 +124,15 @@ struct DevMesh {
                                   // fp_node, and of the free nodes counted alone
     const int32_t *fp_row;        // per RVE n_free + 1 (from rp0): row offsets into
                                   // fp_csr_slot, free nodes in FP64 order
+    const int4 *ls_slot;          // lead: fp_slot, fp_csr_slot, fp_part_slot and fp_row by the
+    const int32_t *ls_csr_slot;   // mixed solver's parts (the FP64 kernel's may divide them)
+    const int32_t *ls_part_slot;
+    const int32_t *ls_row;
     const uint16_t *qidx;         // FP32 phase, per CSR entry of a free node: the neighbour's
                                   // place in the part's increment array
     const int32_t *push_off;      // per RVE n_free + 1 (from rp0): copies of a free node in
                                   // other parts, offsets from push0
-    const uint32_t *lead_ends;    // lead, per element slot (fp_slot): places of its ends in the
+    const uint32_t *lead_ends;    // lead, per element slot (ls_slot): places of its ends in the
                                   // part's displacement array, first | second << 16
     const int32_t *lead_fix;      // lead: per part the fixed neighbours of its free nodes
                                   // (RVE-local ids, from fix0)

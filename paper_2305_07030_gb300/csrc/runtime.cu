@@ -136,7 +136,8 @@ struct fe2_batch {
     DevBuf<float> d_Xh, d_Xl, d_imh, d_iml;
     DevBuf<int32_t> d_rowptr, d_col, d_col_part, d_part_off, d_el_a, d_el_b, d_csr_el;
     DevBuf<int32_t> d_fp_csr_slot, d_fp_part_slot, d_fp_node, d_fp_part_off, d_fp_row;
-    DevBuf<int4> d_fp_slot;
+    DevBuf<int4> d_fp_slot, d_ls_slot;
+    DevBuf<int32_t> d_ls_csr_slot, d_ls_part_slot, d_ls_row;
     DevBuf<double> d_ualt, d_fpt;
     DevBuf<uint16_t> d_qidx;
     DevBuf<int32_t> d_push_off;
@@ -217,6 +218,10 @@ struct fe2_batch {
         m.fp_node = d_fp_node.p;
         m.fp_part_off = d_fp_part_off.p;
         m.fp_row = d_fp_row.p;
+        m.ls_slot = d_ls_slot.p ? d_ls_slot.p : d_fp_slot.p;
+        m.ls_csr_slot = d_ls_slot.p ? d_ls_csr_slot.p : d_fp_csr_slot.p;
+        m.ls_part_slot = d_ls_slot.p ? d_ls_part_slot.p : d_fp_part_slot.p;
+        m.ls_row = d_ls_slot.p ? d_ls_row.p : d_fp_row.p;
         m.qidx = d_qidx.p;
         m.push_off = d_push_off.p;
         m.push = d_push.p;
@@ -255,7 +260,7 @@ struct fe2_batch {
         d_rve.release(); d_X.release(); d_mass.release(); d_EA_csr.release(); d_L_csr.release();
         d_el_EA.release(); d_el_L.release(); d_Xh.release(); d_Xl.release(); d_imh.release();
         d_iml.release(); d_rowptr.release(); d_col.release(); d_col_part.release();
-        d_part_off.release(); d_el_a.release(); d_el_b.release(); d_csr_el.release(); d_fp_csr_slot.release(); d_fp_part_slot.release(); d_fp_node.release(); d_fp_part_off.release(); d_fp_row.release(); d_fp_slot.release(); d_ualt.release(); d_fpt.release(); d_qidx.release(); d_push_off.release(); d_push.release(); d_lead_ends.release(); d_lead_fix.release(); d_lead_fix_off.release(); d_ek0.release(); d_ek1.release(); d_tf.release(); d_sv.release(); d_sa.release(); d_eaf.release();
+        d_part_off.release(); d_el_a.release(); d_el_b.release(); d_csr_el.release(); d_fp_csr_slot.release(); d_fp_part_slot.release(); d_fp_node.release(); d_fp_part_off.release(); d_fp_row.release(); d_fp_slot.release(); d_ls_slot.release(); d_ls_csr_slot.release(); d_ls_part_slot.release(); d_ls_row.release(); d_ualt.release(); d_fpt.release(); d_qidx.release(); d_push_off.release(); d_push.release(); d_lead_ends.release(); d_lead_fix.release(); d_lead_fix_off.release(); d_ek0.release(); d_ek1.release(); d_tf.release(); d_sv.release(); d_sa.release(); d_eaf.release();
         d_eaf_lo.release(); d_dh.release(); d_dl.release(); d_u.release(); d_v.release(); d_a.release(); d_xg.release();
         d_uh.release(); d_ul.release(); d_vh.release(); d_vl.release(); d_ah.release();
         d_al.release(); d_fg.release(); d_F.release(); d_sigma.release(); d_rel.release();
@@ -498,7 +503,7 @@ void build_classes(const std::vector<RveDesc> &rve, const std::vector<int32_t> &
             one.lead_staged = mixed_staged(1, mixed_lead_smem(one.part_max, one.free_max, one.elem_max,
                                                               one.slot_max, limit), one.part_max);
             // element constants in shared memory when they fit
-            one.lead = LeadShape{R.n_parts, R.part_u_max, one.free_max, R.fp_slot_max, one.slot_max, R.part_push_max,
+            one.lead = LeadShape{R.n_parts, R.part_u_max, one.free_max, R.ls_slot_max, one.slot_max, R.part_push_max,
                                  one.lead_staged, true};
             if (lead_smem(one.lead) > limit) one.lead.ksm = false;
             one.lead_kernel = R.part_max <= 0xffff && lead_smem(one.lead) <= limit;
@@ -651,6 +656,9 @@ struct HostLayout {
     // FP64 order of the nodes, the parts' offsets in it, and the free nodes'
     // row offsets (DevMesh::fp_node, fp_part_off, fp_row)
     std::vector<int32_t> fpSlot, fpCsrSlot, fpPartSlot, fpNode, fpPartOff, fpRow;
+    // the same slot tables by the mixed solver's parts (for its lead), where the
+    // FP64 ones are split further; empty otherwise
+    std::vector<int32_t> lsSlot, lsCsrSlot, lsPartSlot, lsRow;
     // FP32-phase kernel: DevMesh::qidx, push_off and push; total global row slots
     std::vector<uint16_t> qidx;
     std::vector<int32_t> pushOff;
@@ -661,18 +669,60 @@ struct HostLayout {
     int64_t n_ell = 0;
 };
 
+// Factor by which the FP64 cluster kernel's parts divide the mixed solver's. The
+// FP64 pipe is 2 operations per clock and SM, so a batch that leaves SMs idle
+// spreads each RVE over more of them, up to 128 CTAs in all and 16 per RVE, as
+// long as a part keeps kSplitNodes nodes: below that the latency of an iteration
+// (4 to 5 us) is no longer the work's. Displacements are the same bits for any
+// split. One RVE, us per iteration, unsplit and split: 512 nodes 13.0, 5.0 (16
+// parts 5.3); 700 nodes 17, 5.3 (8 parts 5.6); 4000 nodes 15 (8 CTAs), 9.6.
+constexpr int kSplitNodes = 40;
+int fp64_split(const HostLayout &L, const RveDesc &R) {
+    int64_t ctas = 0;
+    for (const RveDesc &q : L.rve) ctas += q.n_parts;
+    int f = 1;
+    while (2 * f * ctas <= 128 && 2 * f * R.n_parts <= kMaxParts && R.n_nodes >= 2 * f * R.n_parts * kSplitNodes) f *= 2;
+    return f;
+}
+
 // The FP64 cluster kernel's part of the layout (see HostLayout): its parts are
-// the mixed solver's.
-void build_fp64_parts(const int64_t *elem_off, HostLayout &L) {
+// the mixed solver's, or with `split` a bisection into fp64_split times as many.
+void build_fp64_parts(const int64_t *elem_off, bool split, HostLayout &L) {
     const int32_t n_rve = (int32_t)L.rve.size();
+    const int64_t N = (int64_t)L.perm_to_orig.size(), E = elem_off[n_rve];
+    L.fpCsrSlot.assign(2 * E, -1);
+    L.fpPartSlot.assign((size_t)n_rve * (kMaxParts + 1), 0);
+    L.fpNode.assign(N, 0);
+    L.fpPartOff.assign((size_t)n_rve * 2 * (kMaxParts + 1), 0);
+    L.fpRow.assign((size_t)N + n_rve, 0);
+    L.fpSlot.clear();
     for (int32_t p = 0; p < n_rve; ++p) {
         RveDesc &R = L.rve[p];
-        const int n = R.n_nodes, nf = R.n_free, C = R.n_parts;
+        const int n = R.n_nodes, nf = R.n_free, C = R.n_parts * (split ? fp64_split(L, R) : 1);
         const int32_t *pf = L.part.data() + (size_t)p * 2 * (kMaxParts + 1), *pg = pf + (kMaxParts + 1);
         std::vector<std::vector<int>> fr(C), fx(C);  // per part: free and fixed nodes
-        for (int r = 0; r < C; ++r) {
-            for (int k = pf[r]; k < pf[r + 1]; ++k) fr[r].push_back(k);
-            for (int k = pg[r]; k < pg[r + 1]; ++k) fx[r].push_back(nf + k);
+        if (C == R.n_parts) {
+            for (int r = 0; r < C; ++r) {
+                for (int k = pf[r]; k < pf[r + 1]; ++k) fr[r].push_back(k);
+                for (int k = pg[r]; k < pg[r + 1]; ++k) fx[r].push_back(nf + k);
+            }
+        } else {
+            std::vector<double> X(3 * (size_t)n);
+            for (int k = 0; k < n; ++k)
+                for (int c = 0; c < 3; ++c) X[3 * k + c] = L.X[c * N + R.node0 + k];
+            std::vector<int> all(n);
+            std::iota(all.begin(), all.end(), 0);
+            std::vector<std::vector<int>> parts;
+            rcb(all, C, X.data(), 0, parts);
+            const int32_t *deg = L.row.data() + R.rp0;
+            for (int r = 0; r < C; ++r) {
+                for (int k : parts[r]) (k < nf ? fr[r] : fx[r]).push_back(k);
+                std::sort(fx[r].begin(), fx[r].end());
+                std::sort(fr[r].begin(), fr[r].end(), [&](int x, int y) {
+                    const int dx = deg[x + 1] - deg[x], dy = deg[y + 1] - deg[y];
+                    return dx > dy || (dx == dy && x < y);
+                });
+            }
         }
         int32_t *node = L.fpNode.data() + R.node0, *frow = L.fpRow.data() + R.rp0;
         int32_t *off = L.fpPartOff.data() + (size_t)p * 2 * (kMaxParts + 1), *ffree = off + (kMaxParts + 1);
@@ -861,12 +911,7 @@ void build_layout(int32_t n_rve, const int64_t *node_off, const double *X, const
     L.col.assign(2 * E, 0);
     L.colp.assign(2 * E, 0);
     L.csrEl.assign(2 * E, 0);
-    L.fpCsrSlot.assign(2 * E, -1);
-    L.fpPartSlot.assign((size_t)n_rve * (kMaxParts + 1), 0);
-    L.fpNode.assign(N, 0);
-    L.fpPartOff.assign((size_t)n_rve * 2 * (kMaxParts + 1), 0);
-    L.fpRow.assign((size_t)N + n_rve, 0);
-    L.fpSlot.clear();
+    for (auto *v : {&L.lsSlot, &L.lsCsrSlot, &L.lsPartSlot, &L.lsRow}) v->clear();
     L.Ela.assign(E, 0);
     L.Elb.assign(E, 0);
     L.ElemOf.assign(2 * E, 0);
@@ -1019,8 +1064,20 @@ void build_layout(int32_t n_rve, const int64_t *node_off, const double *X, const
             hElEA[e] = EA[e];
         }
     }
-    build_fp64_parts(elem_off, L);
+    build_fp64_parts(elem_off, false, L);
     build_node_tables(smem_cap, L);
+    bool split = false;
+    for (RveDesc &R : L.rve) {
+        R.ls_slot0 = R.slot0;
+        R.ls_slot_max = R.fp_slot_max;
+        split |= fp64_split(L, R) > 1;
+    }
+    if (!split) return;
+    L.lsSlot = std::move(L.fpSlot);
+    L.lsCsrSlot = std::move(L.fpCsrSlot);
+    L.lsPartSlot = std::move(L.fpPartSlot);
+    L.lsRow = std::move(L.fpRow);
+    build_fp64_parts(elem_off, true, L);
 }
 
 }  // namespace
@@ -1099,6 +1156,10 @@ extern "C" fe2_status fe2_batch_create(int32_t n_rve, const int64_t *node_off, c
     A(b->d_fp_slot.alloc(std::max<size_t>(1, n_fslots)), "fp_slot");
     A(b->d_fp_csr_slot.alloc(2 * E), "fp_csr_slot");
     A(b->d_fp_part_slot.alloc(L.fpPartSlot.size()), "fp_part_slot");
+    A(b->d_ls_slot.alloc(L.lsSlot.size() / 4), "ls_slot");
+    A(b->d_ls_csr_slot.alloc(L.lsCsrSlot.size()), "ls_csr_slot");
+    A(b->d_ls_part_slot.alloc(L.lsPartSlot.size()), "ls_part_slot");
+    A(b->d_ls_row.alloc(L.lsRow.size()), "ls_row");
     A(b->d_fp_node.alloc(N), "fp_node");
     A(b->d_fp_part_off.alloc(L.fpPartOff.size()), "fp_part_off");
     A(b->d_fp_row.alloc(N + n_rve), "fp_row");
@@ -1159,6 +1220,10 @@ extern "C" fe2_status fe2_batch_create(int32_t n_rve, const int64_t *node_off, c
     H2D(b->d_col_part.p, hcolp.data(), sizeof(int32_t) * 2 * E, "col_part");
     H2D(b->d_csr_el.p, L.csrEl.data(), sizeof(int32_t) * 2 * E, "csr_el");
     if (n_fslots) H2D(b->d_fp_slot.p, L.fpSlot.data(), sizeof(int4) * n_fslots, "fp_slot");
+    H2D(b->d_ls_slot.p, L.lsSlot.data(), sizeof(int32_t) * L.lsSlot.size(), "ls_slot");
+    H2D(b->d_ls_csr_slot.p, L.lsCsrSlot.data(), sizeof(int32_t) * L.lsCsrSlot.size(), "ls_csr_slot");
+    H2D(b->d_ls_part_slot.p, L.lsPartSlot.data(), sizeof(int32_t) * L.lsPartSlot.size(), "ls_part_slot");
+    H2D(b->d_ls_row.p, L.lsRow.data(), sizeof(int32_t) * L.lsRow.size(), "ls_row");
     H2D(b->d_fp_csr_slot.p, L.fpCsrSlot.data(), sizeof(int32_t) * 2 * E, "fp_csr_slot");
     H2D(b->d_fp_part_slot.p, L.fpPartSlot.data(), sizeof(int32_t) * L.fpPartSlot.size(), "fp_part_slot");
     H2D(b->d_fp_node.p, L.fpNode.data(), sizeof(int32_t) * N, "fp_node");
@@ -1299,13 +1364,15 @@ extern "C" fe2_status fe2_batch_fp64_slots(int32_t n_rve, const int64_t *node_of
     HostLayout L;
     build_layout(n_rve, node_off, X, elem_off, conn, EA, fixed, nullptr, nullptr, target,
                  (size_t)smem_optin - 16384, L);
-    const int64_t ns = (int64_t)(L.fpSlot.size() / 4);
+    const bool ls = !L.lsSlot.empty();
+    const auto &sl = ls ? L.lsSlot : L.fpSlot, &cs = ls ? L.lsCsrSlot : L.fpCsrSlot, &pp = ls ? L.lsPartSlot : L.fpPartSlot;
+    const int64_t ns = (int64_t)(sl.size() / 4);
     if (n_slots) *n_slots = ns;
     if (slot0)
-        for (int32_t p = 0; p < n_rve; ++p) slot0[p] = L.rve[p].slot0;
-    if (part_slot) std::copy(L.fpPartSlot.begin(), L.fpPartSlot.end(), part_slot);
-    if (slot) std::copy(L.fpSlot.begin(), L.fpSlot.begin() + 4 * std::min(ns, std::max<int64_t>(cap, 0)), slot);
-    if (csr_slot) std::copy(L.fpCsrSlot.begin(), L.fpCsrSlot.end(), csr_slot);
+        for (int32_t p = 0; p < n_rve; ++p) slot0[p] = L.rve[p].ls_slot0;
+    if (part_slot) std::copy(pp.begin(), pp.end(), part_slot);
+    if (slot) std::copy(sl.begin(), sl.begin() + 4 * std::min(ns, std::max<int64_t>(cap, 0)), slot);
+    if (csr_slot) std::copy(cs.begin(), cs.end(), csr_slot);
     return FE2_OK;
 }
 
