@@ -462,12 +462,12 @@ const char *fe2_last_error(void);
  * own every device allocation through their own pools). It allocates nothing:
  * inputs and outputs are the caller's DEVICE buffers, and all working memory
  * is one file-scope device array of fe2_noalloc_scratch_bytes() bytes (about
- * 1.6 MB) that every GPU loading the library holds until the process exits.
+ * 3.5 MB) that every GPU loading the library holds until the process exits.
  *
  * It runs the same per-RVE FP64 solver as fe2_batch_solve with
- * FE2_PREC_FP64, in one CTA. Every node's update is the same sequence of IEEE
- * operations as on that path, but the free nodes are held in the caller's
- * order rather than the batch's spatial order, so the residual sum is
+ * FE2_PREC_FP64, on a thread-block cluster of 1 to 16 CTAs by the node count.
+ * Every node's update is the same sequence of IEEE operations as on that path,
+ * but the nodes are split into parts differently, so the residual sum is
  * associated differently: rel_res agrees with the batched path to about
  * 1e-12, and where the two iteration counts agree (they can differ by one
  * when the residual lands within rounding of the threshold) the

@@ -139,6 +139,15 @@ __device__ __forceinline__ void slot_force(const Slot &e, uint32_t boff, uint32_
     T[2 * ts] = dmul(q, d2);
 }
 
+// Dynamic shared memory of a launch shape (layout: cluster_tables).
+__host__ __device__ inline size_t cluster_bytes(const Fp64Shape &sp) {
+    size_t b = sizeof(double) * (6 * (size_t)sp.part_max + (sp.ssm ? kStateDoubles * (size_t)sp.free_max : 0));
+    if (sp.tsm)
+        b += sizeof(double) * 3 * (size_t)sp.slot_max + sizeof(int32_t) * ((size_t)sp.free_max + 1) +
+             sizeof(uint16_t) * (size_t)sp.row_max;
+    return (b + 15) & ~size_t(15);
+}
+
 }  // namespace
 
 // One RVE on the cluster. XB (smem) is this CTA's [2][3][part_cap] position
@@ -442,32 +451,70 @@ __device__ void solve_rve_fp64_cluster(cg::cluster_group &cl, Fp64ClusterShared 
     cl.sync();  // the next RVE may overwrite the buffers
 }
 
+namespace {
+__device__ __forceinline__ void map_shared(cg::cluster_group &cl, Fp64ClusterShared &sh) {
+    if ((int)threadIdx.x < (int)cl.num_blocks()) {
+        const int r = threadIdx.x;
+        sh.partp[r] = cl.map_shared_rank(&sh.part[0][0], r);
+    }
+    if (threadIdx.x == 0) sh.sigp = cl.map_shared_rank(&sh.sig[0][0], 0);
+}
+
+// One RVE with the tables of a launch shape in `base` (cluster_bytes).
+template <bool TSM, bool SSM>
+__device__ __forceinline__ void solve_in(cg::cluster_group &cl, Fp64ClusterShared &sh, const DevMesh &M,
+                                         const DevState &S, const DevResults &O, const SolveParams &P, int p,
+                                         const Fp64Shape &sp, double *base) {
+    double *XB = base;
+    double *ST = XB + 6 * sp.part_max;
+    double *T = ST + (SSM ? kStateDoubles * (size_t)sp.free_max : 0);
+    int32_t *RS = reinterpret_cast<int32_t *>(T + (TSM ? 3 * (size_t)sp.slot_max : 0));
+    uint16_t *RE = reinterpret_cast<uint16_t *>(RS + (TSM ? sp.free_max + 1 : 0));
+    solve_rve_fp64_cluster<TSM, SSM>(cl, sh, M, S, O, P, p, XB, ST, T, RS, RE, sp.part_max, sp.free_max, sp.slot_max);
+}
+}  // namespace
+
 template <bool TSM, bool SSM>
 __global__ void __launch_bounds__(kMaxThreads, 1)
     dr_fp64_cluster_kernel(DevMesh M, DevState S, DevResults O, SolveParams P, Fp64Shape sp) {
     extern __shared__ __align__(16) double dsm_fp64[];
     __shared__ Fp64ClusterShared sh;
     cg::cluster_group cl = cg::this_cluster();
-    // layout as in fp64_cluster_smem
-    double *XB = dsm_fp64;
-    double *ST = XB + 6 * sp.part_max;
-    double *T = ST + (SSM ? kStateDoubles * (size_t)sp.free_max : 0);
-    int32_t *RS = reinterpret_cast<int32_t *>(T + (TSM ? 3 * (size_t)sp.slot_max : 0));
-    uint16_t *RE = reinterpret_cast<uint16_t *>(RS + (TSM ? sp.free_max + 1 : 0));
-    if ((int)threadIdx.x < (int)cl.num_blocks()) {
-        const int r = threadIdx.x;
-        sh.partp[r] = cl.map_shared_rank(&sh.part[0][0], r);
-    }
-    if (threadIdx.x == 0) sh.sigp = cl.map_shared_rank(&sh.sig[0][0], 0);
+    map_shared(cl, sh);
     for (;;) {
         if (cl.block_rank() == 0 && threadIdx.x == 0) sh.item = atomicAdd(P.counter, 1);
         cl.sync();
         const int item = *cl.map_shared_rank(&sh.item, 0);
         cl.sync();
         if (item >= P.queue_len) return;
-        solve_rve_fp64_cluster<TSM, SSM>(cl, sh, M, S, O, P, P.queue[item], XB, ST, T, RS, RE, sp.part_max,
-                                         sp.free_max, sp.slot_max);
+        solve_in<TSM, SSM>(cl, sh, M, S, O, P, P.queue[item], sp, dsm_fp64);
     }
+}
+
+// The allocation-free call: RVE 0, whose tables a packing kernel left in M's
+// arrays, with the shared-memory variant its own capacities allow in `bytes`; the
+// displacement goes to u in the caller's order (perm). Nothing is done when the
+// packing kernel found the inputs invalid (*skip).
+__global__ void __launch_bounds__(kMaxThreads, 1)
+    dr_fp64_single_kernel(DevMesh M, DevState S, DevResults O, SolveParams P, size_t bytes, const int *skip,
+                          const int32_t *perm, double *u) {
+    extern __shared__ __align__(16) double dsm_fp64[];
+    __shared__ Fp64ClusterShared sh;
+    if (*skip) return;
+    cg::cluster_group cl = cg::this_cluster();
+    map_shared(cl, sh);
+    cl.sync();
+    const RveDesc &R = M.rve[0];
+    Fp64Shape sp = {R.fp_parts, R.fp_part_max, R.fp_free_max, R.fp_slot_max, R.fp_row_max, true, true};
+    if (cluster_bytes(sp) <= bytes) {
+        solve_in<true, true>(cl, sh, M, S, O, P, 0, sp, dsm_fp64);
+    } else {
+        sp.tsm = sp.ssm = false;
+        solve_in<false, false>(cl, sh, M, S, O, P, 0, sp, dsm_fp64);
+    }
+    const double *uo[3] = {S.u0, S.u1, S.u2};
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < R.n_nodes; k += gridDim.x * blockDim.x)
+        for (int c = 0; c < 3; ++c) u[3 * perm[k] + c] = uo[c][k];
 }
 
 namespace {
@@ -513,13 +560,7 @@ void prepare_fp64_cluster(Fp64ClusterKernel k, size_t smem) {
 }
 }  // namespace
 
-size_t fp64_cluster_smem(const Fp64Shape &sp) {
-    size_t b = sizeof(double) * (6 * (size_t)sp.part_max + (sp.ssm ? kStateDoubles * (size_t)sp.free_max : 0));
-    if (sp.tsm)
-        b += sizeof(double) * 3 * (size_t)sp.slot_max + sizeof(int32_t) * ((size_t)sp.free_max + 1) +
-             sizeof(uint16_t) * (size_t)sp.row_max;
-    return (b + 15) & ~size_t(15);
-}
+size_t fp64_cluster_smem(const Fp64Shape &sp) { return cluster_bytes(sp); }
 
 int launch_dr_fp64_cluster(const DevMesh &m, const DevState &s, const DevResults &r, const SolveParams &p,
                            int clusters, int block, const Fp64Shape &sp, void *stream) {
@@ -543,6 +584,27 @@ int occupancy_dr_fp64_cluster(int block, const Fp64Shape &sp) {
         return 0;
     }
     return n;
+}
+
+constexpr size_t kSingleBytes = 200 * 1024;
+
+cudaError_t prepare_dr_fp64_single() {
+    const cudaError_t e = cudaFuncSetAttribute(dr_fp64_single_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)kSingleBytes);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(dr_fp64_single_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+}
+
+int launch_dr_fp64_single(const DevMesh &m, const DevState &s, const DevResults &r, const SolveParams &p, int parts,
+                          const int *skip, const int32_t *perm, double *u, void *stream) {
+    cudaLaunchAttribute attr[1];
+    Fp64Shape sp = {};
+    sp.parts = parts;
+    cudaLaunchConfig_t cfg = fp64_cluster_config(1, sp, kMaxThreads, attr, static_cast<cudaStream_t>(stream));
+    cfg.dynamicSmemBytes = kSingleBytes;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, dr_fp64_single_kernel, m, s, r, p, kSingleBytes, skip, perm, u);
+    if (e != cudaSuccess) return (int)e;
+    return (int)cudaGetLastError();
 }
 
 }  // namespace fe2
