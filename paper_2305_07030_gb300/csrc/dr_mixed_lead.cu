@@ -160,7 +160,7 @@ __device__ __forceinline__ double lead_norm(LeadShared &sh, float acc, int me, i
 // Initial displacement, velocity and acceleration into the state arrays;
 // returns f_ref. With the affine start both reference forces are the same.
 __device__ __noinline__ double lead_start(LeadShared &sh, const DevMesh &M, const DevState &S, const SolveParams &P,
-                                          int p, const RveDesc &R, const Part pt) {
+                                          int p, const RveDesc &R, const Part pt, bool staged) {
     const int n = R.n_nodes, m = pt.m();
     const int64_t n0 = R.node0, b3 = 3 * n0;
     float *uh = S.uh + b3, *ul = S.ul + b3, *vh = S.vh + b3, *vl = S.vl + b3;
@@ -186,21 +186,28 @@ __device__ __noinline__ double lead_start(LeadShared &sh, const DevMesh &M, cons
         }
     }
     cg::this_cluster().sync();
+    // |g|^2 in the two orders of its fused products: parts without the table have
+    // always summed the affine force's (AFF) and the initial force's in different
+    // ones, and keep them; the others use the second for both.
+    auto square = [&](const df *g, bool aff) {
+        const float x = g[0].hi, y = g[1].hi, z = g[2].hi;
+        return aff && !staged ? dot3(y, x, z, y, x, z) : dot3(x, y, z, x, y, z);
+    };
     double f_aff = 0.0;
     df g[3];
+    float acc = 0.f, acc_aff = 0.f;
     if (P.init != 1) {
-        float acc = 0.f;
         for (int k = threadIdx.x; k < m; k += blockDim.x) {
             lead_gather(M, R, vh, vl, pt.gidx(k), g);
-            acc = fadd(acc, dot3(g[0].hi, g[1].hi, g[2].hi, g[0].hi, g[1].hi, g[2].hi));
+            acc_aff = fadd(acc_aff, square(g, true));
         }
-        f_aff = lead_norm(sh, acc, pt.me, pt.C);
+        f_aff = lead_norm(sh, acc_aff, pt.me, pt.C);
     }
-    float acc = 0.f;
     for (int k = threadIdx.x; k < m; k += blockDim.x) {
         const int i = pt.gidx(k);
         lead_gather(M, R, uh, ul, i, g);
-        acc = fadd(acc, dot3(g[0].hi, g[1].hi, g[2].hi, g[0].hi, g[1].hi, g[2].hi));
+        acc = fadd(acc, square(g, false));
+        if (P.init == 1) acc_aff = fadd(acc_aff, square(g, true));
         if (k < pt.nfr) {
             const df im = {M.imh[n0 + i], M.iml[n0 + i]};
             for (int r = 0; r < 3; ++r) {
@@ -213,6 +220,7 @@ __device__ __noinline__ double lead_start(LeadShared &sh, const DevMesh &M, cons
             }
         }
     }
+    if (P.init == 1 && !staged) f_aff = lead_norm(sh, acc_aff, pt.me, pt.C);
     const double f0 = lead_norm(sh, acc, pt.me, pt.C);
     return f_aff > f0 ? f_aff : f0;
 }
@@ -484,7 +492,7 @@ __device__ __forceinline__ void lead_rve(LeadShared &sh, const DevMesh &M, const
         cl.sync();  // every CTA has read the status before rank 0 rewrites it
         if (st0 != RVE_STALLED) return;
     } else {
-        f_ref = lead_start(sh, M, S, P, p, R, pt);
+        f_ref = lead_start(sh, M, S, P, p, R, pt, STAGED);
     }
     const df thresh2 = df_from_double(dmul(dmul(P.tol, f_ref), dmul(P.tol, f_ref)));
     // a resumed RVE runs in double-float until it converges
