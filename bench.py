@@ -127,12 +127,12 @@ class ClockSampler:
                 "samples": len(rows)}
 
 
-# DRAM bytes (read + write) of one dr_mixed_fp32_kernel launch, scaled from
+# DRAM bytes (read + write) of one dr_mixed_node_kernel launch, scaled from
 # one ncu capture of the same kernel: a 5000-node RVE of the 64 x 5000
-# workload for 30,000 iterations read 1,940,224 B and wrote 5,888 B. The
+# workload for 20,000 iterations read 2,051,328 B and wrote 12,800 B. The
 # traffic is each RVE's data and state read once; it does not grow with
 # iterations, so a launch's traffic scales with its number of RVEs.
-FP32_DRAM_BYTES_PER_RVE = 1_940_224 + 5_888
+FP32_DRAM_BYTES_PER_RVE = 2_051_328 + 12_800
 
 
 def fp32_dram_traffic(n_rve):
@@ -310,7 +310,7 @@ def run_ours(args, rank, world):
         achieved = alg / (kms * 1e-3) / 1e9
         roof = {"bound": "smem", "achieved": achieved, "peak": smem_gbs, "unit": "GB/s",
                 "frac": achieved / smem_gbs, "traffic": fp32_dram_traffic(n_in),
-                "kernel": "dr_mixed_fp32_kernel", "kernel_ms": kms,
+                "kernel": "dr_mixed_node_kernel", "kernel_ms": kms,
                 "lead_kernel_ms": statistics.mean(sum(k[per_launch * c] for c in range(n_cls))
                                                   for k in kernel_ms),
                 "resume_kernel_ms": statistics.mean(sum(k[per_launch * c + 2] for c in range(n_cls))

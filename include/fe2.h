@@ -68,9 +68,10 @@ typedef enum {
      * in the same order as a serial element-scatter implementation in the
      * caller's node order, no fused multiply-add, correctly rounded sqrt and
      * divide. The trajectory is bit for bit that of such an implementation;
-     * only the residual and stress sums are reassociated. An RVE of one
-     * spatial part runs on one CTA; an RVE of several parts on a
-     * thread-block cluster, one part per CTA, with the same operations (set
+     * only the residual and stress sums are reassociated. An RVE runs on a
+     * thread-block cluster of 1 to 16 CTAs, one spatial part per CTA (more
+     * and smaller parts in batches that leave SMs idle; the residual's last
+     * bits may depend on it), with the same operations (set
      * FE2_FP64_CLUSTER=0 in the environment before fe2_batch_create to keep
      * every RVE on one CTA). Any RVE size. */
     FE2_PREC_FP64 = 0,
@@ -81,9 +82,8 @@ typedef enum {
      * forces about a double-float reference state refreshed every
      * rebase_every iterations. The residual is totalled in double-float and
      * compared with (tol f_ref)^2 formed in FP64; the stress sum is FP64.
-     * Each CTA holds its part's node state in shared memory: 96 bytes per
-     * node for the FP32 kernel without its element table (velocity and
-     * acceleration then live in global memory), which bounds an RVE to 16
+     * Each CTA holds its part's node state in shared memory; 96 bytes per
+     * node (the FP32 kernel without row tables) bound an RVE to 16
      * parts of 2,186 nodes (34,976 nodes) on a GB300; a solve with a larger
      * RVE returns FE2_EINVAL (use FE2_PREC_FP64). */
     FE2_PREC_MIXED = 1
