@@ -240,9 +240,11 @@ fe2_status fe2_batch_layout(int32_t n_rve, const int64_t *node_off, const double
 
 /*
  * Inspection call, host only: the element slot tables of the FP64 cluster
- * kernel for these inputs (Algorithm 1, getInternalForces on a cluster: each
- * CTA evaluates the elements with an end among its part's free nodes once per
- * iteration). Inputs as for fe2_batch_layout. Outputs (HOST, caller-allocated,
+ * kernel and the mixed lead for these inputs (Algorithm 1, getInternalForces on
+ * a cluster: each CTA evaluates the elements with an end among its part's free
+ * nodes once per iteration), by the parts of fe2_batch_layout. (In batches that
+ * leave SMs idle the FP64 kernel divides the parts further and has tables of its
+ * own of the same form.) Inputs as for fe2_batch_layout. Outputs (HOST, caller-allocated,
  * each may be NULL):
  * n_slots    total slots of the batch.
  * slot0      n_rve: the RVE's first slot.
@@ -278,9 +280,9 @@ fe2_status fe2_batch_fp64_slots(int32_t n_rve, const int64_t *node_off, const do
  * class_rves   per class: number of RVEs.
  * smem         2 per class: dynamic shared memory per CTA in bytes, for the
  *              lead kernel then for the FP32 kernel.
- * staged       2 per class (same order): 1 if that kernel keeps its
- *              element table in shared memory, 0 if it re-reads the CSR rows
- *              from global memory every iteration.
+ * staged       2 per class (same order): 1 if the class's parts meet that
+ *              kernel's footprint rule (its tables are in shared memory), 0 if
+ *              they do not (part of the tables may be in global memory).
  * block        2 per class (same order): threads per CTA.
  *
  * Returns FE2_EINVAL for the inputs fe2_batch_layout rejects.

@@ -1371,7 +1371,9 @@ extern "C" fe2_status fe2_batch_fp64_slots(int32_t n_rve, const int64_t *node_of
     if (slot0)
         for (int32_t p = 0; p < n_rve; ++p) slot0[p] = L.rve[p].ls_slot0;
     if (part_slot) std::copy(pp.begin(), pp.end(), part_slot);
-    if (slot) std::copy(sl.begin(), sl.begin() + 4 * std::min(ns, std::max<int64_t>(cap, 0)), slot);
+    const int64_t nc = std::min(ns, std::max<int64_t>(cap, 0));
+    if (slot) std::copy(sl.begin(), sl.begin() + 4 * nc, slot);
+    for (int64_t k = 0; slot && k < nc; ++k) slot[4 * k + 3] = 0;  // internal: the slot's CSR entry
     if (csr_slot) std::copy(cs.begin(), cs.end(), csr_slot);
     return FE2_OK;
 }
