@@ -136,13 +136,16 @@ struct fe2_batch {
     DevBuf<float> d_Xh, d_Xl, d_imh, d_iml;
     DevBuf<int32_t> d_rowptr, d_col, d_col_part, d_part_off, d_el_a, d_el_b, d_csr_el;
     DevBuf<int32_t> d_fp_csr_slot, d_fp_part_slot, d_fp_node, d_fp_part_off, d_fp_row;
-    DevBuf<int4> d_fp_slot, d_ls_slot;
-    DevBuf<int32_t> d_ls_csr_slot, d_ls_part_slot, d_ls_row;
+    DevBuf<int4> d_fp_slot;
     DevBuf<double> d_ualt, d_fpt;
-    DevBuf<uint16_t> d_qidx;
-    DevBuf<int32_t> d_push_off;
-    DevBuf<uint32_t> d_push, d_lead_ends;
-    DevBuf<int32_t> d_lead_fix, d_lead_fix_off;
+    // tables of the mixed kernels (HostLayout) in one allocation, and each one's
+    // offset; the lead's slot tables only where the FP64 ones are split
+    DevBuf<unsigned char> d_tables;
+    enum { kQidx, kPushOff, kPush, kLeadEnds, kLeadFix, kLeadFixOff, kLsSlot, kLsCsrSlot, kLsPartSlot, kLsRow, kTables };
+    size_t table_off[kTables] = {};
+    bool ls_tables = false;
+    template <class T>
+    const T *table(int k) const { return reinterpret_cast<const T *>(d_tables.p + table_off[k]); }
     DevBuf<float4> d_ek0;
     DevBuf<float> d_ek1;
     DevBuf<float2> d_eaf, d_eaf_lo, d_sa;
@@ -218,16 +221,16 @@ struct fe2_batch {
         m.fp_node = d_fp_node.p;
         m.fp_part_off = d_fp_part_off.p;
         m.fp_row = d_fp_row.p;
-        m.ls_slot = d_ls_slot.p ? d_ls_slot.p : d_fp_slot.p;
-        m.ls_csr_slot = d_ls_slot.p ? d_ls_csr_slot.p : d_fp_csr_slot.p;
-        m.ls_part_slot = d_ls_slot.p ? d_ls_part_slot.p : d_fp_part_slot.p;
-        m.ls_row = d_ls_slot.p ? d_ls_row.p : d_fp_row.p;
-        m.qidx = d_qidx.p;
-        m.push_off = d_push_off.p;
-        m.push = d_push.p;
-        m.lead_ends = d_lead_ends.p;
-        m.lead_fix = d_lead_fix.p;
-        m.lead_fix_off = d_lead_fix_off.p;
+        m.ls_slot = ls_tables ? table<int4>(kLsSlot) : d_fp_slot.p;
+        m.ls_csr_slot = ls_tables ? table<int32_t>(kLsCsrSlot) : d_fp_csr_slot.p;
+        m.ls_part_slot = ls_tables ? table<int32_t>(kLsPartSlot) : d_fp_part_slot.p;
+        m.ls_row = ls_tables ? table<int32_t>(kLsRow) : d_fp_row.p;
+        m.qidx = table<uint16_t>(kQidx);
+        m.push_off = table<int32_t>(kPushOff);
+        m.push = table<uint32_t>(kPush);
+        m.lead_ends = table<uint32_t>(kLeadEnds);
+        m.lead_fix = table<int32_t>(kLeadFix);
+        m.lead_fix_off = table<int32_t>(kLeadFixOff);
         return m;
     }
     DevState state() const {
@@ -260,7 +263,7 @@ struct fe2_batch {
         d_rve.release(); d_X.release(); d_mass.release(); d_EA_csr.release(); d_L_csr.release();
         d_el_EA.release(); d_el_L.release(); d_Xh.release(); d_Xl.release(); d_imh.release();
         d_iml.release(); d_rowptr.release(); d_col.release(); d_col_part.release();
-        d_part_off.release(); d_el_a.release(); d_el_b.release(); d_csr_el.release(); d_fp_csr_slot.release(); d_fp_part_slot.release(); d_fp_node.release(); d_fp_part_off.release(); d_fp_row.release(); d_fp_slot.release(); d_ls_slot.release(); d_ls_csr_slot.release(); d_ls_part_slot.release(); d_ls_row.release(); d_ualt.release(); d_fpt.release(); d_qidx.release(); d_push_off.release(); d_push.release(); d_lead_ends.release(); d_lead_fix.release(); d_lead_fix_off.release(); d_ek0.release(); d_ek1.release(); d_tf.release(); d_sv.release(); d_sa.release(); d_eaf.release();
+        d_part_off.release(); d_el_a.release(); d_el_b.release(); d_csr_el.release(); d_fp_csr_slot.release(); d_fp_part_slot.release(); d_fp_node.release(); d_fp_part_off.release(); d_fp_row.release(); d_fp_slot.release(); d_ualt.release(); d_fpt.release(); d_tables.release(); d_ek0.release(); d_ek1.release(); d_tf.release(); d_sv.release(); d_sa.release(); d_eaf.release();
         d_eaf_lo.release(); d_dh.release(); d_dl.release(); d_u.release(); d_v.release(); d_a.release(); d_xg.release();
         d_uh.release(); d_ul.release(); d_vh.release(); d_vl.release(); d_ah.release();
         d_al.release(); d_fg.release(); d_F.release(); d_sigma.release(); d_rel.release();
@@ -677,9 +680,12 @@ struct HostLayout {
 // split. One RVE, us per iteration, unsplit and split: 512 nodes 13.0, 5.0 (16
 // parts 5.3); 700 nodes 17, 5.3 (8 parts 5.6); 4000 nodes 15 (8 CTAs), 9.6.
 constexpr int kSplitNodes = 40;
-int fp64_split(const HostLayout &L, const RveDesc &R) {
+int64_t mixed_ctas(const HostLayout &L) {
     int64_t ctas = 0;
     for (const RveDesc &q : L.rve) ctas += q.n_parts;
+    return ctas;
+}
+int fp64_split(int64_t ctas, const RveDesc &R) {
     int f = 1;
     while (2 * f * ctas <= 128 && 2 * f * R.n_parts <= kMaxParts && R.n_nodes >= 2 * f * R.n_parts * kSplitNodes) f *= 2;
     return f;
@@ -689,7 +695,7 @@ int fp64_split(const HostLayout &L, const RveDesc &R) {
 // the mixed solver's, or with `split` a bisection into fp64_split times as many.
 void build_fp64_parts(const int64_t *elem_off, bool split, HostLayout &L) {
     const int32_t n_rve = (int32_t)L.rve.size();
-    const int64_t N = (int64_t)L.perm_to_orig.size(), E = elem_off[n_rve];
+    const int64_t N = (int64_t)L.perm_to_orig.size(), E = elem_off[n_rve], ctas = mixed_ctas(L);
     L.fpCsrSlot.assign(2 * E, -1);
     L.fpPartSlot.assign((size_t)n_rve * (kMaxParts + 1), 0);
     L.fpNode.assign(N, 0);
@@ -698,7 +704,7 @@ void build_fp64_parts(const int64_t *elem_off, bool split, HostLayout &L) {
     L.fpSlot.clear();
     for (int32_t p = 0; p < n_rve; ++p) {
         RveDesc &R = L.rve[p];
-        const int n = R.n_nodes, nf = R.n_free, C = R.n_parts * (split ? fp64_split(L, R) : 1);
+        const int n = R.n_nodes, nf = R.n_free, C = R.n_parts * (split ? fp64_split(ctas, R) : 1);
         const int32_t *pf = L.part.data() + (size_t)p * 2 * (kMaxParts + 1), *pg = pf + (kMaxParts + 1);
         std::vector<std::vector<int>> fr(C), fx(C);  // per part: free and fixed nodes
         if (C == R.n_parts) {
@@ -1067,10 +1073,11 @@ void build_layout(int32_t n_rve, const int64_t *node_off, const double *X, const
     build_fp64_parts(elem_off, false, L);
     build_node_tables(smem_cap, L);
     bool split = false;
+    const int64_t ctas = mixed_ctas(L);
     for (RveDesc &R : L.rve) {
         R.ls_slot0 = R.slot0;
         R.ls_slot_max = R.fp_slot_max;
-        split |= fp64_split(L, R) > 1;
+        split |= fp64_split(ctas, R) > 1;
     }
     if (!split) return;
     L.lsSlot = std::move(L.fpSlot);
@@ -1156,20 +1163,33 @@ extern "C" fe2_status fe2_batch_create(int32_t n_rve, const int64_t *node_off, c
     A(b->d_fp_slot.alloc(std::max<size_t>(1, n_fslots)), "fp_slot");
     A(b->d_fp_csr_slot.alloc(2 * E), "fp_csr_slot");
     A(b->d_fp_part_slot.alloc(L.fpPartSlot.size()), "fp_part_slot");
-    A(b->d_ls_slot.alloc(L.lsSlot.size() / 4), "ls_slot");
-    A(b->d_ls_csr_slot.alloc(L.lsCsrSlot.size()), "ls_csr_slot");
-    A(b->d_ls_part_slot.alloc(L.lsPartSlot.size()), "ls_part_slot");
-    A(b->d_ls_row.alloc(L.lsRow.size()), "ls_row");
     A(b->d_fp_node.alloc(N), "fp_node");
     A(b->d_fp_part_off.alloc(L.fpPartOff.size()), "fp_part_off");
     A(b->d_fp_row.alloc(N + n_rve), "fp_row");
     A(b->d_ualt.alloc(9 * N), "ualt");
-    A(b->d_qidx.alloc(2 * E), "qidx");
-    A(b->d_push_off.alloc(N + n_rve), "push_off");
-    A(b->d_push.alloc(std::max<size_t>(1, L.push.size())), "push");
-    A(b->d_lead_ends.alloc(std::max<size_t>(1, L.leadEnds.size())), "lead_ends");
-    A(b->d_lead_fix.alloc(std::max<size_t>(1, L.leadFix.size())), "lead_fix");
-    A(b->d_lead_fix_off.alloc(L.leadFixOff.size()), "lead_fix_off");
+    std::vector<unsigned char> tables;
+    {
+        auto put = [&](int k, const auto &v) {
+            b->table_off[k] = (tables.size() + 255) & ~size_t(255);
+            const size_t bytes = v.size() * sizeof(v[0]);
+            tables.resize(b->table_off[k] + bytes);
+            if (bytes) std::memcpy(tables.data() + b->table_off[k], v.data(), bytes);
+        };
+        tables.reserve(16 * E + 8 * N + 4096);
+        put(fe2_batch::kQidx, L.qidx);
+        put(fe2_batch::kPushOff, L.pushOff);
+        put(fe2_batch::kPush, L.push);
+        put(fe2_batch::kLeadEnds, L.leadEnds);
+        put(fe2_batch::kLeadFix, L.leadFix);
+        put(fe2_batch::kLeadFixOff, L.leadFixOff);
+        put(fe2_batch::kLsSlot, L.lsSlot);
+        put(fe2_batch::kLsCsrSlot, L.lsCsrSlot);
+        put(fe2_batch::kLsPartSlot, L.lsPartSlot);
+        put(fe2_batch::kLsRow, L.lsRow);
+        b->ls_tables = !L.lsSlot.empty();
+        tables.resize(tables.size() + 256);
+    }
+    A(b->d_tables.alloc(tables.size()), "tables");
     A(b->d_ek0.alloc(L.n_ell), "ek0");
     A(b->d_ek1.alloc(L.n_ell), "ek1");
     A(b->d_fpt.alloc(3 * std::max<size_t>(1, n_fslots)), "fpt");
@@ -1220,21 +1240,12 @@ extern "C" fe2_status fe2_batch_create(int32_t n_rve, const int64_t *node_off, c
     H2D(b->d_col_part.p, hcolp.data(), sizeof(int32_t) * 2 * E, "col_part");
     H2D(b->d_csr_el.p, L.csrEl.data(), sizeof(int32_t) * 2 * E, "csr_el");
     if (n_fslots) H2D(b->d_fp_slot.p, L.fpSlot.data(), sizeof(int4) * n_fslots, "fp_slot");
-    H2D(b->d_ls_slot.p, L.lsSlot.data(), sizeof(int32_t) * L.lsSlot.size(), "ls_slot");
-    H2D(b->d_ls_csr_slot.p, L.lsCsrSlot.data(), sizeof(int32_t) * L.lsCsrSlot.size(), "ls_csr_slot");
-    H2D(b->d_ls_part_slot.p, L.lsPartSlot.data(), sizeof(int32_t) * L.lsPartSlot.size(), "ls_part_slot");
-    H2D(b->d_ls_row.p, L.lsRow.data(), sizeof(int32_t) * L.lsRow.size(), "ls_row");
     H2D(b->d_fp_csr_slot.p, L.fpCsrSlot.data(), sizeof(int32_t) * 2 * E, "fp_csr_slot");
     H2D(b->d_fp_part_slot.p, L.fpPartSlot.data(), sizeof(int32_t) * L.fpPartSlot.size(), "fp_part_slot");
     H2D(b->d_fp_node.p, L.fpNode.data(), sizeof(int32_t) * N, "fp_node");
     H2D(b->d_fp_part_off.p, L.fpPartOff.data(), sizeof(int32_t) * L.fpPartOff.size(), "fp_part_off");
     H2D(b->d_fp_row.p, L.fpRow.data(), sizeof(int32_t) * (N + n_rve), "fp_row");
-    H2D(b->d_qidx.p, L.qidx.data(), sizeof(uint16_t) * 2 * E, "qidx");
-    H2D(b->d_push_off.p, L.pushOff.data(), sizeof(int32_t) * (N + n_rve), "push_off");
-    H2D(b->d_lead_ends.p, L.leadEnds.data(), sizeof(uint32_t) * L.leadEnds.size(), "lead_ends");
-    H2D(b->d_lead_fix.p, L.leadFix.data(), sizeof(int32_t) * L.leadFix.size(), "lead_fix");
-    H2D(b->d_lead_fix_off.p, L.leadFixOff.data(), sizeof(int32_t) * L.leadFixOff.size(), "lead_fix_off");
-    H2D(b->d_push.p, L.push.data(), sizeof(uint32_t) * L.push.size(), "push");
+    H2D(b->d_tables.p, tables.data(), tables.size(), "tables");
     H2D(b->d_rowptr.p, hrow.data(), sizeof(int32_t) * (N + n_rve), "rowptr");
     H2D(b->d_part_off.p, hpart.data(), sizeof(int32_t) * hpart.size(), "part_off");
     H2D(b->d_el_a.p, hEla.data(), sizeof(int32_t) * E, "el_a");
