@@ -81,6 +81,7 @@ struct SizeClass {
     bool lead_kernel = false;
     LeadShape lead = {};
     std::vector<int32_t> rves;  // in scheduling order
+    double it_sum = 0.0, it_max = 0.0;  // iterations of its RVEs in the last batched solve (0: unknown)
     int32_t queue_off = 0;      // offset of its queue in the device queue buffer
 };
 
@@ -187,6 +188,7 @@ struct fe2_batch {
     cudaGraphExec_t graph = nullptr;
     cudaStream_t cap = nullptr;           // private capture stream
     fe2_opts graph_opts = {};
+    std::vector<int> graph_pairs;         // its FP32 launches' pair_clusters, per class
     int graph_launches = 0, graph_timed = 0;
 
     DevMesh mesh() const {
@@ -1471,6 +1473,11 @@ fe2_status reorder_queues(fe2_batch *b) {
         for (auto &c : classes) {
             std::stable_sort(c.rves.begin(), c.rves.end(), [&](int32_t x, int32_t y) { return cost(x) > cost(y); });
             std::copy(c.rves.begin(), c.rves.end(), b->h_queue + which * P + c.queue_off);
+            c.it_sum = c.it_max = 0.0;
+            for (int32_t p : c.rves) {
+                c.it_sum += (double)b->h_iters[p];
+                c.it_max = std::max(c.it_max, (double)b->h_iters[p]);
+            }
         }
     }
     CUDA_TRY(cudaMemcpyAsync(b->d_queue.p, b->h_queue, sizeof(int32_t) * 2 * P, cudaMemcpyHostToDevice, b->aux));
@@ -1521,6 +1528,22 @@ int resident_mixed(fe2_batch *b, const SizeClass &c, int lead, int block, size_t
     const int r = occupancy_dr_mixed_node(block, smem, c.node, pair);
     b->occ[key] = r;
     return r;
+}
+
+// Clusters of the FP32 phase with two CTAs per SM, or 0 where one per SM is the
+// better launch. Two per SM when the queue is longer than one round at one per SM:
+// an iteration then takes 1.2 to 1.6 times as long on twice the clusters (64 RVEs
+// of 5000 nodes x 3600 iterations 22.2 ms against 30.5, 256 of 1000 x 1800 9.0
+// against 11.2). But an RVE that needs many more iterations than the others ends
+// the launch alone, and an iteration with 64 registers takes 1.35 times as long
+// (2.3 us against 1.7 at 5000 nodes), so where the last solve's iterations are
+// known the longer of both ends is compared.
+int pair_clusters(fe2_batch *b, const SizeClass &c, int block, size_t smem, int nq, int one) {
+    if (nq <= one || c.node_kind != 2 || c.node.alt) return 0;
+    const int two = resident_mixed(b, c, 0, block, smem, true);
+    if (two < 2 * one) return 0;
+    const double t_one = std::max(c.it_sum / one, c.it_max), t_two = std::max(1.25 * c.it_sum / two, 1.35 * c.it_max);
+    return t_two <= t_one ? two : 0;
 }
 
 // Timing event around a launch: recorded as a graph node while capturing.
@@ -1580,14 +1603,9 @@ fe2_status launch_class(fe2_batch *b, const fe2_opts &o, const SizeClass &c, Sol
             const size_t smem = class_smem(c, lead);
             const int block = class_block(c, lead, o.block_threads);
             const bool node = !lead && c.node_kind > 0;
-            // FP32 phase with two CTAs per SM when the queue is longer than one
-            // round at one per SM. An iteration then takes 1.2 to 1.6 times as
-            // long on twice the clusters: 64 RVEs of 5000 nodes x 3600
-            // iterations 22.2 ms against 30.5, 256 of 1000 x 1800 9.0 against
-            // 11.2.
             const int one = resident_mixed(b, c, lead, block, smem);
-            const int two = node && nq > one && c.node_kind == 2 && !c.node.alt ? resident_mixed(b, c, lead, block, smem, true) : 0;
-            const bool pair = two >= 2 * one;
+            const int two = node ? pair_clusters(b, c, block, smem, nq, one) : 0;
+            const bool pair = two > 0;
             const int resident = pair ? two : one;
             if (timed) {
                 if (*timed + 2 > (int)b->tev.size()) return fail(FE2_ECUDA, "too many launch classes");
@@ -1721,7 +1739,16 @@ fe2_status launch_solve(fe2_batch *b, const fe2_opts &o, cudaStream_t st) {
     } else {
         // one CUDA graph per option set: captured on the first solve with
         // these options, replayed by every later one
-        if (!b->graph || !same_solve_opts(b->graph_opts, o)) {
+        std::vector<int> pairs;
+        if (o.precision == FE2_PREC_MIXED)
+            for (const SizeClass &c : b->classes_mixed) {
+                const int block = class_block(c, 0, o.block_threads);
+                const size_t smem = class_smem(c, 0);
+                pairs.push_back(c.node_kind > 0 ? pair_clusters(b, c, block, smem, (int)c.rves.size(),
+                                                                resident_mixed(b, c, 0, block, smem))
+                                                : 0);
+            }
+        if (!b->graph || !same_solve_opts(b->graph_opts, o) || pairs != b->graph_pairs) {
             if (b->graph) CUDA_TRY(cudaGraphExecDestroy(b->graph));
             b->graph = nullptr;
             CUDA_TRY(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
@@ -1740,6 +1767,7 @@ fe2_status launch_solve(fe2_batch *b, const fe2_opts &o, cudaStream_t st) {
                 return fail(FE2_ECUDA, std::string("graph instantiate: ") + cudaGetErrorString(ei));
             }
             b->graph_opts = o;
+            b->graph_pairs = pairs;
             b->graph_launches = launches;
             b->graph_timed = timed;
         }
