@@ -70,8 +70,9 @@ typedef enum {
      * divide. The trajectory is bit for bit that of such an implementation;
      * only the residual and stress sums are reassociated. An RVE runs on a
      * thread-block cluster of 1 to 16 CTAs, one spatial part per CTA (more
-     * and smaller parts in batches that leave SMs idle; the residual's last
-     * bits may depend on it), with the same operations (set
+     * and smaller parts in batches that leave SMs idle; every result is the
+     * same bits whatever the parts, the CTA size and the batch), with the
+     * same operations (set
      * FE2_FP64_CLUSTER=0 in the environment before fe2_batch_create to keep
      * every RVE on one CTA). Any RVE size. */
     FE2_PREC_FP64 = 0,
@@ -464,7 +465,7 @@ const char *fe2_last_error(void);
  * own every device allocation through their own pools). It allocates nothing:
  * inputs and outputs are the caller's DEVICE buffers, and all working memory
  * is one file-scope device array of fe2_noalloc_scratch_bytes() bytes (about
- * 3.5 MB) that every GPU loading the library holds until the process exits.
+ * 3.7 MB) that every GPU loading the library holds until the process exits.
  *
  * It runs the same per-RVE FP64 solver as fe2_batch_solve with
  * FE2_PREC_FP64, on a thread-block cluster of 1 to 16 CTAs by the node count.

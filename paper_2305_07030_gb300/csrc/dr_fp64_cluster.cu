@@ -19,13 +19,22 @@
 //
 // Synchronisation. One cluster barrier per iteration, before the element
 // forces, and one CTA barrier after them. The residual test runs beside the
-// element forces, in one judging warp per CTA that does nothing else: at
-// evaluation i it sums this CTA's partials of evaluation i-1, and totals
-// evaluation i-2 across the cluster (a tree, the same bits in every CTA; on
-// parts of few nodes its chain of dependent additions is the iteration's longest:
-// 700 nodes on 16 CTAs 5.7 us with a serial sum over all workers and ranks, 4.95). The workers read its verdict after the CTA barrier. The displacements
+// element forces: at evaluation i the terms of evaluation i-1 are summed by a few
+// warps of each CTA, and one judging warp per CTA, which evaluates no elements,
+// totals evaluation i-2 across the cluster (a tree, the same bits in every CTA).
+// The workers read its verdict after the CTA barrier. The displacements
 // of the last three evaluations rotate through a ring in global memory (L2),
 // so the tested evaluation's state is still there.
+//
+// Sums. Every sum over the nodes goes leaf by leaf (Leaves below), so an RVE's
+// results do not depend on how many CTAs its batch leaves for it. The chains of
+// dependent additions are what a test costs: under load an FP64 instruction of a
+// warp waits for the pipe for 100 to 250 cycles. A leaf's terms are therefore spread over
+// 32 lanes, two leaves share a warp's tree, and warps without elements do it first.
+// Against sums by thread, warp and CTA in the judging warp alone: 512 nodes on 8
+// CTAs 4.45 -> 3.67 us per iteration, 300 RVEs of 200 to 1000 nodes with energies
+// x 200 iterations 9.7 -> 8.8 ms, 32 of 5000 x 300 unchanged (14.2 ms). With the
+// judging warp adding every leaf by itself, 32 / leaves lanes each: 6.1 us and 12.2 ms.
 //
 // What bounds it: the FP64 pipe, 2 operations per clock and SM. Per element 13
 // additions and multiplications, per free node 45 at degree 5; divisions and
@@ -33,7 +42,7 @@
 // same for the whole CTA is kept off that pipe: a residual total or a square
 // root computed by every thread costs 16 warps' slots. Measured per
 // iteration, before (totals in every thread, the acceleration stored, the
-// update a phase of its own, one-part RVEs on the single-CTA kernel) and now:
+// update a phase of its own, one-part RVEs on the single-CTA kernel) and after:
 // 5000 nodes on 8 CTAs 23.4 -> 16.0 us, 512 nodes on one CTA 18.8 -> 13.0 us.
 #include <cooperative_groups.h>
 
@@ -53,16 +62,12 @@ namespace {
 // Threads per CTA at most; the last warp judges. 16 warps are 4 per scheduler
 // and leave 128 registers per thread (17 would leave 96, and spills).
 constexpr int kMaxThreads = 512;
-constexpr int kMaxWorkers = kMaxThreads - 32;
 constexpr int kRegElems = 3;      // table elements a worker keeps in registers
 
 struct Fp64ClusterShared {
-    double part[2][4];               // this CTA's sums of evaluation n (parity n & 1):
+    double part[2][4][kMaxParts];    // sums of this CTA's leaves for evaluation n (parity n & 1):
                                      // squared residual, kinetic energy, work terms
     const double *partp[kMaxParts];  // every CTA's `part`
-    double red[32];                  // set-up reductions
-    double rs[kMaxWorkers];          // the workers' squared residuals of one evaluation
-    double wpart[3][kMaxWorkers / 32];  // per worker warp: kinetic energy, work terms
     double sig[kStressWarps][9];     // stress partials (rank 0's copy is the target)
     double *sigp;                    // rank 0's sig
     int code;                        // verdict: -1 = go on, else the RVE status
@@ -76,14 +81,44 @@ __device__ __forceinline__ void cl_wait() {
     asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }
 
-// Sum over the cluster of one value per thread (set-up only; `parity` picks
-// the publication buffer). Every thread gets the total; a cluster barrier.
-__device__ __forceinline__ double cluster_sum(cg::cluster_group &cl, Fp64ClusterShared &sh, double v, int parity) {
-    const double t = block_sum(v, sh.red);
-    if (threadIdx.x == 0) sh.part[parity][0] = t;
+// The leaves of an RVE (fe2_internal.h): its sums are formed leaf by leaf, each
+// in an order of its own, so they are the same bits whatever the cluster size,
+// the CTA size and the other RVEs of the batch.
+struct Leaves {
+    const uint16_t *list;  // this CTA's nodes by leaf; null: one leaf, in order
+    const int32_t *off;    // first entries of this CTA's leaves, counted from the RVE's
+    const int32_t *free;   // their free nodes
+    int own, total;        // leaves of this CTA and of the RVE (powers of two)
+    int base;              // the CTA's first entry
+};
+__device__ __forceinline__ Leaves make_leaves(const DevMesh &M, const RveDesc &R, int p, int me, int C, int c0) {
+    Leaves l;
+    l.total = R.fp_leaves;
+    l.own = l.total / C;
+    l.base = c0;
+    l.list = l.own > 1 ? M.fp_leaf + R.node0 + c0 : nullptr;
+    l.off = M.fp_leaf_off + (int64_t)p * 2 * (kMaxParts + 1) + me * l.own;
+    l.free = l.off + (kMaxParts + 1);
+    return l;
+}
+
+// Sum over the RVE of one value per own node (set-up only; `parity` picks the
+// publication buffer). Every thread gets the total; a cluster barrier.
+__device__ __forceinline__ double node_sum(cg::cluster_group &cl, Fp64ClusterShared &sh, const Leaves &lv,
+                                           const double *v, int m, int parity) {
+    const int lane = threadIdx.x & 31;
+    __syncthreads();
+    for (int j = threadIdx.x >> 5; j < lv.own; j += blockDim.x >> 5) {
+        const int beg = lv.list ? lv.off[j] - lv.base : 0, end = lv.list ? lv.off[j + 1] - lv.base : m;
+        double t = 0.0;
+        for (int q = beg + lane; q < end; q += 32) t = dadd(t, v[lv.list ? lv.list[q] : q]);
+        for (int o = 16; o > 0; o >>= 1) t = dadd(t, __shfl_xor_sync(0xffffffffu, t, o));
+        if (lane == 0) sh.part[parity][0][j] = t;
+    }
     cl.sync();
     double s = 0.0;
-    for (int r = 0; r < (int)cl.num_blocks(); ++r) s = dadd(s, sh.partp[r][parity * 4]);
+    for (int l = 0; l < lv.total; ++l)
+        s = dadd(s, sh.partp[l / lv.own][parity * 4 * kMaxParts + l % lv.own]);
     return s;
 }
 
@@ -146,6 +181,7 @@ __host__ __device__ inline size_t cluster_bytes(const Fp64Shape &sp) {
     if (sp.tsm)
         b += sizeof(double) * 3 * (size_t)sp.slot_max + sizeof(int32_t) * ((size_t)sp.free_max + 1) +
              sizeof(uint16_t) * (size_t)sp.row_max;
+    if (sp.ssm) b += sizeof(uint16_t) * (size_t)sp.part_max;
     return (b + 15) & ~size_t(15);
 }
 
@@ -156,17 +192,18 @@ __host__ __device__ inline size_t cluster_bytes(const Fp64Shape &sp) {
 // entry of each free node, RE: entries slot << 1 | second end) are in shared
 // memory, otherwise in global memory. With SSM the own free nodes' state (ST:
 // velocity, displacement, reference position [3][free_cap] each, mass and
-// damping factor -c m [free_cap] each, and the mass's division estimates) is in
-// shared memory, otherwise in global memory (L2).
+// damping factor -c m [free_cap] each, the mass's division estimates and the
+// force's squares) and the list of the nodes by leaf (LS) are in shared memory,
+// otherwise in global memory (L2).
 template <bool TSM, bool SSM>
 __device__ void solve_rve_fp64_cluster(cg::cluster_group &cl, Fp64ClusterShared &sh, const DevMesh &M,
                                        const DevState &S, const DevResults &O, const SolveParams &P, int p,
-                                       double *XB, double *ST, double *Tsm, int32_t *RS, uint16_t *RE,
+                                       double *XB, double *ST, double *Tsm, int32_t *RS, uint16_t *RE, uint16_t *LS,
                                        int part_cap, int free_cap, int slot_cap) {
     const RveDesc R = M.rve[p];
     const int me = (int)cl.block_rank(), C = (int)cl.num_blocks();
     const int W = blockDim.x - 32;  // workers; the last warp judges
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31;
     const bool judge = tid >= W;
     const int32_t *po = M.fp_part_off + (int64_t)p * 2 * (kMaxParts + 1);
     const int n = R.n_nodes;
@@ -199,6 +236,13 @@ __device__ void solve_rve_fp64_cluster(cg::cluster_group &cl, Fp64ClusterShared 
     double *const gv = S.v0 + n0 + c0;  // !SSM: component c at c * vstride
     const int64_t vstride = S.v1 - S.v0;
     const double mc = -R.c;
+    // squares of the free nodes' forces; kinetic energies and work terms
+    double *const G2 = SSM ? ST + 12 * free_cap : xg + c0;
+    const int gs = SSM ? free_cap : n;
+    double *const kt = S.a0 + n0 + c0, *const wt = S.we + 6 * n0 + c0;
+    const int64_t kstride = S.a1 - S.a0;
+    const Leaves lv = make_leaves(M, R, p, me, C, c0);
+    double *const nn = ring + 2 * rstride;  // set-up: one value per own node
 
     // f_ref, part 1: forces in the affine configuration x = F X (all DOFs)
     for (int k = tid; k < m; k += blockDim.x) {
@@ -208,13 +252,12 @@ __device__ void solve_rve_fp64_cluster(cg::cluster_group &cl, Fp64ClusterShared 
             xg[r * n + i] = dadd(dadd(dmul(F[3 * r], Xv[0]), dmul(F[3 * r + 1], Xv[1])), dmul(F[3 * r + 2], Xv[2]));
     }
     cl.sync();
-    double acc = 0.0;
     for (int k = tid; k < m; k += blockDim.x) {
         double g0, g1, g2;
         gather_force_fp64(M, rowptr, R.csr0, node[k], xg, xg + n, xg + 2 * n, g0, g1, g2);
-        acc += dadd(dadd(dmul(g0, g0), dmul(g1, g1)), dmul(g2, g2));
+        nn[k] = dadd(dadd(dmul(g0, g0), dmul(g1, g1)), dmul(g2, g2));
     }
-    const double f_aff = dsqrt(cluster_sum(cl, sh, acc, 0));
+    const double f_aff = dsqrt(node_sum(cl, sh, lv, nn, m, 0));
 
     // Algorithm 1: displacement BCs on fixed nodes, initial free displacement
     for (int k = tid; k < m; k += blockDim.x) {
@@ -248,6 +291,8 @@ __device__ void solve_rve_fp64_cluster(cg::cluster_group &cl, Fp64ClusterShared 
         const int ne = frow[nfr] - frow[0];
         for (int q = tid; q < ne; q += blockDim.x) RE[q] = (uint16_t)fent[frow[0] + q];
     }
+    if (SSM && lv.list)
+        for (int k = tid; k < m; k += blockDim.x) LS[k] = lv.list[k];
     Slot el[kRegElems];
 #pragma unroll
     for (int j = 0; j < kRegElems; ++j) {
@@ -260,12 +305,11 @@ __device__ void solve_rve_fp64_cluster(cg::cluster_group &cl, Fp64ClusterShared 
     const double hdt = dmul(0.5, dt);
     // getInternalForces(u); accelerations; the first partial velocity update
     // and displacement (free DOFs)
-    acc = 0.0;
     for (int k = tid; k < m; k += blockDim.x) {
         const int i = node[k];
         double g[3];
         gather_force_fp64(M, rowptr, R.csr0, i, xg, xg + n, xg + 2 * n, g[0], g[1], g[2]);
-        acc += dadd(dadd(dmul(g[0], g[0]), dmul(g[1], g[1])), dmul(g[2], g[2]));
+        nn[k] = dadd(dadd(dmul(g[0], g[0]), dmul(g[1], g[1])), dmul(g[2], g[2]));
         if (k < nfr) {
             const double mm = M.mass[n0 + i];
             const double Xv[3] = {X0[i], X1[i], X2[i]};
@@ -288,12 +332,49 @@ __device__ void solve_rve_fp64_cluster(cg::cluster_group &cl, Fp64ClusterShared 
             }
         }
     }
-    const double f0v = dsqrt(cluster_sum(cl, sh, acc, 1));
+    const double f0v = dsqrt(node_sum(cl, sh, lv, nn, m, 1));
     const double f_ref = f_aff > f0v ? f_aff : f0v;
     const double thresh = P.tol * f_ref;
     double res = 0.0, ke = 0.0, wint = 0.0, wext = 0.0;  // judging warp: of the last tested evaluation
     int rc = 1;                                          // ring index of evaluation i
-    const int nres = min(W, 3 * nfr);                    // workers with a residual
+    // Sums of the terms of evaluation i - 1, for every kind of term and leaf: entry
+    // y = 3 j + c (component c of the leaf's free node j) belongs to lane y mod 32,
+    // and the lanes' sums are added as a tree. A warp takes one kind and two leaves
+    // at a time (one if there is but one); the last warps, which have the fewest
+    // elements, begin, and the judging warp comes last where others have none.
+    const int own_sh = 31 - __clz(lv.own), pair = lv.own > 1 ? 1 : 0, grp_sh = own_sh - pair;
+    const int n_sums = (energy ? 4 : P.want_ke ? 2 : 1) << grp_sh;
+    const int nw = (int)(blockDim.x >> 5), from_end = nw - 1 - (tid >> 5);
+    const int first_sum = ns > W - 32 ? from_end : from_end == 0 ? nw - 1 : from_end - 1;
+    const double *const lsum =  // the leaf's sums that this lane adds to the totals
+        (lane & 15) < lv.total ? sh.partp[(lane & 15) >> own_sh] + ((lane & 15) & (lv.own - 1)) : nullptr;
+    auto lane_sum = [&](const double *v, int64_t vs, int l) {
+        const int beg = lv.list ? lv.off[l] - lv.base : 0, cnt = 3 * (lv.list ? lv.free[l] : nfr);
+        double t = 0.0;
+#pragma unroll 4
+        for (int y = lane; y < cnt; y += 32) {
+            const int j = beg + y / 3;
+            const int k = lv.list ? (SSM ? LS[j] : lv.list[j]) : j;
+            t = dadd(t, v[(y % 3) * vs + k]);
+        }
+        return t;
+    };
+    auto leaf_sums = [&](int64_t ev) {
+        for (int x = first_sum; x < n_sums; x += nw) {
+            const int kind = x >> grp_sh, l = (x & ((1 << grp_sh) - 1)) << pair;
+            const double *v = kind == 0 ? G2 : kind == 1 ? kt : kind == 2 ? wt : wt + 3 * n;
+            const int64_t vs = kind == 0 ? gs : kind == 1 ? kstride : n;
+            double t = lane_sum(v, vs, l), o = t;
+            if (pair) {  // lanes 0 to 15 go on with the first leaf, 16 to 31 with the second
+                const double t2 = lane_sum(v, vs, l + 1);
+                o = (lane & 16) ? t : t2;
+                t = (lane & 16) ? t2 : t;
+            }
+            t = dadd(t, __shfl_xor_sync(0xffffffffu, o, 16));
+            for (int d = 8; d > 0; d >>= 1) t = dadd(t, __shfl_xor_sync(0xffffffffu, t, d));
+            if ((lane & 15) == 0 && (lane == 0 || pair)) sh.part[ev & 1][kind][l + (lane >> 4)] = t;
+        }
+    };
     int64_t i = 1;
     for (;; ++i) {
         const uint32_t boff = (i & 1) ? 3 * cb : 0u;
@@ -311,33 +392,17 @@ __device__ void solve_rve_fp64_cluster(cg::cluster_group &cl, Fp64ClusterShared 
                 if (tid + j * W < ns) slot_force(el[j], boff, cb, T + tid + j * W, ts);
             for (int s = tid + kRegElems * W; s < ns; s += W)
                 slot_force(load_slot(M, R, slots, s, XB, me), boff, cb, T + s, ts);
+            if (i >= 2) leaf_sums(i - 1);
         } else {
-            if (i >= 2) {  // this CTA's sums of evaluation i-1
-                double t = 0.0;
-                for (int w = lane; w < nres; w += 32) t = dadd(t, sh.rs[w]);
-                for (int o = 16; o > 0; o >>= 1) t = dadd(t, __shfl_xor_sync(0xffffffffu, t, o));
-                double e[3] = {0.0, 0.0, 0.0};
-                if (P.want_ke) {
-                    for (int c = 0; c < (energy ? 3 : 1); ++c) {
-                        e[c] = lane < (W >> 5) ? sh.wpart[c][lane] : 0.0;
-                        for (int o = 16; o > 0; o >>= 1) e[c] = dadd(e[c], __shfl_xor_sync(0xffffffffu, e[c], o));
-                    }
-                }
-                double *const out = sh.part[(i - 1) & 1];
-                if (lane == 0) {
-                    out[0] = t;
-                    out[1] = e[0]; out[2] = e[1]; out[3] = e[2];
-                }
-            }
+            if (i >= 2) leaf_sums(i - 1);
             if (i >= 3) {  // verdict on evaluation i-2
-                const double *mine = (lane & 15) < C ? sh.partp[lane & 15] + (i & 1) * 4 : nullptr;
                 double tot[4] = {0.0, 0.0, 0.0, 0.0};
                 for (int c = 0; c < 4; ++c) {
                     if (c > 0 && !P.want_ke) break;
                     if (c > 1 && !energy) break;
-                    tot[c] = mine ? mine[c] : 0.0;
-                    // a tree over the CTAs: the same bits in every CTA
-                    for (int o = 1; o < C; o <<= 1) tot[c] = dadd(tot[c], __shfl_xor_sync(0xffffffffu, tot[c], o));
+                    tot[c] = lsum ? lsum[((i & 1) * 4 + c) * kMaxParts] : 0.0;
+                    // a tree over the leaves: the same bits in every CTA
+                    for (int o = 1; o < lv.total; o <<= 1) tot[c] = dadd(tot[c], __shfl_xor_sync(0xffffffffu, tot[c], o));
                 }
                 res = dsqrt(tot[0]);
                 ke = tot[1];
@@ -360,7 +425,6 @@ __device__ void solve_rve_fp64_cluster(cg::cluster_group &cl, Fp64ClusterShared 
             double *const xn = XB + ((i & 1) ? 0 : 3 * part_cap);
             const double *const up = ring + rc * rstride;
             double *const un = ring + rn * rstride;
-            double rs = 0.0, kes = 0.0, wis = 0.0, wes = 0.0;
             for (int x = tid; x < 3 * nfr; x += W) {
                 const int c = (x >= nfr) + (x >= 2 * nfr), k = x - c * nfr;
                 const double *Tc = T + c * ts;
@@ -385,17 +449,17 @@ __device__ void solve_rve_fp64_cluster(cg::cluster_group &cl, Fp64ClusterShared 
                     vv = gv[c * vstride + k]; uu = up[c * n + k]; xr = c == 0 ? X0[id] : (c == 1 ? X1[id] : X2[id]);
                 }
                 const double fd = dmul(cm, vv);
-                rs = dadd(rs, dmul(g, g));
+                G2[c * gs + k] = dmul(g, g);
                 if (energy) {
                     const double du = dmul(dt, vv);
-                    wis = dadd(wis, dmul(du, dadd(gp[c * n + k], g)));
-                    wes = dadd(wes, dmul(du, dadd(fdp[c * n + k], fd)));
+                    wt[c * n + k] = dmul(du, dadd(gp[c * n + k], g));
+                    wt[(3 + c) * n + k] = dmul(du, dadd(fdp[c * n + k], fd));
                     gp[c * n + k] = g;
                     fdp[c * n + k] = fd;
                 }
                 const double ha = dmul(hdt, f64_div_v<false>(dadd(g, fd), mm, vm));
                 const double v1 = dadd(vv, ha);
-                if (P.want_ke) kes += 0.5 * mm * (v1 * v1);
+                if (P.want_ke) kt[c * kstride + k] = dmul(dmul(0.5, mm), dmul(v1, v1));
                 const double vh = dadd(v1, ha);
                 const double u = dadd(uu, dmul(dt, vh));
                 if (SSM) {
@@ -406,20 +470,6 @@ __device__ void solve_rve_fp64_cluster(cg::cluster_group &cl, Fp64ClusterShared 
                 }
                 un[c * n + k] = u;
                 xn[c * part_cap + k] = dadd(xr, u);
-            }
-            sh.rs[tid] = rs;
-            if (P.want_ke) {
-                for (int o = 16; o > 0; o >>= 1) kes = dadd(kes, __shfl_xor_sync(0xffffffffu, kes, o));
-                if (energy)
-                    for (int o = 16; o > 0; o >>= 1) {
-                        wis = dadd(wis, __shfl_xor_sync(0xffffffffu, wis, o));
-                        wes = dadd(wes, __shfl_xor_sync(0xffffffffu, wes, o));
-                    }
-                if (lane == 0) {
-                    sh.wpart[0][warp] = kes;
-                    sh.wpart[1][warp] = wis;
-                    sh.wpart[2][warp] = wes;
-                }
             }
         }
         rc = rn;
@@ -458,7 +508,7 @@ namespace {
 __device__ __forceinline__ void map_shared(cg::cluster_group &cl, Fp64ClusterShared &sh) {
     if ((int)threadIdx.x < (int)cl.num_blocks()) {
         const int r = threadIdx.x;
-        sh.partp[r] = cl.map_shared_rank(&sh.part[0][0], r);
+        sh.partp[r] = cl.map_shared_rank(&sh.part[0][0][0], r);
     }
     if (threadIdx.x == 0) sh.sigp = cl.map_shared_rank(&sh.sig[0][0], 0);
 }
@@ -473,7 +523,8 @@ __device__ __forceinline__ void solve_in(cg::cluster_group &cl, Fp64ClusterShare
     double *T = ST + (SSM ? kStateDoubles * (size_t)sp.free_max : 0);
     int32_t *RS = reinterpret_cast<int32_t *>(T + (TSM ? 3 * (size_t)sp.slot_max : 0));
     uint16_t *RE = reinterpret_cast<uint16_t *>(RS + (TSM ? sp.free_max + 1 : 0));
-    solve_rve_fp64_cluster<TSM, SSM>(cl, sh, M, S, O, P, p, XB, ST, T, RS, RE, sp.part_max, sp.free_max, sp.slot_max);
+    uint16_t *LS = RE + (TSM ? sp.row_max : 0);
+    solve_rve_fp64_cluster<TSM, SSM>(cl, sh, M, S, O, P, p, XB, ST, T, RS, RE, LS, sp.part_max, sp.free_max, sp.slot_max);
 }
 }  // namespace
 

@@ -49,6 +49,7 @@ struct RveDesc {
     int32_t fp_free_max;
     int32_t fp_slot_max;
     int32_t fp_row_max;
+    int32_t fp_leaves;  // groups of nodes whose sums are formed first (a multiple of fp_parts)
     // FP32 phase of the mixed solver (dr_mixed_node.cu): most entries of a part's
     // increment array (free nodes, the zero entry, copies of other parts' nodes)
     // and most copies of its own nodes elsewhere; first copy; first global slot
@@ -87,8 +88,8 @@ struct LeadShape {
     bool staged, ksm;
 };
 // doubles per free node of the FP64 cluster kernel's state: velocity, displacement, reference
-// position, mass, damping factor, the mass's division estimate
-constexpr int kStateDoubles = 12;
+// position, mass, damping factor, the mass's division estimate, the force's squares
+constexpr int kStateDoubles = 15;
 
 // Read-only, create-time arrays.
 struct DevMesh {
@@ -124,6 +125,10 @@ struct DevMesh {
                                   // fp_node, and of the free nodes counted alone
     const int32_t *fp_row;        // per RVE n_free + 1 (from rp0): row offsets into
                                   // fp_csr_slot, free nodes in FP64 order
+    const uint16_t *fp_leaf;      // the nodes again leaf by leaf, ascending RVE-local ids in a
+                                  // leaf: index inside the part (null: a part is a leaf)
+    const int32_t *fp_leaf_off;   // per RVE 2*(kMaxParts+1): the leaves' first entries of
+                                  // fp_leaf (from node0), and each leaf's free nodes
     const int4 *ls_slot;          // lead: fp_slot, fp_csr_slot, fp_part_slot and fp_row by the
     const int32_t *ls_csr_slot;   // mixed solver's parts (the FP64 kernel's may divide them)
     const int32_t *ls_part_slot;
@@ -156,6 +161,8 @@ struct DevState {
     float2 *sa;                   //   (v, a.x) and (a.y, a.z)
     double *gp, *fdp;             // FP64 energy check: previous internal and damping
                                   // force per free DOF [3][N]
+    double *we;                   // FP64 cluster kernel, energy check: work terms per free
+                                  // DOF, per RVE [2][3][n] at 6 node0 (kinetic: a0, a1, a2)
     double *ualt;                 // FP64 cluster kernel: displacements of the last three
                                   // evaluations, per RVE [3][3][n] at 9 node0, FP64 order;
                                   // FP32 phase: increments of the last four, float4 [4][n]

@@ -72,7 +72,8 @@ constexpr size_t kOffNode = align256(kOffPartSlot + sizeof(int32_t) * (kMaxParts
 constexpr size_t kOffRef = align256(kOffNode + sizeof(int32_t) * kNaMaxNodes);   // (part << 16 | index in part)
 constexpr size_t kOffPartOff = align256(kOffRef + sizeof(int32_t) * kNaMaxNodes);
 constexpr size_t kOffFrow = align256(kOffPartOff + sizeof(int32_t) * 2 * (kMaxParts + 1));
-constexpr size_t kNoallocScratchBytes = align256(kOffFrow + sizeof(int32_t) * (kNaMaxNodes + 1));
+constexpr size_t kOffKin = align256(kOffFrow + sizeof(int32_t) * (kNaMaxNodes + 1));  // kinetic energies
+constexpr size_t kNoallocScratchBytes = align256(kOffKin + sizeof(double) * 3 * kNaMaxNodes);
 
 // Parts for n nodes: at least 40 nodes each, below which the latency of an
 // iteration (4 to 5 us) is no longer the work's.
@@ -463,7 +464,7 @@ __global__ void __launch_bounds__(kNaThreads) k_noalloc_pack(NaArgs A, int warm,
         RveDesc R = {};
         R.n_nodes = n; R.n_free = nf; R.n_elems = E; R.n_parts = C;
         R.dtc = dtc; R.c = A.c; R.V0 = A.V0;
-        R.fp_parts = C;
+        R.fp_parts = R.fp_leaves = C;
         R.fp_slot_max = slot_max;
         for (int r = 0; r < C; ++r) {
             R.fp_part_max = max(R.fp_part_max, part_off[r + 1] - part_off[r]);
@@ -606,6 +607,7 @@ extern "C" fe2_status fe2_rve_solve_noalloc(int32_t n_nodes, int32_t n_elems, co
     S.u0 = D(kOffU); S.u1 = S.u0 + n; S.u2 = S.u0 + 2 * n;
     S.v0 = D(kOffV); S.v1 = S.v0 + n; S.v2 = S.v0 + 2 * n;
     S.xg = D(kOffA);
+    S.a0 = D(kOffKin); S.a1 = S.a0 + n; S.a2 = S.a0 + 2 * n;
     S.ualt = D(kOffRing);
     S.fpt = D(kOffForce);
     DevResults O = {};

@@ -142,7 +142,7 @@ struct fe2_batch {
     // tables of the mixed kernels (HostLayout) in one allocation, and each one's
     // offset; the lead's slot tables only where the FP64 ones are split
     DevBuf<unsigned char> d_tables;
-    enum { kQidx, kPushOff, kPush, kLeadEnds, kLeadFix, kLeadFixOff, kLsSlot, kLsCsrSlot, kLsPartSlot, kLsRow, kTables };
+    enum { kQidx, kPushOff, kPush, kLeadEnds, kLeadFix, kLeadFixOff, kLsSlot, kLsCsrSlot, kLsPartSlot, kLsRow, kFpLeaf, kFpLeafOff, kTables };
     size_t table_off[kTables] = {};
     bool ls_tables = false;
     template <class T>
@@ -227,6 +227,8 @@ struct fe2_batch {
         m.ls_csr_slot = ls_tables ? table<int32_t>(kLsCsrSlot) : d_fp_csr_slot.p;
         m.ls_part_slot = ls_tables ? table<int32_t>(kLsPartSlot) : d_fp_part_slot.p;
         m.ls_row = ls_tables ? table<int32_t>(kLsRow) : d_fp_row.p;
+        m.fp_leaf = table<uint16_t>(kFpLeaf);
+        m.fp_leaf_off = table<int32_t>(kFpLeafOff);
         m.qidx = table<uint16_t>(kQidx);
         m.push_off = table<int32_t>(kPushOff);
         m.push = table<uint32_t>(kPush);
@@ -246,6 +248,7 @@ struct fe2_batch {
         s.tf = d_tf.p;
         s.sv = d_sv.p;
         s.gp = d_gp.p;
+        s.we = d_a.p + 3 * n_nodes;
         s.ualt = d_ualt.p;
         s.fpt = d_fpt.p;
         s.ek0 = d_ek0.p;
@@ -661,6 +664,8 @@ struct HostLayout {
     // FP64 order of the nodes, the parts' offsets in it, and the free nodes'
     // row offsets (DevMesh::fp_node, fp_part_off, fp_row)
     std::vector<int32_t> fpSlot, fpCsrSlot, fpPartSlot, fpNode, fpPartOff, fpRow;
+    std::vector<uint16_t> fpLeaf;    // DevMesh::fp_leaf, fp_leaf_off
+    std::vector<int32_t> fpLeafOff;
     // the same slot tables by the mixed solver's parts (for its lead), where the
     // FP64 ones are split further; empty otherwise
     std::vector<int32_t> lsSlot, lsCsrSlot, lsPartSlot, lsRow;
@@ -678,8 +683,9 @@ struct HostLayout {
 // FP64 pipe is 2 operations per clock and SM, so a batch that leaves SMs idle
 // spreads each RVE over more of them, up to 128 CTAs in all and 16 per RVE, as
 // long as a part keeps kSplitNodes nodes: below that the latency of an iteration
-// (4 to 5 us) is no longer the work's. Displacements are the same bits for any
-// split. One RVE, us per iteration, unsplit and split: 512 nodes 13.0, 5.0 (16
+// (4 to 5 us) is no longer the work's. Results are the same bits for any split:
+// the parts of the largest split (its leaves) are formed for every RVE and the
+// sums go leaf by leaf. One RVE, us per iteration, unsplit and split: 512 nodes 13.0, 5.0 (16
 // parts 5.3); 700 nodes 17, 5.3 (8 parts 5.6); 4000 nodes 15 (8 CTAs), 9.6.
 constexpr int kSplitNodes = 40;
 int64_t mixed_ctas(const HostLayout &L) {
@@ -687,9 +693,15 @@ int64_t mixed_ctas(const HostLayout &L) {
     for (const RveDesc &q : L.rve) ctas += q.n_parts;
     return ctas;
 }
+// Largest factor an RVE may be split by, whatever its batch.
+int fp64_leaves(const RveDesc &R) {
+    int f = 1;
+    while (2 * f * R.n_parts <= kMaxParts && R.n_nodes >= 2 * f * R.n_parts * kSplitNodes) f *= 2;
+    return f;
+}
 int fp64_split(int64_t ctas, const RveDesc &R) {
     int f = 1;
-    while (2 * f * ctas <= 128 && 2 * f * R.n_parts <= kMaxParts && R.n_nodes >= 2 * f * R.n_parts * kSplitNodes) f *= 2;
+    while (2 * f * ctas <= 128 && 2 * f <= fp64_leaves(R)) f *= 2;
     return f;
 }
 
@@ -704,34 +716,40 @@ void build_fp64_parts(const int64_t *elem_off, bool split, HostLayout &L) {
     L.fpPartOff.assign((size_t)n_rve * 2 * (kMaxParts + 1), 0);
     L.fpRow.assign((size_t)N + n_rve, 0);
     L.fpSlot.clear();
+    L.fpLeaf.assign(N, 0);
+    L.fpLeafOff.assign((size_t)n_rve * 2 * (kMaxParts + 1), 0);
+    std::vector<double> X;
+    std::vector<int> ids;
     for (int32_t p = 0; p < n_rve; ++p) {
         RveDesc &R = L.rve[p];
         const int n = R.n_nodes, nf = R.n_free, C = R.n_parts * (split ? fp64_split(ctas, R) : 1);
         const int32_t *pf = L.part.data() + (size_t)p * 2 * (kMaxParts + 1), *pg = pf + (kMaxParts + 1);
-        std::vector<std::vector<int>> fr(C), fx(C);  // per part: free and fixed nodes
-        if (C == R.n_parts) {
-            for (int r = 0; r < C; ++r) {
-                for (int k = pf[r]; k < pf[r + 1]; ++k) fr[r].push_back(k);
-                for (int k = pg[r]; k < pg[r + 1]; ++k) fx[r].push_back(nf + k);
-            }
-        } else {
-            std::vector<double> X(3 * (size_t)n);
+        // leaves: the mixed solver's parts, each bisected; RVE-local ids
+        const int F = fp64_leaves(R), G = R.n_parts * F / C;  // leaves per FP64 part
+        std::vector<std::vector<int>> leaf;
+        X.clear();
+        if (F > 1) {
+            X.resize(3 * (size_t)n);
             for (int k = 0; k < n; ++k)
                 for (int c = 0; c < 3; ++c) X[3 * k + c] = L.X[c * N + R.node0 + k];
-            std::vector<int> all(n);
-            std::iota(all.begin(), all.end(), 0);
-            std::vector<std::vector<int>> parts;
-            rcb(all, C, X.data(), 0, parts);
-            const int32_t *deg = L.row.data() + R.rp0;
-            for (int r = 0; r < C; ++r) {
-                for (int k : parts[r]) (k < nf ? fr[r] : fx[r]).push_back(k);
-                std::sort(fx[r].begin(), fx[r].end());
-                std::sort(fr[r].begin(), fr[r].end(), [&](int x, int y) {
-                    const int dx = deg[x + 1] - deg[x], dy = deg[y + 1] - deg[y];
-                    return dx > dy || (dx == dy && x < y);
-                });
-            }
         }
+        for (int r = 0; r < R.n_parts; ++r) {
+            ids.clear();
+            for (int k = pf[r]; k < pf[r + 1]; ++k) ids.push_back(k);
+            for (int k = pg[r]; k < pg[r + 1]; ++k) ids.push_back(nf + k);
+            rcb(ids, F, X.data(), 0, leaf);
+        }
+        // FP64 parts: G leaves each; ascending ids (free nodes by degree, then fixed ones)
+        std::vector<std::vector<int>> fr(C), fx(C);
+        for (int l = 0; l < R.n_parts * F; ++l) {
+            std::sort(leaf[l].begin(), leaf[l].end());
+            for (int k : leaf[l]) (k < nf ? fr : fx)[l / G].push_back(k);
+        }
+        if (G > 1)
+            for (int r = 0; r < C; ++r) {
+                std::sort(fr[r].begin(), fr[r].end());
+                std::sort(fx[r].begin(), fx[r].end());
+            }
         int32_t *node = L.fpNode.data() + R.node0, *frow = L.fpRow.data() + R.rp0;
         int32_t *off = L.fpPartOff.data() + (size_t)p * 2 * (kMaxParts + 1), *ffree = off + (kMaxParts + 1);
         int32_t *ps = L.fpPartSlot.data() + (size_t)p * (kMaxParts + 1);
@@ -751,6 +769,16 @@ void build_fp64_parts(const int64_t *elem_off, bool split, HostLayout &L) {
         for (int r = C; r <= kMaxParts; ++r) {
             off[r] = at;
             ffree[r] = nfree;
+        }
+        R.fp_leaves = R.n_parts * F;
+        int32_t *lo = L.fpLeafOff.data() + (size_t)p * 2 * (kMaxParts + 1), *lfree = lo + (kMaxParts + 1);
+        uint16_t *lp = L.fpLeaf.data() + R.node0;
+        for (int l = 0; l < R.fp_leaves; ++l) {
+            for (int k : leaf[l]) {
+                *lp++ = (uint16_t)ref[k];  // the index: parts of the cluster kernel are small
+                lfree[l] += k < nf;
+            }
+            lo[l + 1] = lo[l] + (int32_t)leaf[l].size();
         }
         R.slot0 = (int64_t)(L.fpSlot.size() / 4);
         R.fp_parts = C;
@@ -1188,6 +1216,8 @@ extern "C" fe2_status fe2_batch_create(int32_t n_rve, const int64_t *node_off, c
         put(fe2_batch::kLsCsrSlot, L.lsCsrSlot);
         put(fe2_batch::kLsPartSlot, L.lsPartSlot);
         put(fe2_batch::kLsRow, L.lsRow);
+        put(fe2_batch::kFpLeaf, L.fpLeaf);
+        put(fe2_batch::kFpLeafOff, L.fpLeafOff);
         b->ls_tables = !L.lsSlot.empty();
         tables.resize(tables.size() + 256);
     }
@@ -1206,7 +1236,7 @@ extern "C" fe2_status fe2_batch_create(int32_t n_rve, const int64_t *node_off, c
     A(b->d_el_L.alloc(E), "el_L");
     A(b->d_u.alloc(3 * N), "u");
     A(b->d_v.alloc(3 * N), "v");
-    A(b->d_a.alloc(3 * N), "a");
+    A(b->d_a.alloc(9 * N), "a");
     A(b->d_xg.alloc(3 * N), "xg");
     A(b->d_uh.alloc(3 * N), "uh");
     A(b->d_ul.alloc(3 * N), "ul");
