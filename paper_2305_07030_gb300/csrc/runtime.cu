@@ -368,30 +368,41 @@ int node_bucket(int n) {
     return b;  // 2^b <= n < 2^(b+1)
 }
 
-// Recursive coordinate bisection of `ids` into `parts` (a power of two) sets.
-void rcb(std::vector<int> ids, int parts, const double *X, int64_t base,
-         std::vector<std::vector<int>> &out) {
+// Recursive coordinate bisection of ids[at, end) in place into `parts` (a power
+// of two) consecutive pieces, whose ends are appended to `ends`. Ties go by id.
+void rcb(std::vector<int> &ids, int at, int end, int parts, const double *X, std::vector<int> &ends) {
     if (parts == 1) {
-        out.push_back(std::move(ids));
+        ends.push_back(end);
         return;
     }
     double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {-1e300, -1e300, -1e300};
-    for (int i : ids)
+    for (int q = at; q < end; ++q)
         for (int c = 0; c < 3; ++c) {
-            const double v = X[3 * (base + i) + c];
+            const double v = X[3 * (int64_t)ids[q] + c];
             lo[c] = std::min(lo[c], v);
             hi[c] = std::max(hi[c], v);
         }
     int ax = 0;
     for (int c = 1; c < 3; ++c)
         if (hi[c] - lo[c] > hi[ax] - lo[ax]) ax = c;
-    std::stable_sort(ids.begin(), ids.end(), [&](int a, int b) {
-        const double va = X[3 * (base + a) + ax], vb = X[3 * (base + b) + ax];
+    const int half = at + (end - at) / 2;
+    std::nth_element(ids.begin() + at, ids.begin() + half, ids.begin() + end, [&](int a, int b) {
+        const double va = X[3 * (int64_t)a + ax], vb = X[3 * (int64_t)b + ax];
         return va < vb || (va == vb && a < b);
     });
-    const size_t half = ids.size() / 2;
-    rcb(std::vector<int>(ids.begin(), ids.begin() + half), parts / 2, X, base, out);
-    rcb(std::vector<int>(ids.begin() + half, ids.end()), parts / 2, X, base, out);
+    rcb(ids, at, half, parts / 2, X, ends);
+    rcb(ids, half, end, parts / 2, X, ends);
+}
+// Each piece (given by its end) into `parts`.
+void rcb_each(std::vector<int> &ids, std::vector<int> &ends, int parts, const double *X) {
+    if (parts == 1) return;
+    std::vector<int> out;
+    int at = 0;
+    for (int e : ends) {
+        rcb(ids, at, e, parts, X, out);
+        at = e;
+    }
+    ends = std::move(out);
 }
 
 // How the FP32 phase holds an RVE's (or a class's) row tables: 2 = in shared
@@ -664,6 +675,7 @@ struct HostLayout {
     // FP64 order of the nodes, the parts' offsets in it, and the free nodes'
     // row offsets (DevMesh::fp_node, fp_part_off, fp_row)
     std::vector<int32_t> fpSlot, fpCsrSlot, fpPartSlot, fpNode, fpPartOff, fpRow;
+    std::vector<uint8_t> leafOf;     // each node's leaf (fp64_leaves) in its RVE
     std::vector<uint16_t> fpLeaf;    // DevMesh::fp_leaf, fp_leaf_off
     std::vector<int32_t> fpLeafOff;
     // the same slot tables by the mixed solver's parts (for its lead), where the
@@ -718,95 +730,67 @@ void build_fp64_parts(const int64_t *elem_off, bool split, HostLayout &L) {
     L.fpSlot.clear();
     L.fpLeaf.assign(N, 0);
     L.fpLeafOff.assign((size_t)n_rve * 2 * (kMaxParts + 1), 0);
-    std::vector<double> X;
-    std::vector<int> ids;
+    L.fpSlot.reserve(6 * E);
+    std::vector<int32_t> ref, slot_of;
     for (int32_t p = 0; p < n_rve; ++p) {
         RveDesc &R = L.rve[p];
         const int n = R.n_nodes, nf = R.n_free, C = R.n_parts * (split ? fp64_split(ctas, R) : 1);
-        const int32_t *pf = L.part.data() + (size_t)p * 2 * (kMaxParts + 1), *pg = pf + (kMaxParts + 1);
-        // leaves: the mixed solver's parts, each bisected; RVE-local ids
-        const int F = fp64_leaves(R), G = R.n_parts * F / C;  // leaves per FP64 part
-        std::vector<std::vector<int>> leaf;
-        X.clear();
-        if (F > 1) {
-            X.resize(3 * (size_t)n);
-            for (int k = 0; k < n; ++k)
-                for (int c = 0; c < 3; ++c) X[3 * k + c] = L.X[c * N + R.node0 + k];
-        }
-        for (int r = 0; r < R.n_parts; ++r) {
-            ids.clear();
-            for (int k = pf[r]; k < pf[r + 1]; ++k) ids.push_back(k);
-            for (int k = pg[r]; k < pg[r + 1]; ++k) ids.push_back(nf + k);
-            rcb(ids, F, X.data(), 0, leaf);
-        }
+        const int leaves = R.n_parts * fp64_leaves(R), G = leaves / C;  // G leaves in an FP64 part
         // FP64 parts: G leaves each; ascending ids (free nodes by degree, then fixed ones)
-        std::vector<std::vector<int>> fr(C), fx(C);
-        for (int l = 0; l < R.n_parts * F; ++l) {
-            std::sort(leaf[l].begin(), leaf[l].end());
-            for (int k : leaf[l]) (k < nf ? fr : fx)[l / G].push_back(k);
-        }
-        if (G > 1)
-            for (int r = 0; r < C; ++r) {
-                std::sort(fr[r].begin(), fr[r].end());
-                std::sort(fx[r].begin(), fx[r].end());
-            }
+        const uint8_t *leaf = L.leafOf.data() + R.node0;
         int32_t *node = L.fpNode.data() + R.node0, *frow = L.fpRow.data() + R.rp0;
         int32_t *off = L.fpPartOff.data() + (size_t)p * 2 * (kMaxParts + 1), *ffree = off + (kMaxParts + 1);
         int32_t *ps = L.fpPartSlot.data() + (size_t)p * (kMaxParts + 1);
-        std::vector<int32_t> ref(n);  // (part << 16 | index in part)
-        int32_t at = 0, nfree = 0;
-        for (int r = 0; r < C; ++r) {
-            off[r] = at;
-            ffree[r] = nfree;
-            nfree += (int32_t)fr[r].size();
-            int32_t k = 0;
-            for (const auto *ids : {&fr[r], &fx[r]})
-                for (int i : *ids) {
-                    ref[i] = (r << 16) | k++;
-                    node[at++] = i;
-                }
-        }
-        for (int r = C; r <= kMaxParts; ++r) {
-            off[r] = at;
-            ffree[r] = nfree;
-        }
-        R.fp_leaves = R.n_parts * F;
         int32_t *lo = L.fpLeafOff.data() + (size_t)p * 2 * (kMaxParts + 1), *lfree = lo + (kMaxParts + 1);
-        uint16_t *lp = L.fpLeaf.data() + R.node0;
-        for (int l = 0; l < R.fp_leaves; ++l) {
-            for (int k : leaf[l]) {
-                *lp++ = (uint16_t)ref[k];  // the index: parts of the cluster kernel are small
-                lfree[l] += k < nf;
-            }
-            lo[l + 1] = lo[l] + (int32_t)leaf[l].size();
+        int32_t size[kMaxParts] = {};
+        for (int k = 0; k < n; ++k) {
+            ++size[leaf[k]];
+            lfree[leaf[k]] += k < nf;
         }
+        for (int l = 0; l < leaves; ++l) lo[l + 1] = lo[l] + size[l];
+        for (int r = 0; r <= kMaxParts; ++r) {
+            off[r] = lo[std::min(r, C) * G];
+            ffree[r] = r == 0 ? 0 : ffree[r - 1];
+            for (int l = (r - 1) * G; r > 0 && r <= C && l < r * G; ++l) ffree[r] += lfree[l];
+        }
+        int32_t at[kMaxParts], to[kMaxParts];  // next index in each part, next entry of each leaf
+        for (int r = 0; r < C; ++r) at[r] = 0;
+        for (int l = 0; l < leaves; ++l) to[l] = lo[l];
+        ref.resize(n);  // (part << 16 | index in part)
+        for (int k = 0; k < n; ++k) {
+            const int l = leaf[k], r = l / G, i = at[r]++;
+            ref[k] = (r << 16) | i;
+            node[off[r] + i] = k;
+            L.fpLeaf[R.node0 + to[l]++] = (uint16_t)i;  // parts of the cluster kernel are small
+        }
+        R.fp_leaves = leaves;
         R.slot0 = (int64_t)(L.fpSlot.size() / 4);
         R.fp_parts = C;
         R.fp_part_max = R.fp_free_max = R.fp_slot_max = R.fp_row_max = 0;
-        std::vector<int32_t> slot_of(R.n_elems, -1);
+        slot_of.assign(R.n_elems, -1);
         const int32_t *row = L.row.data() + R.rp0;
         const int64_t e0 = elem_off[p];
         int32_t ns = 0, pos = 0, x = 0;
         for (int r = 0; r < C; ++r) {
             ps[r] = ns;
             const int32_t first = ns, pos0 = pos;
-            for (int k : fr[r]) {
+            const int nfr = ffree[r + 1] - ffree[r];
+            for (int i = 0; i < nfr; ++i) {
+                const int k = node[off[r] + i];
                 frow[x++] = pos;
                 for (int32_t q = row[k]; q < row[k + 1]; ++q, ++pos) {
                     const int32_t w = L.csrEl[R.csr0 + q];
                     const int32_t e = w >> 1;
                     if (slot_of[e] < first) {  // not yet a slot of this part
                         slot_of[e] = ns++;
-                        L.fpSlot.push_back(e);
-                        L.fpSlot.push_back(ref[L.Ela[e0 + e]]);
-                        L.fpSlot.push_back(ref[L.Elb[e0 + e]]);
-                        L.fpSlot.push_back((q << 1) | (w & 1));
+                        const int32_t slot[4] = {e, ref[L.Ela[e0 + e]], ref[L.Elb[e0 + e]], (q << 1) | (w & 1)};
+                        L.fpSlot.insert(L.fpSlot.end(), slot, slot + 4);
                     }
                     L.fpCsrSlot[R.csr0 + pos] = ((slot_of[e] - first) << 1) | (w & 1);
                 }
             }
-            R.fp_part_max = std::max(R.fp_part_max, (int32_t)(fr[r].size() + fx[r].size()));
-            R.fp_free_max = std::max(R.fp_free_max, (int32_t)fr[r].size());
+            R.fp_part_max = std::max(R.fp_part_max, off[r + 1] - off[r]);
+            R.fp_free_max = std::max(R.fp_free_max, nfr);
             R.fp_slot_max = std::max(R.fp_slot_max, ns - first);
             R.fp_row_max = std::max(R.fp_row_max, pos - pos0);
         }
@@ -959,23 +943,36 @@ void build_layout(int32_t n_rve, const int64_t *node_off, const double *X, const
     std::vector<int32_t> &hcol = L.col, &hcolp = L.colp, &hEla = L.Ela, &hElb = L.Elb, &hrow = L.row,
                          &hpart = L.part;
     std::vector<int64_t> &hElemOf = L.ElemOf, &hGa = L.Ga, &hGb = L.Gb;
+    L.leafOf.assign(N, 0);
     int64_t csr_pos = 0;
+    // one RVE's degrees, fixed flags, rows, parts (node ids in `all`) and new ids
+    std::vector<int> deg, rowp, fill, all, ends, owner, local, newid;
+    std::vector<uint64_t> adj;
+    std::vector<uint8_t> fx;
+    std::vector<std::vector<int>> fr, fxd;
     for (int32_t p = 0; p < n_rve; ++p) {
         const int64_t base = node_off[p];
+        const double *Xp = X + 3 * base;
         const int n = (int)(node_off[p + 1] - base);
         const int64_t e0 = elem_off[p], ne = elem_off[p + 1] - e0;
-        std::vector<int> deg(n, 0);
+        deg.assign(n, 0);
         for (int64_t e = e0; e < e0 + ne; ++e) { deg[conn[2 * e]]++; deg[conn[2 * e + 1]]++; }
-        std::vector<uint8_t> fx(n);
+        fx.resize(n);
         for (int i = 0; i < n; ++i) fx[i] = (fixed[base + i] != 0) || deg[i] == 0;
-        // CSR rows (caller ids), independent of the partition
-        std::vector<std::vector<std::pair<int, int64_t>>> rows(n);
-        for (int64_t e = e0; e < e0 + ne; ++e) {
-            const int a = conn[2 * e], c = conn[2 * e + 1];
-            rows[a].push_back({c, e});
-            rows[c].push_back({a, e});
+        // CSR rows (caller ids), independent of the partition: (neighbour << 32 | element)
+        rowp.assign(n + 1, 0);
+        for (int i = 0; i < n; ++i) rowp[i + 1] = rowp[i] + deg[i];
+        adj.resize(2 * ne);
+        fill.assign(rowp.begin(), rowp.end() - 1);
+        for (int64_t e = 0; e < ne; ++e) {
+            const int a = conn[2 * (e0 + e)], c = conn[2 * (e0 + e) + 1];
+            adj[fill[a]++] = ((uint64_t)c << 32) | (uint64_t)e;
+            adj[fill[c]++] = ((uint64_t)a << 32) | (uint64_t)e;
         }
-        for (auto &row : rows) std::sort(row.begin(), row.end());
+        for (int i = 0; i < n; ++i) {
+            const auto r0 = adj.begin() + rowp[i], r1 = adj.begin() + rowp[i + 1];
+            if (!std::is_sorted(r0, r1)) std::sort(r0, r1);
+        }
         // Parts: the smallest cluster that holds the plain state, doubled
         // (up to 16) while the FP32 kernel's element table does not fit in
         // shared memory; the autotuner may fix the count per size bucket.
@@ -983,19 +980,19 @@ void build_layout(int32_t n_rve, const int64_t *node_off, const double *X, const
         const int want = g_tuning.parts[node_bucket(n)];
         const bool forced = want >= C && want <= kMaxParts && (want & (want - 1)) == 0;
         if (forced) C = want;
-        std::vector<std::vector<int>> fr, fxd;
-        std::vector<int> owner(n), local(n);
+        owner.resize(n);
+        local.resize(n);
         int part_max = 0, free_max = 0, elem_max = 0, slot_max = 0;
+        all.resize(n);
+        std::iota(all.begin(), all.end(), 0);
+        ends.assign(1, n);
+        rcb_each(all, ends, C, Xp);
         for (;;) {
-            std::vector<int> all(n);
-            std::iota(all.begin(), all.end(), 0);
-            std::vector<std::vector<int>> parts;
-            rcb(all, C, X, base, parts);
             fr.assign(C, {});
             fxd.assign(C, {});
-            for (int r = 0; r < C; ++r) {
-                for (int i : parts[r]) (fx[i] ? fxd[r] : fr[r]).push_back(i);
-                std::stable_sort(fr[r].begin(), fr[r].end(), [&](int x, int y) {
+            for (int r = 0, q = 0; r < C; ++r) {
+                for (; q < ends[r]; ++q) (fx[all[q]] ? fxd[r] : fr[r]).push_back(all[q]);
+                std::sort(fr[r].begin(), fr[r].end(), [&](int x, int y) {
                     return deg[x] > deg[y] || (deg[x] == deg[y] && x < y);
                 });
                 std::sort(fxd[r].begin(), fxd[r].end());
@@ -1016,8 +1013,8 @@ void build_layout(int32_t n_rve, const int64_t *node_off, const double *X, const
                 int elems = 0, slots = 0;
                 for (size_t k = 0; k < fr[r].size(); ++k) {
                     const int i = fr[r][k];
-                    for (const auto &pr : rows[i]) {
-                        const int j = pr.first;
+                    for (int q = rowp[i]; q < rowp[i + 1]; ++q) {
+                        const int j = (int)(adj[q] >> 32);
                         elems += !(owner[j] == r && !fx[j] && local[j] < (int)k);
                     }
                 }
@@ -1033,6 +1030,7 @@ void build_layout(int32_t n_rve, const int64_t *node_off, const double *X, const
                                              part_max);
             if (staged || C >= kMaxParts || forced) break;
             C *= 2;
+            rcb_each(all, ends, 2, Xp);
         }
         // order: free nodes part by part (degree-sorted), then fixed part by part
         std::vector<int> order;
@@ -1053,7 +1051,7 @@ void build_layout(int32_t n_rve, const int64_t *node_off, const double *X, const
             nfixed += (int)fxd[r].size();
         }
         for (int r = C; r <= kMaxParts; ++r) pg[r] = nfixed;
-        std::vector<int> newid(n);
+        newid.resize(n);
         for (int k = 0; k < n; ++k) newid[order[k]] = k;
         RveDesc &R = L.rve[p];
         R.node0 = base;
@@ -1077,20 +1075,22 @@ void build_layout(int32_t n_rve, const int64_t *node_off, const double *X, const
             const int orig = order[k];
             L.perm_to_orig[base + k] = base + orig;
             for (int r = 0; r < 3; ++r) hX[r * N + base + k] = X[3 * (base + orig) + r];
-            auto &row = rows[orig];
-            std::sort(row.begin(), row.end());
             hrow[R.rp0 + k] = pos;
-            for (auto &pr : row) {
-                hcol[csr_pos + pos] = newid[pr.first];
-                hcolp[csr_pos + pos] = (owner[pr.first] << 16) | local[pr.first];
-                hElemOf[csr_pos + pos] = pr.second;
-                L.csrEl[csr_pos + pos] = (int32_t)(((pr.second - e0) << 1) | (conn[2 * pr.second + 1] == orig ? 1 : 0));
-                hEAcsr[csr_pos + pos] = EA[pr.second];
-                ++pos;
+            for (int q = rowp[orig]; q < rowp[orig + 1]; ++q, ++pos) {
+                const int j = (int)(adj[q] >> 32);
+                const int64_t e = e0 + (int64_t)(adj[q] & 0xffffffffu);
+                hcol[csr_pos + pos] = newid[j];
+                hcolp[csr_pos + pos] = (owner[j] << 16) | local[j];
+                hElemOf[csr_pos + pos] = e;
+                L.csrEl[csr_pos + pos] = (int32_t)(((e - e0) << 1) | (conn[2 * e + 1] == orig ? 1 : 0));
+                hEAcsr[csr_pos + pos] = EA[e];
             }
         }
         hrow[R.rp0 + n] = pos;
         csr_pos += pos;
+        rcb_each(all, ends, fp64_leaves(R), Xp);
+        for (int l = 0, q = 0; l < (int)ends.size(); ++l)
+            for (; q < ends[l]; ++q) L.leafOf[base + newid[all[q]]] = (uint8_t)l;
         for (int64_t e = e0; e < e0 + ne; ++e) {
             // the caller's orientation (a, b) is kept for lengths and the stress sum
             hEla[e] = newid[conn[2 * e]];
