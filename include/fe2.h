@@ -109,7 +109,8 @@ typedef struct {
                                external work of the energy balance check
                                (fe2_batch_energy) */
     int32_t block_threads;  /* threads per CTA: 0 = default (512, the paper's
-                               team size), else a multiple of 32 in [64, 512] */
+                               team size), else a multiple of 32 in [64, 512]
+                               (FP64 clusters add a warp for the residual test) */
     int64_t lead_iters;   /* MIXED: < 0 = lead until the relative residual
                              <= lead_tol (default); >= 0 = exactly that many
                              double-float iterations */

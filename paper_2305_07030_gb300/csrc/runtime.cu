@@ -1515,8 +1515,6 @@ fe2_status reorder_queues(fe2_batch *b) {
     return FE2_OK;
 }
 
-// Launch the solver kernels of one class on `s` for `nq` queued RVEs. Timing
-// events (tev) are recorded only when `timed` is non-null.
 int resident_of(fe2_batch *b, int kind, int parts, int block, size_t smem, int part_cap) {
     const auto key = std::make_tuple(kind, parts, block, smem, part_cap);
     auto it = b->occ.find(key);
@@ -1581,6 +1579,13 @@ cudaError_t record_timing(cudaEvent_t e, cudaStream_t s, bool capturing) {
     return capturing ? cudaEventRecordWithFlags(e, s, cudaEventRecordExternal) : cudaEventRecord(e, s);
 }
 
+// CTA size of the FP64 cluster kernel: the requested threads and the judging warp,
+// at most 512. A request for 64 threads would otherwise leave one warp for the
+// work: 152 RVEs of 400 nodes 59 us per iteration, so 30 (the single-CTA kernel 47).
+int fp64_block(const fe2_opts &o) { return o.block_threads ? std::min(512, o.block_threads + 32) : 512; }
+
+// Launch the solver kernels of one class on `s` for `nq` queued RVEs. Timing
+// events (tev) are recorded only when `timed` is non-null.
 fe2_status launch_class(fe2_batch *b, const fe2_opts &o, const SizeClass &c, SolveParams P,
                         const int32_t *queue, int nq, int32_t *counters, cudaStream_t s, int *timed,
                         int *launches, bool capturing = false) {
@@ -1593,7 +1598,7 @@ fe2_status launch_class(fe2_batch *b, const fe2_opts &o, const SizeClass &c, Sol
     P.counter = counters;
     P.smem_positions = c.smem_positions;
     if (fp64 && c.fp64_cluster) {
-        const int block = o.block_threads ? o.block_threads : 512;
+        const int block = fp64_block(o);
         const int resident = resident_fp64_cluster(b, c, block);
         if (resident < 1)
             return fail(FE2_ECUDA, "no FP64 cluster of " + std::to_string(c.parts) + " CTAs fits");
@@ -1718,7 +1723,7 @@ fe2_status warm_shapes(fe2_batch *b, const fe2_opts &o) {
     const size_t limit = b->smem_optin - 16384;
     for (const SizeClass &c : fp64 ? b->classes_fp64 : b->classes_mixed) {
         if (fp64 && c.fp64_cluster) {
-            const int block = o.block_threads ? o.block_threads : 512;
+            const int block = fp64_block(o);
             if (resident_fp64_cluster(b, c, block) < 1)
                 return fail(FE2_ECUDA, "no FP64 cluster of " + std::to_string(c.parts) + " CTAs fits");
             continue;
