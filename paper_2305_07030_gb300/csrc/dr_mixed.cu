@@ -6,7 +6,7 @@
 // dr_mixed_node.cu's, both with their tables on chip. The kernels of this file,
 // which re-read the CSR rows from L2, remain for parts whose displacements or
 // increments (with the copies of neighbours in other parts) do not fit in shared
-// memory, and for lengths and rigidities near the limits of FP32.
+// memory.
 //
 // Layout. The RVE is split spatially into `parts` pieces, one per CTA of the
 // cluster; a CTA stages the state of its own nodes in its shared memory and (in

@@ -87,12 +87,19 @@ struct NodeTables {
     int ks;         // slots in shared memory
 };
 
-__device__ __forceinline__ float rsqrt_ftz(float x) {
+// Reciprocal square root and division, with FTZ the forms that flush subnormals to
+// zero (fewer instructions): equal where nothing is subnormal (runtime.cu,
+// node_range_ok), so RVEs near FP32's limits get the others.
+template <bool FTZ>
+__device__ __forceinline__ float rsqrt_of(float x) {
+    if (!FTZ) return rsqrtf(x);
     float y;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-__device__ __forceinline__ float div_ftz(float a, float b) {
+template <bool FTZ>
+__device__ __forceinline__ float div_of(float a, float b) {
+    if (!FTZ) return __fdividef(a, b);
     float y;
     asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
     return y;
@@ -104,7 +111,7 @@ __device__ __forceinline__ float div_ftz(float a, float b) {
 // ALT: the order of the fused products in the two inner products that form h;
 // parts without tables were evaluated in that order, and keep it, so that a
 // solve's trajectory does not depend on where its tables are.
-template <int N, bool ALT>
+template <int N, bool ALT, bool FTZ>
 __device__ __forceinline__ void entry_forces(float q0, float q1, float q2, const float4 *qj, const float4 *k0,
                                              const float *qref, float &g0, float &g1, float &g2) {
     float t0[N], t1[N], t2[N];
@@ -112,12 +119,12 @@ __device__ __forceinline__ void entry_forces(float q0, float q1, float q2, const
     for (int i = 0; i < N; ++i) {
         const float r0 = k0[i].x, r1 = k0[i].y, r2 = k0[i].z, ea = k0[i].w;
         const float lr2 = dot3(r0, r1, r2, r0, r1, r2);
-        const float ril = rsqrt_ftz(lr2);
+        const float ril = rsqrt_of<FTZ>(lr2);
         const float e0 = fsub(qj[i].x, q0), e1 = fsub(qj[i].y, q1), e2 = fsub(qj[i].z, q2);
         const float h = ALT ? __fmaf_rn(2.f, dot3(r1, r0, r2, e1, e0, e2), dot3(e1, e0, e2, e1, e0, e2))
                             : __fmaf_rn(2.f, dot3(r0, r1, r2, e0, e1, e2), dot3(e0, e1, e2, e0, e1, e2));
-        const float l2 = fadd(lr2, h), rl = rsqrt_ftz(l2);
-        const float dq = div_ftz(fmul(fmul(fmul(ea, h), rl), ril), __fmaf_rn(lr2, ril, fmul(l2, rl)));
+        const float l2 = fadd(lr2, h), rl = rsqrt_of<FTZ>(l2);
+        const float dq = div_of<FTZ>(fmul(fmul(fmul(ea, h), rl), ril), __fmaf_rn(lr2, ril, fmul(l2, rl)));
         t0[i] = __fmaf_rn(qref[i], e0, fmul(dq, fadd(r0, e0)));
         t1[i] = __fmaf_rn(qref[i], e1, fmul(dq, fadd(r1, e1)));
         t2[i] = __fmaf_rn(qref[i], e2, fmul(dq, fadd(r2, e2)));
@@ -131,7 +138,7 @@ __device__ __forceinline__ void entry_forces(float q0, float q1, float q2, const
 }
 
 // The same with the entries' tables in memory; NI, K0, K1 point at the first.
-template <int N, bool ALT>
+template <int N, bool ALT, bool FTZ>
 __device__ __forceinline__ void table_forces(const float4 &qi, const float4 *Qc, const uint16_t *NI, const float4 *K0,
                                              const float *K1, float &g0, float &g1, float &g2) {
     float4 qj[N], k0[N];
@@ -142,20 +149,20 @@ __device__ __forceinline__ void table_forces(const float4 &qi, const float4 *Qc,
         k0[i] = K0[32 * i];
         qref[i] = K1[32 * i];
     }
-    entry_forces<N, ALT>(qi.x, qi.y, qi.z, qj, k0, qref, g0, g1, g2);
+    entry_forces<N, ALT, FTZ>(qi.x, qi.y, qi.z, qj, k0, qref, g0, g1, g2);
 }
 
 // A slab's row sums from memory: w entries per node.
-template <int N, bool ALT>
+template <int N, bool ALT, bool FTZ>
 __device__ __forceinline__ void row_forces(const float4 &qi, const float4 *Qc, const uint16_t *NI, const float4 *K0,
                                            const float *K1, int w, float &g0, float &g1, float &g2) {
     for (; w >= N; w -= N, NI += 32 * N, K0 += 32 * N, K1 += 32 * N)
-        table_forces<N, ALT>(qi, Qc, NI, K0, K1, g0, g1, g2);
+        table_forces<N, ALT, FTZ>(qi, Qc, NI, K0, K1, g0, g1, g2);
     if (N > 2 && w >= 2) {
-        table_forces<2, ALT>(qi, Qc, NI, K0, K1, g0, g1, g2);
+        table_forces<2, ALT, FTZ>(qi, Qc, NI, K0, K1, g0, g1, g2);
         w -= 2, NI += 64, K0 += 64, K1 += 64;
     }
-    if (w > 0) table_forces<1, ALT>(qi, Qc, NI, K0, K1, g0, g1, g2);
+    if (w > 0) table_forces<1, ALT, FTZ>(qi, Qc, NI, K0, K1, g0, g1, g2);
 }
 
 // One node's state between iterations: half-step velocity, acceleration.
@@ -244,6 +251,7 @@ __device__ __noinline__ float3 node_gref(const DevMesh &M, const DevState &S, co
 
 // Row constants of the own free nodes from the reference positions in global
 // memory; with `regather` the reference forces too.
+template <bool FTZ>
 __device__ __noinline__ void node_constants(const DevMesh &M, const DevState &S, const RveDesc &R, const Part pt,
                                             const NodeTables T, bool regather) {
     const int n = R.n_nodes, ns = (pt.nfr + 31) >> 5;
@@ -274,7 +282,7 @@ __device__ __noinline__ void node_constants(const DevMesh &M, const DevState &S,
                 const int j = M.col[kk];
                 const float2 ei = M.eaf[kk];
                 const float r0 = xr[j] - x0, r1 = xr[n + j] - x1, r2 = xr[2 * n + j] - x2;
-                const float ril = rsqrt_ftz(dot3(r0, r1, r2, r0, r1, r2));
+                const float ril = rsqrt_of<FTZ>(dot3(r0, r1, r2, r0, r1, r2));
                 k0 = make_float4(r0, r1, r2, ei.x);
                 k1 = fmul(ei.x, fsub(ei.y, ril));
             }
@@ -310,7 +318,7 @@ __device__ __noinline__ void node_finish(NodeShared &sh, const DevMesh &M, const
 // One RVE. ONE: every warp has at most one slab, whose state and first
 // kRegEntries entries per node stay in registers. MINB: CTAs per SM that the
 // registers are bounded for. The arithmetic is the same in all of them.
-template <bool ONE, int MINB, bool ALT>
+template <bool ONE, int MINB, bool ALT, bool FTZ>
 __device__ __forceinline__ void node_rve(NodeShared &sh, const DevMesh &M, const DevState &S, const DevResults &O,
                                          const SolveParams &P, const NodeShape &sp, int p, const NodeTables &T0) {
     cg::cluster_group cl = cg::this_cluster();
@@ -367,7 +375,7 @@ __device__ __forceinline__ void node_rve(NodeShared &sh, const DevMesh &M, const
             sh.st_e = first;
         }
         cl.sync();
-        node_constants(M, S, R, pt, T, false);
+        node_constants<FTZ>(M, S, R, pt, T, false);
         // Own node k's increment of the next evaluation (array par) and its
         // copies `po` in other CTAs.
         auto place = [&](int k, const float4 &next, int par, uint32_t po) {
@@ -484,7 +492,7 @@ __device__ __forceinline__ void node_rve(NodeShared &sh, const DevMesh &M, const
                 }
                 node_positions(M, S, R, pt, T.Q + par * sp.q_cap, true);
                 cl.sync();
-                node_constants(M, S, R, pt, T, true);
+                node_constants<FTZ>(M, S, R, pt, T, true);
                 for (int k = threadIdx.x; k < nfr; k += blockDim.x) {
                     const float4 g = T.G[k];
                     Motion s = load(k);
@@ -504,16 +512,16 @@ __device__ __forceinline__ void node_rve(NodeShared &sh, const DevMesh &M, const
                         float4 qj[4];
 #pragma unroll
                         for (int j = 0; j < 4; ++j) qj[j] = Qc[ci[j]];
-                        entry_forces<4, ALT>(q.x, q.y, q.z, qj, c0, c1, g0, g1, g2);
+                        entry_forces<4, ALT, FTZ>(q.x, q.y, q.z, qj, c0, c1, g0, g1, g2);
                         if (w1 == 5) {
                             qj[0] = Qc[ci[4]];
-                            entry_forces<1, ALT>(q.x, q.y, q.z, qj, c0 + 4, c1 + 4, g0, g1, g2);
+                            entry_forces<1, ALT, FTZ>(q.x, q.y, q.z, qj, c0 + 4, c1 + 4, g0, g1, g2);
                         } else if (w1 > 5) {
                             qj[0] = Qc[ci[4]];
                             qj[1] = Qc[ci[5]];
-                            entry_forces<2, ALT>(q.x, q.y, q.z, qj, c0 + 4, c1 + 4, g0, g1, g2);
+                            entry_forces<2, ALT, FTZ>(q.x, q.y, q.z, qj, c0 + 4, c1 + 4, g0, g1, g2);
                             constexpr int x = 32 * kRegEntries;
-                            row_forces<4, ALT>(q, Qc, T.NI + sl1 + x, T.K0 + sl1 + x, T.K1 + sl1 + x, w1 - kRegEntries, g0, g1, g2);
+                            row_forces<4, ALT, FTZ>(q, Qc, T.NI + sl1 + x, T.K0 + sl1 + x, T.K1 + sl1 + x, w1 - kRegEntries, g0, g1, g2);
                         }
                         if (k1 < nfr) {
                             g0 = fadd(g0, G.x); g1 = fadd(g1, G.y); g2 = fadd(g2, G.z);
@@ -529,8 +537,8 @@ __device__ __forceinline__ void node_rve(NodeShared &sh, const DevMesh &M, const
                         if (k < nfr) now[k] = qi;
                         float g0 = 0.f, g1 = 0.f, g2 = 0.f;
                         const int sl = s0 + lane;
-                        if (MINB > 1 || end <= T.ks) row_forces<MINB == 1 ? 4 : 3, ALT>(qi, Qc, T.NI + sl, T.K0 + sl, T.K1 + sl, w, g0, g1, g2);
-                        else row_forces<4, ALT>(qi, Qc, T.NI + sl, T.X0 + sl, T.X1 + sl, w, g0, g1, g2);
+                        if (MINB > 1 || end <= T.ks) row_forces<MINB == 1 ? 4 : 3, ALT, FTZ>(qi, Qc, T.NI + sl, T.K0 + sl, T.K1 + sl, w, g0, g1, g2);
+                        else row_forces<4, ALT, FTZ>(qi, Qc, T.NI + sl, T.X0 + sl, T.X1 + sl, w, g0, g1, g2);
                         if (k < nfr) {
                             const float4 g = T.G[k];
                             Motion m = load(k);
@@ -590,7 +598,7 @@ __device__ __forceinline__ void node_rve(NodeShared &sh, const DevMesh &M, const
     node_finish(sh, M, S, O, P, p, R, pt, fin >= 0 ? ring + fin * n : nullptr, status, it, r2, k2, f_ref);
 }
 
-template <bool ONE, int MINB, bool ALT>
+template <bool ONE, int MINB, bool ALT, bool FTZ>
 __global__ void __launch_bounds__(kThreads, MINB)
     dr_mixed_node_kernel(const __grid_constant__ DevMesh M, const __grid_constant__ DevState S,
                          const __grid_constant__ DevResults O, const __grid_constant__ SolveParams P,
@@ -620,7 +628,7 @@ __global__ void __launch_bounds__(kThreads, MINB)
         const int item = *cl.map_shared_rank(&sh.item, 0);
         cl.sync();
         if (item >= P.queue_len) return;
-        node_rve<ONE, MINB, ALT>(sh, M, S, O, P, sp, P.queue[item], T);
+        node_rve<ONE, MINB, ALT, FTZ>(sh, M, S, O, P, sp, P.queue[item], T);
     }
 }
 
@@ -630,10 +638,11 @@ using NodeKernel = void (*)(DevMesh, DevState, DevResults, SolveParams, NodeShap
 // pair: two CTAs per SM at 64 registers a thread hide each other's barriers and
 // gathers, for launches of more clusters than fit at one per SM (runtime.cu).
 NodeKernel pick_node(const NodeShape &sp, int block, bool pair) {
-    if (sp.alt) return dr_mixed_node_kernel<false, 1, true>;
-    if (pair) return dr_mixed_node_kernel<false, 2, false>;
-    return sp.free_cap <= block && sp.smem_slots >= sp.slot_cap ? dr_mixed_node_kernel<true, 1, false>
-                                                                : dr_mixed_node_kernel<false, 1, false>;
+    if (!sp.flush) return sp.alt ? dr_mixed_node_kernel<false, 1, true, false> : dr_mixed_node_kernel<false, 1, false, false>;
+    if (sp.alt) return dr_mixed_node_kernel<false, 1, true, true>;
+    if (pair) return dr_mixed_node_kernel<false, 2, false, true>;
+    return sp.free_cap <= block && sp.smem_slots >= sp.slot_cap ? dr_mixed_node_kernel<true, 1, false, true>
+                                                                : dr_mixed_node_kernel<false, 1, false, true>;
 }
 
 cudaLaunchConfig_t node_config(int clusters, int parts, int block, size_t smem, cudaLaunchAttribute *attr,

@@ -77,7 +77,8 @@ struct Fp64Shape {
 // shared memory (the others are streamed from global memory).
 struct NodeShape {
     int parts, q_cap, free_cap, slot_cap, push_cap, smem_slots;
-    int alt;  // order of the fused operations in an element's force (entry_forces)
+    int alt;    // order of the fused operations in an element's force (entry_forces)
+    int flush;  // RveDesc::flush_ok
 };
 // CTAs per cluster of the lead kernel (dr_mixed_lead.cu) and capacities of one
 // CTA: displacement entries, free nodes, element slots, row entries (ELL), copies

@@ -528,18 +528,19 @@ void build_classes(const std::vector<RveDesc> &rve, const std::vector<int32_t> &
             one.lead_kernel = R.part_max <= 0xffff && lead_smem(one.lead) <= limit;
             one.lead_staged = one.lead_staged && one.lead_kernel;
             one.node = NodeShape{R.n_parts, R.part_q_max, one.free_max, one.slot_max, R.part_push_max, one.slot_max, 0};
-            one.node_kind = R.flush_ok ? node_kind_of(one.node, limit) : 0;
+            one.node_kind = node_kind_of(one.node, limit);
             one.fp32_staged = one.node_kind > 0 &&
                               mixed_staged(0, mixed_fp32_smem(one.part_max, one.free_max, one.elem_max,
                                                               one.slot_max, limit), one.part_max);
             one.node.alt = !one.fp32_staged;
+            one.node.flush = R.flush_ok;
             const int bk = node_bucket(R.n_nodes);
             one.block_lead = g_tuning.block_lead[bk];
             one.block_fp32 = g_tuning.block_fp32[bk];
             bool placed = false;
             for (auto &c : out) {
                 if (c.parts != one.parts || c.lead_staged != one.lead_staged || c.fp32_staged != one.fp32_staged ||
-                    c.node_kind != one.node_kind || c.lead_kernel != one.lead_kernel || c.lead.ksm != one.lead.ksm ||
+                    c.node_kind != one.node_kind || c.node.flush != one.node.flush || c.lead_kernel != one.lead_kernel || c.lead.ksm != one.lead.ksm ||
                     c.block_lead != one.block_lead || c.block_fp32 != one.block_fp32)
                     continue;
                 SizeClass t = c;
@@ -804,7 +805,7 @@ void build_fp64_parts(const int64_t *elem_off, bool split, HostLayout &L) {
 // or a force is subnormal. A squared length of the iterations is lr2 + h, zero or
 // at least 6e-8 lr2, so lengths from 1e-12 to 1e6 keep it normal; with
 // rigidities from 1e-15 to 1e15 a flushed force term is below 1e-31 of the force
-// at unit strain.
+// at unit strain. Other RVEs run the same kernel without the flush.
 bool node_range_ok(const HostLayout &L, const RveDesc &R) {
     const int64_t N = (int64_t)L.perm_to_orig.size();
     for (int64_t e = R.elem0; e < R.elem0 + R.n_elems; ++e) {
@@ -914,7 +915,7 @@ void build_node_tables(size_t smem_cap, HostLayout &L) {
         // when the RVE shares a launch with others)
         const NodeShape sp = {C, R.part_q_max, R.part_free_max, R.part_slot_max, R.part_push_max, R.part_slot_max, 0};
         R.flush_ok = node_range_ok(L, R);
-        if (R.flush_ok && node_kind_of(sp, smem_cap) == 1) L.n_ell += (int64_t)C * R.part_slot_max;
+        if (node_kind_of(sp, smem_cap) == 1) L.n_ell += (int64_t)C * R.part_slot_max;
     }
 }
 
@@ -1550,7 +1551,8 @@ int resident_mixed(fe2_batch *b, const SizeClass &c, int lead, int block, size_t
         return r;
     }
     if (lead || c.node_kind == 0) return resident_of(b, lead, c.parts, block, smem, c.part_max);
-    const auto key = std::make_tuple(7 + (c.node_kind == 1) + 2 * pair, c.parts, block, smem, c.node.free_cap);
+    const auto key = std::make_tuple(7 + (c.node_kind == 1) + 2 * pair, c.parts, block, smem,
+                                     4 * c.node.free_cap + 2 * c.node.alt + c.node.flush);
     auto it = b->occ.find(key);
     if (it != b->occ.end()) return it->second;
     const int r = occupancy_dr_mixed_node(block, smem, c.node, pair);
@@ -1567,7 +1569,7 @@ int resident_mixed(fe2_batch *b, const SizeClass &c, int lead, int block, size_t
 // (2.3 us against 1.7 at 5000 nodes), so where the last solve's iterations are
 // known the longer of both ends is compared.
 int pair_clusters(fe2_batch *b, const SizeClass &c, int block, size_t smem, int nq, int one) {
-    if (nq <= one || c.node_kind != 2 || c.node.alt) return 0;
+    if (nq <= one || c.node_kind != 2 || c.node.alt || !c.node.flush) return 0;
     const int two = resident_mixed(b, c, 0, block, smem, true);
     if (two < 2 * one) return 0;
     const double t_one = std::max(c.it_sum / one, c.it_max), t_two = std::max(1.25 * c.it_sum / two, 1.35 * c.it_max);
