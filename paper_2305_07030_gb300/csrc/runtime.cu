@@ -849,6 +849,7 @@ void build_node_tables(size_t smem_cap, HostLayout &L) {
             continue;
         }
         for (int s = 0; s < C; ++s) {
+            const size_t before = L.push.size();
             for (int k = pf[s]; k < pf[s + 1]; ++k) {
                 off[k] = (int32_t)(L.push.size() - R.push0);
                 uint32_t seen = 0;
@@ -859,7 +860,7 @@ void build_node_tables(size_t smem_cap, HostLayout &L) {
                     L.push.push_back(((uint32_t)r << 16) | (uint32_t)(q[r]++ & 0xffff));
                 }
             }
-            R.part_push_max = std::max(R.part_push_max, (int32_t)(L.push.size() - R.push0) - off[pf[s]]);
+            R.part_push_max = std::max(R.part_push_max, (int32_t)(L.push.size() - before));
         }
         off[R.n_free] = (int32_t)(L.push.size() - R.push0);
         for (int s = 0; s < C; ++s)
