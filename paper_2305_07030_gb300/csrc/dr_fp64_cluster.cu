@@ -640,23 +640,65 @@ int occupancy_dr_fp64_cluster(int block, const Fp64Shape &sp) {
     return n;
 }
 
-constexpr size_t kSingleBytes = 200 * 1024;
-
-cudaError_t prepare_dr_fp64_single() {
-    const cudaError_t e = cudaFuncSetAttribute(dr_fp64_single_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)kSingleBytes);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(dr_fp64_single_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+// Largest power of two up to kMaxParts of CTAs with `smem` bytes each that fit on
+// the device as one cluster (0: not even one CTA).
+template <class K>
+static int largest_cluster(K kernel, size_t smem) {
+    for (int c = kMaxParts; c > 0; c /= 2) {
+        cudaLaunchAttribute attr[1];
+        Fp64Shape sp = {};
+        sp.parts = c;
+        cudaLaunchConfig_t cfg = fp64_cluster_config(1, sp, kMaxThreads, attr, nullptr);
+        cfg.dynamicSmemBytes = smem;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n > 0) return c;
+        cudaGetLastError();
+    }
+    return 0;
 }
 
-int launch_dr_fp64_single(const DevMesh &m, const DevState &s, const DevResults &r, const SolveParams &p, int parts,
-                          const int *skip, const int32_t *perm, double *u, void *stream) {
+// The same for the cluster kernel, once per device and size.
+int fp64_max_cluster(size_t smem) {
+    static std::mutex mutex;
+    static std::map<std::pair<int, size_t>, int> known;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> lock(mutex);
+    const auto key = std::make_pair(dev, smem);
+    const auto it = known.find(key);
+    if (it != known.end()) return it->second;
+    const Fp64ClusterKernel k = dr_fp64_cluster_kernel<true, true>;
+    prepare_fp64_cluster(k, smem);
+    return known[key] = largest_cluster(k, smem);
+}
+
+// Dynamic shared memory of the allocation-free call's kernel: enough for every table
+// of n nodes in `parts` pieces with n_elems elements, at most kSingleBytes.
+constexpr size_t kSingleBytes = 200 * 1024;
+static size_t single_bytes(int n, int n_elems, int parts) {
+    const int m = (n + parts - 1) / parts;
+    const Fp64Shape most = {parts, m, m, n_elems, 2 * n_elems, true, true};
+    return std::min(kSingleBytes, cluster_bytes(most));
+}
+
+cudaError_t prepare_dr_fp64_single(int *max_cluster) {
+    cudaError_t e = cudaFuncSetAttribute(dr_fp64_single_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kSingleBytes);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(dr_fp64_single_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    *max_cluster = largest_cluster(dr_fp64_single_kernel, kSingleBytes);
+    return *max_cluster > 0 ? cudaSuccess : cudaErrorLaunchOutOfResources;
+}
+
+int launch_dr_fp64_single(const DevMesh &m, const DevState &s, const DevResults &r, const SolveParams &p, int n,
+                          int n_elems, int parts, const int *skip, const int32_t *perm, double *u, void *stream) {
     cudaLaunchAttribute attr[1];
     Fp64Shape sp = {};
     sp.parts = parts;
     cudaLaunchConfig_t cfg = fp64_cluster_config(1, sp, kMaxThreads, attr, static_cast<cudaStream_t>(stream));
-    cfg.dynamicSmemBytes = kSingleBytes;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, dr_fp64_single_kernel, m, s, r, p, kSingleBytes, skip, perm, u);
+    cfg.dynamicSmemBytes = single_bytes(n, n_elems, parts);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, dr_fp64_single_kernel, m, s, r, p, cfg.dynamicSmemBytes, skip, perm, u);
     if (e != cudaSuccess) return (int)e;
     return (int)cudaGetLastError();
 }

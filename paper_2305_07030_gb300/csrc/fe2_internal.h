@@ -254,11 +254,14 @@ size_t fp64_cluster_smem(const Fp64Shape &sp);
 int launch_dr_fp64_cluster(const DevMesh &m, const DevState &s, const DevResults &r, const SolveParams &p,
                            int clusters, int block, const Fp64Shape &sp, void *stream);
 int occupancy_dr_fp64_cluster(int block, const Fp64Shape &sp);
+// CTAs of the largest cluster of that kernel, each with smem bytes, that the device
+// can hold.
+int fp64_max_cluster(size_t smem);
 // The same solver for the allocation-free call: one cluster of `parts` CTAs for
-// RVE 0 of m, tables in the caller's arrays; nothing to do when *skip.
-cudaError_t prepare_dr_fp64_single();
-int launch_dr_fp64_single(const DevMesh &m, const DevState &s, const DevResults &r, const SolveParams &p, int parts,
-                          const int *skip, const int32_t *perm, double *u, void *stream);
+// RVE 0 of m (n nodes), tables in the caller's arrays; nothing to do when *skip.
+cudaError_t prepare_dr_fp64_single(int *max_cluster);
+int launch_dr_fp64_single(const DevMesh &m, const DevState &s, const DevResults &r, const SolveParams &p, int n,
+                          int n_elems, int parts, const int *skip, const int32_t *perm, double *u, void *stream);
 // Shared memory per node of a kernel without its element table.
 size_t mixed_plain_node_bytes(int lead);
 // Resident CTAs per SM (FP64) / co-resident clusters (mixed) for a launch shape.

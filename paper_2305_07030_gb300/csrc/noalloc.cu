@@ -29,6 +29,7 @@
 
 #include "../../include/fe2.h"
 #include "dr_device.cuh"
+#include "fp64_parts.h"
 
 namespace fe2 {
 namespace {
@@ -36,7 +37,6 @@ namespace {
 constexpr int kNaMaxNodes = 4096;
 constexpr int kNaMaxElems = 16384;
 constexpr int kNaThreads = 512;
-constexpr int kNaMaxParts = kMaxParts;
 
 // Byte layout of the scratch array (every block 256-byte aligned).
 constexpr size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -74,14 +74,6 @@ constexpr size_t kOffPartOff = align256(kOffRef + sizeof(int32_t) * kNaMaxNodes)
 constexpr size_t kOffFrow = align256(kOffPartOff + sizeof(int32_t) * 2 * (kMaxParts + 1));
 constexpr size_t kOffKin = align256(kOffFrow + sizeof(int32_t) * (kNaMaxNodes + 1));  // kinetic energies
 constexpr size_t kNoallocScratchBytes = align256(kOffKin + sizeof(double) * 3 * kNaMaxNodes);
-
-// Parts for n nodes: at least 40 nodes each, below which the latency of an
-// iteration (4 to 5 us) is no longer the work's.
-int na_parts(int n) {
-    int c = 1;
-    while (c < kNaMaxParts && n >= 2 * c * 40) c *= 2;
-    return c;
-}
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocScratchBytes];
 
@@ -478,7 +470,7 @@ __global__ void __launch_bounds__(kNaThreads) k_noalloc_pack(NaArgs A, int warm,
 
 std::mutex g_na_mutex;
 void *g_na_ptr[64] = {};
-bool g_na_attr[64] = {};
+int g_na_cluster[64] = {};  // largest cluster of the solver's kernel; 0: not yet known
 thread_local std::string g_na_err;
 
 }  // namespace
@@ -532,6 +524,7 @@ extern "C" fe2_status fe2_rve_solve_noalloc(int32_t n_nodes, int32_t n_elems, co
         return FE2_ECUDA;
     }
     void *scratch = nullptr;
+    int max_cluster = 0;
     {
         // once per device, with that device current: the device address of the
         // scratch array (its name in host code is not a device address)
@@ -544,14 +537,15 @@ extern "C" fe2_status fe2_rve_solve_noalloc(int32_t n_nodes, int32_t n_elems, co
                 return FE2_ECUDA;
             }
         }
-        if (!g_na_attr[dev]) {
-            e = prepare_dr_fp64_single();
+        if (!g_na_cluster[dev]) {
+            e = prepare_dr_fp64_single(&g_na_cluster[dev]);
             if (e != cudaSuccess) {
-                g_na_err = std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e);
+                g_na_cluster[dev] = 0;
+                g_na_err = std::string("solver kernel: ") + cudaGetErrorString(e);
                 return FE2_ECUDA;
             }
-            g_na_attr[dev] = true;
         }
+        max_cluster = g_na_cluster[dev];
         scratch = g_na_ptr[dev];
     }
     NaArgs A;
@@ -577,7 +571,7 @@ extern "C" fe2_status fe2_rve_solve_noalloc(int32_t n_nodes, int32_t n_elems, co
     P.init = o.init;
     P.want_ke = o.kinetic_energy != 0 ? 1 : 0;  // kinetic energy only: no work-sum scratch here
     unsigned char *scr = static_cast<unsigned char *>(scratch);
-    const int n = n_nodes, C = na_parts(n);
+    const int n = n_nodes, C = fp64_single_parts(n, max_cluster);
     int np = 1;
     while (np < n) np *= 2;
     k_noalloc_pack<<<1, kNaThreads, sizeof(uint64_t) * np, static_cast<cudaStream_t>(stream)>>>(A, o.init == 2, C, scr);
@@ -613,7 +607,7 @@ extern "C" fe2_status fe2_rve_solve_noalloc(int32_t n_nodes, int32_t n_elems, co
     DevResults O = {};
     O.sigma = A.sigma; O.iters = A.iters; O.rel_res = A.rel_res; O.status = A.status;
     O.f_ref = D(kOffMisc); O.ke = D(kOffMisc) + 1;
-    e = (cudaError_t)launch_dr_fp64_single(M, S, O, P, C, reinterpret_cast<int *>(scr + kOffMisc + 2 * sizeof(double)),
+    e = (cudaError_t)launch_dr_fp64_single(M, S, O, P, n, n_elems, C, reinterpret_cast<int *>(scr + kOffMisc + 2 * sizeof(double)),
                                            I(kOffPerm), A.u, stream);
     if (e != cudaSuccess) {
         g_na_err = std::string("launch: ") + cudaGetErrorString(e);

@@ -23,6 +23,7 @@
 
 #include "../../include/fe2.h"
 #include "fe2_internal.h"
+#include "fp64_parts.h"
 
 using namespace fe2;
 
@@ -690,32 +691,18 @@ struct HostLayout {
     std::vector<uint32_t> leadEnds;
     std::vector<int32_t> leadFix, leadFixOff;
     int64_t n_ell = 0;
+    int max_cluster = kMaxParts;  // of the FP64 cluster kernel, on the device it is for
 };
 
-// Factor by which the FP64 cluster kernel's parts divide the mixed solver's. The
-// FP64 pipe is 2 operations per clock and SM, so a batch that leaves SMs idle
-// spreads each RVE over more of them, up to 128 CTAs in all and 16 per RVE, as
-// long as a part keeps kSplitNodes nodes: below that the latency of an iteration
-// (4 to 5 us) is no longer the work's. Results are the same bits for any split:
-// the parts of the largest split (its leaves) are formed for every RVE and the
-// sums go leaf by leaf. One RVE, us per iteration, unsplit and split: 512 nodes 13.0, 5.0 (16
-// parts 5.3); 700 nodes 17, 5.3 (8 parts 5.6); 4000 nodes 15 (8 CTAs), 9.6.
-constexpr int kSplitNodes = 40;
+// The FP64 cluster kernel's parts divide the mixed solver's (fp64_parts.h).
 int64_t mixed_ctas(const HostLayout &L) {
     int64_t ctas = 0;
     for (const RveDesc &q : L.rve) ctas += q.n_parts;
     return ctas;
 }
-// Largest factor an RVE may be split by, whatever its batch.
-int fp64_leaves(const RveDesc &R) {
-    int f = 1;
-    while (2 * f * R.n_parts <= kMaxParts && R.n_nodes >= 2 * f * R.n_parts * kSplitNodes) f *= 2;
-    return f;
-}
-int fp64_split(int64_t ctas, const RveDesc &R) {
-    int f = 1;
-    while (2 * f * ctas <= 128 && 2 * f <= fp64_leaves(R)) f *= 2;
-    return f;
+int fp64_leaves(const RveDesc &R) { return fp64_leaf_factor(R.n_nodes, R.n_parts); }
+int fp64_split(const HostLayout &L, int64_t ctas, const RveDesc &R) {
+    return fp64_split_factor(ctas, R.n_nodes, R.n_parts, L.max_cluster);
 }
 
 // The FP64 cluster kernel's part of the layout (see HostLayout): its parts are
@@ -735,7 +722,7 @@ void build_fp64_parts(const int64_t *elem_off, bool split, HostLayout &L) {
     std::vector<int32_t> ref, slot_of;
     for (int32_t p = 0; p < n_rve; ++p) {
         RveDesc &R = L.rve[p];
-        const int n = R.n_nodes, nf = R.n_free, C = R.n_parts * (split ? fp64_split(ctas, R) : 1);
+        const int n = R.n_nodes, nf = R.n_free, C = R.n_parts * (split ? fp64_split(L, ctas, R) : 1);
         const int leaves = R.n_parts * fp64_leaves(R), G = leaves / C;  // G leaves in an FP64 part
         // FP64 parts: G leaves each; ascending ids (free nodes by degree, then fixed ones)
         const uint8_t *leaf = L.leafOf.data() + R.node0;
@@ -1109,7 +1096,7 @@ void build_layout(int32_t n_rve, const int64_t *node_off, const double *X, const
     for (RveDesc &R : L.rve) {
         R.ls_slot0 = R.slot0;
         R.ls_slot_max = R.fp_slot_max;
-        split |= fp64_split(ctas, R) > 1;
+        split |= fp64_split(L, ctas, R) > 1;
     }
     if (!split) return;
     L.lsSlot = std::move(L.fpSlot);
@@ -1156,6 +1143,7 @@ extern "C" fe2_status fe2_batch_create(int32_t n_rve, const int64_t *node_off, c
 
     // ---- packing: parts, permutation, CSR rows, element list ----
     HostLayout L;
+    L.max_cluster = fp64_max_cluster(smem_cap);
     build_layout(n_rve, node_off, X, elem_off, conn, EA, fixed, V0, damping, target, smem_cap, L);
     b->rve = L.rve;
     b->perm_to_orig = L.perm_to_orig;
