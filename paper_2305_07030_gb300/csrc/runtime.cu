@@ -82,7 +82,7 @@ struct SizeClass {
     bool lead_kernel = false;
     LeadShape lead = {};
     std::vector<int32_t> rves;  // in scheduling order
-    double it_sum = 0.0, it_max = 0.0;  // iterations of its RVEs in the last batched solve (0: unknown)
+    double it_sum = 0.0, it_max = 0.0;  // mixed: iterations of its RVEs in the last batched mixed solve (0: unknown)
     int32_t queue_off = 0;      // offset of its queue in the device queue buffer
 };
 
@@ -165,6 +165,7 @@ struct fe2_batch {
     int32_t last_launches = 0;
     int32_t last_timed = 0;               // persistent launches bracketed by tev
     int last_energy = 0;                  // kinetic_energy option of the last batched solve
+    bool last_mixed = false;              // whether it was a mixed one
     cudaStream_t last_stream = nullptr;
     std::vector<cudaStream_t> side;       // forked streams for concurrent classes
     std::vector<cudaEvent_t> ev;
@@ -184,13 +185,18 @@ struct fe2_batch {
     // resident CTAs (FP64) or clusters (mixed) per launch shape, queried once
     // so that nothing but launches happens while a solve is captured
     std::map<std::tuple<int, int, int, size_t, int>, int> occ;
-    // the batched solve as a CUDA graph, valid for the options it was
-    // captured with (the kernels read F, queues and state from device memory)
-    cudaGraphExec_t graph = nullptr;
+    // the batched solve as a CUDA graph, for the options and the FP32 launches'
+    // pair_clusters (per class) that it was captured with. The last two are kept, the
+    // one in use first: a change of pair_clusters, or an affine solve and a warm one
+    // in turn, would otherwise capture in every solve.
+    struct SolveGraph {
+        cudaGraphExec_t exec = nullptr;
+        fe2_opts opts = {};
+        std::vector<int> pairs;
+        int launches = 0, timed = 0;
+    };
+    SolveGraph graphs[2];
     cudaStream_t cap = nullptr;           // private capture stream
-    fe2_opts graph_opts = {};
-    std::vector<int> graph_pairs;         // its FP32 launches' pair_clusters, per class
-    int graph_launches = 0, graph_timed = 0;
 
     DevMesh mesh() const {
         DevMesh m;
@@ -284,8 +290,10 @@ struct fe2_batch {
         aux = nullptr;
         if (ev_done) cudaEventDestroy(ev_done);
         ev_done = nullptr;
-        if (graph) cudaGraphExecDestroy(graph);
-        graph = nullptr;
+        for (auto &g : graphs) {
+            if (g.exec) cudaGraphExecDestroy(g.exec);
+            g.exec = nullptr;
+        }
         if (cap) cudaStreamDestroy(cap);
         cap = nullptr;
         if (h_iters) cudaFreeHost(h_iters);
@@ -1493,6 +1501,7 @@ fe2_status reorder_queues(fe2_batch *b) {
         for (auto &c : classes) {
             std::stable_sort(c.rves.begin(), c.rves.end(), [&](int32_t x, int32_t y) { return cost(x) > cost(y); });
             std::copy(c.rves.begin(), c.rves.end(), b->h_queue + which * P + c.queue_off);
+            if (which == 0 || !b->last_mixed) continue;  // a mixed solve's counts (pair_clusters)
             c.it_sum = c.it_max = 0.0;
             for (int32_t p : c.rves) {
                 c.it_sum += (double)b->h_iters[p];
@@ -1556,12 +1565,14 @@ int resident_mixed(fe2_batch *b, const SizeClass &c, int lead, int block, size_t
 // against 11.2). But an RVE that needs many more iterations than the others ends
 // the launch alone, and an iteration with 64 registers takes 1.35 times as long
 // (2.3 us against 1.7 at 5000 nodes), so where the last solve's iterations are
-// known the longer of both ends is compared.
+// known the longer of both ends is compared (for nq of the class's RVEs their share
+// of the total).
 int pair_clusters(fe2_batch *b, const SizeClass &c, int block, size_t smem, int nq, int one) {
     if (nq <= one || c.node_kind != 2 || c.node.alt || !c.node.flush) return 0;
     const int two = resident_mixed(b, c, 0, block, smem, true);
     if (two < 2 * one) return 0;
-    const double t_one = std::max(c.it_sum / one, c.it_max), t_two = std::max(1.25 * c.it_sum / two, 1.35 * c.it_max);
+    const double total = c.it_sum * nq / (double)c.rves.size();
+    const double t_one = std::max(total / one, c.it_max), t_two = std::max(1.25 * total / two, 1.35 * c.it_max);
     return t_two <= t_one ? two : 0;
 }
 
@@ -1763,8 +1774,6 @@ fe2_status launch_solve(fe2_batch *b, const fe2_opts &o, cudaStream_t st) {
         const fe2_status r = record_solve(b, o, st, false, &launches, &timed);
         if (r != FE2_OK) return r;
     } else {
-        // one CUDA graph per option set: captured on the first solve with
-        // these options, replayed by every later one
         std::vector<int> pairs;
         if (o.precision == FE2_PREC_MIXED)
             for (const SizeClass &c : b->classes_mixed) {
@@ -1774,9 +1783,16 @@ fe2_status launch_solve(fe2_batch *b, const fe2_opts &o, cudaStream_t st) {
                                                                 resident_mixed(b, c, 0, block, smem))
                                                 : 0);
             }
-        if (!b->graph || !same_solve_opts(b->graph_opts, o) || pairs != b->graph_pairs) {
-            if (b->graph) CUDA_TRY(cudaGraphExecDestroy(b->graph));
-            b->graph = nullptr;
+        // a graph is captured where neither of the last two has these options and
+        // launch shapes, and replayed by every later solve that has them
+        auto valid = [&](const fe2_batch::SolveGraph &g) {
+            return g.exec && same_solve_opts(g.opts, o) && g.pairs == pairs;
+        };
+        fe2_batch::SolveGraph &G = b->graphs[0];
+        if (!valid(G)) std::swap(b->graphs[0], b->graphs[1]);
+        if (!valid(G)) {
+            if (G.exec) CUDA_TRY(cudaGraphExecDestroy(G.exec));
+            G.exec = nullptr;
             CUDA_TRY(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
             const fe2_status r = record_solve(b, o, b->cap, true, &launches, &timed);
             cudaGraph_t g = nullptr;
@@ -1786,23 +1802,24 @@ fe2_status launch_solve(fe2_batch *b, const fe2_opts &o, cudaStream_t st) {
                 return r;
             }
             if (e != cudaSuccess) return fail(FE2_ECUDA, std::string("graph capture: ") + cudaGetErrorString(e));
-            const cudaError_t ei = cudaGraphInstantiate(&b->graph, g, 0);
+            const cudaError_t ei = cudaGraphInstantiate(&G.exec, g, 0);
             cudaGraphDestroy(g);
             if (ei != cudaSuccess) {
-                b->graph = nullptr;
+                G.exec = nullptr;
                 return fail(FE2_ECUDA, std::string("graph instantiate: ") + cudaGetErrorString(ei));
             }
-            b->graph_opts = o;
-            b->graph_pairs = pairs;
-            b->graph_launches = launches;
-            b->graph_timed = timed;
+            G.opts = o;
+            G.pairs = pairs;
+            G.launches = launches;
+            G.timed = timed;
         }
-        CUDA_TRY(cudaGraphLaunch(b->graph, st));
-        launches = b->graph_launches;
-        timed = b->graph_timed;
+        CUDA_TRY(cudaGraphLaunch(G.exec, st));
+        launches = G.launches;
+        timed = G.timed;
     }
     b->last_launches = launches;
     b->last_energy = o.kinetic_energy;
+    b->last_mixed = o.precision == FE2_PREC_MIXED;
     b->last_timed = timed / 2;
     b->last_stream = st;
     b->solved = true;
@@ -2037,6 +2054,7 @@ extern "C" fe2_status fe2_batch_solve_naive(fe2_batch *b, const double *F, const
     CUDA_TRY(cudaStreamSynchronize(st));
     b->last_launches = launches;
     b->last_energy = 0;
+    b->last_mixed = false;
     b->last_timed = 0;
     b->last_stream = st;
     b->solved = true;
