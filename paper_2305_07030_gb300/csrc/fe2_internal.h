@@ -92,12 +92,8 @@ struct LeadShape {
 // position, mass, damping factor, the mass's division estimate, the force's squares
 constexpr int kStateDoubles = 15;
 
-// The kernels' argument blocks begin on 16 bytes: with a DevState of 8 modulo 16 the
-// FP32 phase read the arguments behind it in smaller pieces, 1.7 % more time per
-// iteration (one RVE of 5000 nodes, 38.4 -> 39.1 ms for 20,000).
-
 // Read-only, create-time arrays.
-struct alignas(16) DevMesh {
+struct DevMesh {
     const RveDesc *rve;
     const double *X0, *X1, *X2;   // reference coordinates (permuted)
     const float *Xh, *Xl;         // reference coordinates as double-float, [3][N]
@@ -152,7 +148,7 @@ struct alignas(16) DevMesh {
 };
 
 // Mutable solver state (device).
-struct alignas(16) DevState {
+struct DevState {
     double *u0, *u1, *u2;         // displacement (output of every mode)
     double *v0, *v1, *v2;         // FP64 velocity
     double *a0, *a1, *a2;         // FP64 acceleration
