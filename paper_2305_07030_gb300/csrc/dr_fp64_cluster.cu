@@ -239,8 +239,8 @@ __device__ void solve_rve_fp64_cluster(cg::cluster_group &cl, Fp64ClusterShared 
     // squares of the free nodes' forces; kinetic energies and work terms
     double *const G2 = SSM ? ST + 12 * free_cap : xg + c0;
     const int gs = SSM ? free_cap : n;
-    double *const kt = S.a0 + n0 + c0, *const wt = S.we + 6 * n0 + c0;
     const int64_t kstride = S.a1 - S.a0;
+    double *const kt = S.a0 + n0 + c0, *const wt = S.a0 + 3 * kstride + 6 * n0 + c0;
     const Leaves lv = make_leaves(M, R, p, me, C, c0);
     double *const nn = ring + 2 * rstride;  // set-up: one value per own node
 

@@ -255,7 +255,6 @@ struct fe2_batch {
         s.tf = d_tf.p;
         s.sv = d_sv.p;
         s.gp = d_gp.p;
-        s.we = d_a.p + 3 * n_nodes;
         s.ualt = d_ualt.p;
         s.fpt = d_fpt.p;
         s.ek0 = d_ek0.p;
@@ -1234,7 +1233,7 @@ extern "C" fe2_status fe2_batch_create(int32_t n_rve, const int64_t *node_off, c
     A(b->d_el_L.alloc(E), "el_L");
     A(b->d_u.alloc(3 * N), "u");
     A(b->d_v.alloc(3 * N), "v");
-    A(b->d_a.alloc(9 * N), "a");
+    A(b->d_a.alloc(9 * N), "a");  // and the work terms (DevState::a0)
     A(b->d_xg.alloc(3 * N), "xg");
     A(b->d_uh.alloc(3 * N), "uh");
     A(b->d_ul.alloc(3 * N), "ul");
