@@ -179,8 +179,8 @@ def stress_errors(args, sigma, status):
 
 
 def fp64_alu_seconds(nets, iters, rates):
-    """Lower bound on the FP64 kernel's time from its operation counts and the
-    measured FP64 rates: per element with a free end 13 add/multiply, 2
+    """Time of an FP64 kernel that does every operation on the FP64 pipe, from the
+    measured rates: per element with a free end 13 add/multiply, 2
     divisions and 1 square root; per free node 34 + 3 x degree add/multiply
     and 3 divisions (the update, the element-table sum, damping, residual,
     acceleration and velocity), every operation on the FP64 pipe."""
@@ -193,6 +193,19 @@ def fp64_alu_seconds(nets, iters, rates):
         nf = int(free.sum())
         addmul = 13 * ef + 34 * nf + 3 * int(deg[free].sum())
         t += int(it) * (addmul / fma + (2 * ef + 3 * nf) / div + ef / sqrt)
+    return t
+
+
+def fp64_pipe_seconds(nets, iters, fma):
+    """Lower bound on the FP64 cluster kernel's time from the operations it leaves
+    on the FP64 pipe (divisions and square roots run on the integer pipes): per
+    element with a free end 13 add/multiply, per free node 30 + 3 x degree."""
+    t = 0.0
+    for n, it in zip(nets, iters):
+        deg = np.bincount(n.elems.ravel(), minlength=n.n_nodes)
+        free = (n.fixed == 0) & (deg > 0)
+        ef = int((free[n.elems[:, 0]] | free[n.elems[:, 1]]).sum())
+        t += int(it) * (13 * ef + 30 * int(free.sum()) + 3 * int(deg[free].sum())) / fma
     return t
 
 
@@ -326,15 +339,16 @@ def run_ours(args, rank, world):
         rates = fe2.probe_fp64_rates()
         kms = statistics.mean(sum(k) for k in kernel_ms) / max(1, n_cls)
         kmax = statistics.mean(max(k) for k in kernel_ms)
-        t_alu = fp64_alu_seconds(nets, iters, rates)
+        t_alu = fp64_pipe_seconds(nets, iters, rates[0])
         node_iters = float((nn * iters).sum())
         roof = {"bound": "alu", "achieved": node_iters / (kmax * 1e-3) / 1e9,
                 "peak": node_iters / t_alu / 1e9, "unit": "G node-iterations/s",
                 "frac": t_alu / (kmax * 1e-3), "traffic": None, "kernel": "dr_fp64_kernel / dr_fp64_cluster_kernel",
                 "kernel_ms": kmax, "kernel_ms_mean_per_class": kms,
                 "fp64_rates_per_s": {"fma": rates[0], "div": rates[1], "sqrt": rates[2]},
-                "peak_source": "derived: the kernel's FP64 operation counts per element and free "
-                               "node at the rates measured live by fe2_probe_fp64_rates",
+                "peak_source": "derived: the kernel's FP64 additions and multiplications per element "
+                               "and free node at the rate measured live by fe2_probe_fp64_rates",
+                "frac_div_sqrt_at_hw_rate": fp64_alu_seconds(nets, iters, rates) / (kmax * 1e-3),
                 "smem_view": {"bytes_per_node_iter": BYTES_PER_NODE_ITER["fp64"],
                               "GBps": BYTES_PER_NODE_ITER["fp64"] * node_iters / (kmax * 1e-3) / 1e9,
                               "frac_of_smem": BYTES_PER_NODE_ITER["fp64"] * node_iters /

@@ -137,8 +137,9 @@ void fe2_opts_default(fe2_opts *opts);
  * 2^b <= n_nodes < 2^(b+1): the cluster size (CTAs, i.e. spatial parts, per
  * RVE; a power of two <= 16) and the CTA sizes of the FP32 and lead kernels
  * (multiples of 32 in [64, 512]). Zero entries mean automatic: the smallest
- * cluster whose parts hold at most 1024 nodes, doubled while the FP32
- * kernel's element table does not fit in shared memory, and 512 threads.
+ * cluster whose parts hold at most 1024 nodes, doubled while the parts do not
+ * meet the FP32 phase's footprint rule (120 bytes per node and 52 per element
+ * within shared memory), and 512 threads.
  * The paper found the best team size to depend on the sub-problem size
  * (Section III); fe2_autotune measures it on this GPU.
  *

@@ -42,8 +42,8 @@
 // same for the whole CTA is kept off that pipe: a residual total or a square
 // root computed by every thread costs 16 warps' slots. Measured per
 // iteration, before (totals in every thread, the acceleration stored, the
-// update a phase of its own, one-part RVEs on the single-CTA kernel) and after:
-// 5000 nodes on 8 CTAs 23.4 -> 16.0 us, 512 nodes on one CTA 18.8 -> 13.0 us.
+// update a phase of its own, one-part RVEs on the single-CTA kernel) and now:
+// 5000 nodes on 8 CTAs 23.4 -> 15.8 us, 512 nodes on one CTA 18.8 -> 12.2 us.
 #include <cooperative_groups.h>
 
 #include <algorithm>

@@ -95,8 +95,6 @@ struct MixedShared {
     // next ones must reach a quarter of, and the evaluation that set it
     float st_h, st_l;
     long long st_e;
-    int elems;                                // FP32 kernel: elements of this CTA's part
-    int slots;                                // FP32 kernel: row slots of this CTA's part
 };
 
 // Double-float total of the cluster's per-warp partials (buffer `buf`),
@@ -452,8 +450,6 @@ __device__ void fp32_rve(cg::cluster_group &cl, MixedShared &sh, const DevMesh &
                 xr[c] = df_add({Xh[c * n + i], Xl[c * n + i]}, {uh[c * n + i], ul[c * n + i]}).hi;
             Pl[k] = make_float4(xr[0], xr[1], xr[2], 0.f);
             for (int b = 0; b < kBufs; ++b) Qb[b][k] = make_float4(0.f, 0.f, 0.f, 0.f);
-            // velocity and acceleration of own free nodes live in shared memory
-            // (rewritten every iteration; global stores would miss L1 each time)
             if (k < pt.nfr) {
                 SV[k] = make_float4(vh[i], vh[n + i], vh[2 * n + i], ah[i]);
                 SA[k] = make_float2(ah[n + i], ah[2 * n + i]);
@@ -801,9 +797,10 @@ void prepare(K kernel, size_t smem) {
 }  // namespace
 
 // Footprint rule of the cluster size: a part's node state (120 B per node) and
-// 52 B per element of its rows within the limit. A part that meets it has its
-// row tables wholly in shared memory in dr_mixed_node.cu's kernel, whose own
-// need is smaller.
+// 52 B per element of its rows within the limit. This is the size of an earlier
+// FP32 kernel; dr_mixed_node.cu's, whose row tables are then wholly in shared memory,
+// needs less. The rule stays because it sets an RVE's parts, CTA sizes and (parts
+// beyond it) order of fused operations: another one would change the trajectories.
 size_t mixed_fp32_smem(int part_cap, int free_cap, int elem_cap, int slot_cap, size_t limit) {
     const size_t plain = kFp32PlainNodeBytes * (size_t)part_cap;
     const size_t F = (size_t)free_cap, U = (size_t)elem_cap, S = (size_t)slot_cap;
@@ -812,9 +809,12 @@ size_t mixed_fp32_smem(int part_cap, int free_cap, int elem_cap, int slot_cap, s
     return staged <= limit ? staged : plain;
 }
 
-// Footprint rule of the lead: with the table (dr_mixed_lead.cu, STAGED) when a
+// Footprint rule of the lead: the staged form (dr_mixed_lead.cu, STAGED) when a
 // part's displacements, state and element records are within the limit by this
-// count; that kernel's own need is smaller.
+// count. It is an earlier lead kernel's size too (the present one needs less: 109 KB
+// at 800 nodes on one CTA, 187 KB at 1250 on each of 16) and stays for the same
+// reason: the form decides the CTA size, the order of the residual's sum and the
+// evaluation at which the lead ends.
 size_t mixed_lead_smem(int part_cap, int free_cap, int elem_cap, int slot_cap, size_t limit) {
     const size_t plain = kLeadPlainNodeBytes * (size_t)part_cap;
     const size_t F = (size_t)free_cap, U = (size_t)elem_cap, S = (size_t)slot_cap;

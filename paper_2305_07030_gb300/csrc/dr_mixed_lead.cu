@@ -31,7 +31,7 @@
 // evaluated from both ends): 64 RVEs of 5000 nodes x 400 iterations 12.6 -> 11.2
 // ms, 256 of 1000 x 200 4.35 -> 3.98, 8 of 37 to 200 x 100 0.31 -> 0.25, 24 of
 // 1k to 33k x 200 10.3 -> 6.9 (the parts without a table), and the one-part RVEs
-// of 780 to 900 nodes, which had none either, 22.7 -> 6.9 us per iteration.
+// of 780 to about 820 nodes, which had none either, 22.2 -> 8.3 us per iteration (790 nodes).
 #include <algorithm>
 #include <map>
 #include <mutex>
@@ -186,9 +186,9 @@ __device__ __noinline__ double lead_start(LeadShared &sh, const DevMesh &M, cons
         }
     }
     cg::this_cluster().sync();
-    // |g|^2 in the two orders of its fused products: parts without the table have
-    // always summed the affine force's (AFF) and the initial force's in different
-    // ones, and keep them; the others use the second for both.
+    // |g|^2 in the two orders of its fused products: parts beyond the footprint rule
+    // have always summed the affine force's (AFF) and the initial force's in different
+    // ones; they keep them (and an affine start its second sum) only for f_ref's bits.
     auto square = [&](const df *g, bool aff) {
         const float x = g[0].hi, y = g[1].hi, z = g[2].hi;
         return aff && !staged ? dot3(y, x, z, y, x, z) : dot3(x, y, z, x, y, z);

@@ -108,9 +108,9 @@ __device__ __forceinline__ float div_of(float a, float b) {
 // Force increments on a node from N row entries, t(d_ref + dd) - t(d_ref) =
 // q_ref dd + dq (r + dd), added to g in row order. N independent chains: one is
 // about 200 cycles of latency, so one at a time would leave the pipes idle.
-// ALT: the order of the fused products in the two inner products that form h;
-// parts without tables were evaluated in that order, and keep it, so that a
-// solve's trajectory does not depend on where its tables are.
+// ALT: the order of the fused products in the two inner products that form h. Parts
+// beyond the footprint rule (mixed_fp32_smem) have the second one, only so that
+// their trajectories keep the bits they have always had.
 template <int N, bool ALT, bool FTZ>
 __device__ __forceinline__ void entry_forces(float q0, float q1, float q2, const float4 *qj, const float4 *k0,
                                              const float *qref, float &g0, float &g1, float &g2) {

@@ -39,7 +39,7 @@ struct RveDesc {
     double V0;        // reference volume
     int32_t part_max;       // largest part (nodes), sizes the shared memory
     int32_t part_free_max;  // most free nodes in one part
-    int32_t part_elem_max;  // FP32 kernel: most table elements of one part
+    int32_t part_elem_max;  // footprint rules: most elements with an end in one part
     int32_t part_slot_max;  // FP32 kernel: most row slots (ELL, 32-node slabs) of one part
     int64_t slot0;          // FP64 cluster kernel: first element slot of this RVE
     // FP64 cluster kernel: its parts (a multiple of n_parts), the largest of
@@ -162,7 +162,7 @@ struct DevState {
     float *fg;                    // MIXED: reference force g_ref, FP32 [3][N]
     double *xg;                   // [3][N] FP64 positions scratch
     double *tf;                   // FP64: per element, its force on the first node (3)
-    float4 *sv;                   // MIXED FP32 kernel without element table: per node
+    float4 *sv;                   // MIXED FP32 kernel without tables: per node
     float2 *sa;                   //   (v, a.x) and (a.y, a.z)
     double *gp, *fdp;             // FP64 energy check: previous internal and damping
                                   // force per free DOF [3][N]
@@ -229,11 +229,10 @@ int launch_dr_fp64(const DevMesh &m, const DevState &s, const DevResults &r,
 int launch_dr_mixed(const DevMesh &m, const DevState &s, const DevResults &r,
                     const SolveParams &p, int lead, int clusters, int parts, int block,
                     size_t smem, int part_cap, void *stream);
-// Dynamic shared memory of the FP32 kernel for a class: the staged node state,
-// plus each part's element table and rows when they fit within `limit` bytes.
+// Footprint rules of the mixed solver (dr_mixed.cu): the bytes of a part with tables
+// where they are within `limit`, else of its plain node state. The first sets the
+// number of parts and the FP32 phase's order of operations, the second the lead's form.
 size_t mixed_fp32_smem(int part_cap, int free_cap, int elem_cap, int slot_cap, size_t limit);
-// Dynamic shared memory of the lead kernel for a class: one double-float
-// displacement per node, or two plus the element table when they fit.
 size_t mixed_lead_smem(int part_cap, int free_cap, int elem_cap, int slot_cap, size_t limit);
 // Lead kernel (dr_mixed_lead.cu): dynamic shared memory, launch, co-resident
 // clusters.
@@ -247,7 +246,7 @@ size_t mixed_node_smem(const NodeShape &sp);
 int launch_dr_mixed_node(const DevMesh &m, const DevState &s, const DevResults &r, const SolveParams &p,
                          int clusters, int block, size_t smem, const NodeShape &sp, bool pair, void *stream);
 int occupancy_dr_mixed_node(int block, size_t smem, const NodeShape &sp, bool pair);
-// Whether a launch with `smem` bytes uses the shared-memory element table.
+// Whether a footprint of `smem` bytes (by the rules above) is one with tables.
 bool mixed_staged(int lead, size_t smem, int part_cap);
 // FP64 cluster kernel (dr_fp64_cluster.cu): dynamic shared memory, launch,
 // co-resident clusters. `block`: threads per CTA, the last warp of which tests
@@ -264,7 +263,7 @@ int fp64_max_cluster(size_t smem);
 cudaError_t prepare_dr_fp64_single(int *max_cluster);
 int launch_dr_fp64_single(const DevMesh &m, const DevState &s, const DevResults &r, const SolveParams &p, int n,
                           int n_elems, int parts, const int *skip, const int32_t *perm, double *u, void *stream);
-// Shared memory per node of a kernel without its element table.
+// Shared memory per node of a kernel without tables (dr_mixed.cu).
 size_t mixed_plain_node_bytes(int lead);
 // Resident CTAs per SM (FP64) / co-resident clusters (mixed) for a launch shape.
 int occupancy_dr_fp64(int smem_positions, int block, size_t smem);

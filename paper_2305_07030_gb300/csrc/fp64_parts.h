@@ -2,9 +2,10 @@
 //
 // The FP64 pipe is 2 operations per clock and SM, so RVEs that leave SMs idle are
 // spread over more of them, up to 16 CTAs each as long as a part keeps kSplitNodes
-// nodes: below that the latency of an iteration (4 to 5 us) is no longer the
-// work's. One RVE, us per iteration, unsplit and split: 512 nodes 13.0, 5.0 (16
-// parts 5.3); 700 nodes 17, 5.3 (8 parts 5.6); 4000 nodes 15 (8 CTAs), 9.6.
+// nodes: below that the latency of an iteration (3.5 us) is no longer the
+// work's. One RVE, us per iteration: 512 nodes on 1 CTA 13.0, on 8 5.0, on 16 5.3;
+// 700 nodes on 1 CTA 17, on 8 5.6, on 16 5.3 (taken with the sums of before; now 3.5 for
+// both on 8 and 16); 5000 nodes on 8 CTAs 15.8, on 16 9.7.
 //
 // max_cluster is the largest cluster that the device can hold (fp64_max_cluster): a
 // larger one could never be placed, and such an RVE runs on fewer CTAs.

@@ -14,7 +14,7 @@
 // The split follows the nodes' Morton order, cut into equal pieces: about the
 // bisection's octants for evenly spread nodes, from one sort. The FP64 pipe of one
 // SM (2 operations per clock) is what a one-CTA solve waits for: 700 nodes x 500
-// iterations on one CTA 14.3 ms, on 16 CTAs 2.6; 4000 nodes on 8 CTAs 18.4 us per
+// iterations on one CTA 14.3 ms, on 16 CTAs 1.95; 4000 nodes on 8 CTAs 18.4 us per
 // iteration, on 16 13.2.
 //
 // The scratch array is shared by every call on a device and keeps the last

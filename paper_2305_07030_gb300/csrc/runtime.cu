@@ -63,8 +63,8 @@ struct DevBuf {
 // One size class: RVEs solved by one persistent launch.
 struct SizeClass {
     int parts = 1;              // mixed: cluster size
-    bool lead_staged = false;   // mixed: lead kernel with its element table
-    bool fp32_staged = false;   // mixed: FP32 kernel with its element table
+    bool lead_staged = false;   // mixed: the lead's staged form (footprint rule)
+    bool fp32_staged = false;   // mixed: parts within the FP32 phase's footprint rule
     int block_lead = 0;         // mixed: tuned CTA sizes (0 = default)
     int block_fp32 = 0;
     int smem_positions = 1;     // FP64: positions in shared memory
@@ -355,8 +355,8 @@ bool finite3(const double *p) { return std::isfinite(p[0]) && std::isfinite(p[1]
 
 // Smallest cluster size (CTAs) for an RVE of n nodes in the mixed solver: a
 // power of two with at most `target` nodes per CTA and room for the node
-// state of the FP32 kernel without its element table (the larger of the two
-// kernels' plain footprints, with slack for an uneven bisection), at most 16.
+// state of the FP32 kernel without tables (the larger of the two kernels' plain
+// footprints, with slack for an uneven bisection), at most 16.
 int min_parts(int n, int target, size_t smem_cap) {
     const size_t per_node = std::max(mixed_plain_node_bytes(0), mixed_plain_node_bytes(1));
     int C = 1;
@@ -498,8 +498,8 @@ void build_classes(const std::vector<RveDesc> &rve, const std::vector<int32_t> &
         for (auto &c : cls)
             if (!c.rves.empty()) out.push_back(c);
     } else {
-        // A class is keyed by the cluster size and by whether each kernel keeps
-        // its element table in shared memory, both decided by the RVE alone
+        // A class is keyed by the cluster size and by each kernel's form (where its
+        // tables are, order of operations), all decided by the RVE alone
         // (its own parts and table sizes), so an RVE runs the same code path,
         // with the same CTA size, whatever batch it is in. RVEs of one key are
         // packed first-fit into classes whose combined tables still fit.
@@ -600,8 +600,7 @@ void build_classes(const std::vector<RveDesc> &rve, const std::vector<int32_t> &
 
 int mixed_block(int requested, bool lead, bool staged);
 
-// Dynamic shared memory of a mixed class's lead (lead = 1) or FP32 kernel:
-// with the element table when the class is staged for that kernel.
+// Dynamic shared memory of a mixed class's lead (lead = 1) or FP32 kernel.
 size_t class_smem(const SizeClass &c, int lead) {
     const bool st = lead ? c.lead_staged : c.fp32_staged;
     const size_t plain = mixed_plain_node_bytes(lead) * (size_t)c.part_max;
@@ -970,8 +969,8 @@ void build_layout(int32_t n_rve, const int64_t *node_off, const double *X, const
             if (!std::is_sorted(r0, r1)) std::sort(r0, r1);
         }
         // Parts: the smallest cluster that holds the plain state, doubled
-        // (up to 16) while the FP32 kernel's element table does not fit in
-        // shared memory; the autotuner may fix the count per size bucket.
+        // (up to 16) while the parts do not meet the FP32 phase's footprint
+        // rule; the autotuner may fix the count per size bucket.
         int C = min_parts(n, target, smem_cap);
         const int want = g_tuning.parts[node_bucket(n)];
         const bool forced = want >= C && want <= kMaxParts && (want & (want - 1)) == 0;
@@ -1472,11 +1471,11 @@ fe2_status check_opts(const fe2_opts &o) {
     return FE2_OK;
 }
 
-// CTA size of a mixed launch: 512 threads, except the lead kernel without its
-// element table (256: two CTAs per SM, its registers allow no more). The size
-// is a function of the RVE (its bucket's tuning) and never of the batch, which
-// keeps every RVE's result independent of which other RVEs share its launch
-// (partial sums follow the thread mapping).
+// CTA size of a mixed launch: 512 threads, except the lead of parts beyond its
+// footprint rule (256, from a kernel that ran two CTAs per SM; kept because the
+// residual's partial sums follow the thread mapping). The size is a function of
+// the RVE (its bucket's tuning) and never of the batch, which keeps every RVE's
+// result independent of which other RVEs share its launch.
 int mixed_block(int requested, bool lead, bool staged) {
     const int cap = lead && !staged ? 256 : 512;
     return requested ? std::min(requested, cap) : cap;
@@ -2157,13 +2156,15 @@ extern "C" fe2_status fe2_batch_submit(fe2_batch *b, int32_t n, const int32_t *r
         cudaStream_t ls = s;
         const int k = used++ % (kSlotSides + 1) - 1;
         if (k >= 0) {
-            if ((int)sl.side.size() <= k) {
-                cudaStream_t ns;
+            if ((int)sl.side_end.size() <= k) {
                 cudaEvent_t ne;
-                CUDA_TRY(cudaStreamCreateWithFlags(&ns, cudaStreamNonBlocking));
-                sl.side.push_back(ns);
                 CUDA_TRY(cudaEventCreateWithFlags(&ne, cudaEventDisableTiming));
                 sl.side_end.push_back(ne);
+            }
+            if ((int)sl.side.size() <= k) {
+                cudaStream_t ns;
+                CUDA_TRY(cudaStreamCreateWithFlags(&ns, cudaStreamNonBlocking));
+                sl.side.push_back(ns);
             }
             ls = sl.side[k];
             CUDA_TRY(cudaStreamWaitEvent(ls, sl.fork, 0));
