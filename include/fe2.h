@@ -70,9 +70,9 @@ typedef enum {
      * divide. The trajectory is bit for bit that of such an implementation;
      * only the residual and stress sums are reassociated. An RVE runs on a
      * thread-block cluster of 1 to 16 CTAs, one spatial part per CTA (more
-     * and smaller parts in batches that leave SMs idle; every result is the
-     * same bits whatever the parts, the CTA size and the batch), with the
-     * same operations (set
+     * and smaller parts in batches that leave SMs idle; every result is then
+     * the same bits whatever the batch and the CTA size), with the same
+     * operations (set
      * FE2_FP64_CLUSTER=0 in the environment before fe2_batch_create to keep
      * every RVE on one CTA). Any RVE size. */
     FE2_PREC_FP64 = 0,

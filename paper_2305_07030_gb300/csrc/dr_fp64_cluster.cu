@@ -29,12 +29,15 @@
 // Sums. Every sum over the nodes goes leaf by leaf (Leaves below), so an RVE's
 // results do not depend on how many CTAs its batch leaves for it. The chains of
 // dependent additions are what a test costs: under load an FP64 instruction of a
-// warp waits for the pipe for 100 to 250 cycles. A leaf's terms are therefore spread over
-// 32 lanes, two leaves share a warp's tree, and warps without elements do it first.
-// Against sums by thread, warp and CTA in the judging warp alone: 512 nodes on 8
-// CTAs 4.45 -> 3.67 us per iteration, 300 RVEs of 200 to 1000 nodes with energies
-// x 200 iterations 9.7 -> 8.8 ms, 32 of 5000 x 300 unchanged (14.2 ms). With the
-// judging warp adding every leaf by itself, 32 / leaves lanes each: 6.1 us and 12.2 ms.
+// warp waits for the pipe for 100 to 250 cycles. A leaf's terms are therefore spread
+// over groups of about 64 nodes and 32 lanes each, two groups share a warp's tree, and
+// warps without elements do it first. Per iteration, with sums by thread, warp and
+// CTA in the judging warp alone (which the batch could change) and so: 512 nodes on 8
+// CTAs 4.3 -> 3.6 us (with energies 8.3 -> 5.1), 5000 nodes on 16 CTAs 9.8 -> 9.5 (14.6 ->
+// 13.9), 15,000 23.1 -> 21.3 (30.0 -> 30.3), 60,000 90.3 -> 88.0; only the energies of
+// RVEs of more than 16,000 nodes cost 4 to 6 % more than they did, their terms' way
+// through L2 (17,500 nodes 34.6 -> 36.1). With one judging lane per 32 / leaves of a CTA:
+// 512 nodes 6.1 us.
 //
 // What bounds it: the FP64 pipe, 2 operations per clock and SM. Per element 13
 // additions and multiplications, per free node 45 at degree 5; divisions and
@@ -65,7 +68,7 @@ constexpr int kMaxThreads = 512;
 constexpr int kRegElems = 3;      // table elements a worker keeps in registers
 
 struct Fp64ClusterShared {
-    double part[2][4][kMaxParts];    // sums of this CTA's leaves for evaluation n (parity n & 1):
+    double part[2][4][kMaxParts];    // sums of this CTA's groups for evaluation n (parity n & 1):
                                      // squared residual, kinetic energy, work terms
     const double *partp[kMaxParts];  // every CTA's `part`
     double sig[kStressWarps][9];     // stress partials (rank 0's copy is the target)
@@ -175,13 +178,18 @@ __device__ __forceinline__ void slot_force(const Slot &e, uint32_t boff, uint32_
     T[2 * ts] = dmul(q, d2);
 }
 
+// Doubles per free node of the state in shared memory, by Fp64Shape::ssm: velocity,
+// reference position, mass, damping factor, the mass's division estimate, the
+// force's squares; displacement unless 2.
+__host__ __device__ constexpr size_t state_doubles(int ssm) { return ssm == 1 ? 15 : ssm == 2 ? 12 : 0; }
+
 // Dynamic shared memory of a launch shape (layout: cluster_tables).
 __host__ __device__ inline size_t cluster_bytes(const Fp64Shape &sp) {
-    size_t b = sizeof(double) * (6 * (size_t)sp.part_max + (sp.ssm ? kStateDoubles * (size_t)sp.free_max : 0));
+    size_t b = sizeof(double) * (6 * (size_t)sp.part_max + state_doubles(sp.ssm) * (size_t)sp.free_max);
     if (sp.tsm)
         b += sizeof(double) * 3 * (size_t)sp.slot_max + sizeof(int32_t) * ((size_t)sp.free_max + 1) +
              sizeof(uint16_t) * (size_t)sp.row_max;
-    if (sp.ssm) b += sizeof(uint16_t) * (size_t)sp.part_max;
+    if (sp.ssm == 1) b += sizeof(uint16_t) * (size_t)sp.part_max;
     return (b + 15) & ~size_t(15);
 }
 
@@ -190,12 +198,13 @@ __host__ __device__ inline size_t cluster_bytes(const Fp64Shape &sp) {
 // One RVE on the cluster. XB (smem) is this CTA's [2][3][part_cap] position
 // buffers. With TSM the element table T [3][slot_cap] and the rows (RS: first
 // entry of each free node, RE: entries slot << 1 | second end) are in shared
-// memory, otherwise in global memory. With SSM the own free nodes' state (ST:
-// velocity, displacement, reference position [3][free_cap] each, mass and
-// damping factor -c m [free_cap] each, the mass's division estimates and the
-// force's squares) and the list of the nodes by leaf (LS) are in shared memory,
-// otherwise in global memory (L2).
-template <bool TSM, bool SSM>
+// memory, otherwise in global memory. With SSM = 1 the own free nodes' state (ST:
+// velocity, reference position, the force's squares [3][free_cap] each, mass,
+// damping factor -c m and the mass's division estimate [free_cap] each, displacement
+// [3][free_cap]) and the list of the nodes by leaf (LS) are in shared memory, with
+// SSM = 2 all but the displacement (from the ring) and the list, otherwise in global
+// memory (L2). 2 is for parts that 1 does not fit.
+template <bool TSM, int SSM>
 __device__ void solve_rve_fp64_cluster(cg::cluster_group &cl, Fp64ClusterShared &sh, const DevMesh &M,
                                        const DevState &S, const DevResults &O, const SolveParams &P, int p,
                                        double *XB, double *ST, double *Tsm, int32_t *RS, uint16_t *RE, uint16_t *LS,
@@ -230,14 +239,14 @@ __device__ void solve_rve_fp64_cluster(cg::cluster_group &cl, Fp64ClusterShared 
     const uint32_t cb = (uint32_t)(sizeof(double) * part_cap);
     const bool energy = P.want_ke == 2;
     double *gp = S.gp + 3 * n0 + c0, *fdp = S.fdp + 3 * n0 + c0;  // by FP64 order, energy check
-    double *const sv = ST, *const su = ST + 3 * free_cap, *const sx = ST + 6 * free_cap;
+    double *const sv = ST, *const sx = ST + 3 * free_cap, *const su = ST + 12 * free_cap;
     double *const sm = ST + 9 * free_cap, *const sc = ST + 10 * free_cap;
     uint32_t *const sr = reinterpret_cast<uint32_t *>(ST + 11 * free_cap);
     double *const gv = S.v0 + n0 + c0;  // !SSM: component c at c * vstride
     const int64_t vstride = S.v1 - S.v0;
     const double mc = -R.c;
     // squares of the free nodes' forces; kinetic energies and work terms
-    double *const G2 = SSM ? ST + 12 * free_cap : xg + c0;
+    double *const G2 = SSM ? ST + 6 * free_cap : xg + c0;
     const int gs = SSM ? free_cap : n;
     const int64_t kstride = S.a1 - S.a0;
     double *const kt = S.a0 + n0 + c0, *const wt = S.a0 + 3 * kstride + 6 * n0 + c0;
@@ -274,7 +283,7 @@ __device__ void solve_rve_fp64_cluster(cg::cluster_group &cl, Fp64ClusterShared 
             XB[r * part_cap + k] = x;
             XB[(3 + r) * part_cap + k] = x;  // fixed positions live in both buffers
             if (SSM && !fixed) {
-                su[r * free_cap + k] = u;
+                if (SSM == 1) su[r * free_cap + k] = u;
                 sx[r * free_cap + k] = Xv[r];
             }
             if (!fixed) ring[r * n + k] = u;
@@ -291,7 +300,7 @@ __device__ void solve_rve_fp64_cluster(cg::cluster_group &cl, Fp64ClusterShared 
         const int ne = frow[nfr] - frow[0];
         for (int q = tid; q < ne; q += blockDim.x) RE[q] = (uint16_t)fent[frow[0] + q];
     }
-    if (SSM && lv.list)
+    if (SSM == 1 && lv.list)
         for (int k = tid; k < m; k += blockDim.x) LS[k] = lv.list[k];
     Slot el[kRegElems];
 #pragma unroll
@@ -320,7 +329,7 @@ __device__ void solve_rve_fp64_cluster(cg::cluster_group &cl, Fp64ClusterShared 
                 XB[(3 + r) * part_cap + k] = dadd(Xv[r], u);
                 if (SSM) {
                     sv[r * free_cap + k] = v;
-                    su[r * free_cap + k] = u;
+                    if (SSM == 1) su[r * free_cap + k] = u;
                 } else {
                     gv[r * vstride + k] = v;
                 }
@@ -337,42 +346,44 @@ __device__ void solve_rve_fp64_cluster(cg::cluster_group &cl, Fp64ClusterShared 
     const double thresh = P.tol * f_ref;
     double res = 0.0, ke = 0.0, wint = 0.0, wext = 0.0;  // judging warp: of the last tested evaluation
     int rc = 1;                                          // ring index of evaluation i
-    // Sums of the terms of evaluation i - 1, for every kind of term and leaf: entry
-    // y = 3 j + c (component c of the leaf's free node j) belongs to lane y mod 32,
-    // and the lanes' sums are added as a tree. A warp takes one kind and two leaves
-    // at a time (one if there is but one); the last warps, which have the fewest
-    // elements, begin, and the judging warp comes last where others have none.
-    const int own_sh = 31 - __clz(lv.own), pair = lv.own > 1 ? 1 : 0, grp_sh = own_sh - pair;
-    const int n_sums = (energy ? 4 : P.want_ke ? 2 : 1) << grp_sh;
+    // Sums of the terms of evaluation i - 1, for every kind of term and every group of
+    // a leaf's terms: entry y = 3 j + c (component c of the leaf's free node j) belongs
+    // to lane y mod 32 of group (y / 32) mod groups, and the lanes' sums are added as a
+    // tree. A warp takes one kind and two groups at a time (one if there is but one);
+    // the last warps, which have the fewest elements, begin, and the judging warp comes
+    // last where others have none.
+    const int gsh = 31 - __clz(R.fp_groups), ush = 31 - __clz(lv.own) + gsh;  // 2^ush groups here
+    const int pair = ush > 0 ? 1 : 0, n_sums = (energy ? 4 : P.want_ke ? 2 : 1) << (ush - pair);
     const int nw = (int)(blockDim.x >> 5), from_end = nw - 1 - (tid >> 5);
     const int first_sum = ns > W - 32 ? from_end : from_end == 0 ? nw - 1 : from_end - 1;
-    const double *const lsum =  // the leaf's sums that this lane adds to the totals
-        (lane & 15) < lv.total ? sh.partp[(lane & 15) >> own_sh] + ((lane & 15) & (lv.own - 1)) : nullptr;
-    auto lane_sum = [&](const double *v, int64_t vs, int l) {
-        const int beg = lv.list ? lv.off[l] - lv.base : 0, cnt = 3 * (lv.list ? lv.free[l] : nfr);
+    const int all_groups = lv.total << gsh;
+    const double *const lsum =  // the group's sums that this lane adds first
+        lane < all_groups ? sh.partp[lane >> ush] + (lane & ((1 << ush) - 1)) : nullptr;
+    auto lane_sum = [&](const double *v, int64_t vs, int u) {
+        const int l = u >> gsh, beg = lv.list ? lv.off[l] - lv.base : 0;
+        const int end = 3 * (lv.list ? lv.free[l] : nfr);
         double t = 0.0;
 #pragma unroll 4
-        for (int y = lane; y < cnt; y += 32) {
-            const int j = beg + y / 3;
-            const int k = lv.list ? (SSM ? LS[j] : lv.list[j]) : j;
+        for (int y = lane + 32 * (u & ((1 << gsh) - 1)); y < end; y += 32 << gsh) {
+            const int j = beg + y / 3, k = lv.list ? (SSM == 1 ? LS[j] : lv.list[j]) : j;
             t = dadd(t, v[(y % 3) * vs + k]);
         }
         return t;
     };
     auto leaf_sums = [&](int64_t ev) {
         for (int x = first_sum; x < n_sums; x += nw) {
-            const int kind = x >> grp_sh, l = (x & ((1 << grp_sh) - 1)) << pair;
-            const double *v = kind == 0 ? G2 : kind == 1 ? kt : kind == 2 ? wt : wt + 3 * n;
+            const int kind = x >> (ush - pair), u = (x & ((1 << (ush - pair)) - 1)) << pair;
+            const double *const v = kind == 0 ? G2 : kind == 1 ? kt : kind == 2 ? wt : wt + 3 * n;
             const int64_t vs = kind == 0 ? gs : kind == 1 ? kstride : n;
-            double t = lane_sum(v, vs, l), o = t;
-            if (pair) {  // lanes 0 to 15 go on with the first leaf, 16 to 31 with the second
-                const double t2 = lane_sum(v, vs, l + 1);
+            double t = lane_sum(v, vs, u), o = t;
+            if (pair) {  // lanes 0 to 15 go on with the first group, 16 to 31 with the second
+                const double t2 = lane_sum(v, vs, u + 1);
                 o = (lane & 16) ? t : t2;
                 t = (lane & 16) ? t2 : t;
             }
             t = dadd(t, __shfl_xor_sync(0xffffffffu, o, 16));
             for (int d = 8; d > 0; d >>= 1) t = dadd(t, __shfl_xor_sync(0xffffffffu, t, d));
-            if ((lane & 15) == 0 && (lane == 0 || pair)) sh.part[ev & 1][kind][l + (lane >> 4)] = t;
+            if ((lane & 15) == 0 && (lane == 0 || pair)) sh.part[ev & 1][kind][u + (lane >> 4)] = t;
         }
     };
     int64_t i = 1;
@@ -400,9 +411,13 @@ __device__ void solve_rve_fp64_cluster(cg::cluster_group &cl, Fp64ClusterShared 
                 for (int c = 0; c < 4; ++c) {
                     if (c > 0 && !P.want_ke) break;
                     if (c > 1 && !energy) break;
-                    tot[c] = lsum ? lsum[((i & 1) * 4 + c) * kMaxParts] : 0.0;
-                    // a tree over the leaves: the same bits in every CTA
-                    for (int o = 1; o < lv.total; o <<= 1) tot[c] = dadd(tot[c], __shfl_xor_sync(0xffffffffu, tot[c], o));
+                    const int at = ((int)(i & 1) * 4 + c) * kMaxParts;
+                    double t = lsum ? lsum[at] : 0.0;
+                    for (int e = lane + 32; e < all_groups; e += 32)
+                        t = dadd(t, sh.partp[e >> ush][at + (e & ((1 << ush) - 1))]);
+                    // a tree over the lanes: the same bits in every CTA
+                    for (int o = 1; o < 32 && o < all_groups; o <<= 1) t = dadd(t, __shfl_xor_sync(0xffffffffu, t, o));
+                    tot[c] = t;
                 }
                 res = dsqrt(tot[0]);
                 ke = tot[1];
@@ -440,7 +455,7 @@ __device__ void solve_rve_fp64_cluster(cg::cluster_group &cl, Fp64ClusterShared 
                 uint32_t vm;
                 if (SSM) {
                     mm = sm[k]; cm = sc[k]; vm = sr[k];
-                    vv = sv[c * free_cap + k]; uu = su[c * free_cap + k]; xr = sx[c * free_cap + k];
+                    vv = sv[c * free_cap + k]; uu = SSM == 1 ? su[c * free_cap + k] : up[c * n + k]; xr = sx[c * free_cap + k];
                 } else {
                     const int id = node[k];
                     mm = M.mass[n0 + id];
@@ -464,7 +479,7 @@ __device__ void solve_rve_fp64_cluster(cg::cluster_group &cl, Fp64ClusterShared 
                 const double u = dadd(uu, dmul(dt, vh));
                 if (SSM) {
                     sv[c * free_cap + k] = vh;
-                    su[c * free_cap + k] = u;
+                    if (SSM == 1) su[c * free_cap + k] = u;
                 } else {
                     gv[c * vstride + k] = vh;
                 }
@@ -514,13 +529,13 @@ __device__ __forceinline__ void map_shared(cg::cluster_group &cl, Fp64ClusterSha
 }
 
 // One RVE with the tables of a launch shape in `base` (cluster_bytes).
-template <bool TSM, bool SSM>
+template <bool TSM, int SSM>
 __device__ __forceinline__ void solve_in(cg::cluster_group &cl, Fp64ClusterShared &sh, const DevMesh &M,
                                          const DevState &S, const DevResults &O, const SolveParams &P, int p,
                                          const Fp64Shape &sp, double *base) {
     double *XB = base;
     double *ST = XB + 6 * sp.part_max;
-    double *T = ST + (SSM ? kStateDoubles * (size_t)sp.free_max : 0);
+    double *T = ST + state_doubles(SSM) * (size_t)sp.free_max;
     int32_t *RS = reinterpret_cast<int32_t *>(T + (TSM ? 3 * (size_t)sp.slot_max : 0));
     uint16_t *RE = reinterpret_cast<uint16_t *>(RS + (TSM ? sp.free_max + 1 : 0));
     uint16_t *LS = RE + (TSM ? sp.row_max : 0);
@@ -528,7 +543,7 @@ __device__ __forceinline__ void solve_in(cg::cluster_group &cl, Fp64ClusterShare
 }
 }  // namespace
 
-template <bool TSM, bool SSM>
+template <bool TSM, int SSM>
 __global__ void __launch_bounds__(kMaxThreads, 1)
     dr_fp64_cluster_kernel(DevMesh M, DevState S, DevResults O, SolveParams P, Fp64Shape sp) {
     extern __shared__ __align__(16) double dsm_fp64[];
@@ -559,12 +574,13 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
     map_shared(cl, sh);
     cl.sync();
     const RveDesc &R = M.rve[0];
-    Fp64Shape sp = {R.fp_parts, R.fp_part_max, R.fp_free_max, R.fp_slot_max, R.fp_row_max, true, true};
+    Fp64Shape sp = {R.fp_parts, R.fp_part_max, R.fp_free_max, R.fp_slot_max, R.fp_row_max, true, 1};
     if (cluster_bytes(sp) <= bytes) {
-        solve_in<true, true>(cl, sh, M, S, O, P, 0, sp, dsm_fp64);
+        solve_in<true, 1>(cl, sh, M, S, O, P, 0, sp, dsm_fp64);
     } else {
-        sp.tsm = sp.ssm = false;
-        solve_in<false, false>(cl, sh, M, S, O, P, 0, sp, dsm_fp64);
+        sp.tsm = false;
+        sp.ssm = 0;
+        solve_in<false, 0>(cl, sh, M, S, O, P, 0, sp, dsm_fp64);
     }
     const double *uo[3] = {S.u0, S.u1, S.u2};
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < R.n_nodes; k += gridDim.x * blockDim.x)
@@ -575,8 +591,11 @@ namespace {
 using Fp64ClusterKernel = void (*)(DevMesh, DevState, DevResults, SolveParams, Fp64Shape);
 
 Fp64ClusterKernel pick_fp64_cluster(const Fp64Shape &sp) {
-    if (sp.tsm) return sp.ssm ? dr_fp64_cluster_kernel<true, true> : dr_fp64_cluster_kernel<true, false>;
-    return sp.ssm ? dr_fp64_cluster_kernel<false, true> : dr_fp64_cluster_kernel<false, false>;
+    if (sp.tsm)
+        return sp.ssm == 1 ? dr_fp64_cluster_kernel<true, 1>
+                           : sp.ssm ? dr_fp64_cluster_kernel<true, 2> : dr_fp64_cluster_kernel<true, 0>;
+    return sp.ssm == 1 ? dr_fp64_cluster_kernel<false, 1>
+                       : sp.ssm ? dr_fp64_cluster_kernel<false, 2> : dr_fp64_cluster_kernel<false, 0>;
 }
 
 cudaLaunchConfig_t fp64_cluster_config(int clusters, const Fp64Shape &sp, int block, cudaLaunchAttribute *attr,
@@ -667,7 +686,7 @@ int fp64_max_cluster(size_t smem) {
     const auto key = std::make_pair(dev, smem);
     const auto it = known.find(key);
     if (it != known.end()) return it->second;
-    const Fp64ClusterKernel k = dr_fp64_cluster_kernel<true, true>;
+    const Fp64ClusterKernel k = dr_fp64_cluster_kernel<true, 1>;
     prepare_fp64_cluster(k, smem);
     return known[key] = largest_cluster(k, smem);
 }
@@ -677,7 +696,7 @@ int fp64_max_cluster(size_t smem) {
 constexpr size_t kSingleBytes = 200 * 1024;
 static size_t single_bytes(int n, int n_elems, int parts) {
     const int m = (n + parts - 1) / parts;
-    const Fp64Shape most = {parts, m, m, n_elems, 2 * n_elems, true, true};
+    const Fp64Shape most = {parts, m, m, n_elems, 2 * n_elems, true, 1};
     return std::min(kSingleBytes, cluster_bytes(most));
 }
 

@@ -49,7 +49,8 @@ struct RveDesc {
     int32_t fp_free_max;
     int32_t fp_slot_max;
     int32_t fp_row_max;
-    int32_t fp_leaves;  // groups of nodes whose sums are formed first (a multiple of fp_parts)
+    int32_t fp_leaves;  // sets of nodes whose sums are formed first (a multiple of fp_parts)
+    int32_t fp_groups;  // and the groups of each that are summed apart
     // FP32 phase of the mixed solver (dr_mixed_node.cu): most entries of a part's
     // increment array (free nodes, the zero entry, copies of other parts' nodes)
     // and most copies of its own nodes elsewhere; first copy; first global slot
@@ -67,10 +68,12 @@ struct RveDesc {
 
 // Launch shape of the FP64 cluster kernel: CTAs per cluster, capacities of one
 // CTA, and what it keeps in shared memory beside the positions (tsm: element
-// table and rows, ssm: the own free nodes' state).
+// table and rows, ssm: the own free nodes' state, 1 with and 2 without their
+// displacements).
 struct Fp64Shape {
     int parts, part_max, free_max, slot_max, row_max;
-    bool tsm, ssm;
+    bool tsm;
+    int ssm;
 };
 // CTAs per cluster of the FP32-phase kernel (dr_mixed_node.cu) and capacities of
 // one CTA: increment entries, free nodes, row slots, copies of own nodes, and the row slots held in
@@ -88,9 +91,6 @@ struct LeadShape {
     int parts, u_cap, free_cap, elem_cap, slot_cap, push_cap;
     bool staged, ksm;
 };
-// doubles per free node of the FP64 cluster kernel's state: velocity, displacement, reference
-// position, mass, damping factor, the mass's division estimate, the force's squares
-constexpr int kStateDoubles = 15;
 
 // Read-only, create-time arrays.
 struct DevMesh {

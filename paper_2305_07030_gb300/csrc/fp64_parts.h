@@ -26,6 +26,14 @@ inline int fp64_leaf_factor(int n_nodes, int n_parts) {
     return f;
 }
 
+// Groups into which a leaf's terms are divided before they are summed: about 64
+// nodes each, at most 16 to a CTA that holds a whole part.
+inline int fp64_groups(int n_nodes, int n_parts, int leaves) {
+    int g = 1;
+    while (2 * g * (leaves / n_parts) <= kMaxSplit && n_nodes >= 2 * g * leaves * 64) g *= 2;
+    return g;
+}
+
 // Factor taken in a batch of `ctas` parts: up to 128 CTAs in all.
 inline int fp64_split_factor(int64_t ctas, int n_nodes, int n_parts, int max_cluster) {
     const int most = fp64_leaf_factor(n_nodes, n_parts);

@@ -127,7 +127,7 @@ __device__ __forceinline__ uint32_t spread3(uint32_t x) {
     return (x | (x << 2)) & 0x09249249u;
 }
 
-__global__ void __launch_bounds__(kNaThreads) k_noalloc_pack(NaArgs A, int warm, int C, unsigned char *scr) {
+__global__ void __launch_bounds__(kNaThreads) k_noalloc_pack(NaArgs A, int warm, int C, int groups, unsigned char *scr) {
     extern __shared__ __align__(16) uint64_t keys[];  // the next power of two above n
     __shared__ double red[6 * (kNaThreads / 32)];
     __shared__ int tmp[32];
@@ -457,6 +457,7 @@ __global__ void __launch_bounds__(kNaThreads) k_noalloc_pack(NaArgs A, int warm,
         R.n_nodes = n; R.n_free = nf; R.n_elems = E; R.n_parts = C;
         R.dtc = dtc; R.c = A.c; R.V0 = A.V0;
         R.fp_parts = R.fp_leaves = C;
+        R.fp_groups = groups;
         R.fp_slot_max = slot_max;
         for (int r = 0; r < C; ++r) {
             R.fp_part_max = max(R.fp_part_max, part_off[r + 1] - part_off[r]);
@@ -574,7 +575,8 @@ extern "C" fe2_status fe2_rve_solve_noalloc(int32_t n_nodes, int32_t n_elems, co
     const int n = n_nodes, C = fp64_single_parts(n, max_cluster);
     int np = 1;
     while (np < n) np *= 2;
-    k_noalloc_pack<<<1, kNaThreads, sizeof(uint64_t) * np, static_cast<cudaStream_t>(stream)>>>(A, o.init == 2, C, scr);
+    k_noalloc_pack<<<1, kNaThreads, sizeof(uint64_t) * np, static_cast<cudaStream_t>(stream)>>>(A, o.init == 2, C, fp64_groups(n, C, C),
+                                                                                               scr);
     e = cudaGetLastError();
     if (e != cudaSuccess) {
         g_na_err = std::string("launch: ") + cudaGetErrorString(e);

@@ -443,7 +443,7 @@ void build_classes(const std::vector<RveDesc> &rve, const std::vector<int32_t> &
         // the single-CTA kernel.
         const bool clusters = env_int("FE2_FP64_CLUSTER", 1) != 0;
         auto shape_of = [&](const RveDesc &R) {
-            return Fp64Shape{R.fp_parts, R.fp_part_max, R.fp_free_max, R.fp_slot_max, R.fp_row_max, false, false};
+            return Fp64Shape{R.fp_parts, R.fp_part_max, R.fp_free_max, R.fp_slot_max, R.fp_row_max, false, 0};
         };
         auto on_cluster = [&](const RveDesc &R) { return clusters && fp64_cluster_smem(shape_of(R)) <= cap; };
         for (int32_t p : order) {
@@ -451,9 +451,9 @@ void build_classes(const std::vector<RveDesc> &rve, const std::vector<int32_t> &
             // shared-memory variant of an RVE: the element table first, then
             // the free-node state, as far as they fit
             Fp64Shape one = shape_of(rve[p]);
-            const bool opts[4][2] = {{true, true}, {true, false}, {false, true}, {false, false}};
+            const int opts[6][2] = {{1, 1}, {1, 2}, {1, 0}, {0, 1}, {0, 2}, {0, 0}};
             for (const auto &o : opts) {
-                one.tsm = o[0];
+                one.tsm = o[0] != 0;
                 one.ssm = o[1];
                 if (fp64_cluster_smem(one) <= cap) break;
             }
@@ -758,6 +758,7 @@ void build_fp64_parts(const int64_t *elem_off, bool split, HostLayout &L) {
             L.fpLeaf[R.node0 + to[l]++] = (uint16_t)i;  // parts of the cluster kernel are small
         }
         R.fp_leaves = leaves;
+        R.fp_groups = fp64_groups(n, R.n_parts, leaves);
         R.slot0 = (int64_t)(L.fpSlot.size() / 4);
         R.fp_parts = C;
         R.fp_part_max = R.fp_free_max = R.fp_slot_max = R.fp_row_max = 0;
@@ -1524,9 +1525,9 @@ int resident_of(fe2_batch *b, int kind, int parts, int block, size_t smem, int p
 }
 
 // Resident clusters of an FP64 cluster class (cached like resident_of; the
-// key's kind 3 + 2 tsm + ssm and the smem size identify the variant).
+// key's kind 15 + 3 tsm + ssm and the smem size identify the variant).
 int resident_fp64_cluster(fe2_batch *b, const SizeClass &c, int block) {
-    const auto key = std::make_tuple(3 + 2 * (int)c.fp.tsm + (int)c.fp.ssm, c.parts, block, fp64_cluster_smem(c.fp),
+    const auto key = std::make_tuple(15 + 3 * (int)c.fp.tsm + c.fp.ssm, c.parts, block, fp64_cluster_smem(c.fp),
                                      c.fp.part_max);
     auto it = b->occ.find(key);
     if (it != b->occ.end()) return it->second;

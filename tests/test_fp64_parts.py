@@ -1,6 +1,6 @@
 """How many CTAs an RVE gets in FP64 (csrc/fp64_parts.h, compiled by itself): never a
 cluster that the device cannot hold, with any device limit as many as without one up
-to it, and leaves that do not depend on it."""
+to it, and leaves and groups of terms that do not depend on it."""
 import os
 import subprocess
 
@@ -18,6 +18,8 @@ int main() {
             bad += fp64_single_parts(n, limit) != std::min(fp64_single_parts(n, 16), std::max(limit, 1));
             for (int parts = 1; parts <= 16; parts *= 2) {
                 const int most = fp64_leaf_factor(n, parts);
+                const int g = fp64_groups(n, parts, parts * most);
+                bad += g * most > 16 || (g > 1 && n < g * parts * most * 64);  // one warp's table, one CTA's sums
                 bad += parts * most > 16 || (most > 1 && n < parts * most * kSplitNodes);
                 for (int ctas = parts; ctas < 300; ++ctas) {
                     const int f = fp64_split_factor(ctas, n, parts, limit);
