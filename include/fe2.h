@@ -467,7 +467,7 @@ const char *fe2_last_error(void);
  * own every device allocation through their own pools). It allocates nothing:
  * inputs and outputs are the caller's DEVICE buffers, and all working memory
  * is one file-scope device array of fe2_noalloc_scratch_bytes() bytes (about
- * 3.7 MB) that every GPU loading the library holds until the process exits.
+ * 3.9 MB) that every GPU loading the library holds until the process exits.
  *
  * It runs the same per-RVE FP64 solver as fe2_batch_solve with
  * FE2_PREC_FP64, on a thread-block cluster of 1 to 16 CTAs by the node count.

@@ -30,14 +30,15 @@
 // results do not depend on how many CTAs its batch leaves for it. The chains of
 // dependent additions are what a test costs: under load an FP64 instruction of a
 // warp waits for the pipe for 100 to 250 cycles. A leaf's terms are therefore spread
-// over groups of about 64 nodes and 32 lanes each, two groups share a warp's tree, and
-// warps without elements do it first. Per iteration, with sums by thread, warp and
-// CTA in the judging warp alone (which the batch could change) and so: 512 nodes on 8
-// CTAs 4.3 -> 3.6 us (with energies 8.3 -> 5.1), 5000 nodes on 16 CTAs 9.8 -> 9.5 (14.6 ->
-// 13.9), 15,000 23.1 -> 21.3 (30.0 -> 30.3), 60,000 90.3 -> 88.0; only the energies of
-// RVEs of more than 16,000 nodes cost 4 to 6 % more than they did, their terms' way
-// through L2 (17,500 nodes 34.6 -> 36.1). With one judging lane per 32 / leaves of a CTA:
-// 512 nodes 6.1 us.
+// over groups of about 64 nodes and 32 lanes each, one group to a warp, and warps
+// without elements do it first; kinetic energies are kept for three evaluations and
+// summed at the end. Per iteration, with sums by thread, warp and CTA in the judging
+// warp alone (which the batch could change) and so: 512 nodes on 8 CTAs 4.3 -> 3.8 us
+// (energy check 8.4 -> 5.3), 152 RVEs of 200 nodes 6.45 -> 6.35 (10.5 -> 8.1), of 800 17.9 ->
+// 17.5 (23.8 -> 25.3), 5000 nodes on 16 CTAs 9.85 -> 9.2 (14.6 -> 12.6), 60,000 90.3 -> 86.7
+// (117 -> 123). The energy check costs up to 6 % more than it did where its terms are
+// many (parts of 800 nodes and more). Two groups to a warp: 200 nodes 6.85, 5000 9.6 us;
+// four: 7.6, 10.2; with one judging lane per 32 / leaves of a CTA 512 nodes 6.1.
 //
 // What bounds it: the FP64 pipe, 2 operations per clock and SM. Per element 13
 // additions and multiplications, per free node 45 at degree 5; divisions and
@@ -183,9 +184,12 @@ __device__ __forceinline__ void slot_force(const Slot &e, uint32_t boff, uint32_
 // force's squares; displacement unless 2.
 __host__ __device__ constexpr size_t state_doubles(int ssm) { return ssm == 1 ? 15 : ssm == 2 ? 12 : 0; }
 
+// Doubles per free node of the energy terms in shared memory.
+__host__ __device__ constexpr size_t term_doubles(bool terms) { return terms ? 9 : 0; }
+
 // Dynamic shared memory of a launch shape (layout: cluster_tables).
 __host__ __device__ inline size_t cluster_bytes(const Fp64Shape &sp) {
-    size_t b = sizeof(double) * (6 * (size_t)sp.part_max + state_doubles(sp.ssm) * (size_t)sp.free_max);
+    size_t b = sizeof(double) * (6 * (size_t)sp.part_max + (state_doubles(sp.ssm) + term_doubles(sp.terms)) * (size_t)sp.free_max);
     if (sp.tsm)
         b += sizeof(double) * 3 * (size_t)sp.slot_max + sizeof(int32_t) * ((size_t)sp.free_max + 1) +
              sizeof(uint16_t) * (size_t)sp.row_max;
@@ -203,11 +207,13 @@ __host__ __device__ inline size_t cluster_bytes(const Fp64Shape &sp) {
 // damping factor -c m and the mass's division estimate [free_cap] each, displacement
 // [3][free_cap]) and the list of the nodes by leaf (LS) are in shared memory, with
 // SSM = 2 all but the displacement (from the ring) and the list, otherwise in global
-// memory (L2). 2 is for parts that 1 does not fit.
+// memory (L2). 2 is for parts that 1 does not fit. TE: the kinetic energies of three
+// evaluations, or one's with the two work terms (energy check), of the free nodes,
+// [3][free_cap] each, null for global memory.
 template <bool TSM, int SSM>
 __device__ void solve_rve_fp64_cluster(cg::cluster_group &cl, Fp64ClusterShared &sh, const DevMesh &M,
                                        const DevState &S, const DevResults &O, const SolveParams &P, int p,
-                                       double *XB, double *ST, double *Tsm, int32_t *RS, uint16_t *RE, uint16_t *LS,
+                                       double *XB, double *ST, double *TE, double *Tsm, int32_t *RS, uint16_t *RE, uint16_t *LS,
                                        int part_cap, int free_cap, int slot_cap) {
     const RveDesc R = M.rve[p];
     const int me = (int)cl.block_rank(), C = (int)cl.num_blocks();
@@ -248,8 +254,15 @@ __device__ void solve_rve_fp64_cluster(cg::cluster_group &cl, Fp64ClusterShared 
     // squares of the free nodes' forces; kinetic energies and work terms
     double *const G2 = SSM ? ST + 6 * free_cap : xg + c0;
     const int gs = SSM ? free_cap : n;
-    const int64_t kstride = S.a1 - S.a0;
-    double *const kt = S.a0 + n0 + c0, *const wt = S.a0 + 3 * kstride + 6 * n0 + c0;
+    // Without the energy check the kinetic energies are wanted at the end only: those of
+    // the last three evaluations are kept (slot by displacement ring index).
+    const bool ke_ring = P.want_ke == 1;
+    const int64_t gstride = S.a1 - S.a0, kstride = TE ? free_cap : gstride;
+    double *const kt = TE ? TE : S.a0 + n0 + c0;
+    double *const wt = TE ? TE + 3 * free_cap : S.a0 + 3 * gstride + 6 * n0 + c0;
+    const int wts = TE ? free_cap : n;
+    auto ke_slot = [&](int slot) { return slot == 0 ? kt : wt + 3 * (slot - 1) * wts; };
+    auto ke_stride = [&](int slot) { return slot == 0 ? kstride : (int64_t)wts; };
     const Leaves lv = make_leaves(M, R, p, me, C, c0);
     double *const nn = ring + 2 * rstride;  // set-up: one value per own node
 
@@ -349,42 +362,59 @@ __device__ void solve_rve_fp64_cluster(cg::cluster_group &cl, Fp64ClusterShared 
     // Sums of the terms of evaluation i - 1, for every kind of term and every group of
     // a leaf's terms: entry y = 3 j + c (component c of the leaf's free node j) belongs
     // to lane y mod 32 of group (y / 32) mod groups, and the lanes' sums are added as a
-    // tree. A warp takes one kind and two groups at a time (one if there is but one);
-    // the last warps, which have the fewest elements, begin, and the judging warp comes
-    // last where others have none.
+    // tree. A warp takes one kind and one group at a time, two where there are more
+    // than warps; the last warps, which have the fewest elements, begin, and the judging
+    // warp comes last where others have none.
     const int gsh = 31 - __clz(R.fp_groups), ush = 31 - __clz(lv.own) + gsh;  // 2^ush groups here
-    const int pair = ush > 0 ? 1 : 0, n_sums = (energy ? 4 : P.want_ke ? 2 : 1) << (ush - pair);
+    const int kinds = energy ? 4 : 1;
     const int nw = (int)(blockDim.x >> 5), from_end = nw - 1 - (tid >> 5);
     const int first_sum = ns > W - 32 ? from_end : from_end == 0 ? nw - 1 : from_end - 1;
     const int all_groups = lv.total << gsh;
+    auto pair_of = [&](int kinds_now) { return ush > 0 && kinds_now << ush > nw ? 1 : 0; };
+    const int pair = pair_of(kinds);
     const double *const lsum =  // the group's sums that this lane adds first
         lane < all_groups ? sh.partp[lane >> ush] + (lane & ((1 << ush) - 1)) : nullptr;
     auto lane_sum = [&](const double *v, int64_t vs, int u) {
         const int l = u >> gsh, beg = lv.list ? lv.off[l] - lv.base : 0;
         const int end = 3 * (lv.list ? lv.free[l] : nfr);
-        double t = 0.0;
-#pragma unroll 4
-        for (int y = lane + 32 * (u & ((1 << gsh) - 1)); y < end; y += 32 << gsh) {
+        auto term = [&](int y) {
             const int j = beg + y / 3, k = lv.list ? (SSM == 1 ? LS[j] : lv.list[j]) : j;
-            t = dadd(t, v[(y % 3) * vs + k]);
-        }
+            return v[(y % 3) * vs + k];
+        };
+        int y = lane + 32 * (u & ((1 << gsh) - 1));
+        double t = y < end ? term(y) : 0.0;
+#pragma unroll 4
+        for (y += 32 << gsh; y < end; y += 32 << gsh) t = dadd(t, term(y));
         return t;
     };
-    auto leaf_sums = [&](int64_t ev) {
-        for (int x = first_sum; x < n_sums; x += nw) {
-            const int kind = x >> (ush - pair), u = (x & ((1 << (ush - pair)) - 1)) << pair;
-            const double *const v = kind == 0 ? G2 : kind == 1 ? kt : kind == 2 ? wt : wt + 3 * n;
-            const int64_t vs = kind == 0 ? gs : kind == 1 ? kstride : n;
-            double t = lane_sum(v, vs, u), o = t;
-            if (pair) {  // lanes 0 to 15 go on with the first group, 16 to 31 with the second
-                const double t2 = lane_sum(v, vs, u + 1);
-                o = (lane & 16) ? t : t2;
-                t = (lane & 16) ? t2 : t;
-            }
-            t = dadd(t, __shfl_xor_sync(0xffffffffu, o, 16));
-            for (int d = 8; d > 0; d >>= 1) t = dadd(t, __shfl_xor_sync(0xffffffffu, t, d));
-            if ((lane & 15) == 0 && (lane == 0 || pair)) sh.part[ev & 1][kind][u + (lane >> 4)] = t;
+    // terms `v` ([3] components `vs` apart) of group u (and u + 1 with `two`) into out
+    auto group_sums = [&](const double *v, int64_t vs, int u, int two, double *out) {
+        double t = lane_sum(v, vs, u), o = t;
+        if (two) {  // lanes 0 to 15 go on with the first group, 16 to 31 with the second
+            const double t2 = lane_sum(v, vs, u + 1);
+            o = (lane & 16) ? t : t2;
+            t = (lane & 16) ? t2 : t;
         }
+        t = dadd(t, __shfl_xor_sync(0xffffffffu, o, 16));
+        for (int d = 8; d > 0; d >>= 1) t = dadd(t, __shfl_xor_sync(0xffffffffu, t, d));
+        if ((lane & 15) == 0 && (lane == 0 || two)) out[u + (lane >> 4)] = t;
+    };
+    auto leaf_sums = [&](int64_t ev) {
+        for (int x = first_sum; x < kinds << (ush - pair); x += nw) {
+            const int kind = x >> (ush - pair), u = (x & ((1 << (ush - pair)) - 1)) << pair;
+            const double *const v = kind == 0 ? G2 : kind == 1 ? kt : kind == 2 ? wt : wt + 3 * wts;
+            group_sums(v, kind == 0 ? gs : kind == 1 ? kstride : wts, u, pair, sh.part[ev & 1][kind]);
+        }
+    };
+    // the RVE's total of one kind, from the groups' sums of parity q: a tree over the
+    // lanes, the same bits in every CTA
+    auto total = [&](int kind, int q) {
+        const int at = (q * 4 + kind) * kMaxParts;
+        double t = lsum ? lsum[at] : 0.0;
+        for (int e = lane + 32; e < all_groups; e += 32)
+            t = dadd(t, sh.partp[e >> ush][at + (e & ((1 << ush) - 1))]);
+        for (int o = 1; o < 32 && o < all_groups; o <<= 1) t = dadd(t, __shfl_xor_sync(0xffffffffu, t, o));
+        return t;
     };
     int64_t i = 1;
     for (;; ++i) {
@@ -407,23 +437,12 @@ __device__ void solve_rve_fp64_cluster(cg::cluster_group &cl, Fp64ClusterShared 
         } else {
             if (i >= 2) leaf_sums(i - 1);
             if (i >= 3) {  // verdict on evaluation i-2
-                double tot[4] = {0.0, 0.0, 0.0, 0.0};
-                for (int c = 0; c < 4; ++c) {
-                    if (c > 0 && !P.want_ke) break;
-                    if (c > 1 && !energy) break;
-                    const int at = ((int)(i & 1) * 4 + c) * kMaxParts;
-                    double t = lsum ? lsum[at] : 0.0;
-                    for (int e = lane + 32; e < all_groups; e += 32)
-                        t = dadd(t, sh.partp[e >> ush][at + (e & ((1 << ush) - 1))]);
-                    // a tree over the lanes: the same bits in every CTA
-                    for (int o = 1; o < 32 && o < all_groups; o <<= 1) t = dadd(t, __shfl_xor_sync(0xffffffffu, t, o));
-                    tot[c] = t;
-                }
-                res = dsqrt(tot[0]);
-                ke = tot[1];
+                const int q = (int)(i & 1);
+                res = dsqrt(total(0, q));
                 if (energy) {
-                    wint = dsub(wint, dmul(0.5, tot[2]));
-                    wext = dadd(wext, dmul(0.5, tot[3]));
+                    ke = total(1, q);
+                    wint = dsub(wint, dmul(0.5, total(2, q)));
+                    wext = dadd(wext, dmul(0.5, total(3, q)));
                 }
                 const int code = !isfinite(res) ? RVE_NAN : res <= thresh ? RVE_OK : i - 2 >= P.max_iter ? RVE_MAXITER : -1;
                 if (lane == 0) sh.code = code;
@@ -440,6 +459,8 @@ __device__ void solve_rve_fp64_cluster(cg::cluster_group &cl, Fp64ClusterShared 
             double *const xn = XB + ((i & 1) ? 0 : 3 * part_cap);
             const double *const up = ring + rc * rstride;
             double *const un = ring + rn * rstride;
+            double *const kn = ke_slot(ke_ring ? rc : 0);
+            const int64_t kns = ke_stride(ke_ring ? rc : 0);
             for (int x = tid; x < 3 * nfr; x += W) {
                 const int c = (x >= nfr) + (x >= 2 * nfr), k = x - c * nfr;
                 const double *Tc = T + c * ts;
@@ -467,14 +488,14 @@ __device__ void solve_rve_fp64_cluster(cg::cluster_group &cl, Fp64ClusterShared 
                 G2[c * gs + k] = dmul(g, g);
                 if (energy) {
                     const double du = dmul(dt, vv);
-                    wt[c * n + k] = dmul(du, dadd(gp[c * n + k], g));
-                    wt[(3 + c) * n + k] = dmul(du, dadd(fdp[c * n + k], fd));
+                    wt[c * wts + k] = dmul(du, dadd(gp[c * n + k], g));
+                    wt[(3 + c) * wts + k] = dmul(du, dadd(fdp[c * n + k], fd));
                     gp[c * n + k] = g;
                     fdp[c * n + k] = fd;
                 }
                 const double ha = dmul(hdt, f64_div_v<false>(dadd(g, fd), mm, vm));
                 const double v1 = dadd(vv, ha);
-                if (P.want_ke) kt[c * kstride + k] = dmul(dmul(0.5, mm), dmul(v1, v1));
+                if (P.want_ke) kn[c * kns + k] = dmul(dmul(0.5, mm), dmul(v1, v1));
                 const double vh = dadd(v1, ha);
                 const double u = dadd(uu, dmul(dt, vh));
                 if (SSM) {
@@ -491,7 +512,13 @@ __device__ void solve_rve_fp64_cluster(cg::cluster_group &cl, Fp64ClusterShared 
     }
     // The stopping evaluation is i - 2, ring index (i - 2) % 3 = (i + 1) % 3:
     // final displacement to the output arrays, positions to the global scratch
-    const double *const uf = ring + (rc == 2 ? 0 : rc + 1) * rstride;
+    const int rf = rc == 2 ? 0 : rc + 1;
+    const double *const uf = ring + rf * rstride;
+    if (ke_ring) {
+        const int two = pair_of(1);
+        for (int x = tid >> 5; x < 1 << (ush - two); x += nw)
+            group_sums(ke_slot(rf), ke_stride(rf), x << two, two, sh.part[0][1]);
+    }
     for (int k = tid; k < m; k += blockDim.x) {
         const int id = node[k];
         double *const uo[3] = {S.u0 + n0, S.u1 + n0, S.u2 + n0};
@@ -506,6 +533,7 @@ __device__ void solve_rve_fp64_cluster(cg::cluster_group &cl, Fp64ClusterShared 
     cl.sync();
     if (me == 0) {
         stress_total(R, F, &sh.sig[0][0], O.sigma + 9 * (int64_t)p);
+        if (judge && ke_ring) ke = total(1, 0);
         if (judge && lane == 0) {
             O.iters[p] = i - 2;
             O.rel_res[p] = f_ref > 0.0 ? res / f_ref : (res > 0.0 ? INFINITY : 0.0);
@@ -535,11 +563,13 @@ __device__ __forceinline__ void solve_in(cg::cluster_group &cl, Fp64ClusterShare
                                          const Fp64Shape &sp, double *base) {
     double *XB = base;
     double *ST = XB + 6 * sp.part_max;
-    double *T = ST + state_doubles(SSM) * (size_t)sp.free_max;
+    double *TE = ST + state_doubles(SSM) * (size_t)sp.free_max;
+    double *T = TE + term_doubles(sp.terms) * (size_t)sp.free_max;
     int32_t *RS = reinterpret_cast<int32_t *>(T + (TSM ? 3 * (size_t)sp.slot_max : 0));
     uint16_t *RE = reinterpret_cast<uint16_t *>(RS + (TSM ? sp.free_max + 1 : 0));
     uint16_t *LS = RE + (TSM ? sp.row_max : 0);
-    solve_rve_fp64_cluster<TSM, SSM>(cl, sh, M, S, O, P, p, XB, ST, T, RS, RE, LS, sp.part_max, sp.free_max, sp.slot_max);
+    solve_rve_fp64_cluster<TSM, SSM>(cl, sh, M, S, O, P, p, XB, ST, sp.terms ? TE : nullptr, T, RS, RE, LS, sp.part_max,
+                                     sp.free_max, sp.slot_max);
 }
 }  // namespace
 
@@ -574,7 +604,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
     map_shared(cl, sh);
     cl.sync();
     const RveDesc &R = M.rve[0];
-    Fp64Shape sp = {R.fp_parts, R.fp_part_max, R.fp_free_max, R.fp_slot_max, R.fp_row_max, true, 1};
+    Fp64Shape sp = {R.fp_parts, R.fp_part_max, R.fp_free_max, R.fp_slot_max, R.fp_row_max, true, 1, false};
     if (cluster_bytes(sp) <= bytes) {
         solve_in<true, 1>(cl, sh, M, S, O, P, 0, sp, dsm_fp64);
     } else {
@@ -696,7 +726,7 @@ int fp64_max_cluster(size_t smem) {
 constexpr size_t kSingleBytes = 200 * 1024;
 static size_t single_bytes(int n, int n_elems, int parts) {
     const int m = (n + parts - 1) / parts;
-    const Fp64Shape most = {parts, m, m, n_elems, 2 * n_elems, true, 1};
+    const Fp64Shape most = {parts, m, m, n_elems, 2 * n_elems, true, 1, false};
     return std::min(kSingleBytes, cluster_bytes(most));
 }
 

@@ -69,11 +69,12 @@ struct RveDesc {
 // Launch shape of the FP64 cluster kernel: CTAs per cluster, capacities of one
 // CTA, and what it keeps in shared memory beside the positions (tsm: element
 // table and rows, ssm: the own free nodes' state, 1 with and 2 without their
-// displacements).
+// displacements, terms: the energy terms).
 struct Fp64Shape {
     int parts, part_max, free_max, slot_max, row_max;
     bool tsm;
     int ssm;
+    bool terms;
 };
 // CTAs per cluster of the FP32-phase kernel (dr_mixed_node.cu) and capacities of
 // one CTA: increment entries, free nodes, row slots, copies of own nodes, and the row slots held in
@@ -154,8 +155,9 @@ struct DevState {
     double *u0, *u1, *u2;         // displacement (output of every mode)
     double *v0, *v1, *v2;         // FP64 velocity
     double *a0, *a1, *a2;         // FP64 acceleration; FP64 cluster kernel: kinetic
-                                  // energies, and behind the three arrays the work terms,
-                                  // per RVE [2][3][n] at 6 node0 (batches only)
+                                  // energies, and behind the three arrays those of two
+                                  // more evaluations or the work terms, per RVE
+                                  // [2][3][n] at 6 node0
     float *uh, *ul;               // MIXED: displacement, double-float [3][N]
     float *vh, *vl;               // MIXED: velocity (lead: double-float; FP32 phase: vh)
     float *ah, *al;               // MIXED: acceleration (same convention)

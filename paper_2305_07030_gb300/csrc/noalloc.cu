@@ -73,7 +73,7 @@ constexpr size_t kOffRef = align256(kOffNode + sizeof(int32_t) * kNaMaxNodes);  
 constexpr size_t kOffPartOff = align256(kOffRef + sizeof(int32_t) * kNaMaxNodes);
 constexpr size_t kOffFrow = align256(kOffPartOff + sizeof(int32_t) * 2 * (kMaxParts + 1));
 constexpr size_t kOffKin = align256(kOffFrow + sizeof(int32_t) * (kNaMaxNodes + 1));  // kinetic energies
-constexpr size_t kNoallocScratchBytes = align256(kOffKin + sizeof(double) * 3 * kNaMaxNodes);
+constexpr size_t kNoallocScratchBytes = align256(kOffKin + sizeof(double) * 9 * kNaMaxNodes);
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocScratchBytes];
 

@@ -443,7 +443,7 @@ void build_classes(const std::vector<RveDesc> &rve, const std::vector<int32_t> &
         // the single-CTA kernel.
         const bool clusters = env_int("FE2_FP64_CLUSTER", 1) != 0;
         auto shape_of = [&](const RveDesc &R) {
-            return Fp64Shape{R.fp_parts, R.fp_part_max, R.fp_free_max, R.fp_slot_max, R.fp_row_max, false, 0};
+            return Fp64Shape{R.fp_parts, R.fp_part_max, R.fp_free_max, R.fp_slot_max, R.fp_row_max, false, 0, false};
         };
         auto on_cluster = [&](const RveDesc &R) { return clusters && fp64_cluster_smem(shape_of(R)) <= cap; };
         for (int32_t p : order) {
@@ -1524,16 +1524,51 @@ int resident_of(fe2_batch *b, int kind, int parts, int block, size_t smem, int p
     return r;
 }
 
-// Resident clusters of an FP64 cluster class (cached like resident_of; the
-// key's kind 15 + 3 tsm + ssm and the smem size identify the variant).
-int resident_fp64_cluster(fe2_batch *b, const SizeClass &c, int block) {
-    const auto key = std::make_tuple(15 + 3 * (int)c.fp.tsm + c.fp.ssm, c.parts, block, fp64_cluster_smem(c.fp),
-                                     c.fp.part_max);
+// Resident clusters of an FP64 cluster launch (cached like resident_of; the key's
+// kind and the smem size identify the variant).
+int resident_fp64_cluster(fe2_batch *b, const Fp64Shape &sp, int block) {
+    const auto key = std::make_tuple(15 + 3 * (int)sp.tsm + sp.ssm, sp.parts, block, fp64_cluster_smem(sp),
+                                     sp.part_max);
     auto it = b->occ.find(key);
     if (it != b->occ.end()) return it->second;
-    const int r = occupancy_dr_fp64_cluster(block, c.fp);
+    const int r = occupancy_dr_fp64_cluster(block, sp);
     b->occ[key] = r;
     return r;
+}
+
+// Launch of nq of an FP64 cluster class's RVEs: shape, CTA size, resident clusters.
+// Results do not depend on any of them.
+struct Fp64Launch {
+    Fp64Shape sp;
+    int block, resident;
+};
+Fp64Launch fp64_launch(fe2_batch *b, const SizeClass &c, const fe2_opts &o, int nq) {
+    Fp64Launch l = {c.fp, o.block_threads ? o.block_threads : 512, 0};
+    l.resident = resident_fp64_cluster(b, l.sp, l.block);
+    if (l.block < 512 && l.resident > 0) {
+        // The judging warp comes on top of the requested threads where that costs the
+        // launch no resident cluster. 64 threads, 152 RVEs of 400 nodes: 59 us per
+        // iteration with one working warp, 30 with two (the single-CTA kernel 47); 256
+        // threads, 1000 RVEs of 100 nodes: 24 us with two CTAs per SM, 37 with one.
+        const int more = resident_fp64_cluster(b, l.sp, l.block + 32);
+        if (std::min(nq, more) >= std::min(nq, l.resident)) {
+            l.block += 32;
+            l.resident = more;
+        }
+    }
+    if (o.kinetic_energy) {
+        // energy terms in shared memory where they cost no resident cluster
+        Fp64Shape t = l.sp;
+        t.terms = true;
+        if (fp64_cluster_smem(t) <= b->smem_optin - 16384) {
+            const int with = resident_fp64_cluster(b, t, l.block);
+            if (std::min(nq, with) >= std::min(nq, l.resident)) {
+                l.sp = t;
+                l.resident = with;
+            }
+        }
+    }
+    return l;
 }
 
 // Resident clusters of a mixed class's kernel (cached likewise; kinds 7 to 10:
@@ -1580,11 +1615,6 @@ cudaError_t record_timing(cudaEvent_t e, cudaStream_t s, bool capturing) {
     return capturing ? cudaEventRecordWithFlags(e, s, cudaEventRecordExternal) : cudaEventRecord(e, s);
 }
 
-// CTA size of the FP64 cluster kernel: the requested threads and the judging warp,
-// at most 512. A request for 64 threads would otherwise leave one warp for the
-// work: 152 RVEs of 400 nodes 59 us per iteration, so 30 (the single-CTA kernel 47).
-int fp64_block(const fe2_opts &o) { return o.block_threads ? std::min(512, o.block_threads + 32) : 512; }
-
 // Launch the solver kernels of one class on `s` for `nq` queued RVEs. Timing
 // events (tev) are recorded only when `timed` is non-null.
 fe2_status launch_class(fe2_batch *b, const fe2_opts &o, const SizeClass &c, SolveParams P,
@@ -1599,15 +1629,14 @@ fe2_status launch_class(fe2_batch *b, const fe2_opts &o, const SizeClass &c, Sol
     P.counter = counters;
     P.smem_positions = c.smem_positions;
     if (fp64 && c.fp64_cluster) {
-        const int block = fp64_block(o);
-        const int resident = resident_fp64_cluster(b, c, block);
-        if (resident < 1)
+        const Fp64Launch l = fp64_launch(b, c, o, nq);
+        if (l.resident < 1)
             return fail(FE2_ECUDA, "no FP64 cluster of " + std::to_string(c.parts) + " CTAs fits");
         if (timed) {
             if (*timed + 2 > (int)b->tev.size()) return fail(FE2_ECUDA, "too many launch classes");
             CUDA_TRY(record_timing(b->tev[*timed], s, capturing));
         }
-        const int e = launch_dr_fp64_cluster(M, S, R, P, std::min(nq, resident), block, c.fp, s);
+        const int e = launch_dr_fp64_cluster(M, S, R, P, std::min(nq, l.resident), l.block, l.sp, s);
         if (e != 0) return fail(FE2_ECUDA, std::string("launch: ") + cudaGetErrorString((cudaError_t)e));
         if (timed) {
             CUDA_TRY(record_timing(b->tev[*timed + 1], s, capturing));
@@ -1724,8 +1753,7 @@ fe2_status warm_shapes(fe2_batch *b, const fe2_opts &o) {
     const size_t limit = b->smem_optin - 16384;
     for (const SizeClass &c : fp64 ? b->classes_fp64 : b->classes_mixed) {
         if (fp64 && c.fp64_cluster) {
-            const int block = fp64_block(o);
-            if (resident_fp64_cluster(b, c, block) < 1)
+            if (fp64_launch(b, c, o, (int)c.rves.size()).resident < 1)
                 return fail(FE2_ECUDA, "no FP64 cluster of " + std::to_string(c.parts) + " CTAs fits");
             continue;
         }
