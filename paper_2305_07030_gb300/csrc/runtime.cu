@@ -1549,7 +1549,7 @@ Fp64Launch fp64_launch(fe2_batch *b, const SizeClass &c, const fe2_opts &o, int 
         // The judging warp comes on top of the requested threads where that costs the
         // launch no resident cluster. 64 threads, 152 RVEs of 400 nodes: 59 us per
         // iteration with one working warp, 30 with two (the single-CTA kernel 47); 256
-        // threads, 1000 RVEs of 100 nodes: 24 us with two CTAs per SM, 37 with one.
+        // threads, 1000 RVEs of 100 nodes: 26 us with two CTAs per SM, 37 with one.
         const int more = resident_fp64_cluster(b, l.sp, l.block + 32);
         if (std::min(nq, more) >= std::min(nq, l.resident)) {
             l.block += 32;
